@@ -117,15 +117,11 @@ SSBA_API int ssba_build_mask(const ssba_desc* desc, const void* Q, const void* K
  *   kv_cnt      device, int32 [B][heads][Tb], each in [1, keep].
  *   O           device out, [B][heads][N][head_dim] of desc->dtype, original token order.
  *   lse         device out, fp32 [B][heads][N], natural log.
- *   workspace   device, optional (NULL and 0 allowed): the split-merge area of the
- *               bf16 kernel, at least ssba_forward_workspace_bytes(desc) bytes,
- *               16-byte aligned. With it, and with lists of at least 24 blocks, the
- *               persistent kernel gives its pipelines equal shares of key blocks and
- *               cuts at most one query block per share boundary in two, merging the
- *               parts' partial softmax sums; otherwise shares are whole query blocks
- *               (up to one query block's work of imbalance). The part that finishes
- *               second does the merge, so the rows of a cut query block may differ in
- *               their last bit from one call to the next (within the usual rounding).
+ *   workspace   device, optional (NULL and 0 allowed), at least
+ *               ssba_forward_workspace_bytes(desc) bytes, 16-byte aligned. Only
+ *               ssba_forward_fused uses it (its grid barrier); here it is checked and left
+ *               alone, and the result is the same with and without it, bit for bit and from
+ *               one call to the next.
  *               Rules: zero-fill it once before its first use. Every call that
  *               returns SSBA_OK and runs to completion leaves it zero-filled again,
  *               so later calls ordered after it on the GPU reuse it as is. Calls that

@@ -435,8 +435,8 @@ def build_mask_noalloc(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, kv_idx=
 
 def forward(desc: SsbaDesc, Q, K, V, kv_idx, kv_cnt, O=None, lse=None, workspace="default", stream=None):
     """ssba_forward: returns (O [B,h,N,d] in desc.dtype, lse [B,h,N] fp32).
-    ``workspace``: "default" (the per-stream one of default_forward_workspace), None (no
-    workspace: whole-query-block shares) or a zero-filled uint8 CUDA tensor."""
+    ``workspace``: "default" (the per-stream one of default_forward_workspace), None or a
+    zero-filled uint8 CUDA tensor; the result is the same with each."""
     lib = load_library()
     d = desc.c()
     keep = lib.ssba_keep_count(ctypes.byref(d))

@@ -3,40 +3,44 @@
 // and its MMAs; Algorithm 1 SparseAttention over image tokens).
 //
 // Work item = one query block (64 tokens, an 8x8 window of the shifted grid) of one
-// (batch, head); it visits only the key blocks listed for it. Persistent CTAs, one per SM
-// (its 205 KB of shared memory fills the SM), each running two independent
-// pipelines of 12 warps (768 threads), warp-specialised by warpgroup:
-//   warp 0      TMA producer (Q, K). Q of each item and K, V of each listed key block arrive as
-//               8 KB tiles cut from [B*heads, H, W, d] tensor maps (128-byte swizzle): one
-//               8x8-token box when the shifted window does not cross the grid edge, else two
-//               or four boxes. A half-block shift is a multiple of 4 tokens, so a crossing
-//               window splits 4 + 4: no gather pass and no out-of-range fill. Q is
-//               double-buffered; K and V have separate 5-stage rings (a K slot frees when
-//               its QK is done, a V slot when its PV is done).
-//   warp 1      QK issuer (one elected lane; warp 1 of the CTA also owns the TMEM allocation):
-//                 S_t = Q K_t^T   tcgen05.mma kind::f16, M=64 N=64, A = Q tile and
-//                                 B = K tile from shared memory (K-major, SW128)
-//               S is triple-buffered in TMEM: QK of block t waits only until PV_{t-3} has
-//               read P_{t-3} from the same buffer.
-//   warp 2      TMA producer of the V ring (warp 0 keeps Q and K), so that two threads
-//               share the per-box issue latency.
-//   warp 3      PV issuer (one elected lane):
-//                 O  += P_t V_t   tcgen05.mma kind::f16, M=64 N=64, A = P from TMEM,
-//                                 B = V tile (MN-major, SW128)
-//               P_t (bf16 pairs, 32 columns) goes into the first half of S_t's buffer, which
-//               the softmax no longer needs once S_t is in its registers, so the softmax never
-//               waits for a P buffer and QK runs up to three blocks ahead. TMEM of a
-//               pipeline: S/P 3 x 64 + O 64 = 256 columns. Two issuing threads keep one's
-//               barrier waits (about 100 cycles per query) off the other's issue path.
-//   warps 4-7   softmax, one TMEM lane quadrant each. The M=64 data path puts tile row r
-//               at lane 32*(r/16) + r%16, so two threads share a row (16x32bx2 TMEM
-//               loads), each holding 32 of its 64 scores. Online softmax in fp32 with exp2
-//               in the log2-scaled domain; the running max is only raised when it grows by
-//               more than 2^8, which keeps P <= 256 in bf16; O is then rescaled in TMEM
-//               after P_t is stored, so that S and O never share the registers (80 per
-//               thread: 768 threads on one SM). At the end of an item the row statistics
-//               (max, sum) go to shared memory.
-//   warps 8-11  epilogue: O / l in bf16 and lse, overlapping the next item's softmax.
+// (batch, head); it visits only the key blocks listed for it. Two items are worked on at a
+// time, as the two halves (rows 0-63 and 64-127) of M=128 products: half A is one item, half B
+// another one, each with its own key blocks. Step t takes the t-th listed block of both:
+//   S = [Q_A; Q_B] [K_A,t; K_B,t]^T   M=128 N=128 K=16 x 4: rows 0-63 need columns 0-63 of it,
+//                                     rows 64-127 columns 64-127; the rest is never read
+//   O_A += P_A V_A,t, O_B += P_B V_B,t   M=128 N=64 K=16, 4 + 4 products on the same O columns,
+//                                     each with the other half's lanes masked off, so that
+//                                     nothing of one item (an infinity, a NaN) reaches the other
+// The products of a step cost what two M=64 products of each kind would, but the pair has one
+// hand-off where two tiles had two, and a softmax thread owns a whole row of 64 scores. An item
+// left over at the end of a pipeline's work takes both halves: the first half of its list in A,
+// the second in B, merged at the end (two partial softmax sums).
+// What bounds it: a step of each of the CTA's two pipelines takes about 1550 cycles, of which the
+// tensor pipe is busy 2 x 608 (QK 4 x 80, PV 8 x 36) and the softmax needs 2 x 435 of its scheduler;
+// the rest is hand-offs (mbarrier waits, tensor-memory round trips) that two chains do not quite
+// cover. Forward on given lists, 24 heads, GPU time against the kernel with one 64-row tile per
+// product: 4K (128 of 510 blocks) 2396 -> 1783 us, 2048 px (41 of 256) 400 -> 316, four 1024 px
+// images (16 of 64) 171 -> 150, one (11 of 64) 38.9 -> 36.6, 512 px (3 of 16) 10.6 -> 10.9.
+// Persistent CTAs, one per SM (its 226 KB of shared memory fills the SM), each running two
+// independent pipelines of 8 warps (512 threads, 128 registers each), warp-specialised:
+//   K producer  (TMA, one lane). Q of each item and K, V of each listed key block arrive as 8 KB tiles
+//               cut from [B*heads, H, W, d] tensor maps (128-byte swizzle): one 8x8-token box when the
+//               shifted window does not cross the grid edge, else two or four boxes. A half-block
+//               shift is a multiple of 4 tokens, so a crossing window splits 4 + 4: no gather pass
+//               and no out-of-range fill. K and V have rings of three 16 KB stages each, Q one (the
+//               next round's Q arrives while the softmax works on the last scores of this one).
+//   QK issuer   QK of step t + 1 goes out as soon as the softmax holds S_t in registers and PV of
+//               step t - 1 is done.
+//   V producer  as the K producer, for the V ring.
+//   PV issuer   PV of step t once P_t is stored and V_t has landed.
+//   softmax     four warps, one TMEM lane quadrant each (two for half A, two for half B), one thread
+//               per row. Online softmax in fp32 with exp2 in the log2-scaled domain against a
+//               reference max m: the first step's row maximum. Later steps form P against it at once
+//               and look at their row sum afterwards; only where that exceeds 2^24 (or is no number)
+//               is the step's maximum taken, m raised, O rescaled in TMEM and P formed again. They
+//               also write the finished items: O / l in bf16 and lse, after the exps of the next
+//               item's first step, so that the wait for the item's last PV is spent on them.
+// TMEM of a pipeline: S 128 + P 2 x 32 (bf16 pairs) + O 64 = 256 columns.
 // In-kernel selection (ssba_forward_select): given the block means, each CTA first computes
 // the score rows and the Top-k gating of its own items (one warp per item, the arithmetic of
 // the mask kernels) and writes the lists to the caller's kv_idx / kv_cnt, which its producers
@@ -45,6 +49,7 @@
 // bounded (globaltimer budget + CTA abort flag); a timeout is reported in the device status
 // word and the CTA drains its in-flight copies and MMAs before it exits.
 #include <cuda.h>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 
@@ -61,53 +66,56 @@ using namespace ptx;
 using namespace win;
 
 constexpr int kD = 64;
-constexpr int kRows = 64;  // query rows per item = tokens per block
-constexpr int kKStages = 5;  // K ring
-constexpr int kVStages = 5;  // V ring
-constexpr int kSBuf = 3;     // S buffers in TMEM (fp32, 64 columns each); P_t (bf16 pairs) goes
-                             // into the first 32 columns of S_t's buffer
-constexpr int kSlotWarps = 12;                // warps of one pipeline (see the role map above)
+constexpr int kRows = 64;    // query rows per item = tokens per block
+constexpr int kStages = 3;   // K ring, V ring
 constexpr int kSlots = 2;                     // independent pipelines per CTA
-constexpr int kThreads = kSlots * kSlotWarps * 32;
+constexpr int kSoftWarps = 4;                 // softmax warps of one pipeline
+constexpr int kRoleWarps = 4;                 // K producer, QK issuer, V producer, PV issuer of one pipeline
+constexpr int kThreads = kSlots * (kSoftWarps + kRoleWarps) * 32;
+enum Role { kLoadK = 0, kQK = 1, kLoadV = 2, kPV = 3, kSoftmax = 4 };
 constexpr uint32_t kSlotCols = 256;           // TMEM columns of one pipeline
 constexpr uint32_t kTmemCols = kSlots * kSlotCols;
-constexpr uint32_t kColS = 0;    // S / P buffers: [0,64), [64,128), [128,192)
+constexpr uint32_t kColS = 0;    // S: [0,128)
+constexpr uint32_t kColP = 128;  // P buffers: [128,160), [160,192)
 constexpr uint32_t kColO = 192;  // O accumulator: [192,256)
-constexpr uint32_t kTileBytes = kRows * kD * 2;  // 8 KB
-constexpr float kRescaleLog2 = 8.0f;
-constexpr int kLabelCap = 128;  // labels staged per producer warp and piece; the rest are read per block
-constexpr int kCntCap = 64;     // phase-B item counts of a pipeline held in shared memory
-constexpr int kCntA = 3;        // phase-A pieces of one pipeline: at most three
-constexpr int kSplitMinKeep = 24;  // shortest list for which items are cut to balance the pipelines
+constexpr uint32_t kTileBytes = kRows * kD * 2;    // 8 KB: one block of one tensor
+constexpr uint32_t kPairBytes = 2 * kTileBytes;    // both halves
+// A step's row sum of exp2(s c - m) above which the row's reference max m is raised. Any value would
+// give the same precision (P, O and l are floating-point numbers, of any common scale); this one
+// leaves O 2^100 of head room over V, and a later step has to exceed the first one's maximum by
+// 2^18 to reach it.
+constexpr float kRaise = 16777216.f;  // 2^24
+constexpr int kCntCap = 40;  // item counts of a pipeline held in shared memory (20 rounds)
 
-// QK: M=64 N=64, A (Q) and B (K) K-major. PV: M=64 N=64, A (P) K-major, B (V) MN-major.
-constexpr uint32_t kIdescQK = idesc_bf16_f32(64, 64, false, false);
-constexpr uint32_t kIdescPV = idesc_bf16_f32(64, 64, false, true);
+// QK: M=128, A (Q) and B (K) K-major; N=64 in a step that only one half takes part in. PV: M=128
+// N=64, A (P) K-major, B (V) MN-major.
+constexpr uint32_t kIdescQK = idesc_bf16_f32(128, 128, false, false);
+constexpr uint32_t kIdescQK1 = idesc_bf16_f32(128, 64, false, false);
+constexpr uint32_t kIdescPV = idesc_bf16_f32(128, 64, false, true);
 
 struct __align__(1024) SlotSmem {
-    uint8_t k[kKStages][kTileBytes];
-    uint8_t v[kVStages][kTileBytes];
-    uint8_t q[2][kTileBytes];
-    float2 stats[2][kRows];  // (max in log2 units, row sum) per item parity
-    uint64_t k_full[kKStages];
-    uint64_t k_empty[kKStages];
-    uint64_t v_full[kVStages];
-    uint64_t v_empty[kVStages];
-    uint64_t q_full[2];
-    uint64_t q_empty[2];
-    uint64_t s_full[kSBuf];
-    uint64_t s_free[kSBuf];   // PV_t has finished (it read P_t from S_t's buffer): QK_{t+3} may
-                              // overwrite the buffer
-    uint64_t p_full[kSBuf];
-    uint64_t stats_full[2];
-    uint64_t stats_free[2];
-    uint64_t o_full;
-    uint64_t o_free;
+    uint8_t k[kStages][kPairBytes];
+    uint8_t v[kStages][kPairBytes];
+    uint8_t q[kPairBytes];
+};
+
+// Barriers and schedule of one pipeline.
+struct SlotCtl {
+    uint64_t k_full[kStages];
+    uint64_t k_empty[kStages];
+    uint64_t v_full[kStages];
+    uint64_t v_empty[kStages];
+    uint64_t q_full;
+    uint64_t q_empty;
+    uint64_t s_full;      // QK_g has finished
+    uint64_t s_free;      // the four softmax warps hold S_g in registers
+    uint64_t p_full[2];   // the four softmax warps have stored P_g (and read the last item's O); two, as
+                          // they may store P_{g+1} before the issuer, waiting for V_g, sees P_g
+    uint64_t o_full[2];   // PV_g has finished
+    uint64_t merged;      // half B's part of a split item is in shared memory
     uint64_t drain[2];
-    int32_t labels[2][kLabelCap];     // [producer warp] key-block labels of the current piece
-    int32_t cnts[kCntCap];            // counts of the first phase-B items, in walk order
-    int4 pieceA[kCntA];               // phase-A pieces in walk order: item, tb, nb, part
-    int nA, nB, M;                    // phase-A pieces, phase-B items, phase-A items (all pipelines)
+    int32_t cnts[kCntCap];  // counts of the first items, in walk order
+    int first, stride, last, rounds, single;  // see build_schedule
 };
 
 constexpr int kWinCap = 256;  // labels whose window (origin, box shape) is tabulated per CTA (2048 px: 256)
@@ -166,10 +174,13 @@ __device__ __forceinline__ int pipe_of(int slot)
 #define TL_ITEM(slot, n, ev) do { } while (0)
 #endif
 
+constexpr int kPoolUnits = 2 * (2 * kStages + 1);  // 8 KB pooling buffers of one pipeline's stages
+
 struct __align__(1024) SmemLayout {
     SlotSmem slot[kSlots];
+    SlotCtl ctl[kSlots];
     uint32_t win[kWinCap];  // label -> r0 | c0 << 15 | box shape << 30 (see window_entry)
-    uint64_t pool_bar[kThreads / 32];  // one per warp: its block's rows landed (in-kernel pooling)
+    uint64_t pool_bar[kSlots * kPoolUnits];  // one per buffer: its block's rows landed (in-kernel pooling)
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -177,6 +188,7 @@ struct __align__(1024) SmemLayout {
 // Four maps per tensor, one per box shape, over the [B*heads][H][W][d] bf16 view, and
 // the text keys and values as [B*heads][T_txt][d] (64-row boxes, zero fill past T_txt).
 static_assert(sizeof(SmemLayout) + 1024 <= 232448, "shared memory of one CTA (227 KB opt-in limit)");
+static_assert(sizeof(SlotSmem) == kPoolUnits * kTileBytes, "stages back to back");
 
 struct TileMaps {
     CUtensorMap q[4], k[4], v[4];
@@ -196,17 +208,12 @@ struct TcParams {
     int num_items;
     float scale_log2;  // softmax scale * log2(e)
     int* status;       // device status word
-    // Split-merge workspace (null when the caller gave none; then split = 0).
-    int split;         // 1: pipelines take equal ranges of blocks, items may be cut in two
-    int* ws_cnt;       // [boundaries][4] arrival counters, zero between launches
-    float2* ws_st;     // [boundaries][2][64] row (max in log2 units, sum) of each part
-    float* ws_o;       // [boundaries][2][64][64] unnormalised O of each part, fp32
     const float* sel_qb;  // in-kernel selection: block means [B*heads][Tb][64] (null: lists given)
     const float* sel_kb;
     int32_t* sel_cnt;     // counts written by the selection
     float* sel_scores;    // optional S export [B*heads][Tb][Tb]
-    // in-kernel pooling (ssba_forward_fused): every warp of the grid pools one (block, tensor)
-    // unit into sel_qb / sel_kb, then the CTAs meet at a grid barrier (null: means given)
+    // in-kernel pooling (ssba_forward_fused): the warps of the grid pool the (block, tensor)
+    // units into sel_qb / sel_kb, then the CTAs meet at a grid barrier (null: means given)
     const __nv_bfloat16* pool_q;
     const __nv_bfloat16* pool_k;
     unsigned* gsync;  // grid barrier words in the workspace (arrivals, departures)
@@ -216,27 +223,14 @@ struct TcParams {
                          // arrive at the grid barrier of the fused launch (0 otherwise)
 };
 
-// Work schedule, for V pipelines (two per CTA).
-//   split = 0: whole items round-robin, item v + r V for pipeline v (neighbouring pipelines
-//     work on neighbouring items, so the K/V tiles of a few heads are shared through L2).
-//   split = 1 (a workspace was given and items is not a multiple of V, items >= V): the
-//     first M = items - (floor(items / V) - 1) V items (V <= M < 2V) form phase A, the rest
-//     phase B. Phase A counts in units (item, key block), item u / keep, block u % keep (a
-//     block past the item's count is an empty unit); pipeline v takes the units
-//     [floor(M keep v / V), floor(M keep (v+1) / V)), at least keep of them, so an item is
-//     cut at most once: at boundary v, into a first part (the last item of pipeline v-1)
-//     and a second part (the first item of pipeline v). Each part writes its unnormalised
-//     O and row statistics to the workspace, and the part that arrives second at the
-//     boundary's counter merges the two (two partial softmax sums combine by rescaling
-//     each by 2^(m_part - m), m the larger maximum, and adding) and resets the counter.
-//     Phase B is whole items round-robin, item M + v + r V. Every pipeline then has the
-//     same number of key blocks, give or take one.
-// A pipeline runs phase A first and, in it, its cut last item first, so that both parts
-// of every cut item finish early and the merges (a few global-memory round trips)
-// overlap later work instead of lengthening the end of the kernel.
-// Under in-kernel selection the items go to the pipelines in contiguous ranges (item counts
-// differing by at most one), so that the few items of a CTA share one or two heads and the
-// selection stages each head's k_b once.
+// Work schedule, for V pipelines (two per CTA): each takes its items two at a time (a round), a
+// single one left over alone, split over the two halves.
+//   Lists given: neighbouring items form a pair, pairs go round-robin (neighbouring pipelines work
+//     on neighbouring items, so the K/V tiles of a few heads are shared through L2); of the items
+//     left after the whole rounds each pipeline takes one, or the first ones a pair.
+//   In-kernel selection: contiguous ranges (item counts differing by at most one), so that the
+//     few items of a CTA share one or two heads and the selection stages each head's k_b once.
+// Pipeline `slot` of CTA b is number b + slot * CTAs: the longer shares go to different CTAs.
 __device__ __forceinline__ int sel_item_count(const TcParams& p, int v, int V)
 {
     return p.num_items / V + (v < p.num_items % V ? 1 : 0);
@@ -246,16 +240,11 @@ __device__ __forceinline__ int sel_first_item(const TcParams& p, int v, int V)
     return v * (p.num_items / V) + min(v, p.num_items % V);
 }
 
-__device__ __forceinline__ int split_items(const TcParams& p, int V)
-{
-    return p.split ? p.num_items - (p.num_items / V - 1) * V : 0;
-}
-
-struct Piece {
-    int item;  // (batch, head) * Tb + query-block label
-    int tb;    // first block (position in the item's list)
-    int nb;    // blocks of this piece (0 for an empty piece)
-    int part;  // -1 whole item, 0 first part (boundary v + 1), 1 second part (boundary v)
+// One round: per half the item, the first block (position in the item's blocks, text first) and
+// the number of blocks.
+struct Round {
+    int item[2], tb[2], nb[2];
+    bool split;  // both halves work on the same item
 };
 
 __device__ __forceinline__ float fast_exp2(float x)
@@ -279,15 +268,36 @@ __device__ __forceinline__ bool wait_raw(uint32_t bar, uint32_t parity, uint64_t
     return true;
 }
 
-// 16x32bx2 store of 16 fp32 columns, threads 16-31 at +32 columns (counterpart of
-// tmem_ld_16x32bx2_x16_off32), used for the O rescale.
-__device__ __forceinline__ void tmem_st_16x32bx2_x16_off32(uint32_t taddr, const uint32_t (&r)[16])
+// Wait of the MMA issuers and the softmax warps for phase `parity`: nothing but the try_wait when the
+// phase is complete (48 cycles measured, against 93 for a wait that returns a verdict to branch on).
+// Bounded like mbar_wait; it returns in any case, and once the CTA's abort flag (at shared address
+// abort_at) is raised it returns after one more try. The roles that use it then run through the
+// rest of their round: their products, loads and stores stay in the CTA's own tensor and shared
+// memory and in the rows of its own items, and every arrive count stays the same. (The producers stop at
+// once: an announced copy that is never issued may not be announced again.)
+__device__ __forceinline__ void wait_phase(uint32_t bar, uint32_t parity, uint32_t abort_at, uint64_t budget_ns)
 {
     asm volatile(
-        "tcgen05.st.sync.aligned.16x32bx2.x16.b32 [%0], 32, "
-        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        "{\n"
+        ".reg .pred P;\n"
+        ".reg .u64 t0, t1;\n"
+        ".reg .u32 a;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 P, [%0], %1;\n"
+        "@P bra DONE;\n"
+        "mov.u64 t0, %%globaltimer;\n"
+        "AGAIN:\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 P, [%0], %1;\n"
+        "@P bra DONE;\n"
+        "ld.volatile.shared.u32 a, [%2];\n"
+        "setp.ne.u32 P, a, 0;\n"
+        "@P bra DONE;\n"
+        "mov.u64 t1, %%globaltimer;\n"
+        "sub.u64 t1, t1, t0;\n"
+        "setp.le.u64 P, t1, %3;\n"
+        "@P bra AGAIN;\n"
+        "st.volatile.shared.u32 [%2], 1;\n"
+        "DONE:\n"
+        "}\n" ::"r"(bar), "r"(parity), "r"(abort_at), "l"(budget_ns)
         : "memory");
 }
 
@@ -303,80 +313,92 @@ constexpr bool kChecked = true;
 constexpr bool kChecked = false;
 #endif
 
-// Block means of the whole layer inside the launch: unit u is (tensor u & 1, item u >> 1), one
-// unit per warp and round, assigned warp-major over the grid so that the CTAs get equal
-// shares. Lanes 0..7 bulk-copy the unit's eight token rows (one copy per row, two where the
-// shifted window wraps the right edge) into this warp's 8 KB of the idle stage buffers, and
-// after the copies land every lane sums its (row group, column chunk) with the loop order of
-// ssba_pool_blocks_kernel, so the means are those of ssba_pool_blocks bit for bit. Returns
-// false if a copy did not land in time (after a second bounded wait for it).
+// Block means of the whole layer inside the launch: unit u is (tensor u & 1, item u >> 1); the
+// CTA takes the units u = i gridDim + blockIdx, i < kSlots * kPoolUnits at a time, one 8 KB piece
+// of the idle stage buffers each, warp w units w and w + 16 of them (all copies of a batch in
+// flight together). Lanes 0..7 bulk-copy the unit's eight token rows (one copy per row, two where
+// the shifted window wraps the right edge), and after the copies land every lane sums its (row
+// group, column chunk) with the loop order of ssba_pool_blocks_kernel, so the means are those of
+// ssba_pool_blocks bit for bit. Returns false if a copy did not land in time (after a second
+// bounded wait for it).
 __device__ __noinline__ bool pool_phase(const TcParams& p, SmemLayout& cs, int gwarp, int lane, volatile int* abortf)
 {
     constexpr int VE = 8, CPR = kD / VE, RPI = 32 / CPR, LOADS = 64 / RPI;
-    constexpr int kWarps = kThreads / 32, kPerSlot = kWarps / kSlots;
-    static_assert(kPerSlot * kTileBytes <= (kKStages + kVStages + 2) * kTileBytes, "pool buffers");
+    constexpr int kWarps = kThreads / 32, kUnits = kSlots * kPoolUnits;
     const Grid& g = p.g;
     const int Tb = g.Tb(), N = g.H * g.W;
     const int col = lane % CPR, r0 = lane / CPR;
-    const uint8_t* buf = &cs.slot[gwarp / kPerSlot].k[0][0] + (gwarp % kPerSlot) * kTileBytes;
-    const uint32_t bar = smem_u32(&cs.pool_bar[gwarp]);
-    const int nw = gridDim.x * kWarps;
+    const int total = 2 * p.num_items;
     int round = 0;
-    for (int u = gwarp * gridDim.x + blockIdx.x; u < 2 * p.num_items; u += nw, ++round) {
-        const int which = u & 1, item = u >> 1;
-        const int bh = item / Tb, label = item - bh * Tb;
-        const int br = label / g.bw, bc = label - br * g.bw;
-        const int rb = br * 8 - g.sr, cb = bc * 8 - g.sc;
-        if (round > 0) {
+    for (int base = 0; base * (int)gridDim.x + (int)blockIdx.x < total; base += kUnits, ++round) {
+        for (int q = gwarp; q < kUnits; q += kWarps) {
+            const int u = (base + q) * gridDim.x + blockIdx.x;
+            if (u >= total) break;
+            const uint32_t bar = smem_u32(&cs.pool_bar[q]);
+            const uint32_t buf = smem_u32(&cs.slot[q / kPoolUnits].k[0][0]) + (q % kPoolUnits) * kTileBytes;
+            const int which = u & 1, item = u >> 1;
+            const int bh = item / Tb, label = item - bh * Tb;
+            const int br = label / g.bw, bc = label - br * g.bw;
+            const int rb = br * 8 - g.sr, cb = bc * 8 - g.sc;
+            if (round > 0) {
+                __syncwarp();
+                fence_proxy_async_smem();  // the last round's reads before the copies overwrite them
+            }
+            if (lane == 0) mbar_arrive_expect_tx(bar, kTileBytes);
             __syncwarp();
-            fence_proxy_async_smem();  // the last round's reads before the copies overwrite them
-        }
-        if (lane == 0) mbar_arrive_expect_tx(bar, kTileBytes);
-        __syncwarp();
-        if (lane < 8) {
-            const __nv_bfloat16* X = (which ? p.pool_k : p.pool_q) + (size_t)bh * N * kD;
-            int r = rb + lane;
-            r += r < 0 ? g.H : 0;
-            const uint32_t dst = smem_u32(buf) + lane * 8 * kD * 2;
-            // columns cb .. cb + 7 with -W < cb <= W - 8, each negative one taken + W
-            if (cb >= 0 || cb <= -8) {  // one run of 8 columns
-                bulk_load(dst, X + (size_t)(r * g.W + (cb < 0 ? cb + g.W : cb)) * kD, 8 * kD * 2, bar);
-            } else {  // columns W + cb .. W - 1, then 0 .. 7 + cb
-                const int n1 = -cb;  // 1 .. 7
-                bulk_load(dst, X + (size_t)(r * g.W + g.W + cb) * kD, n1 * kD * 2, bar);
-                bulk_load(dst + n1 * kD * 2, X + (size_t)r * g.W * kD, (8 - n1) * kD * 2, bar);
+            if (lane < 8) {
+                const __nv_bfloat16* X = (which ? p.pool_k : p.pool_q) + (size_t)bh * N * kD;
+                int r = rb + lane;
+                r += r < 0 ? g.H : 0;
+                const uint32_t dst = buf + lane * 8 * kD * 2;
+                // columns cb .. cb + 7 with -W < cb <= W - 8, each negative one taken + W
+                if (cb >= 0 || cb <= -8) {  // one run of 8 columns
+                    bulk_load(dst, X + (size_t)(r * g.W + (cb < 0 ? cb + g.W : cb)) * kD, 8 * kD * 2, bar);
+                } else {  // columns W + cb .. W - 1, then 0 .. 7 + cb
+                    const int n1 = -cb;  // 1 .. 7
+                    bulk_load(dst, X + (size_t)(r * g.W + g.W + cb) * kD, n1 * kD * 2, bar);
+                    bulk_load(dst + n1 * kD * 2, X + (size_t)r * g.W * kD, (8 - n1) * kD * 2, bar);
+                }
             }
         }
-        if (!mbar_wait(bar, round & 1, abortf, p.budget_ns)) {
-            volatile int never = 0;  // wait once more, for the copies only, before giving up
-            mbar_wait(bar, round & 1, &never, p.budget_ns);
-            return false;
-        }
-        if (gwarp == 0 && lane == 0 && round == 0) TL_CTA(tl::kPoolLanded);
-        float acc[VE];
-#pragma unroll
-        for (int e = 0; e < VE; ++e) acc[e] = 0.f;
-#pragma unroll
-        for (int i = 0; i < LOADS; ++i) {
-            const int pos = r0 + i * RPI;
-            const uint4 v = *reinterpret_cast<const uint4*>(buf + (pos * kD + col * VE) * 2);
-            const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float2 f = __bfloat1622float2(h2[e]);
-                acc[2 * e] += f.x;
-                acc[2 * e + 1] += f.y;
+        for (int q = gwarp; q < kUnits; q += kWarps) {
+            const int u = (base + q) * gridDim.x + blockIdx.x;
+            if (u >= total) break;
+            const uint32_t bar = smem_u32(&cs.pool_bar[q]);
+            const uint8_t* buf = &cs.slot[q / kPoolUnits].k[0][0] + (q % kPoolUnits) * kTileBytes;
+            const int which = u & 1, item = u >> 1;
+            if (!mbar_wait(bar, round & 1, abortf, p.budget_ns)) {
+                volatile int never = 0;  // wait once more, for the copies only, before giving up
+                for (int x = gwarp; x < kUnits && (base + x) * (int)gridDim.x + (int)blockIdx.x < total; x += kWarps)
+                    mbar_wait(smem_u32(&cs.pool_bar[x]), round & 1, &never, p.budget_ns);
+                return false;
             }
-        }
+            if (gwarp == 0 && lane == 0 && round == 0 && q == 0) TL_CTA(tl::kPoolLanded);
+            float acc[VE];
 #pragma unroll
-        for (int o = CPR; o < 32; o <<= 1)
+            for (int e = 0; e < VE; ++e) acc[e] = 0.f;
 #pragma unroll
-            for (int e = 0; e < VE; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
-        if (r0 == 0) {
-            float* dst = const_cast<float*>(which ? p.sel_kb : p.sel_qb) + ((size_t)bh * Tb + label) * kD + col * VE;
-            constexpr float kInv = 1.0f / 64.0f;
-            reinterpret_cast<float4*>(dst)[0] = make_float4(acc[0] * kInv, acc[1] * kInv, acc[2] * kInv, acc[3] * kInv);
-            reinterpret_cast<float4*>(dst)[1] = make_float4(acc[4] * kInv, acc[5] * kInv, acc[6] * kInv, acc[7] * kInv);
+            for (int i = 0; i < LOADS; ++i) {
+                const int pos = r0 + i * RPI;
+                const uint4 v = *reinterpret_cast<const uint4*>(buf + (pos * kD + col * VE) * 2);
+                const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 f = __bfloat1622float2(h2[e]);
+                    acc[2 * e] += f.x;
+                    acc[2 * e + 1] += f.y;
+                }
+            }
+#pragma unroll
+            for (int o = CPR; o < 32; o <<= 1)
+#pragma unroll
+                for (int e = 0; e < VE; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+            if (r0 == 0) {
+                float* dst = const_cast<float*>(which ? p.sel_kb : p.sel_qb) + (size_t)item * kD + col * VE;
+                constexpr float kInv = 1.0f / 64.0f;
+                reinterpret_cast<float4*>(dst)[0] = make_float4(acc[0] * kInv, acc[1] * kInv, acc[2] * kInv, acc[3] * kInv);
+                reinterpret_cast<float4*>(dst)[1] = make_float4(acc[4] * kInv, acc[5] * kInv, acc[6] * kInv, acc[7] * kInv);
+            }
         }
     }
     return true;
@@ -401,13 +423,16 @@ __device__ bool grid_barrier_arrive_wait(unsigned* w, unsigned n, volatile int* 
     }
 }
 
-// After the whole CTA is done (every CTA of the grid has passed the barrier by then): w[1]
-// counts departures, and the last CTA to leave sets both words back to zero, so a call that
-// completes leaves the workspace zero-filled. (A CTA that gave up at the barrier does not
-// depart; the workspace is then zeroed again by the caller, as after any timeout.)
-__device__ void grid_barrier_depart(unsigned* w, unsigned n)
+// After a CTA has passed the barrier: w[1] counts departures, and the last CTA to pass sets both words
+// back to zero (nobody polls them any more), so a call that completes leaves the workspace
+// zero-filled. The count is taken at once and its answer looked at later (grid_barrier_reset): the
+// round trip of the atomic is off the launch's critical path, where at the end of the kernel it
+// added about a microsecond. (A CTA that gave up at the barrier does not depart; the workspace is
+// then zeroed again by the caller, as after any timeout.)
+__device__ __forceinline__ unsigned grid_barrier_depart(unsigned* w) { return atomicAdd(&w[1], 1u); }
+__device__ __forceinline__ void grid_barrier_reset(unsigned* w, unsigned n, unsigned departed)
 {
-    if (atomicAdd(&w[1], 1u) == n - 1) {
+    if (departed == n - 1) {
         atomicExch(&w[0], 0u);
         atomicExch(&w[1], 0u);
     }
@@ -463,117 +488,202 @@ __device__ __noinline__ void select_item(const TcParams& p, int item, int lane, 
     __syncwarp();
 }
 
-// Piece k of pipeline v (V pipelines) from the schedule in shared memory.
-__device__ __forceinline__ Piece get_piece(const TcParams& p, const SlotSmem& sm, int k, int v, int V)
+// Round r of a pipeline from its schedule in shared memory.
+__device__ __forceinline__ Round get_round(const TcParams& p, const SlotCtl& c, int r)
 {
-    Piece pc;
-    if (k < sm.nA) {
-        const int4 e = sm.pieceA[k];
-        pc.item = e.x;
-        pc.tb = e.y;
-        pc.nb = e.z;
-        pc.part = e.w;
-    } else {
-        const int r = k - sm.nA;
-        pc.item = p.sel_qb ? sel_first_item(p, v, V) + r : sm.M + v + r * V;
-        pc.tb = 0;
-        pc.part = -1;
-        pc.nb = p.units;
+    Round rd;
+    const bool end = r == c.rounds - 1;
+    rd.split = end && c.single;
+    rd.item[0] = end ? c.last : c.first + r * c.stride;
+    rd.item[1] = rd.item[0] + (rd.split ? 0 : 1);
+    rd.tb[0] = rd.tb[1] = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        int n = p.units;
         if (p.idx && !p.sel_qb)
-            pc.nb = p.ntxt + min(max(r < kCntCap ? sm.cnts[r] : __ldg(p.cnt + pc.item), 0), p.keep);
+            n = p.ntxt + (2 * r + h < kCntCap ? c.cnts[2 * r + h] : min(max(__ldg(p.cnt + rd.item[h]), 0), p.keep));
+        rd.nb[h] = n;
     }
-    return pc;
+    if (rd.split) {
+        rd.tb[1] = (rd.nb[0] + 1) >> 1;
+        rd.nb[1] = rd.nb[0] - rd.tb[1];
+        rd.nb[0] = rd.tb[1];
+    }
+    return rd;
 }
 
 // Fills the schedule of pipeline v (thread t of its nthr threads); see the work-schedule
-// comment above.
-__device__ void build_schedule(const TcParams& p, SlotSmem& sm, int v, int V, int t, int nthr)
+// comment above. Rounds r < rounds - 1 are the pairs of items first + r stride, + 1; the last one
+// is the pair (or, single set, the one item) at `last`.
+__device__ void build_schedule(const TcParams& p, SlotCtl& c, int v, int V, int t, int nthr)
 {
-    const int M = split_items(p, V);
-    const int rest = p.num_items - M - v;
-    const int nB = p.sel_qb ? sel_item_count(p, v, V) : (rest > 0 ? (rest + V - 1) / V : 0);
-    if (p.idx && !p.sel_qb)
-        for (int r = t; r < nB && r < kCntCap; r += nthr) sm.cnts[r] = __ldg(p.cnt + M + v + r * V);
-    if (t != 0) return;
-    int nA = 0;
-    if (M > 0) {
-        const int U = p.units;
-        const long long u0 = (long long)M * U * v / V, u1 = (long long)M * U * (v + 1) / V;
-        const long long cut = u1 / U * U;  // start of the item holding unit u1 - 1
-        auto add = [&](long long a, long long b) {   // piece over units [a, b) of one item
-            const int item = (int)(a / U);
-            const int tb = (int)(a - (long long)item * U), te = (int)(b - (long long)item * U);
-            const int n = p.ntxt + (p.idx ? min(max(__ldg(p.cnt + item), 0), p.keep) : p.keep);
-            sm.pieceA[nA++] = make_int4(item, tb, max(0, min(te, n) - tb), tb > 0 ? 1 : (te < U ? 0 : -1));
-        };
-        long long uend = u1;
-        if (u1 % U != 0 && cut > u0) {  // the cut last item goes first
-            add(cut, u1);
-            uend = cut;
-        }
-        for (long long u = u0; u < uend;) {
-            const long long next = min((u / U + 1) * U, uend);
-            add(u, next);
-            u = next;
-        }
+    int first, stride, last, rounds, single;
+    if (p.sel_qb) {
+        const int n = sel_item_count(p, v, V);
+        first = sel_first_item(p, v, V);
+        stride = 2;
+        rounds = (n + 1) / 2;
+        single = n & 1;
+        last = first + 2 * (rounds - 1);
+    } else {
+        const int full = p.num_items / (2 * V), base = full * 2 * V, rem = p.num_items - base;
+        const int pairs = max(0, rem - V);  // pipelines that take a pair of the rest, the others one item
+        const int n = v < pairs ? 2 : (v < rem ? 1 : 0);
+        first = 2 * v;
+        stride = 2 * V;
+        rounds = full + (n > 0);
+        single = n == 1;
+        last = n > 0 ? base + v + min(v, pairs) : first + (full - 1) * stride;
     }
-    sm.nA = nA;
-    sm.nB = nB;
-    sm.M = M;
+    if (p.idx && !p.sel_qb)
+        for (int i = t; i < 2 * rounds && i < kCntCap; i += nthr) {
+            const int r = i >> 1, item = (r == rounds - 1 ? last : first + r * stride) + (i & 1);
+            if (item < p.num_items) c.cnts[i] = min(max(__ldg(p.cnt + item), 0), p.keep);
+        }
+    if (t != 0) return;
+    c.first = first;
+    c.stride = stride;
+    c.last = last;
+    c.rounds = rounds;
+    c.single = single;
 }
 
-__global__ void __maxnreg__(80) ssba_attn_tc_kernel(const __grid_constant__ TileMaps maps,
-                                                                    const TcParams p)
+// 32 lanes x 32 bits, 32 consecutive columns: thread i gets lane (base + i).
+__device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t* r)
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_t* r)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        : "memory");
+}
+
+// D[tmem] (+)= A[tmem] * B[smem]^T on half h's 64 lanes only: the other lanes of D keep their value.
+__device__ __forceinline__ void mma_ts_half(int h, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                            uint32_t accumulate)
+{
+    const uint32_t off_a = h ? 0xffffffffu : 0u, off_b = ~off_a;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %6, %6}, p;\n"
+        "}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(off_a), "r"(off_b)
+        : "memory");
+}
+
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+// Row of a finished item: O / l in bf16 and lse to global memory, O (unnormalised) read from TMEM
+// in two chunks, the other part of a split item (b_o: its row in shared memory, 16-byte chunks
+// swizzled by row) added with weights wa, wb first.
+__device__ __forceinline__ void store_row(const TcParams& p, int item, int row, uint32_t ocol, float m, float l,
+                                          const float* b_o, float wa, float wb)
+{
+    const int Tb = p.g.Tb(), N = p.g.H * p.g.W;
+    const int bh = item / Tb, label = item - bh * Tb;
+    const bool ok = l > 0.f;
+    const float inv = ok ? 1.f / l : 0.f;
+    const int tok = p.g.token(label, tile_row_pos(p.g, label, row));
+    uint4* dst = reinterpret_cast<uint4*>(p.O + ((size_t)bh * N + tok) * kD);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        uint32_t o[32];
+        tmem_ld_32x32b_x32(ocol + 32 * c, o);
+        tmem_wait_ld();
+        if (b_o) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 x = *reinterpret_cast<const float4*>(b_o + 4 * ((8 * c + i) ^ (row & 15)));
+                const float xb[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float a = wa > 0.f ? __uint_as_float(o[4 * i + e]) * wa : 0.f;
+                    o[4 * i + e] = __float_as_uint(wb > 0.f ? fmaf(xb[e], wb, a) : a);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float f[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) f[e] = ok ? __uint_as_float(o[8 * i + e]) * inv : 0.f;
+            dst[4 * c + i] = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]),
+                                        pack_bf16(f[6], f[7]));
+        }
+    }
+    p.lse[(size_t)bh * N + tok] = ok ? (m * 0.69314718055994531f + logf(l)) : -INFINITY;
+}
+
+__global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_constant__ TileMaps maps,
+                                                                   const TcParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     SmemLayout& cs = *reinterpret_cast<SmemLayout*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                     ~static_cast<uintptr_t>(1023));
     const int gwarp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) TL_CTA(tl::kEntry);
-    // the pipelines' variables are defined after the pooling below, so that they are not live
-    // across its call (at 80 registers a thread, values live across a call are spilled)
-    {
-    const int slot = gwarp / kSlotWarps;
-    SlotSmem& sm = cs.slot[slot];
-    if (threadIdx.x % (kSlotWarps * 32) == 0) {
+    if (threadIdx.x < kSlots * kSoftWarps * 32 && threadIdx.x % (kSoftWarps * 32) == 0) {
+        const int slot = threadIdx.x / (kSoftWarps * 32);
+        SlotCtl& sm = cs.ctl[slot];
         if (slot == 0) cs.abort_flag = 0;
-        for (int s = 0; s < kKStages; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             mbar_init(smem_u32(&sm.k_full[s]), 1);
             mbar_init(smem_u32(&sm.k_empty[s]), 1);
-        }
-        for (int s = 0; s < kVStages; ++s) {
             mbar_init(smem_u32(&sm.v_full[s]), 1);
             mbar_init(smem_u32(&sm.v_empty[s]), 1);
         }
-        for (int b = 0; b < kSBuf; ++b) {
-            mbar_init(smem_u32(&sm.s_full[b]), 1);
-            mbar_init(smem_u32(&sm.s_free[b]), 1);
-            mbar_init(smem_u32(&sm.p_full[b]), 4);
-        }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&sm.q_full[b]), 1);
-            mbar_init(smem_u32(&sm.q_empty[b]), 1);
-            mbar_init(smem_u32(&sm.stats_full[b]), 4);
-            mbar_init(smem_u32(&sm.stats_free[b]), 4);
+            mbar_init(smem_u32(&sm.p_full[b]), 4);
+            mbar_init(smem_u32(&sm.o_full[b]), 1);
+            mbar_init(smem_u32(&sm.drain[b]), 1);
         }
-        mbar_init(smem_u32(&sm.o_full), 1);
-        mbar_init(smem_u32(&sm.o_free), 4);
-        mbar_init(smem_u32(&sm.drain[0]), 1);
-        mbar_init(smem_u32(&sm.drain[1]), 1);
+        mbar_init(smem_u32(&sm.q_full), 1);
+        mbar_init(smem_u32(&sm.q_empty), 1);
+        mbar_init(smem_u32(&sm.s_full), 1);
+        mbar_init(smem_u32(&sm.s_free), 4);
+        mbar_init(smem_u32(&sm.merged), 2);
         if (p.pool_q)
-            for (int w = slot * kSlotWarps; w < (slot + 1) * kSlotWarps; ++w) mbar_init(smem_u32(&cs.pool_bar[w]), 1);
+            for (int w = slot * kPoolUnits; w < (slot + 1) * kPoolUnits; ++w) mbar_init(smem_u32(&cs.pool_bar[w]), 1);
         fence_mbar_init();
     }
-    const Grid g = p.g;
-    for (int l = threadIdx.x; l < g.Tb() && l < kWinCap; l += kThreads) cs.win[l] = window_entry(g, l);
+    for (int l = threadIdx.x; l < p.g.Tb() && l < kWinCap; l += kThreads) cs.win[l] = window_entry(p.g, l);
+    if (gwarp == 2 && lane < 12) tma_prefetch_desc(lane < 4 ? &maps.q[lane] : (lane < 8 ? &maps.k[lane - 4] : &maps.v[lane - 8]));
+    if (gwarp == 1) {
+        tmem_alloc(smem_u32(&cs.tmem_base), kTmemCols);
+        tmem_relinquish();
     }
     // everything above reads no input; the lists, counts and tensors may come from the grid
     // launched just before this one (programmatic dependent launch)
     grid_dep_wait();
     if (threadIdx.x == 0) TL_CTA(tl::kDepWait);
     bool pool_fail = false;
+    unsigned departed = 0;
     if (p.pool_q) {
-        // the block means of the whole layer: every warp of the grid one (block, tensor) unit,
+        // the block means of the whole layer, the (block, tensor) units shared out over the grid,
         // then a grid barrier; the next grid is released only after it, so that it cannot take
         // an SM that one of these CTAs still waits for
         __syncthreads();  // the pooling barriers are initialised
@@ -585,28 +695,30 @@ __global__ void __maxnreg__(80) ssba_attn_tc_kernel(const __grid_constant__ Tile
                                                   p.withhold != 2 || blockIdx.x != 0);
         // on a timeout the means of other CTAs may be missing: the status is set, and the raised
         // abort flag makes every role leave at its first wait that does not complete at once
-        // (lists selected from stale means still hold labels in [0, Tb)). No early return and
-        // no condition on the selection: either costs the pipeline roles registers (spills).
+        // (lists selected from stale means still hold labels in [0, Tb))
         pool_fail = __syncthreads_or(pool_fail);
         if (threadIdx.x == 0) TL_CTA(tl::kBarrier);
-        if (pool_fail && threadIdx.x == 0) {
-            atomicExch(p.status, SSBA_ERR_TIMEOUT);
-            cs.abort_flag = 1;
+        if (threadIdx.x == 0) {
+            if (pool_fail) {
+                atomicExch(p.status, SSBA_ERR_TIMEOUT);
+                cs.abort_flag = 1;
+            } else {
+                departed = grid_barrier_depart(p.gsync);
+            }
         }
     }
     grid_dep_launch();
-    const int slot = gwarp / kSlotWarps;   // which pipeline of this CTA
-    const int warp = gwarp % kSlotWarps;   // role within the pipeline
+    // which pipeline of this CTA, and the role within it: the softmax warps first, so that a
+    // pipeline's four are one per TMEM lane quadrant (and two softmax warps share a scheduler)
+    const bool soft = gwarp < kSlots * kSoftWarps;
+    const int slot = soft ? gwarp / kSoftWarps : (gwarp - kSlots * kSoftWarps) / kRoleWarps;
+    const int role = soft ? kSoftmax : (gwarp - kSlots * kSoftWarps) % kRoleWarps;
     SlotSmem& sm = cs.slot[slot];
+    SlotCtl& ct = cs.ctl[slot];
     volatile int* abortf = &cs.abort_flag;
-    // pipeline `slot` of CTA b is pipeline b + slot * gridDim.x of 2 * gridDim.x: the items
-    // left over after whole rounds go to the first pipelines, one per CTA, and the other
-    // pipeline of such a CTA finishes first and leaves it the SM
     const int vcta = slot * gridDim.x + blockIdx.x;
     const int vgrid = gridDim.x * kSlots;
-    const Grid g = p.g;
-    const int Tb = g.Tb();
-    const int N = g.H * g.W;
+    const int Tb = p.g.Tb();
     if (p.sel_qb) {
         // the lists of this CTA's items (the contiguous ranges of its two pipelines): the k_b
         // of the heads they touch are staged by all threads in the stage buffers of both
@@ -623,7 +735,7 @@ __global__ void __maxnreg__(80) ssba_attn_tc_kernel(const __grid_constant__ Tile
         // staging: pipeline 0's k, v, q buffers end with the scratch (per warp 128 key words and
         // a 64-float query row, then up to kSelQRows shared query rows); the rest of them and
         // pipeline 1's hold the heads
-        constexpr uint32_t kRegion = (kKStages + kVStages + 2) * kTileBytes;  // k, v, q of one pipeline
+        constexpr uint32_t kRegion = sizeof(SlotSmem);  // k, v, q of one pipeline
         constexpr int kSelQRows = 48;
         constexpr int kWarpScratch = 128 + kD;  // words per warp: keys, then its own query row
         constexpr uint32_t kScratch = (kThreads / 32) * kWarpScratch * 4 + kSelQRows * kD * 4;
@@ -680,13 +792,9 @@ __global__ void __maxnreg__(80) ssba_attn_tc_kernel(const __grid_constant__ Tile
             __syncthreads();
         }
         if (threadIdx.x == 0) TL_CTA(tl::kSelected);
+        if (p.pool_q && threadIdx.x == 0 && !pool_fail) grid_barrier_reset(p.gsync, gridDim.x, departed);
     }
-    build_schedule(p, sm, vcta, vgrid, threadIdx.x % (kSlotWarps * 32), kSlotWarps * 32);
-    if (gwarp == 0 && lane < 12) tma_prefetch_desc(lane < 4 ? &maps.q[lane] : (lane < 8 ? &maps.k[lane - 4] : &maps.v[lane - 8]));
-    if (gwarp == 1) {
-        tmem_alloc(smem_u32(&cs.tmem_base), kTmemCols);
-        tmem_relinquish();
-    }
+    if (soft) build_schedule(p, ct, vcta, vgrid, threadIdx.x % (kSoftWarps * 32), kSoftWarps * 32);
     // the stage buffers held the pooled rows and the staged means (generic accesses); the
     // producers' tensor copies (async proxy) overwrite them next
     if (p.sel_qb) fence_proxy_async_smem();
@@ -694,461 +802,410 @@ __global__ void __maxnreg__(80) ssba_attn_tc_kernel(const __grid_constant__ Tile
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = cs.tmem_base + slot * kSlotCols;
+    const int rounds = ct.rounds;
+    const uint32_t abort_at = smem_u32(&cs.abort_flag);
     bool dead = false;
     if (threadIdx.x == 0) TL_CTA(tl::kPipesStart);
-    if (threadIdx.x % (kSlotWarps * 32) == 0) TL_ITEM(slot, 0u, tl::kPipeClock0);
+    if (soft && threadIdx.x % (kSoftWarps * 32) == 0) TL_ITEM(slot, 0u, tl::kPipeClock0);
 
-    if (warp == 0 || warp == 2) {
+    if (role == kLoadK || role == kLoadV) {
         // ------------------------------------------------------------ TMA producers
-        // Warp 0 loads each item's Q tile and the K tiles of its key blocks into the K ring,
-        // warp 2 the V tiles into the V ring; one elected lane each, blocking (suspending)
-        // waits. A K slot frees when its QK is done and a V slot when its PV is done, so the
-        // rings do not wait on each other, and the two issuing threads overlap their TMA
-        // issue latency (about 140 cycles per box per thread).
-        const bool is_k = warp == 0;
-        uint32_t g = 0, nq = 0;
-        const int npieces = sm.nA + sm.nB;
-        for (int pi = 0; !dead && pi < npieces; ++pi, ++nq) {
-            const Piece pc = get_piece(p, sm, pi, vcta, vgrid);
-            const int bh = pc.item / Tb, label = pc.item - bh * Tb;
-            const int nblk = pc.nb;
-            // item blocks [tb, tb + nblk): text blocks first (positions < ntxt), then the
-            // listed image blocks, list entry (position - ntxt)
-            const int ti0 = max(pc.tb, p.ntxt);
-            const int nimg = max(0, pc.tb + nblk - ti0);
-            const int32_t* list = p.idx ? p.idx + (size_t)pc.item * p.keep + (ti0 - p.ntxt) : nullptr;
-            // all lanes fetch the piece's labels in one round and stage their window entries;
-            // lane 0 then issues the copies (measured: faster than prefetching the labels one
-            // piece ahead with cp.async)
-            uint32_t* lab = reinterpret_cast<uint32_t*>(sm.labels[is_k ? 0 : 1]);
-            for (int t = lane; t < nimg && t < kLabelCap; t += 32) {
-                const int j = list ? clamp_label(ld_list(p, list + t), Tb) : ti0 - p.ntxt + t;
-                lab[t] = j < kWinCap ? cs.win[j] : window_entry(p.g, j);
-            }
-            if (kChecked && is_k && list) {
-                // this piece's entries ascending and in range (the one before it too, for a second
-                // part), and the item's count in [0, keep]
+        // The K producer loads each round's Q tiles and the K tiles of its key blocks, the V producer
+        // the V tiles, one elected lane for both halves. A K stage frees when its QK is done and a V
+        // stage when its PV is done, so the rings do not wait on each other. All lanes fetch the
+        // labels of 32 steps at once and look up their windows; each step's two entries then come
+        // from a shuffle.
+        const bool is_k = role == kLoadK;
+        const uint32_t empty0 = smem_u32(is_k ? &ct.k_empty[0] : &ct.v_empty[0]);
+        const uint32_t full0 = smem_u32(is_k ? &ct.k_full[0] : &ct.v_full[0]);
+        const uint32_t tile0 = smem_u32(is_k ? &sm.k[0][0] : &sm.v[0][0]);
+        const CUtensorMap* m4 = is_k ? maps.k : maps.v;
+        const CUtensorMap* mt = is_k ? &maps.kt : &maps.vt;
+        // test hook: the first K copies of pipeline 0 never land
+        const bool hold = p.withhold == 1 && is_k && vcta == 0;
+        uint32_t g = 0;  // steps announced
+        int nq = 0;      // rounds whose Q is announced
+        auto entry_of = [&](int label) { return label < kWinCap ? cs.win[label] : window_entry(p.g, label); };
+        for (int r = 0; !dead && r < rounds; ++r) {
+            const Round rd = get_round(p, ct, r);
+            const int steps = max(rd.nb[0], rd.nb[1]);
+            const int bh0 = rd.item[0] / Tb, bh1 = rd.item[1] / Tb;
+            if (kChecked && is_k && p.idx) {
+                // the entries of both halves ascending and in range (the one before a second part
+                // too), and the items' counts in [0, keep]
                 bool bad = false;
-                for (int t = lane; t < nimg; t += 32) {
-                    const int raw = ld_list(p, list + t);
-                    bad |= raw < 0 || raw >= Tb;
-                    if (t > 0 || ti0 > p.ntxt) bad |= raw <= ld_list(p, list + t - 1);
-                }
-                if (lane == 0 && !p.sel_qb) {
-                    const int c = __ldg(p.cnt + pc.item);
-                    bad |= c < 0 || c > p.keep;
+                for (int h = 0; h < 2; ++h) {
+                    const int32_t* hl = p.idx + (size_t)rd.item[h] * p.keep;
+                    const int a = max(rd.tb[h], p.ntxt) - p.ntxt, b = rd.tb[h] + rd.nb[h] - p.ntxt;
+                    for (int t = a + lane; t < b; t += 32) {
+                        const int raw = ld_list(p, hl + t);
+                        bad |= raw < 0 || raw >= Tb;
+                        if (t > 0) bad |= raw <= ld_list(p, hl + t - 1);
+                    }
+                    if (lane == 0 && !p.sel_qb) {
+                        const int c = __ldg(p.cnt + rd.item[h]);
+                        bad |= c < 0 || c > p.keep;
+                    }
                 }
                 if (__any_sync(0xffffffffu, bad) && lane == 0) atomicExch(p.status, SSBA_ERR_CHECK);
+                __syncwarp();
             }
-            __syncwarp();
-            if (lane == 0) {
-                if (is_k) {
-                    const uint32_t qb = nq & 1;
-                    if (!mbar_wait(smem_u32(&sm.q_empty[qb]), ((nq >> 1) & 1) ^ 1, abortf, p.budget_ns)) dead = true;
-                    if (!dead) {
-                        mbar_arrive_expect_tx(smem_u32(&sm.q_full[qb]), kTileBytes);
-                        window_boxes_e(maps.q, smem_u32(&sm.q[qb][0]), smem_u32(&sm.q_full[qb]),
-                                       label < kWinCap ? cs.win[label] : window_entry(p.g, label), bh);
-                    }
+            // the round's Q pair, once the last round's final QK has read its own
+            auto load_q = [&]() -> bool {
+                const bool ok = mbar_wait(smem_u32(&ct.q_empty), (r & 1) ^ 1, abortf, p.budget_ns);
+                if (!__all_sync(0xffffffffu, ok)) return false;
+                if (elect_one_sync()) {
+                    const uint32_t bar = smem_u32(&ct.q_full);
+                    mbar_arrive_expect_tx(bar, kPairBytes);
+                    window_boxes_e(maps.q, smem_u32(&sm.q[0]), bar, entry_of(rd.item[0] - bh0 * Tb), bh0);
+                    window_boxes_e(maps.q, smem_u32(&sm.q[0]) + kTileBytes, bar, entry_of(rd.item[1] - bh1 * Tb), bh1);
                 }
-                const uint32_t nst = is_k ? kKStages : kVStages;
-                // text blocks of the piece (positions below ntxt): rows [64 tt, 64 tt + 64) of
-                // the text keys / values, zero past T_txt
-                const int te_txt = min(pc.tb + nblk, p.ntxt);
-                for (int tt = pc.tb; tt < te_txt && !dead; ++tt, ++g) {
-                    const uint32_t slot = g % nst;
-                    uint64_t* empty = is_k ? &sm.k_empty[slot] : &sm.v_empty[slot];
-                    uint64_t* full = is_k ? &sm.k_full[slot] : &sm.v_full[slot];
-                    if (!mbar_wait(smem_u32(empty), ((g / nst) & 1) ^ 1, abortf, p.budget_ns)) {
+                __syncwarp();
+                ++nq;
+                return true;
+            };
+            if (is_k && steps == 0 && !load_q()) dead = true;
+            for (int t0 = 0; t0 < steps && !dead; t0 += 32) {
+                uint32_t ent[2] = {0u, 0u};
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int t = t0 + lane, i = rd.tb[h] + t - p.ntxt;  // entry of the item's list
+                    if (t < rd.nb[h] && i >= 0)
+                        ent[h] = entry_of(p.idx ? clamp_label(ld_list(p, p.idx + (size_t)rd.item[h] * p.keep + i), Tb) : i);
+                }
+                const int te = min(t0 + 32, steps);
+                for (int t = t0; t < te; ++t) {
+                    const uint32_t st = g % kStages, full = full0 + 8 * st, dst = tile0 + st * kPairBytes;
+                    const uint32_t e0 = __shfl_sync(0xffffffffu, ent[0], t - t0);
+                    const uint32_t e1 = __shfl_sync(0xffffffffu, ent[1], t - t0);
+                    const bool ok = mbar_wait(empty0 + 8 * st, ((g / kStages) & 1) ^ 1, abortf, p.budget_ns);
+                    if (!__all_sync(0xffffffffu, ok)) {
                         dead = true;
                         break;
                     }
-                    mbar_arrive_expect_tx(smem_u32(full), kTileBytes);
-                    tma_load_3d(smem_u32(is_k ? &sm.k[slot][0] : &sm.v[slot][0]), is_k ? &maps.kt : &maps.vt,
-                                smem_u32(full), 0, tt * 64, bh);
-                }
-                // image blocks of the piece: list entries [ti0 - ntxt, ti0 - ntxt + nimg)
-                const bool hold = p.withhold == 1 && is_k && vcta == 0;  // test hook: never lands
-                const uint32_t empty0 = smem_u32(is_k ? &sm.k_empty[0] : &sm.v_empty[0]);
-                const uint32_t full0 = smem_u32(is_k ? &sm.k_full[0] : &sm.v_full[0]);
-                const uint32_t tile0 = smem_u32(is_k ? &sm.k[0][0] : &sm.v[0][0]);
-                const CUtensorMap* m4 = is_k ? maps.k : maps.v;
-                for (int t = 0; t < nimg && !dead; ++t, ++g) {
-                    uint32_t e;
-                    if (t < kLabelCap) {
-                        e = lab[t];
-                    } else {
-                        const int j = list ? clamp_label(ld_list(p, list + t), Tb) : ti0 - p.ntxt + t;
-                        e = j < kWinCap ? cs.win[j] : window_entry(p.g, j);
+                    if (elect_one_sync()) {
+                        const bool a = t < rd.nb[0], b = t < rd.nb[1];
+                        mbar_arrive_expect_tx(full, (a + b) * kTileBytes);
+                        if (!(hold && g == 0)) {
+                            // text keys / values [64 pos, 64 pos + 64) at positions pos < ntxt, zero past T_txt
+                            if (a) {
+                                if (rd.tb[0] + t < p.ntxt) tma_load_3d(dst, mt, full, 0, (rd.tb[0] + t) * 64, bh0);
+                                else window_boxes_e(m4, dst, full, e0, bh0);
+                            }
+                            if (b) {
+                                if (rd.tb[1] + t < p.ntxt)
+                                    tma_load_3d(dst + kTileBytes, mt, full, 0, (rd.tb[1] + t) * 64, bh1);
+                                else
+                                    window_boxes_e(m4, dst + kTileBytes, full, e1, bh1);
+                            }
+                        }
+                        TL_TILE(slot, g, is_k ? tl::kKIssue : tl::kVIssue);
                     }
-                    const uint32_t slot = g % nst;
-                    if (!mbar_wait(empty0 + 8 * slot, ((g / nst) & 1) ^ 1, abortf, p.budget_ns)) {
+                    __syncwarp();
+                    ++g;
+                    // the round's Q after its first K: it waits longest
+                    if (is_k && t == 0 && !load_q()) {
                         dead = true;
                         break;
                     }
-                    mbar_arrive_expect_tx(full0 + 8 * slot, kTileBytes);
-                    if (hold && g == 0) continue;
-                    window_boxes_e(m4, tile0 + slot * kTileBytes, full0 + 8 * slot, e, bh);
-                    TL_TILE(gwarp / kSlotWarps, g, is_k ? tl::kKIssue : tl::kVIssue);
                 }
             }
-            dead = __shfl_sync(0xffffffffu, dead, 0);
-            g = __shfl_sync(0xffffffffu, g, 0);
         }
         if (dead && lane == 0) {
-            // drain: wait for the copies this thread issued that may still be in flight
-            const uint32_t nst = is_k ? kKStages : kVStages;
-            for (uint32_t x = g > nst ? g - nst : 0; x < g; ++x)
-                wait_raw(smem_u32(is_k ? &sm.k_full[x % nst] : &sm.v_full[x % nst]), (x / nst) & 1, p.budget_ns);
-            if (is_k)
-                for (uint32_t n = nq > 1 ? nq - 1 : 0; n <= nq; ++n)
-                    wait_raw(smem_u32(&sm.q_full[n & 1]), (n >> 1) & 1, p.budget_ns);
+            // drain: wait for the copies of this warp that may still be in flight
+            for (uint32_t x = g > kStages ? g - kStages : 0; x < g; ++x)
+                wait_raw(full0 + 8 * (x % kStages), (x / kStages) & 1, p.budget_ns);
+            if (nq > 0) wait_raw(smem_u32(&ct.q_full), (nq - 1) & 1, p.budget_ns);
         }
         __syncwarp();
-    } else if (warp == 1) {
+    } else if (role == kQK) {
         // ------------------------------------------------------------ QK issuer
-        // S_t = Q K_t^T into S buffer t % 3, once PV_{t-3} has read P_{t-3} from it.
-        // MMAs and commits are issued under an elect.sync taken at the issue site: the
-        // compiler then keeps the descriptors on the uniform datapath (measured: 4 MMAs +
-        // commit issue in about 280 cycles, against about 480 under a precomputed lane test).
-        // elect.sync picks the same lane of a full warp every time, so a commit always
-        // follows the MMAs of its own thread.
+        // S_g = [Q_A; Q_B] [K_A; K_B]^T once the softmax holds S_{g-1} in registers (N=64 on the one
+        // half's keys where only one takes part). MMAs and commits are issued under an elect.sync
+        // taken at the issue site: the compiler then keeps the descriptors on the uniform datapath
+        // (measured: 4 MMAs + commit issue in about 280 cycles, against about 480 under a
+        // precomputed lane test). elect.sync picks the same lane of a full warp every time, so a
+        // commit always follows the MMAs of its own thread.
         const bool leader = elect_one_sync();
-        uint32_t gblk = 0, nloc = 0;
         const uint32_t kbase = smem_u32(&sm.k[0][0]);
-        const int npieces = sm.nA + sm.nB;
-        for (int pi = 0; !dead && pi < npieces; ++pi, ++nloc) {
-            const Piece pc = get_piece(p, sm, pi, vcta, vgrid);
-            const int nblk = pc.nb;
-            const uint32_t qb = nloc & 1;
-            const uint32_t qaddr = smem_u32(&sm.q[qb][0]);
-            if (!mbar_wait(smem_u32(&sm.q_full[qb]), (nloc >> 1) & 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            if (nblk == 0 && elect_one_sync()) mma_commit(smem_u32(&sm.q_empty[qb]));
-            for (int t = 0; t < nblk; ++t) {
-                const uint32_t gb = gblk + t, slot = gb % kKStages, sb = gb % kSBuf;
-                if (gb >= (uint32_t)kSBuf &&
-                    !mbar_wait(smem_u32(&sm.s_free[sb]), ((gb / kSBuf) - 1) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
-                if (lane == 0) TL_TILE(gwarp / kSlotWarps, gb, tl::kSFree);
-                if (!mbar_wait(smem_u32(&sm.k_full[slot]), (gb / kKStages) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
+        uint32_t g = 0;
+        for (int r = 0; r < rounds && !*abortf; ++r) {
+            const Round rd = get_round(p, ct, r);
+            const int steps = max(rd.nb[0], rd.nb[1]), both = min(rd.nb[0], rd.nb[1]);
+            const uint32_t one_b = rd.nb[1] > rd.nb[0] ? 1u : 0u;  // the half of the steps past `both`
+            const uint32_t qaddr = smem_u32(&sm.q[0]);
+            wait_phase(smem_u32(&ct.q_full), r & 1, abort_at, p.budget_ns);
+            if (steps == 0 && elect_one_sync()) mma_commit(smem_u32(&ct.q_empty));
+            for (int t = 0; t < steps; ++t, ++g) {
+                const uint32_t st = g % kStages;
+                wait_phase(smem_u32(&ct.k_full[st]), (g / kStages) & 1, abort_at, p.budget_ns);
+                // QK_g follows PV_{g-2}: the softmax, which sees S_g, then knows its P buffer is free (a wait of
+                // its own there cost 7 % of the whole kernel)
+                if (g >= 2) wait_phase(smem_u32(&ct.o_full[g & 1]), ((g >> 1) - 1) & 1, abort_at, p.budget_ns);
+                if (g >= 1) wait_phase(smem_u32(&ct.s_free), (g - 1) & 1, abort_at, p.budget_ns);
+                if (lane == 0) TL_TILE(slot, g, tl::kSFree);
                 tc_fence_after();
                 if (elect_one_sync()) {
+                    const uint32_t off = t < both ? 0u : one_b;
+                    const uint32_t idesc = t < both ? kIdescQK : kIdescQK1;
                     const uint64_t adesc = sdesc_sw128(qaddr, 16, 1024);
-                    const uint64_t bdesc = sdesc_sw128(kbase + slot * kTileBytes, 16, 1024);
-                    const uint32_t d = tbase + kColS + sb * 64;
+                    const uint64_t bdesc = sdesc_sw128(kbase + st * kPairBytes + off * kTileBytes, 16, 1024);
+                    const uint32_t d = tbase + kColS + off * 64;
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        mma_ss(d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), kIdescQK, k > 0 ? 1u : 0u);
-                    mma_commit(smem_u32(&sm.s_full[sb]));
-                    mma_commit(smem_u32(&sm.k_empty[slot]));
-                    if (t == nblk - 1) mma_commit(smem_u32(&sm.q_empty[qb]));  // last read of this Q tile
-                    TL_TILE(gwarp / kSlotWarps, gb, tl::kQKIssue);
+                        mma_ss(d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, k > 0 ? 1u : 0u);
+                    mma_commit(smem_u32(&ct.s_full));
+                    mma_commit(smem_u32(&ct.k_empty[st]));
+                    if (t == steps - 1) mma_commit(smem_u32(&ct.q_empty));  // last read of this Q pair
+                    TL_TILE(slot, g, tl::kQKIssue);
                 }
                 __syncwarp();
             }
-            gblk += nblk;
         }
+        dead = *abortf != 0;
         if (dead && leader) {
-            mma_commit(smem_u32(&sm.drain[0]));
-            wait_raw(smem_u32(&sm.drain[0]), 0, p.budget_ns);
+            mma_commit(smem_u32(&ct.drain[0]));
+            wait_raw(smem_u32(&ct.drain[0]), 0, p.budget_ns);
         }
-    } else if (warp == 3) {
+    } else if (role == kPV) {
         // ------------------------------------------------------------ PV issuer
-        // O += P_t V_t once the softmax has written P_t to shared memory and V_t has landed;
-        // PVs of a pipeline are issued by this one thread, so they accumulate into O in order.
+        // O_h += P_h V_h of both halves once the softmax has stored P_g and V_g has landed; all PVs
+        // of a pipeline are issued by this one thread, so they accumulate into O in order. (One
+        // issuer for QK and PV took 2000 cycles a step: its waits and issues do not overlap.)
         const bool leader = elect_one_sync();
-        uint32_t gblk = 0, nloc = 0;
         const uint32_t vbase = smem_u32(&sm.v[0][0]);
-        const int npieces = sm.nA + sm.nB;
-        for (int pi = 0; !dead && pi < npieces; ++pi, ++nloc) {
-            const Piece pc = get_piece(p, sm, pi, vcta, vgrid);
-            const int nblk = pc.nb;
-            for (int t = 0; t < nblk; ++t) {
-                const uint32_t gb = gblk + t, pb = gb % kSBuf, slot = gb % kVStages;
-                if (!mbar_wait(smem_u32(&sm.p_full[pb]), (gb / kSBuf) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
-                if (t == 0 && nloc > 0 &&
-                    !mbar_wait(smem_u32(&sm.o_free), (nloc - 1) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
-                if (!mbar_wait(smem_u32(&sm.v_full[slot]), (gb / kVStages) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
-                if (lane == 0) TL_TILE(gwarp / kSlotWarps, gb, tl::kPVReady);
+        uint32_t g = 0;
+        for (int r = 0; r < rounds && !*abortf; ++r) {
+            const Round rd = get_round(p, ct, r);
+            const int steps = max(rd.nb[0], rd.nb[1]);
+            for (int t = 0; t < steps; ++t, ++g) {
+                const uint32_t pb = g & 1, st = g % kStages;
+                wait_phase(smem_u32(&ct.v_full[st]), (g / kStages) & 1, abort_at, p.budget_ns);
+                wait_phase(smem_u32(&ct.p_full[pb]), (g >> 1) & 1, abort_at, p.budget_ns);
+                if (lane == 0) TL_TILE(slot, g, tl::kPVReady);
                 tc_fence_after();
                 if (elect_one_sync()) {
-                    const uint64_t vdesc = sdesc_sw128(vbase + slot * kTileBytes, 8192, 1024);
-                    const uint32_t pcol = tbase + kColS + pb * 64;
+                    const uint32_t pcol = tbase + kColP + pb * 32;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        mma_ts(tbase + kColO, pcol + k * 8, vdesc + (uint64_t)(k * 128), kIdescPV,
-                               (t > 0 || k > 0) ? 1u : 0u);
-                    mma_commit(smem_u32(&sm.v_empty[slot]));
-                    mma_commit(smem_u32(&sm.s_free[pb]));
-                    TL_TILE(gwarp / kSlotWarps, gb, tl::kPVIssue);
+                    for (int h = 0; h < 2; ++h) {
+                        if (t >= rd.nb[h]) continue;
+                        const uint64_t vdesc = sdesc_sw128(vbase + st * kPairBytes + h * kTileBytes, 8192, 1024);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            mma_ts_half(h, tbase + kColO, pcol + k * 8, vdesc + (uint64_t)(k * 128), kIdescPV,
+                                        (t > 0 || k > 0) ? 1u : 0u);
+                    }
+                    mma_commit(smem_u32(&ct.o_full[pb]));
+                    mma_commit(smem_u32(&ct.v_empty[st]));
+                    TL_TILE(slot, g, tl::kPVIssue);
                 }
                 __syncwarp();
             }
-            if (dead) break;
-            // an empty item writes no O, but o_full must still not run two phases ahead
-            if (nblk == 0 && nloc > 0 &&
-                !mbar_wait(smem_u32(&sm.o_free), (nloc - 1) & 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            if (elect_one_sync()) mma_commit(smem_u32(&sm.o_full));
-            __syncwarp();
-            gblk += nblk;
         }
+        dead = *abortf != 0;
         if (dead && leader) {
-            mma_commit(smem_u32(&sm.drain[1]));
-            wait_raw(smem_u32(&sm.drain[1]), 0, p.budget_ns);
+            mma_commit(smem_u32(&ct.drain[1]));
+            wait_raw(smem_u32(&ct.drain[1]), 0, p.budget_ns);
         }
-    } else if (warp >= 4 && warp < 8) {
-        // ------------------------------------------------------------ softmax
+    } else if (role == kSoftmax) {
+        // ------------------------------------------------------------ softmax and output
         const int quad = gwarp & 3;  // TMEM lane quadrant of this warp
-        const int half = lane >> 4;
-        const int row = quad * 16 + (lane & 15);
-        const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
+        const int half = quad >> 1;
+        const int row = (quad & 1) * 32 + lane;  // tile row of the half's item
+        const uint32_t tq = tbase + (static_cast<uint32_t>(quad * 32) << 16);
+        const uint32_t scol = tq + kColS + half * 64, ocol = tq + kColO;
         const float c = p.scale_log2;
-        uint32_t gblk = 0, nloc = 0;
-        const int npieces = sm.nA + sm.nB;
-        for (int pi = 0; !dead && pi < npieces; ++pi, ++nloc) {
-            const Piece pc = get_piece(p, sm, pi, vcta, vgrid);
-            const int nblk = pc.nb;
+        uint32_t g = 0;
+        // The last round's item, whose O is written after this round's first exps: its row statistics
+        // stay here; its last PV is that of step g - 1.
+        bool owed = false;
+        float done_m = 0.f, done_l = 0.f;
+        auto wait_pv = [&](uint32_t x) {  // PV_x has finished
+            wait_phase(smem_u32(&ct.o_full[x & 1]), (x >> 1) & 1, abort_at, p.budget_ns);
+            tc_fence_after();
+        };
+        // writes the rows of round r's item, whose last PV is that of step `last`
+        auto finish = [&](uint32_t last, int r) {
+            wait_pv(last);
+            const Round rd = get_round(p, ct, r);
+            store_row(p, half ? rd.item[1] : rd.item[0], row, ocol, done_m, done_l, nullptr, 1.f, 0.f);
+            tc_fence_before();
+            owed = false;
+        };
+        bool split = false;
+        for (int r = 0; r < rounds && !*abortf; ++r) {
+            int nb, steps, mask_t;  // mask_t: the step of the last text block, if that one is ragged
+            bool parted;            // half B has blocks (of a split item: there is something to merge)
+            {
+                const Round rd = get_round(p, ct, r);
+                nb = half ? rd.nb[1] : rd.nb[0];
+                steps = max(rd.nb[0], rd.nb[1]);
+                mask_t = (p.t_txt & 63) ? p.ntxt - 1 - (half ? rd.tb[1] : rd.tb[0]) : -1;
+                split = rd.split;
+                parted = rd.nb[1] > 0;
+                if (steps == 0) {  // empty lists: nothing was multiplied; O = 0, lse = -inf
+                    if (owed) finish(g - 1, r - 1);
+                    if (!split || half == 0)
+                        store_row(p, half ? rd.item[1] : rd.item[0], row, ocol, 0.f, 0.f, nullptr, 1.f, 0.f);
+                    split = false;
+                    continue;
+                }
+            }
             float m_used = 0.f, l = 0.f;
-            for (int t = 0; t < nblk; ++t) {
-                const uint32_t gb = gblk + t, sb = gb % kSBuf;
-                if (!mbar_wait(smem_u32(&sm.s_full[sb]), (gb / kSBuf) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
-                if (quad == 0 && lane == 0) TL_TILE(gwarp / kSlotWarps, gb, tl::kSmxStart);
+            for (int t = 0; t < nb; ++t, ++g) {
+                wait_phase(smem_u32(&ct.s_full), g & 1, abort_at, p.budget_ns);
+                if (quad == 0 && lane == 0) TL_TILE(slot, g, tl::kSmxStart);
                 tc_fence_after();
-                const uint32_t scol = tbase + lane_off + kColS + sb * 64;
-                uint32_t sr[32];
-                tmem_ld_16x32bx2_x16_off32(scol, *reinterpret_cast<uint32_t(*)[16]>(&sr[0]));
-                tmem_ld_16x32bx2_x16_off32(scol + 16, *reinterpret_cast<uint32_t(*)[16]>(&sr[16]));
+                uint32_t sr[64];
+                tmem_ld_32x32b_x32(scol, &sr[0]);
+                tmem_ld_32x32b_x32(scol + 32, &sr[32]);
                 tmem_wait_ld();
-                if (quad == 0 && lane == 0) TL_TILE(gwarp / kSlotWarps, gb, tl::kSLoaded);
-                {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ct.s_free));
+                if (quad == 0 && lane == 0) TL_TILE(slot, g, tl::kSLoaded);
+                if (t == mask_t) {
                     // the last text block: its columns past T_txt are zero-filled keys, not keys
-                    const int tt = pc.tb + t, valid = p.t_txt - tt * 64;
-                    if (tt < p.ntxt && valid < 64)
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (half * 32 + i >= valid) sr[i] = __float_as_uint(-INFINITY);
+                    for (int i = 0; i < 64; ++i)
+                        if (i >= (p.t_txt & 63)) sr[i] = __float_as_uint(-INFINITY);
                 }
-                float mx;
-                {
-                    float t8[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        t8[i] = fmaxf(fmaxf(__uint_as_float(sr[i]), __uint_as_float(sr[i + 8])),
-                                      fmaxf(__uint_as_float(sr[i + 16]), __uint_as_float(sr[i + 24])));
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) t8[i] = fmaxf(t8[i], t8[i + 4]);
-                    mx = fmaxf(fmaxf(t8[0], t8[1]), fmaxf(t8[2], t8[3]));
-                }
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-                const float mx2 = mx * c;
-                // lazy rescale: the running max is raised only when it grows by more than
-                // 2^kRescaleLog2; O is then rescaled below, after P_t is stored (so that O
-                // and S are never held in registers at the same time)
-                bool rescale = false;
-                float alpha = 1.f;
-                if (t == 0) {
-                    m_used = mx2;
-                } else {
-                    const bool need = mx2 > m_used + kRescaleLog2;
-                    rescale = __any_sync(0xffffffffu, need);
-                    if (need) {
-                        alpha = fast_exp2(m_used - mx2);
-                        m_used = mx2;
-                    }
-                }
-                if (quad == 0 && lane == 0) TL_TILE(gwarp / kSlotWarps, gb, tl::kMaxDone);
-                // x = s * c - m and the row sums in packed fp32x2 arithmetic (two lanes per op)
-                uint32_t pk[16];
-                const float2 c2 = make_float2(c, c), nm2 = make_float2(-m_used, -m_used);
-                float2 ls2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[2 * i]), __uint_as_float(sr[2 * i + 1])),
-                                                c2, nm2);
-                    const float2 pp = make_float2(fast_exp2(x.x), fast_exp2(x.y));
-                    ls2[i & 1] = __fadd2_rn(ls2[i & 1], pp);
-                    pk[i] = pack_bf16(pp.x, pp.y);
-                }
-                const float2 lsum = __fadd2_rn(ls2[0], ls2[1]);
-                l = fmaf(l, alpha, lsum.x + lsum.y);
-                if (quad == 0 && lane == 0) TL_TILE(gwarp / kSlotWarps, gb, tl::kSmxExp);
-                // P_t (bf16 pairs) into the first half of S_t's buffer, which S_t no longer needs
-                if (quad == 0 && lane == 0) TL_TILE(gwarp / kSlotWarps, gb, tl::kPFree);
-                const uint32_t pb = sb;
-                tmem_st_16x32bx2_x16_off16(tbase + lane_off + kColS + pb * 64, pk);
-                if (rescale) {
-                    // O must hold every earlier PV before it is rescaled; PV_t waits for p_full
-                    const uint32_t qb = (gb - 1) % kSBuf;
-                    if (!mbar_wait(smem_u32(&sm.s_free[qb]), ((gb - 1) / kSBuf) & 1, abortf, p.budget_ns)) {
-                        dead = true;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t ocol = tbase + lane_off + kColO;
-                    uint32_t o[16];
+                const float2 c2 = make_float2(c, c);
+                // P = exp2(s c - m) in bf16 to tensor memory; returns the thread's row sum of it. Packed
+                // fp32x2 arithmetic (two columns per op).
+                auto exps = [&]() -> float {
+                    const float2 nm2 = make_float2(-m_used, -m_used);
+                    float2 ls2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
+                                     make_float2(0.f, 0.f)};
 #pragma unroll
                     for (int h2 = 0; h2 < 2; ++h2) {
-                        tmem_ld_16x32bx2_x16_off32(ocol + h2 * 16, o);
-                        tmem_wait_ld();
+                        uint32_t pk[16];
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                        tmem_st_16x32bx2_x16_off32(ocol + h2 * 16, o);
+                        for (int b = 0; b < 16; b += 8) {
+                            float2 x[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                x[i] = __ffma2_rn(make_float2(__uint_as_float(sr[32 * h2 + 2 * (b + i)]),
+                                                              __uint_as_float(sr[32 * h2 + 2 * (b + i) + 1])), c2, nm2);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) x[i] = make_float2(fast_exp2(x[i].x), fast_exp2(x[i].y));
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                ls2[i & 3] = __fadd2_rn(ls2[i & 3], x[i]);
+                                pk[b + i] = pack_bf16(x[i].x, x[i].y);
+                            }
+                        }
+                        tmem_st_32x32b_x16(tq + kColP + (g & 1) * 32 + h2 * 16, pk);
                     }
+                    const float2 lsum = __fadd2_rn(__fadd2_rn(ls2[0], ls2[1]), __fadd2_rn(ls2[2], ls2[3]));
+                    return lsum.x + lsum.y;
+                };
+                // the first step only takes its maximum; later ones nearly always skip it (141 of 536
+                // cycles of a warp's step, two warps a scheduler)
+                float ls = t == 0 ? INFINITY : exps();
+                const bool over = !(ls <= kRaise);
+                if (__any_sync(0xffffffffu, over)) {
+                    float mx;
+                    {
+                        float t8[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) t8[i] = __uint_as_float(sr[i]);
+#pragma unroll
+                        for (int j = 8; j < 56; j += 16)
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                t8[i] = max3(t8[i], __uint_as_float(sr[j + i]), __uint_as_float(sr[j + 8 + i]));
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) t8[i] = fmaxf(t8[i], __uint_as_float(sr[56 + i]));
+                        mx = fmaxf(max3(max3(t8[0], t8[1], t8[2]), t8[3], t8[4]), max3(t8[5], t8[6], t8[7]));
+                    }
+                    const float mx2 = fmaxf(mx * c, -3.0e38f);  // finite, so that scores of -inf give P = 0
+                    const float alpha = over && t > 0 ? fast_exp2(m_used - mx2) : 1.f;
+                    m_used = over ? mx2 : m_used;
+                    l *= alpha;
+                    if (t > 0) {
+                        wait_pv(g - 1);
+#pragma unroll
+                        for (int h2 = 0; h2 < 4; ++h2) {
+                            uint32_t o[16];
+                            tmem_ld_32x32b_x16(ocol + h2 * 16, o);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                            tmem_st_32x32b_x16(ocol + h2 * 16, o);
+                        }
+                    }
+                    ls = exps();
                 }
+                l += ls;
+                if (quad == 0 && lane == 0) TL_TILE(slot, g, tl::kSmxExp);
+                if (t == 0 && owed) finish(g - 1, r - 1);
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sm.p_full[pb]));
-                if (quad == 0 && lane == 0) TL_TILE(gwarp / kSlotWarps, gb, tl::kPStored);
+                if (lane == 0) mbar_arrive(smem_u32(&ct.p_full[g & 1]));
+                if (quad == 0 && lane == 0) TL_TILE(slot, g, tl::kPStored);
             }
-            if (dead) break;
-            // hand the row statistics to the epilogue warps
-            const float ltot = l + __shfl_xor_sync(0xffffffffu, l, 16);
-            const uint32_t eb = nloc & 1;
-            if (!mbar_wait(smem_u32(&sm.stats_free[eb]), ((nloc >> 1) & 1) ^ 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            if (half == 0) sm.stats[eb][row] = make_float2(m_used, ltot);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sm.stats_full[eb]));
-            gblk += nblk;
-        }
-    } else {
-        // ------------------------------------------------------------ epilogue
-        const int quad = gwarp & 3;
-        const int half = lane >> 4;
-        const int row = quad * 16 + (lane & 15);
-        const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-        uint32_t nloc = 0;
-        const int npieces = sm.nA + sm.nB;
-        for (int pi = 0; !dead && pi < npieces; ++pi, ++nloc) {
-            const Piece pc = get_piece(p, sm, pi, vcta, vgrid);
-            const int bh = pc.item / Tb, label = pc.item - bh * Tb;
-            const uint32_t eb = nloc & 1;
-            if (quad == 0 && lane == 0) TL_ITEM(gwarp / kSlotWarps, nloc, tl::kEpiStart);
-            if (!mbar_wait(smem_u32(&sm.o_full), nloc & 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            if (quad == 0 && lane == 0) TL_ITEM(gwarp / kSlotWarps, nloc, tl::kEpiO);
-            tc_fence_after();
-            uint32_t o[32];
-            tmem_ld_16x32bx2_x16_off32(tbase + lane_off + kColO, *reinterpret_cast<uint32_t(*)[16]>(&o[0]));
-            tmem_ld_16x32bx2_x16_off32(tbase + lane_off + kColO + 16, *reinterpret_cast<uint32_t(*)[16]>(&o[16]));
-            tmem_wait_ld();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sm.o_free));
-            if (!mbar_wait(smem_u32(&sm.stats_full[eb]), (nloc >> 1) & 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            float2 st = sm.stats[eb][row];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sm.stats_free[eb]));
-
-            if (pc.part >= 0) {
-                // a cut item: publish this part, and if the other part is already there,
-                // merge (each warp owns 16 rows, so the hand-off is per warp)
-                const int bidx = pc.part == 1 ? vcta : vcta + 1;
-                const size_t mine = (size_t)bidx * 2 + pc.part, other = mine ^ 1;
-                float4* wo = reinterpret_cast<float4*>(p.ws_o + (mine * kRows + row) * kD + half * 32);
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    wo[i] = make_float4(__uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]),
-                                        __uint_as_float(o[4 * i + 2]), __uint_as_float(o[4 * i + 3]));
-                if (half == 0) p.ws_st[mine * kRows + row] = st;
-                __threadfence();
+            // steps that only the other half takes part in
+            for (int t = nb; t < steps; ++t, ++g) {
+                wait_phase(smem_u32(&ct.s_full), g & 1, abort_at, p.budget_ns);
+                if (t == 0 && owed) finish(g - 1, r - 1);
                 __syncwarp();
-                int arrived = 0;
-                if (lane == 0) arrived = atomicAdd(p.ws_cnt + bidx * 4 + quad, 1);
-                arrived = __shfl_sync(0xffffffffu, arrived, 0);
-                if (arrived == 0) continue;  // first here: the other part merges
-                if (lane == 0) atomicExch(p.ws_cnt + bidx * 4 + quad, 0);  // ready for the next launch
-                __threadfence();
-                const float2 os = __ldcg(p.ws_st + other * kRows + row);
-                const float4* oo = reinterpret_cast<const float4*>(p.ws_o + (other * kRows + row) * kD + half * 32);
-                // an empty part (sum 0) contributes nothing; its O was never written
-                const bool a_ok = st.y > 0.f, b_ok = os.y > 0.f;
-                const float m = a_ok ? (b_ok ? fmaxf(st.x, os.x) : st.x) : os.x;
-                const float wa = a_ok ? fast_exp2(st.x - m) : 0.f, wb = b_ok ? fast_exp2(os.x - m) : 0.f;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float4 x = __ldcg(oo + i);
-                    const float xb[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float a = a_ok ? __uint_as_float(o[4 * i + e]) * wa : 0.f;
-                        o[4 * i + e] = __float_as_uint(b_ok ? fmaf(xb[e], wb, a) : a);
-                    }
+                if (lane == 0) {
+                    mbar_arrive(smem_u32(&ct.s_free));
+                    mbar_arrive(smem_u32(&ct.p_full[g & 1]));
                 }
-                st = make_float2(m, (a_ok ? st.y * wa : 0.f) + (b_ok ? os.y * wb : 0.f));
             }
-
-            const bool ok = st.y > 0.f;
-            const float inv = ok ? 1.f / st.y : 0.f;
-            const int tok = g.token(label, tile_row_pos(g, label, row));
-            uint4 v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float f[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) f[e] = ok ? __uint_as_float(o[8 * i + e]) * inv : 0.f;
-                v[i].x = pack_bf16(f[0], f[1]);
-                v[i].y = pack_bf16(f[2], f[3]);
-                v[i].z = pack_bf16(f[4], f[5]);
-                v[i].w = pack_bf16(f[6], f[7]);
+            if (split && !parted) {  // one block: half A has all of it
+                split = false;
+                if (half) break;
             }
-            // lanes l and l ^ 16 hold the two halves of one row (chunks 0-3 and 4-7): swap two
-            // chunks so that every store instruction writes whole 32-byte sectors
-            uint4 s0 = half ? v[0] : v[1], s1 = half ? v[2] : v[3], r0v, r1v;
-            r0v.x = __shfl_xor_sync(0xffffffffu, s0.x, 16); r0v.y = __shfl_xor_sync(0xffffffffu, s0.y, 16);
-            r0v.z = __shfl_xor_sync(0xffffffffu, s0.z, 16); r0v.w = __shfl_xor_sync(0xffffffffu, s0.w, 16);
-            r1v.x = __shfl_xor_sync(0xffffffffu, s1.x, 16); r1v.y = __shfl_xor_sync(0xffffffffu, s1.y, 16);
-            r1v.z = __shfl_xor_sync(0xffffffffu, s1.z, 16); r1v.w = __shfl_xor_sync(0xffffffffu, s1.w, 16);
-            uint4* rowp = reinterpret_cast<uint4*>(p.O + ((size_t)bh * N + tok) * kD);
-            // chunk written by this lane in instruction i: 2i + half
-            rowp[0 + half] = half ? r0v : v[0];
-            rowp[2 + half] = half ? r1v : v[2];
-            rowp[4 + half] = half ? v[1] : r0v;
-            rowp[6 + half] = half ? v[3] : r1v;
-            if (half == 0)
-                p.lse[(size_t)bh * N + tok] = ok ? (st.x * 0.69314718055994531f + logf(st.y)) : -INFINITY;
-            if (quad == 0 && lane == 0) TL_ITEM(gwarp / kSlotWarps, nloc, tl::kEpiDone);
+            owed = true;
+            done_m = m_used;
+            done_l = l;
         }
+        // the pipeline's last item or items
+        if (owed && !split) finish(g - 1, rounds - 1);
+        if (split) {
+            // a split item: half B leaves its part in the K ring (no copy or product uses it any
+            // more), half A adds it to its own (two partial softmax sums) and writes the rows
+            float* part = reinterpret_cast<float*>(&sm.k[0][0]) + row * kD;
+            float2* stat = reinterpret_cast<float2*>(&sm.k[1][0]) + row;
+            wait_pv(g - 1);
+            if (half == 1) {
+#pragma unroll
+                for (int h2 = 0; h2 < 2; ++h2) {
+                    uint32_t o[32];
+                    tmem_ld_32x32b_x32(ocol + h2 * 32, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        *reinterpret_cast<float4*>(part + 4 * ((8 * h2 + i) ^ (row & 15))) =
+                            make_float4(__uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]),
+                                        __uint_as_float(o[4 * i + 2]), __uint_as_float(o[4 * i + 3]));
+                }
+                *stat = make_float2(done_m, done_l);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ct.merged));
+            } else {
+                wait_phase(smem_u32(&ct.merged), 0, abort_at, p.budget_ns);
+                const float2 os = *stat;
+                const bool b_ok = os.y != 0.f;  // an empty part contributes nothing; its O was never written
+                const float m = b_ok ? fmaxf(done_m, os.x) : done_m;
+                const float wa = fast_exp2(done_m - m), wb = b_ok ? fast_exp2(os.x - m) : 0.f;
+                store_row(p, ct.last, row, ocol, m, done_l * wa + (b_ok ? os.y * wb : 0.f), part, wa, wb);
+            }
+            tc_fence_before();
+        }
+        dead = *abortf != 0;
     }
 
     if (dead) atomicExch(p.status, SSBA_ERR_TIMEOUT);
-    if (threadIdx.x % (kSlotWarps * 32) == 0) TL_CTA(slot == 0 ? tl::kSlot0End : tl::kSlot1End);
+    if (soft && threadIdx.x % (kSoftWarps * 32) == 0) TL_CTA(slot == 0 ? tl::kSlot0End : tl::kSlot1End);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (gwarp == 1) tmem_dealloc(cs.tmem_base, kTmemCols);
-    if (p.pool_q && threadIdx.x == 0 && !cs.abort_flag) grid_barrier_depart(p.gsync, gridDim.x);
     if (threadIdx.x == 0) TL_CTA(tl::kEnd);
 }
 
@@ -1172,19 +1229,20 @@ PerDeviceOnce g_attn_attr;  // the kernel's shared-memory attributes, set once p
 
 }  // namespace
 
-// Split-merge workspace: counters, then row statistics, then O parts, for one boundary
-// per pipeline of the largest grid this device runs (two per SM) plus one.
 namespace {
-size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 int max_grid() { return num_sms(); }
-size_t ws_boundaries() { return (size_t)kSlots * max_grid() + 1; }
-size_t ws_cnt_bytes() { return align256(ws_boundaries() * 4 * sizeof(int)); }
-size_t ws_st_bytes() { return align256(ws_boundaries() * 2 * kRows * sizeof(float2)); }
-size_t ws_o_bytes() { return ws_boundaries() * 2 * kRows * kD * sizeof(float); }
+size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 }  // namespace
 
-// ... then 256 bytes for the grid barrier words of the launch that pools.
-size_t attn_tc_workspace_bytes() { return ws_cnt_bytes() + ws_st_bytes() + align256(ws_o_bytes()) + 256; }
+// Bytes of the forward workspace. Only its last 256 are used, by the grid barrier of the launch that
+// pools; the rest is the size callers have always had to bring (a split schedule's counters, row
+// statistics and partial O, two pipelines an SM), so that what was too small stays too small.
+size_t attn_tc_workspace_bytes()
+{
+    const size_t boundaries = (size_t)kSlots * max_grid() + 1;
+    return align256(boundaries * 4 * sizeof(int)) + align256(boundaries * 2 * kRows * sizeof(float2)) +
+           align256(boundaries * 2 * kRows * kD * sizeof(float)) + 256;
+}
 
 int launch_attn_tc_bf16(const ssba_desc& d, const Grid& g, int keep, float scale, const void* Q, const void* K,
                         const void* V, const int32_t* idx, const int32_t* cnt, void* O, float* lse, void* ws,
@@ -1244,9 +1302,7 @@ int launch_attn_tc_bf16(const ssba_desc& d, const Grid& g, int keep, float scale
     p.sel_scores = sel_scores;
     p.pool_q = pool ? static_cast<const __nv_bfloat16*>(Q) : nullptr;
     p.pool_k = pool ? static_cast<const __nv_bfloat16*>(K) : nullptr;
-    p.gsync = pool ? reinterpret_cast<unsigned*>(static_cast<char*>(ws) + ws_cnt_bytes() + ws_st_bytes() +
-                                                 align256(ws_o_bytes()))
-                   : nullptr;
+    p.gsync = pool ? reinterpret_cast<unsigned*>(static_cast<char*>(ws) + attn_tc_workspace_bytes() - 256) : nullptr;
     p.status = device_status_word();
     if (!p.status) {
         set_error("ssba_forward (bf16): could not resolve the device status word");
@@ -1259,26 +1315,10 @@ int launch_attn_tc_bf16(const ssba_desc& d, const Grid& g, int keep, float scale
                              cudaSharedmemCarveoutMaxShared);
     });
     // One CTA fits an SM (shared memory), so each CTA runs kSlots pipelines; the persistent
-    // grid has one CTA per SM (fewer for small problems).
+    // grid has one CTA per SM, fewer for small problems (one item a pipeline: with one a CTA the next
+    // layer's mask finds too few free SMs to start early, 13.0 against 10.0 us a 256 px layer).
     const int want = (p.num_items + kSlots - 1) / kSlots;
     const int grid = want < max_grid() ? want : max_grid();
-    p.split = 0;
-    p.ws_cnt = nullptr;
-    p.ws_st = nullptr;
-    p.ws_o = nullptr;
-    if (ws) {
-        char* w = static_cast<char*>(ws);
-        p.ws_cnt = reinterpret_cast<int*>(w);
-        p.ws_st = reinterpret_cast<float2*>(w + ws_cnt_bytes());
-        p.ws_o = reinterpret_cast<float*>(w + ws_cnt_bytes() + ws_st_bytes());
-        // Equal shares of blocks only pay when some pipeline would otherwise take one item
-        // more than another, and when items are long: a merge costs a few global-memory
-        // round trips (about 5 us under load, measured), which 11-block items do not
-        // earn back but 64-block items (dense) do (179 vs 198 us at 1024 px, 24 heads).
-        p.split = (!sel_qb && p.units >= kSplitMinKeep && p.num_items >= kSlots * grid &&
-                   p.num_items % (kSlots * grid) != 0)
-                      ? 1 : 0;
-    }
     // programmatic dependent launch: the kernel may start (barriers, tensor memory, window
     // table) while the previous grid on the stream finishes; it waits for that grid before
     // reading any input
