@@ -164,11 +164,15 @@ def _raise_on(rc: int) -> None:
 
 
 def _stream_ptr(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is None:  # the current stream, without building a torch.cuda.Stream (0.4 against 3.0 us)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return int(stream.cuda_stream)
 
 
 def _check(t: torch.Tensor, name: str, shape, dtype) -> None:
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.shape == shape
+            and t.is_contiguous()):
+        return
     if not isinstance(t, torch.Tensor):
         raise SsbaError(SSBA_ERR_INVALID, f"{name} must be a torch.Tensor")
     if t.device.type != "cuda":
@@ -181,13 +185,48 @@ def _check(t: torch.Tensor, name: str, shape, dtype) -> None:
         raise SsbaError(SSBA_ERR_INVALID, f"{name} must be contiguous")
 
 
+class _Plan:
+    """What the calls derive from a descriptor's values alone: the C struct, the list length and
+    the tensors' shapes. No tensor, pointer or device is kept."""
+    __slots__ = ("c", "ref", "keep", "dtype", "x", "rows", "means", "lists", "counts", "scores")
+
+    def __init__(self, lib, desc: SsbaDesc, c: _Desc):
+        self.c = c
+        self.ref = ctypes.byref(self.c)
+        self.keep = lib.ssba_keep_count(self.ref)
+        if self.keep < 0:
+            _raise_on(SSBA_ERR_INVALID)
+        B, h, Tb = desc.B, desc.heads, desc.Tb
+        self.dtype = desc.dtype
+        self.x = torch.Size((B, h, desc.N, desc.head_dim))
+        self.rows = self.x[:3]
+        self.means = torch.Size((B, h, Tb, desc.head_dim))
+        self.lists = torch.Size((B, h, Tb, self.keep))
+        self.counts = torch.Size((B, h, Tb))
+        self.scores = torch.Size((B, h, Tb, Tb))
+
+
+_PLAN_CAP = 256
+_plans: dict = {}
+
+
+def _plan(lib, desc: SsbaDesc) -> _Plan:
+    """The plan of a descriptor, kept by the bytes of its C struct (a model's layers share a few
+    descriptors; at the cap the table starts over). The struct is made anew each time, so whatever
+    it refuses is refused on every call."""
+    c = desc.c()
+    key = bytes(c)
+    pl = _plans.get(key)
+    if pl is None:
+        pl = _Plan(lib, desc, c)
+        if len(_plans) >= _PLAN_CAP:
+            _plans.clear()
+        _plans[key] = pl
+    return pl
+
+
 def keep_count(desc: SsbaDesc) -> int:
-    lib = load_library()
-    d = desc.c()
-    k = lib.ssba_keep_count(ctypes.byref(d))
-    if k < 0:
-        _raise_on(SSBA_ERR_INVALID)
-    return k
+    return _plan(load_library(), desc).keep
 
 
 def mask_workspace_bytes(desc: SsbaDesc) -> int:
@@ -202,6 +241,21 @@ def forward_workspace_bytes(desc: SsbaDesc) -> int:
     return int(lib.ssba_forward_workspace_bytes(ctypes.byref(d)))
 
 
+def _out(t, name: str, shape, dtype, dev):
+    """An output: allocated when the caller gave none, else checked."""
+    if t is None:
+        return torch.empty(shape, dtype=dtype, device=dev)
+    _check(t, name, shape, dtype)
+    return t
+
+
+def _scores_out(scores, pl: _Plan, dev):
+    if isinstance(scores, torch.Tensor):
+        _check(scores, "scores", pl.scores, torch.float32)
+        return scores
+    return torch.empty(pl.scores, dtype=torch.float32, device=dev) if scores else None
+
+
 _fwd_ws: dict = {}
 
 
@@ -212,9 +266,13 @@ def default_forward_workspace(desc: SsbaDesc, device, stream=None) -> torch.Tens
     streams get two workspaces, so they never share its counters or barrier words."""
     need = forward_workspace_bytes(desc)
     dev = torch.device(device)
-    idx = dev.index if dev.index is not None else torch.cuda.current_device()
-    with torch.cuda.device(idx):
+    cur = torch.cuda.current_device()
+    idx = dev.index if dev.index is not None else cur
+    if idx == cur:
         key = (idx, _stream_ptr(stream))
+    else:
+        with torch.cuda.device(idx):
+            key = (idx, _stream_ptr(stream))
     with _lock:
         ws = _fwd_ws.get(key)
         if ws is None or ws.numel() < need:
@@ -235,33 +293,18 @@ def build_mask(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, kv_idx=None, kv
                scores: bool | torch.Tensor = False, workspace=None, stream=None):
     """ssba_build_mask: returns (kv_idx [B,h,Tb,keep] int32, kv_cnt [B,h,Tb] int32[, S])."""
     lib = load_library()
-    d = desc.c()
-    keep = lib.ssba_keep_count(ctypes.byref(d))
-    if keep < 0:
-        _raise_on(SSBA_ERR_INVALID)
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
-    _check(Q, "Q", shp, desc.dtype)
-    _check(K, "K", shp, desc.dtype)
+    pl = _plan(lib, desc)
+    _check(Q, "Q", pl.x, pl.dtype)
+    _check(K, "K", pl.x, pl.dtype)
     dev = Q.device
-    if kv_idx is None:
-        kv_idx = torch.empty((desc.B, desc.heads, desc.Tb, keep), dtype=torch.int32, device=dev)
-    if kv_cnt is None:
-        kv_cnt = torch.empty((desc.B, desc.heads, desc.Tb), dtype=torch.int32, device=dev)
-    _check(kv_idx, "kv_idx", (desc.B, desc.heads, desc.Tb, keep), torch.int32)
-    _check(kv_cnt, "kv_cnt", (desc.B, desc.heads, desc.Tb), torch.int32)
-    S = None
-    if isinstance(scores, torch.Tensor):
-        S = scores
-        _check(S, "scores", (desc.B, desc.heads, desc.Tb, desc.Tb), torch.float32)
-    elif scores:
-        S = torch.empty((desc.B, desc.heads, desc.Tb, desc.Tb), dtype=torch.float32, device=dev)
-    ws_need = int(lib.ssba_mask_workspace_bytes(ctypes.byref(d)))
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev)
+    S = _scores_out(scores, pl, dev)
     if workspace is None:
-        workspace = torch.empty(ws_need, dtype=torch.uint8, device=dev)
-    rc = lib.ssba_build_mask(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), kv_idx.data_ptr(),
-                             kv_cnt.data_ptr(), S.data_ptr() if S is not None else None,
-                             workspace.data_ptr(), workspace.numel() * workspace.element_size(),
-                             _stream_ptr(stream))
+        workspace = torch.empty(int(lib.ssba_mask_workspace_bytes(pl.ref)), dtype=torch.uint8, device=dev)
+    rc = lib.ssba_build_mask(pl.ref, Q.data_ptr(), K.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
+                             S.data_ptr() if S is not None else None, workspace.data_ptr(),
+                             workspace.numel() * workspace.element_size(), _stream_ptr(stream))
     _raise_on(rc)
     return (kv_idx, kv_cnt, S) if S is not None else (kv_idx, kv_cnt)
 
@@ -271,25 +314,23 @@ def qkv_rope_pool(desc: SsbaDesc, X: torch.Tensor, Wqkv: torch.Tensor, bias=None
     """ssba_qkv_rope_pool: X [B, N, heads*64] -> (Q, K, V [B, heads, N, 64] bf16 with RoPE on Q
     and K, qb, kb [B, heads, Tb, 64] fp32 block means, or None when pooled is False)."""
     lib = load_library()
-    d = desc.c()
+    pl = _plan(lib, desc)
     Dm = desc.heads * desc.head_dim
     _check(X, "X", (desc.B, desc.N, Dm), torch.bfloat16)
     _check(Wqkv, "Wqkv", (3 * Dm, Dm), torch.bfloat16)
     if bias is not None:
         _check(bias, "bias", (3 * Dm,), torch.float32)
     dev = X.device
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
-    pshp = (desc.B, desc.heads, desc.Tb, desc.head_dim)
     if out is None:
-        out = [torch.empty(shp, dtype=torch.bfloat16, device=dev) for _ in range(3)]
-        out += [torch.empty(pshp, dtype=torch.float32, device=dev) for _ in range(2)] if pooled else [None, None]
+        out = [torch.empty(pl.x, dtype=torch.bfloat16, device=dev) for _ in range(3)]
+        out += [torch.empty(pl.means, dtype=torch.float32, device=dev) for _ in range(2)] if pooled else [None, None]
     Q, K, V, qb, kb = out
     for t, n in ((Q, "Q"), (K, "K"), (V, "V")):
-        _check(t, n, shp, torch.bfloat16)
+        _check(t, n, pl.x, torch.bfloat16)
     for t, n in ((qb, "qb"), (kb, "kb")):
         if t is not None:
-            _check(t, n, pshp, torch.float32)
-    _raise_on(lib.ssba_qkv_rope_pool(ctypes.byref(d), X.data_ptr(), Wqkv.data_ptr(),
+            _check(t, n, pl.means, torch.float32)
+    _raise_on(lib.ssba_qkv_rope_pool(pl.ref, X.data_ptr(), Wqkv.data_ptr(),
                                      bias.data_ptr() if bias is not None else None, Q.data_ptr(), K.data_ptr(),
                                      V.data_ptr(), qb.data_ptr() if qb is not None else None,
                                      kb.data_ptr() if kb is not None else None, _stream_ptr(stream)))
@@ -300,83 +341,51 @@ def select_mask(desc: SsbaDesc, qb: torch.Tensor, kb: torch.Tensor, kv_idx=None,
                 scores: bool | torch.Tensor = False, stream=None):
     """ssba_select_mask: block means -> (kv_idx, kv_cnt[, S]) as build_mask returns them."""
     lib = load_library()
-    d = desc.c()
-    keep = lib.ssba_keep_count(ctypes.byref(d))
-    if keep < 0:
-        _raise_on(SSBA_ERR_INVALID)
-    pshp = (desc.B, desc.heads, desc.Tb, desc.head_dim)
-    _check(qb, "qb", pshp, torch.float32)
-    _check(kb, "kb", pshp, torch.float32)
+    pl = _plan(lib, desc)
+    _check(qb, "qb", pl.means, torch.float32)
+    _check(kb, "kb", pl.means, torch.float32)
     dev = qb.device
-    if kv_idx is None:
-        kv_idx = torch.empty((desc.B, desc.heads, desc.Tb, keep), dtype=torch.int32, device=dev)
-    if kv_cnt is None:
-        kv_cnt = torch.empty((desc.B, desc.heads, desc.Tb), dtype=torch.int32, device=dev)
-    _check(kv_idx, "kv_idx", (desc.B, desc.heads, desc.Tb, keep), torch.int32)
-    _check(kv_cnt, "kv_cnt", (desc.B, desc.heads, desc.Tb), torch.int32)
-    S = None
-    if isinstance(scores, torch.Tensor):
-        S = scores
-        _check(S, "scores", (desc.B, desc.heads, desc.Tb, desc.Tb), torch.float32)
-    elif scores:
-        S = torch.empty((desc.B, desc.heads, desc.Tb, desc.Tb), dtype=torch.float32, device=dev)
-    _raise_on(lib.ssba_select_mask(ctypes.byref(d), qb.data_ptr(), kb.data_ptr(), kv_idx.data_ptr(),
-                                   kv_cnt.data_ptr(), S.data_ptr() if S is not None else None, _stream_ptr(stream)))
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev)
+    S = _scores_out(scores, pl, dev)
+    _raise_on(lib.ssba_select_mask(pl.ref, qb.data_ptr(), kb.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
+                                   S.data_ptr() if S is not None else None, _stream_ptr(stream)))
     return (kv_idx, kv_cnt, S) if S is not None else (kv_idx, kv_cnt)
 
 
 def pool_blocks(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, qb=None, kb=None, stream=None):
     """ssba_pool_blocks: (qb, kb) fp32 [B, heads, Tb, head_dim] block means of Q and K."""
     lib = load_library()
-    d = desc.c()
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
-    _check(Q, "Q", shp, desc.dtype)
-    _check(K, "K", shp, desc.dtype)
-    pshp = (desc.B, desc.heads, desc.Tb, desc.head_dim)
-    qb = torch.empty(pshp, dtype=torch.float32, device=Q.device) if qb is None else qb
-    kb = torch.empty(pshp, dtype=torch.float32, device=Q.device) if kb is None else kb
-    _check(qb, "qb", pshp, torch.float32)
-    _check(kb, "kb", pshp, torch.float32)
-    _raise_on(lib.ssba_pool_blocks(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), qb.data_ptr(), kb.data_ptr(),
+    pl = _plan(lib, desc)
+    _check(Q, "Q", pl.x, pl.dtype)
+    _check(K, "K", pl.x, pl.dtype)
+    qb = _out(qb, "qb", pl.means, torch.float32, Q.device)
+    kb = _out(kb, "kb", pl.means, torch.float32, Q.device)
+    _raise_on(lib.ssba_pool_blocks(pl.ref, Q.data_ptr(), K.data_ptr(), qb.data_ptr(), kb.data_ptr(),
                                    _stream_ptr(stream)))
     return qb, kb
 
 
 def _forward_select_call(fn_name, desc, Q, K, V, qb, kb, kv_idx, kv_cnt, scores, O, lse, workspace, stream):
     lib = load_library()
-    d = desc.c()
-    keep = keep_count(desc)
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
-    for t, n in ((Q, "Q"), (K, "K"), (V, "V")):
-        _check(t, n, shp, desc.dtype)
+    pl = _plan(lib, desc)
+    _check(Q, "Q", pl.x, pl.dtype)
+    _check(K, "K", pl.x, pl.dtype)
+    _check(V, "V", pl.x, pl.dtype)
     dev = Q.device
-    pshp = (desc.B, desc.heads, desc.Tb, desc.head_dim)
-    qb = torch.empty(pshp, dtype=torch.float32, device=dev) if qb is None else qb
-    kb = torch.empty(pshp, dtype=torch.float32, device=dev) if kb is None else kb
-    _check(qb, "qb", pshp, torch.float32)
-    _check(kb, "kb", pshp, torch.float32)
-    kv_idx = torch.empty((desc.B, desc.heads, desc.Tb, keep), dtype=torch.int32, device=dev) if kv_idx is None \
-        else kv_idx
-    kv_cnt = torch.empty((desc.B, desc.heads, desc.Tb), dtype=torch.int32, device=dev) if kv_cnt is None else kv_cnt
-    _check(kv_idx, "kv_idx", (desc.B, desc.heads, desc.Tb, keep), torch.int32)
-    _check(kv_cnt, "kv_cnt", (desc.B, desc.heads, desc.Tb), torch.int32)
-    S = None
-    if isinstance(scores, torch.Tensor):
-        S = scores
-        _check(S, "scores", (desc.B, desc.heads, desc.Tb, desc.Tb), torch.float32)
-    elif scores:
-        S = torch.empty((desc.B, desc.heads, desc.Tb, desc.Tb), dtype=torch.float32, device=dev)
-    O = torch.empty(shp, dtype=desc.dtype, device=dev) if O is None else O
-    lse = torch.empty(shp[:3], dtype=torch.float32, device=dev) if lse is None else lse
-    _check(O, "O", shp, desc.dtype)
-    _check(lse, "lse", shp[:3], torch.float32)
+    qb = _out(qb, "qb", pl.means, torch.float32, dev)
+    kb = _out(kb, "kb", pl.means, torch.float32, dev)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev)
+    S = _scores_out(scores, pl, dev)
+    O = _out(O, "O", pl.x, pl.dtype, dev)
+    lse = _out(lse, "lse", pl.rows, torch.float32, dev)
     if isinstance(workspace, str):
         workspace = default_forward_workspace(desc, dev, stream)
     wp, wn = _ws_args(workspace)
-    _raise_on(getattr(lib, fn_name)(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), V.data_ptr(), qb.data_ptr(),
-                                    kb.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
-                                    S.data_ptr() if S is not None else None, O.data_ptr(), lse.data_ptr(), wp, wn,
-                                    _stream_ptr(stream)))
+    _raise_on(getattr(lib, fn_name)(pl.ref, Q.data_ptr(), K.data_ptr(), V.data_ptr(), qb.data_ptr(), kb.data_ptr(),
+                                    kv_idx.data_ptr(), kv_cnt.data_ptr(), S.data_ptr() if S is not None else None,
+                                    O.data_ptr(), lse.data_ptr(), wp, wn, _stream_ptr(stream)))
     return qb, kb, kv_idx, kv_cnt, S, O, lse
 
 
@@ -406,29 +415,15 @@ def build_mask_noalloc(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, kv_idx=
     """ssba_build_mask_noalloc: build_mask with the library's built-in scratch area (no
     workspace argument; see include/ssba.h for the size limit and the sharing rule)."""
     lib = load_library()
-    d = desc.c()
-    keep = lib.ssba_keep_count(ctypes.byref(d))
-    if keep < 0:
-        _raise_on(SSBA_ERR_INVALID)
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
-    _check(Q, "Q", shp, desc.dtype)
-    _check(K, "K", shp, desc.dtype)
+    pl = _plan(lib, desc)
+    _check(Q, "Q", pl.x, pl.dtype)
+    _check(K, "K", pl.x, pl.dtype)
     dev = Q.device
-    if kv_idx is None:
-        kv_idx = torch.empty((desc.B, desc.heads, desc.Tb, keep), dtype=torch.int32, device=dev)
-    if kv_cnt is None:
-        kv_cnt = torch.empty((desc.B, desc.heads, desc.Tb), dtype=torch.int32, device=dev)
-    _check(kv_idx, "kv_idx", (desc.B, desc.heads, desc.Tb, keep), torch.int32)
-    _check(kv_cnt, "kv_cnt", (desc.B, desc.heads, desc.Tb), torch.int32)
-    S = None
-    if isinstance(scores, torch.Tensor):
-        S = scores
-        _check(S, "scores", (desc.B, desc.heads, desc.Tb, desc.Tb), torch.float32)
-    elif scores:
-        S = torch.empty((desc.B, desc.heads, desc.Tb, desc.Tb), dtype=torch.float32, device=dev)
-    rc = lib.ssba_build_mask_noalloc(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), kv_idx.data_ptr(),
-                                     kv_cnt.data_ptr(), S.data_ptr() if S is not None else None,
-                                     _stream_ptr(stream))
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev)
+    S = _scores_out(scores, pl, dev)
+    rc = lib.ssba_build_mask_noalloc(pl.ref, Q.data_ptr(), K.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
+                                     S.data_ptr() if S is not None else None, _stream_ptr(stream))
     _raise_on(rc)
     return (kv_idx, kv_cnt, S) if S is not None else (kv_idx, kv_cnt)
 
@@ -438,25 +433,19 @@ def forward(desc: SsbaDesc, Q, K, V, kv_idx, kv_cnt, O=None, lse=None, workspace
     ``workspace``: "default" (the per-stream one of default_forward_workspace), None or a
     zero-filled uint8 CUDA tensor; the result is the same with each."""
     lib = load_library()
-    d = desc.c()
-    keep = lib.ssba_keep_count(ctypes.byref(d))
-    if keep < 0:
-        _raise_on(SSBA_ERR_INVALID)
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
-    for t, n in ((Q, "Q"), (K, "K"), (V, "V")):
-        _check(t, n, shp, desc.dtype)
-    _check(kv_idx, "kv_idx", (desc.B, desc.heads, desc.Tb, keep), torch.int32)
-    _check(kv_cnt, "kv_cnt", (desc.B, desc.heads, desc.Tb), torch.int32)
-    if O is None:
-        O = torch.empty(shp, dtype=desc.dtype, device=Q.device)
-    if lse is None:
-        lse = torch.empty(shp[:3], dtype=torch.float32, device=Q.device)
-    _check(O, "O", shp, desc.dtype)
-    _check(lse, "lse", shp[:3], torch.float32)
+    pl = _plan(lib, desc)
+    _check(Q, "Q", pl.x, pl.dtype)
+    _check(K, "K", pl.x, pl.dtype)
+    _check(V, "V", pl.x, pl.dtype)
+    _check(kv_idx, "kv_idx", pl.lists, torch.int32)
+    _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device)
     if isinstance(workspace, str):
-        workspace = default_forward_workspace(desc, Q.device, stream) if desc.dtype == torch.bfloat16 else None
+        # neither kernel uses one here (the fp32 one takes none; bf16 only checks what is given)
+        workspace = None
     wp, wn = _ws_args(workspace)
-    rc = lib.ssba_forward(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), V.data_ptr(), kv_idx.data_ptr(),
+    rc = lib.ssba_forward(pl.ref, Q.data_ptr(), K.data_ptr(), V.data_ptr(), kv_idx.data_ptr(),
                           kv_cnt.data_ptr(), O.data_ptr(), lse.data_ptr(), wp, wn, _stream_ptr(stream))
     _raise_on(rc)
     return O, lse
@@ -468,29 +457,22 @@ def forward_joint(desc: SsbaDesc, Q, K, V, K_txt, V_txt, kv_idx, kv_cnt, O=None,
     its text segment). K_txt, V_txt: [B, heads, T_txt, d] bf16. Returns (O, lse) of the
     image tokens."""
     lib = load_library()
-    d = desc.c()
-    keep = lib.ssba_keep_count(ctypes.byref(d))
-    if keep < 0:
-        _raise_on(SSBA_ERR_INVALID)
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
-    for t, n in ((Q, "Q"), (K, "K"), (V, "V")):
-        _check(t, n, shp, desc.dtype)
+    pl = _plan(lib, desc)
+    _check(Q, "Q", pl.x, pl.dtype)
+    _check(K, "K", pl.x, pl.dtype)
+    _check(V, "V", pl.x, pl.dtype)
     T_txt = int(K_txt.shape[2]) if isinstance(K_txt, torch.Tensor) and K_txt.dim() == 4 else -1
     tshp = (desc.B, desc.heads, max(T_txt, 0), desc.head_dim)
-    _check(K_txt, "K_txt", tshp, desc.dtype)
-    _check(V_txt, "V_txt", tshp, desc.dtype)
-    _check(kv_idx, "kv_idx", (desc.B, desc.heads, desc.Tb, keep), torch.int32)
-    _check(kv_cnt, "kv_cnt", (desc.B, desc.heads, desc.Tb), torch.int32)
-    if O is None:
-        O = torch.empty(shp, dtype=desc.dtype, device=Q.device)
-    if lse is None:
-        lse = torch.empty(shp[:3], dtype=torch.float32, device=Q.device)
-    _check(O, "O", shp, desc.dtype)
-    _check(lse, "lse", shp[:3], torch.float32)
+    _check(K_txt, "K_txt", tshp, pl.dtype)
+    _check(V_txt, "V_txt", tshp, pl.dtype)
+    _check(kv_idx, "kv_idx", pl.lists, torch.int32)
+    _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device)
     if isinstance(workspace, str):
-        workspace = default_forward_workspace(desc, Q.device, stream) if desc.dtype == torch.bfloat16 else None
+        workspace = None  # not used by this call
     wp, wn = _ws_args(workspace)
-    rc = lib.ssba_forward_joint(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), V.data_ptr(),
+    rc = lib.ssba_forward_joint(pl.ref, Q.data_ptr(), K.data_ptr(), V.data_ptr(),
                                 K_txt.data_ptr() if T_txt > 0 else None, V_txt.data_ptr() if T_txt > 0 else None,
                                 T_txt, kv_idx.data_ptr(), kv_cnt.data_ptr(), O.data_ptr(), lse.data_ptr(), wp, wn,
                                 _stream_ptr(stream))
@@ -501,20 +483,16 @@ def forward_joint(desc: SsbaDesc, Q, K, V, K_txt, V_txt, kv_idx, kv_cnt, O=None,
 def forward_dense(desc: SsbaDesc, Q, K, V, O=None, lse=None, workspace="default", stream=None):
     """ssba_forward_dense: dense softmax attention from the same build (workspace as in forward)."""
     lib = load_library()
-    d = desc.c()
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
-    for t, n in ((Q, "Q"), (K, "K"), (V, "V")):
-        _check(t, n, shp, desc.dtype)
-    if O is None:
-        O = torch.empty(shp, dtype=desc.dtype, device=Q.device)
-    if lse is None:
-        lse = torch.empty(shp[:3], dtype=torch.float32, device=Q.device)
-    _check(O, "O", shp, desc.dtype)
-    _check(lse, "lse", shp[:3], torch.float32)
+    pl = _plan(lib, desc)
+    _check(Q, "Q", pl.x, pl.dtype)
+    _check(K, "K", pl.x, pl.dtype)
+    _check(V, "V", pl.x, pl.dtype)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device)
     if isinstance(workspace, str):
-        workspace = default_forward_workspace(desc, Q.device, stream) if desc.dtype == torch.bfloat16 else None
+        workspace = None  # not used by this call
     wp, wn = _ws_args(workspace)
-    rc = lib.ssba_forward_dense(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(),
+    rc = lib.ssba_forward_dense(pl.ref, Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(),
                                 lse.data_ptr(), wp, wn, _stream_ptr(stream))
     _raise_on(rc)
     return O, lse
@@ -574,27 +552,18 @@ def backward(desc: SsbaDesc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, dQ=None, dK=No
     With _timeout_budget_ns set it calls the failure-detection test hook ssba_test_backward_timeout
     instead (see include/ssba.h): the gradients are then undefined."""
     lib = load_library()
-    d = desc.c()
-    keep = lib.ssba_keep_count(ctypes.byref(d))
-    if keep < 0:
-        _raise_on(SSBA_ERR_INVALID)
-    shp = (desc.B, desc.heads, desc.N, desc.head_dim)
+    pl = _plan(lib, desc)
     for t, n in ((Q, "Q"), (K, "K"), (V, "V"), (O, "O"), (dO, "dO")):
-        _check(t, n, shp, desc.dtype)
-    _check(lse, "lse", shp[:3], torch.float32)
-    _check(kv_idx, "kv_idx", (desc.B, desc.heads, desc.Tb, keep), torch.int32)
-    _check(kv_cnt, "kv_cnt", (desc.B, desc.heads, desc.Tb), torch.int32)
-    outs = []
-    for t, n in ((dQ, "dQ"), (dK, "dK"), (dV, "dV")):
-        if t is None:
-            t = torch.empty(shp, dtype=torch.float32, device=Q.device)
-        _check(t, n, shp, torch.float32)
-        outs.append(t)
-    need = int(lib.ssba_backward_workspace_bytes(ctypes.byref(d)))
+        _check(t, n, pl.x, pl.dtype)
+    _check(lse, "lse", pl.rows, torch.float32)
+    _check(kv_idx, "kv_idx", pl.lists, torch.int32)
+    _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
+    outs = [_out(t, n, pl.x, torch.float32, Q.device) for t, n in ((dQ, "dQ"), (dK, "dK"), (dV, "dV"))]
     if workspace is None:
+        need = int(lib.ssba_backward_workspace_bytes(pl.ref))
         workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=Q.device)
     wp, wn = _ws_args(workspace)
-    args = (ctypes.byref(d), Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), lse.data_ptr(), dO.data_ptr(),
+    args = (pl.ref, Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), lse.data_ptr(), dO.data_ptr(),
             kv_idx.data_ptr(), kv_cnt.data_ptr(), outs[0].data_ptr(), outs[1].data_ptr(), outs[2].data_ptr(), wp, wn)
     if _timeout_budget_ns is None:
         rc = lib.ssba_backward(*args, _stream_ptr(stream))
