@@ -6,120 +6,122 @@
 //   dV_m = sum_n p_nm dO_n
 //   ds_nm = p_nm (dO_n . v_m - D_n)
 //   dQ_n = scale sum_m ds_nm k_m,   dK_m = scale sum_n ds_nm q_n.
-// Two kernels, no atomics, deterministic:
-//   ssba_bwd_dq_kernel    one CTA per (batch*head, query block): two threads per query row
-//                         (interleaved halves of head_dim, as the fp32 forward), the kept key
-//                         blocks staged in shared memory in list order; writes dQ and D.
+// Two kernels, no atomics, deterministic, 128 threads a CTA, every product a register-tiled fp32 one
+// of 64 x 64 tiles in shared memory (simt_tile.cuh):
+//   ssba_bwd_dq_kernel    one CTA per (batch*head, query block): the kept key blocks staged in list
+//                         order; S = Q K^T, dP = dO V^T, dQ += dS K. dS takes the place of V, so
+//                         three CTAs fit an SM (70 KB each). Writes dQ and D.
 //   ssba_bwd_dkdv_kernel  one CTA per (batch*head, key block): finds, in ascending order, the
-//                         query blocks whose lists hold it, stages each one's Q and dO, and
-//                         accumulates dK and dV for its 64 key rows (two threads per row).
+//                         query blocks whose lists hold it, stages each one's Q and dO, and forms
+//                         S^T = K Q^T, dP^T = V dO^T, dV += P^T dO, dK += dS^T Q (P^T, then dS^T, in
+//                         one tile; two CTAs an SM, 87 KB each).
 #include "common.cuh"
+#include "simt_tile.cuh"
 
 namespace ssba {
 
 namespace {
 
-constexpr int kD = 64;            // head_dim of these kernels
-constexpr int kP = 64;            // tokens per block (8 x 8)
-constexpr int kThreads = 2 * kP;  // two threads per row
+using namespace simt;
 
-__device__ __forceinline__ float ld_f32(const float* p) { return __ldg(p); }
-__device__ __forceinline__ float ld_f32(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-
-// Stages rows g.token(label, p) of X (64 x 64, any dtype) as fp32 into dst.
-template <typename T>
-__device__ __forceinline__ void stage_block(float (*dst)[kD], const T* X, const Grid& g, int label)
-{
-    for (int e = threadIdx.x; e < kP * kD; e += kThreads) {
-        const int p = e / kD, c = e - p * kD;
-        dst[p][c] = ld_f32(X + (size_t)g.token(label, p) * kD + c);
-    }
-}
+constexpr size_t kDqSmem = 4 * kTileFloats * sizeof(float);
+constexpr size_t kDkvSmem = 5 * kTileFloats * sizeof(float);
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads) ssba_bwd_dq_kernel(
+__global__ void __launch_bounds__(kThreads, 3) ssba_bwd_dq_kernel(
     const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V, const T* __restrict__ O,
     const float* __restrict__ lse, const T* __restrict__ dO, Grid g, int keep, float scale,
     const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt, float* __restrict__ dQ,
     float* __restrict__ Dbuf)
 {
-    __shared__ float Ks[kP][kD];
-    __shared__ float Vs[kP][kD];
+    extern __shared__ float4 raw[];
+    float* Qs = reinterpret_cast<float*>(raw);
+    float* Gs = Qs + kTileFloats;
+    float* Ks = Gs + kTileFloats;
+    float* Vs = Ks + kTileFloats;  // then dS
     const int label = blockIdx.x, bh = blockIdx.y;
     const int Tb = g.Tb();
     const int N = g.H * g.W;
-    const int r = threadIdx.x >> 1, h = threadIdx.x & 1;
-    const int tok = g.token(label, r);
-    const size_t row = (size_t)bh * N + tok;
-
-    float q[kD / 2], go[kD / 2], dq[kD / 2];
-    float D = 0.f;
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    const size_t head = (size_t)bh * N * kD;
+    int qtok[kR];
+    row_tokens(g, label, qtok);
+    stage(Qs, Q + head, qtok);
+    stage(Gs, dO + head, qtok);
+    __syncthreads();
+    float D[kR], L[kR];
+    float2 dq[kR][2];
 #pragma unroll
-    for (int c = 0; c < kD / 2; ++c) {
-        q[c] = ld_f32(Q + row * kD + 2 * c + h);
-        go[c] = ld_f32(dO + row * kD + 2 * c + h);
-        D = fmaf(go[c], ld_f32(O + row * kD + 2 * c + h), D);
-        dq[c] = 0.f;
+    for (int a = 0; a < kR; ++a) {
+        const size_t row = (size_t)bh * N + qtok[a];
+        const float4 o = load4(O + row * kD + 4 * tx);
+        const float4 go = *reinterpret_cast<const float4*>(Gs + (ty + 8 * a) * kLd + 4 * tx);
+        D[a] = row_sum(fmaf(go.x, o.x, go.y * o.y) + fmaf(go.z, o.z, go.w * o.w));
+        L[a] = lse[row];
+        dq[a][0] = dq[a][1] = make_float2(0.f, 0.f);
+        if (tx == 0) Dbuf[row] = D[a];
     }
-    D += __shfl_xor_sync(0xffffffffu, D, 1);
-    const float L = lse[row];
     const int32_t* list = idx + ((size_t)bh * Tb + label) * keep;
     const int nblk = min(max(cnt[(size_t)bh * Tb + label], 0), keep);
     for (int t = 0; t < nblk; ++t) {
         const int j = list[t];
         if ((unsigned)j >= (unsigned)Tb) continue;  // malformed label: skipped, never read out of bounds
+        int tok[kR];
+        row_tokens(g, j, tok);
+        __syncthreads();  // the last block's K and dS are consumed
+        stage(Ks, K + head, tok);
+        stage(Vs, V + head, tok);
         __syncthreads();
-        stage_block(Ks, K + (size_t)bh * N * kD, g, j);
-        stage_block(Vs, V + (size_t)bh * N * kD, g, j);
-        __syncthreads();
-#pragma unroll 4
-        for (int p = 0; p < kP; ++p) {
-            float s = 0.f, dp = 0.f;
+        float s[kR][4], dp[kR][4];
+        dot_rows(s, Qs, Ks);
+        dot_rows(dp, Gs, Vs);
 #pragma unroll
-            for (int c = 0; c < kD / 2; ++c) {
-                s = fmaf(q[c], Ks[p][2 * c + h], s);
-                dp = fmaf(go[c], Vs[p][2 * c + h], dp);
+        for (int a = 0; a < kR; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const float pr = expf(s[a][b] * scale - L[a]);
+                s[a][b] = pr * (dp[a][b] - D[a]) * scale;
             }
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            dp += __shfl_xor_sync(0xffffffffu, dp, 1);
-            const float pr = expf(s * scale - L);
-            const float ds = pr * (dp - D) * scale;
-#pragma unroll
-            for (int c = 0; c < kD / 2; ++c) dq[c] = fmaf(ds, Ks[p][2 * c + h], dq[c]);
-        }
+        __syncthreads();  // V is consumed
+        put(Vs, s);
+        __syncthreads();
+        add_product(dq, Vs, Ks);
     }
 #pragma unroll
-    for (int c = 0; c < kD / 2; ++c) dQ[row * kD + 2 * c + h] = dq[c];
-    if (h == 0) Dbuf[row] = D;
+    for (int a = 0; a < kR; ++a)
+        *reinterpret_cast<float4*>(dQ + ((size_t)bh * N + qtok[a]) * kD + 4 * tx) =
+            make_float4(dq[a][0].x, dq[a][0].y, dq[a][1].x, dq[a][1].y);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads) ssba_bwd_dkdv_kernel(
+__global__ void __launch_bounds__(kThreads, 2) ssba_bwd_dkdv_kernel(
     const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V, const float* __restrict__ lse,
     const T* __restrict__ dO, const float* __restrict__ Dbuf, Grid g, int keep, float scale,
     const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt, float* __restrict__ dK,
     float* __restrict__ dV)
 {
-    __shared__ float Qs[kP][kD];
-    __shared__ float Gs[kP][kD];
+    extern __shared__ float4 raw[];
+    float* Ks = reinterpret_cast<float*>(raw);
+    float* Vs = Ks + kTileFloats;
+    float* Qs = Vs + kTileFloats;
+    float* Gs = Qs + kTileFloats;
+    float* Ps = Gs + kTileFloats;  // P^T, then dS^T
     __shared__ float Ls[kP], Ds[kP];
     __shared__ int qlist[kThreads];
     __shared__ int wcount[kThreads / 32];
     const int label = blockIdx.x, bh = blockIdx.y;
     const int Tb = g.Tb();
     const int N = g.H * g.W;
-    const int r = threadIdx.x >> 1, h = threadIdx.x & 1;
+    const int tx = threadIdx.x & 15;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const size_t krow = (size_t)bh * N + g.token(label, r);
-
-    float k[kD / 2], v[kD / 2], dk[kD / 2], dv[kD / 2];
+    const size_t head = (size_t)bh * N * kD;
+    int ktok[kR];
+    row_tokens(g, label, ktok);
+    stage(Ks, K + head, ktok);
+    stage(Vs, V + head, ktok);
+    float2 dk[kR][2], dv[kR][2];
 #pragma unroll
-    for (int c = 0; c < kD / 2; ++c) {
-        k[c] = ld_f32(K + krow * kD + 2 * c + h);
-        v[c] = ld_f32(V + krow * kD + 2 * c + h);
-        dk[c] = 0.f;
-        dv[c] = 0.f;
-    }
+    for (int a = 0; a < kR; ++a) dk[a][0] = dk[a][1] = dv[a][0] = dv[a][1] = make_float2(0.f, 0.f);
     // query blocks whose lists hold this key block, in ascending order, kThreads at a time
     for (int i0 = 0; i0 < Tb; i0 += kThreads) {
         const int i = i0 + threadIdx.x;
@@ -141,39 +143,43 @@ __global__ void __launch_bounds__(kThreads) ssba_bwd_dkdv_kernel(
         __syncthreads();
         for (int u = 0; u < total; ++u) {
             const int qi = qlist[u];
-            __syncthreads();
-            stage_block(Qs, Q + (size_t)bh * N * kD, g, qi);
-            stage_block(Gs, dO + (size_t)bh * N * kD, g, qi);
+            int tok[kR];
+            row_tokens(g, qi, tok);
+            __syncthreads();  // the last block's tiles are consumed
+            stage(Qs, Q + head, tok);
+            stage(Gs, dO + head, tok);
             if (threadIdx.x < kP) {
                 const size_t qrow = (size_t)bh * N + g.token(qi, threadIdx.x);
                 Ls[threadIdx.x] = lse[qrow];
                 Ds[threadIdx.x] = Dbuf[qrow];
             }
             __syncthreads();
-#pragma unroll 4
-            for (int n = 0; n < kP; ++n) {
-                float s = 0.f, dp = 0.f;
+            float s[kR][4];
+            dot_rows(s, Ks, Qs);
 #pragma unroll
-                for (int c = 0; c < kD / 2; ++c) {
-                    s = fmaf(k[c], Qs[n][2 * c + h], s);
-                    dp = fmaf(v[c], Gs[n][2 * c + h], dp);
-                }
-                s += __shfl_xor_sync(0xffffffffu, s, 1);
-                dp += __shfl_xor_sync(0xffffffffu, dp, 1);
-                const float pr = expf(s * scale - Ls[n]);
-                const float ds = pr * (dp - Ds[n]) * scale;
+            for (int a = 0; a < kR; ++a)
 #pragma unroll
-                for (int c = 0; c < kD / 2; ++c) {
-                    dv[c] = fmaf(pr, Gs[n][2 * c + h], dv[c]);
-                    dk[c] = fmaf(ds, Qs[n][2 * c + h], dk[c]);
-                }
-            }
+                for (int b2 = 0; b2 < 4; ++b2) s[a][b2] = expf(s[a][b2] * scale - Ls[tx + 16 * b2]);
+            put(Ps, s);
+            __syncthreads();
+            add_product(dv, Ps, Gs);
+            float dp[kR][4];
+            dot_rows(dp, Vs, Gs);
+#pragma unroll
+            for (int a = 0; a < kR; ++a)
+#pragma unroll
+                for (int b2 = 0; b2 < 4; ++b2) s[a][b2] = s[a][b2] * (dp[a][b2] - Ds[tx + 16 * b2]) * scale;
+            __syncthreads();  // P^T is consumed
+            put(Ps, s);
+            __syncthreads();
+            add_product(dk, Ps, Qs);
         }
     }
 #pragma unroll
-    for (int c = 0; c < kD / 2; ++c) {
-        dK[krow * kD + 2 * c + h] = dk[c];
-        dV[krow * kD + 2 * c + h] = dv[c];
+    for (int a = 0; a < kR; ++a) {
+        const size_t row = ((size_t)bh * N + ktok[a]) * kD + 4 * tx;
+        *reinterpret_cast<float4*>(dK + row) = make_float4(dk[a][0].x, dk[a][0].y, dk[a][1].x, dk[a][1].y);
+        *reinterpret_cast<float4*>(dV + row) = make_float4(dv[a][0].x, dv[a][0].y, dv[a][1].x, dv[a][1].y);
     }
 }
 
@@ -182,13 +188,18 @@ int launch_bwd_t(const ssba_desc& d, const Grid& g, int keep, float scale, const
                  const void* V, const void* O, const float* lse, const void* dO, const int32_t* idx,
                  const int32_t* cnt, float* dQ, float* dK, float* dV, float* Dbuf, cudaStream_t st)
 {
+    static PerDeviceOnce attr;  // one for each T
+    attr.run([] {
+        cudaFuncSetAttribute(ssba_bwd_dq_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDqSmem);
+        cudaFuncSetAttribute(ssba_bwd_dkdv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDkvSmem);
+    });
     dim3 grid(g.Tb(), d.B * d.heads);
-    ssba_bwd_dq_kernel<T><<<grid, kThreads, 0, st>>>(
+    ssba_bwd_dq_kernel<T><<<grid, kThreads, kDqSmem, st>>>(
         static_cast<const T*>(Q), static_cast<const T*>(K), static_cast<const T*>(V), static_cast<const T*>(O), lse,
         static_cast<const T*>(dO), g, keep, scale, idx, cnt, dQ, Dbuf);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
-        ssba_bwd_dkdv_kernel<T><<<grid, kThreads, 0, st>>>(
+        ssba_bwd_dkdv_kernel<T><<<grid, kThreads, kDkvSmem, st>>>(
             static_cast<const T*>(Q), static_cast<const T*>(K), static_cast<const T*>(V), lse,
             static_cast<const T*>(dO), Dbuf, g, keep, scale, idx, cnt, dK, dV);
         e = cudaGetLastError();

@@ -1,92 +1,102 @@
 // attn_simt.cu -- fp32 block-sparse attention forward on CUDA cores (Sec. 2.2
 // Efficient Sparse Execution; Algorithm 1 SparseAttention over the expanded mask).
 //
-// One CTA per (batch*head, query block), two threads per query row: each thread
-// owns the interleaved half {h, h+2, ...} of head_dim (so the two halves hit
-// adjacent shared-memory banks). The kept key blocks are visited in list order;
-// each block's K and V rows (gathered through the shifted grid, any shift) are
-// staged in shared memory and folded into an online softmax in fp32 with expf.
+// One CTA of 128 threads per (batch*head, query block). The kept key blocks are visited in list
+// order; each block's K and V rows (gathered through the shifted grid, any shift) are staged in
+// shared memory, S = Q K^T and O += P V run as register-tiled fp32 products (simt_tile.cuh), and the
+// block is folded into an online softmax with expf. P takes the place of K once S is done, so three
+// CTAs fit an SM (52 KB each).
 // This path serves fp32 inputs, where the tensor-core path's bf16 operands would
 // not meet fp32 accuracy.
 #include "common.cuh"
+#include "simt_tile.cuh"
 
 namespace ssba {
 
 namespace {
 
-constexpr int kD = 64;             // head_dim of this kernel
-constexpr int kP = 64;             // tokens per block (8 x 8)
-constexpr int kThreads = 2 * kP;   // two threads per query row
+using namespace simt;
 
-__global__ void __launch_bounds__(kThreads) ssba_attn_simt_f32_kernel(
+constexpr size_t kSmem = 3 * kTileFloats * sizeof(float);
+
+__global__ void __launch_bounds__(kThreads, 3) ssba_attn_simt_f32_kernel(
     const float* __restrict__ Q, const float* __restrict__ K, const float* __restrict__ V, Grid g, int keep,
     float scale, const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt, float* __restrict__ O,
     float* __restrict__ lse)
 {
-    __shared__ float Ks[kP][kD];
-    __shared__ float Vs[kP][kD];
+    extern __shared__ float4 raw[];
+    float* Qs = reinterpret_cast<float*>(raw);
+    float* Ks = Qs + kTileFloats;  // then P
+    float* Vs = Ks + kTileFloats;
     const int label = blockIdx.x, bh = blockIdx.y;
     const int Tb = g.Tb();
     const int N = g.H * g.W;
-    const int r = threadIdx.x >> 1, h = threadIdx.x & 1;
-    const int tok = g.token(label, r);
-    const float* Qh = Q + (size_t)bh * N * kD;
+    const int tx = threadIdx.x & 15;
     const float* Kh = K + (size_t)bh * N * kD;
     const float* Vh = V + (size_t)bh * N * kD;
+    int qtok[kR];
+    row_tokens(g, label, qtok);
+    stage(Qs, Q + (size_t)bh * N * kD, qtok);
 
-    float q[kD / 2], o[kD / 2];
+    float2 o[kR][2];
+    float m[kR], l[kR];  // l: this thread's part of the row sums
 #pragma unroll
-    for (int c = 0; c < kD / 2; ++c) {
-        q[c] = Qh[(size_t)tok * kD + 2 * c + h];
-        o[c] = 0.f;
+    for (int a = 0; a < kR; ++a) {
+        o[a][0] = o[a][1] = make_float2(0.f, 0.f);
+        m[a] = -INFINITY;
+        l[a] = 0.f;
     }
-    float m = -INFINITY, l = 0.f;
     const int32_t* list = idx + ((size_t)bh * Tb + label) * keep;
     const int nblk = min(max(cnt[(size_t)bh * Tb + label], 0), keep);
 
     for (int t = 0; t < nblk; ++t) {
         const int j = list[t];
         if ((unsigned)j >= (unsigned)Tb) continue;  // malformed label: skipped, never read out of bounds
+        int tok[kR];
+        row_tokens(g, j, tok);
+        __syncthreads();  // the last block's P and V are consumed
+        stage(Ks, Kh, tok);
+        stage(Vs, Vh, tok);
         __syncthreads();
-        for (int e = threadIdx.x; e < kP * (kD / 4); e += kThreads) {
-            int p = e / (kD / 4), c4 = e - p * (kD / 4);
-            int kt = g.token(j, p);
-            reinterpret_cast<float4*>(&Ks[p][0])[c4] =
-                __ldg(reinterpret_cast<const float4*>(Kh + (size_t)kt * kD) + c4);
-            reinterpret_cast<float4*>(&Vs[p][0])[c4] =
-                __ldg(reinterpret_cast<const float4*>(Vh + (size_t)kt * kD) + c4);
+        float s[kR][4];
+        dot_rows(s, Qs, Ks);
+#pragma unroll
+        for (int a = 0; a < kR; ++a) {
+            float bmax = -INFINITY;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                s[a][b] *= scale;
+                bmax = fmaxf(bmax, s[a][b]);
+            }
+            const float mnew = fmaxf(m[a], row_max(bmax));
+            const float alpha = expf(m[a] - mnew);  // 0 on the first block (m = -inf)
+            m[a] = mnew;
+            l[a] *= alpha;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                s[a][b] = expf(s[a][b] - mnew);
+                l[a] += s[a][b];
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                o[a][h].x *= alpha;
+                o[a][h].y *= alpha;
+            }
         }
+        __syncthreads();  // K is consumed
+        put(Ks, s);
         __syncthreads();
-        float s[kP];
-        float bmax = -INFINITY;
-#pragma unroll 8
-        for (int p = 0; p < kP; ++p) {
-            float acc = 0.f;
-#pragma unroll
-            for (int c = 0; c < kD / 2; ++c) acc = fmaf(q[c], Ks[p][2 * c + h], acc);
-            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-            s[p] = acc * scale;
-            bmax = fmaxf(bmax, s[p]);
-        }
-        const float mnew = fmaxf(m, bmax);
-        const float alpha = expf(m - mnew);  // 0 on the first block (m = -inf)
-        l *= alpha;
-#pragma unroll
-        for (int c = 0; c < kD / 2; ++c) o[c] *= alpha;
-#pragma unroll 8
-        for (int p = 0; p < kP; ++p) {
-            const float pr = expf(s[p] - mnew);
-            l += pr;
-#pragma unroll
-            for (int c = 0; c < kD / 2; ++c) o[c] = fmaf(pr, Vs[p][2 * c + h], o[c]);
-        }
-        m = mnew;
+        add_product(o, Ks, Vs);
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;  // an empty list gives O = 0, lse = -inf
-    float* Oh = O + (size_t)bh * N * kD + (size_t)tok * kD;
 #pragma unroll
-    for (int c = 0; c < kD / 2; ++c) Oh[2 * c + h] = o[c] * inv;
-    if (h == 0) lse[(size_t)bh * N + tok] = l > 0.f ? m + logf(l) : -INFINITY;
+    for (int a = 0; a < kR; ++a) {
+        const float sum = row_sum(l[a]);
+        const float inv = sum > 0.f ? 1.f / sum : 0.f;  // an empty list gives O = 0, lse = -inf
+        const size_t row = (size_t)bh * N + qtok[a];
+        *reinterpret_cast<float4*>(O + row * kD + 4 * tx) =
+            make_float4(o[a][0].x * inv, o[a][0].y * inv, o[a][1].x * inv, o[a][1].y * inv);
+        if (tx == 0) lse[row] = sum > 0.f ? m[a] + logf(sum) : -INFINITY;
+    }
 }
 
 }  // namespace
@@ -99,8 +109,12 @@ int launch_attn_simt_f32(const ssba_desc& d, const Grid& g, int keep, float scal
         set_error("ssba_forward (fp32): needs head_dim=%d and block=8", kD);
         return SSBA_ERR_UNSUPPORTED;
     }
+    static PerDeviceOnce attr;
+    attr.run([] {
+        cudaFuncSetAttribute(ssba_attn_simt_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    });
     dim3 grid(g.Tb(), d.B * d.heads);
-    ssba_attn_simt_f32_kernel<<<grid, kThreads, 0, st>>>(Q, K, V, g, keep, scale, idx, cnt, O, lse);
+    ssba_attn_simt_f32_kernel<<<grid, kThreads, kSmem, st>>>(Q, K, V, g, keep, scale, idx, cnt, O, lse);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("ssba_attn_simt_f32_kernel launch: %s", cudaGetErrorString(e));
