@@ -248,7 +248,9 @@ int ssba_build_mask(const ssba_desc* desc, const void* Q, const void* K, int32_t
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     rc = launch_mask_fused(*desc, g, keep, Q, K, kv_idx, kv_cnt, scores_opt, st);
     if (rc != SSBA_ERR_UNSUPPORTED) return rc;
-    rc = launch_pool(*desc, g, Q, K, qb, kb, st);
+    // rows of up to 256 blocks: the means of ssba_pool_blocks, bit for bit, so that every way to such a
+    // row's list gives the same one
+    rc = g.Tb() <= 256 ? launch_pool_blocks(*desc, g, Q, K, qb, kb, st) : launch_pool(*desc, g, Q, K, qb, kb, st);
     if (rc != SSBA_OK) return rc;
     return launch_select(*desc, g, keep, qb, kb, kv_idx, kv_cnt, scores_opt, st);
 }

@@ -440,11 +440,12 @@ __device__ __forceinline__ void grid_barrier_reset(unsigned* w, unsigned n, unsi
 
 // A list entry: written earlier in this launch under in-kernel selection (read through L2),
 // else read-only input.
-__device__ __forceinline__ int ld_list(const TcParams& p, const int32_t* a) { return p.sel_qb ? __ldcg(a) : __ldg(a); }
+template <bool kSel>
+__device__ __forceinline__ int ld_list(const int32_t* a) { return kSel ? __ldcg(a) : __ldg(a); }
 
 // Score row and Top-k gating of one item (one warp), with the arithmetic and the selection code
 // of the mask kernels (S_j = q_b . k_b[j], four interleaved partial sums over d combined in a
-// fixed order; the total order of sel::rank_select, walked by sel::ballot_select on keys held
+// fixed order; walked by sel::ballot_select on keys held
 // in registers), so the same means give the same lists. kbs: the head's k_b
 // staged in shared memory, the 16-byte chunk c4 of row j at chunk c4 ^ (j & 15) (two lanes per
 // bank at most when 32 lanes read one column); qs: the item's q_b row in shared memory. Not
@@ -456,7 +457,6 @@ __device__ __noinline__ void select_item(const TcParams& p, int item, int lane, 
     const int Tb = p.g.Tb();
     const bool stamp = threadIdx.x == 0 && item == sel_first_item(p, blockIdx.x, gridDim.x * kSlots);
     if (stamp) TL_CTA(tl::kSelStart);
-    const float4* q4 = reinterpret_cast<const float4*>(qs);
     uint32_t key[kPer];
 #pragma unroll
     for (int m = 0; m < kPer; ++m) {
@@ -464,18 +464,9 @@ __device__ __noinline__ void select_item(const TcParams& p, int item, int lane, 
         key[m] = 0u;
         if (j < Tb) {
             const float* row = kbs + j * kD;
-            const int sw = j & 15;
-            float a[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int c4 = 0; c4 < kD / 4; ++c4) {
-                const float4 qv = q4[c4];
-                const float4 kv = *reinterpret_cast<const float4*>(row + 4 * (c4 ^ sw));
-                a[0] = fmaf(qv.x, kv.x, a[0]);
-                a[1] = fmaf(qv.y, kv.y, a[1]);
-                a[2] = fmaf(qv.z, kv.z, a[2]);
-                a[3] = fmaf(qv.w, kv.w, a[3]);
-            }
-            const float acc = (a[0] + a[1]) + (a[2] + a[3]);
+            float s1[1];
+            sel::affinity<1>(s1, qs, kD, [&](int c) { return *reinterpret_cast<const float4*>(row + 4 * (c ^ (j & 15))); });
+            const float acc = s1[0];
             if (p.sel_scores) p.sel_scores[(size_t)item * Tb + j] = acc;
             key[m] = sel::order_key(acc);
         }
@@ -489,6 +480,7 @@ __device__ __noinline__ void select_item(const TcParams& p, int item, int lane, 
 }
 
 // Round r of a pipeline from its schedule in shared memory.
+template <bool kSel>
 __device__ __forceinline__ Round get_round(const TcParams& p, const SlotCtl& c, int r)
 {
     Round rd;
@@ -500,7 +492,7 @@ __device__ __forceinline__ Round get_round(const TcParams& p, const SlotCtl& c, 
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         int n = p.units;
-        if (p.idx && !p.sel_qb)
+        if (!kSel && p.idx)
             n = p.ntxt + (2 * r + h < kCntCap ? c.cnts[2 * r + h] : min(max(__ldg(p.cnt + rd.item[h]), 0), p.keep));
         rd.nb[h] = n;
     }
@@ -515,10 +507,11 @@ __device__ __forceinline__ Round get_round(const TcParams& p, const SlotCtl& c, 
 // Fills the schedule of pipeline v (thread t of its nthr threads); see the work-schedule
 // comment above. Rounds r < rounds - 1 are the pairs of items first + r stride, + 1; the last one
 // is the pair (or, single set, the one item) at `last`.
-__device__ void build_schedule(const TcParams& p, SlotCtl& c, int v, int V, int t, int nthr)
+template <bool kSel>
+__device__ __forceinline__ void build_schedule(const TcParams& p, SlotCtl& c, int v, int V, int t, int nthr)
 {
     int first, stride, last, rounds, single;
-    if (p.sel_qb) {
+    if (kSel) {
         const int n = sel_item_count(p, v, V);
         first = sel_first_item(p, v, V);
         stride = 2;
@@ -535,7 +528,7 @@ __device__ void build_schedule(const TcParams& p, SlotCtl& c, int v, int V, int 
         single = n == 1;
         last = n > 0 ? base + v + min(v, pairs) : first + (full - 1) * stride;
     }
-    if (p.idx && !p.sel_qb)
+    if (!kSel && p.idx)
         for (int i = t; i < 2 * rounds && i < kCntCap; i += nthr) {
             const int r = i >> 1, item = (r == rounds - 1 ? last : first + r * stride) + (i & 1);
             if (item < p.num_items) c.cnts[i] = min(max(__ldg(p.cnt + item), 0), p.keep);
@@ -638,6 +631,11 @@ __device__ __forceinline__ void store_row(const TcParams& p, int item, int row, 
     p.lse[(size_t)bh * N + tok] = ok ? (m * 0.69314718055994531f + logf(l)) : -INFINITY;
 }
 
+// kSel: the lists are selected here, from means given or (p.pool_q) pooled here too; without it they are
+// given. Two kernels, so that the set-up of the one costs the pipelines of the other nothing: the
+// registers and the code of the whole kernel move with every edit of it (7 % of the forward on given
+// lists, measured, for a change inside select_item).
+template <bool kSel>
 __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_constant__ TileMaps maps,
                                                                    const TcParams p)
 {
@@ -666,7 +664,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         mbar_init(smem_u32(&sm.s_full), 1);
         mbar_init(smem_u32(&sm.s_free), 4);
         mbar_init(smem_u32(&sm.merged), 2);
-        if (p.pool_q)
+        if (kSel && p.pool_q)
             for (int w = slot * kPoolUnits; w < (slot + 1) * kPoolUnits; ++w) mbar_init(smem_u32(&cs.pool_bar[w]), 1);
         fence_mbar_init();
     }
@@ -682,7 +680,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
     if (threadIdx.x == 0) TL_CTA(tl::kDepWait);
     bool pool_fail = false;
     unsigned departed = 0;
-    if (p.pool_q) {
+    if (kSel && p.pool_q) {
         // the block means of the whole layer, the (block, tensor) units shared out over the grid,
         // then a grid barrier; the next grid is released only after it, so that it cannot take
         // an SM that one of these CTAs still waits for
@@ -719,7 +717,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
     const int vcta = slot * gridDim.x + blockIdx.x;
     const int vgrid = gridDim.x * kSlots;
     const int Tb = p.g.Tb();
-    if (p.sel_qb) {
+    if (kSel) {
         // the lists of this CTA's items (the contiguous ranges of its two pipelines): the k_b
         // of the heads they touch are staged by all threads in the stage buffers of both
         // pipelines (free until the producers start), one asynchronous round per batch of
@@ -794,10 +792,10 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         if (threadIdx.x == 0) TL_CTA(tl::kSelected);
         if (p.pool_q && threadIdx.x == 0 && !pool_fail) grid_barrier_reset(p.gsync, gridDim.x, departed);
     }
-    if (soft) build_schedule(p, ct, vcta, vgrid, threadIdx.x % (kSoftWarps * 32), kSoftWarps * 32);
+    if (soft) build_schedule<kSel>(p, ct, vcta, vgrid, threadIdx.x % (kSoftWarps * 32), kSoftWarps * 32);
     // the stage buffers held the pooled rows and the staged means (generic accesses); the
     // producers' tensor copies (async proxy) overwrite them next
-    if (p.sel_qb) fence_proxy_async_smem();
+    if (kSel) fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -827,7 +825,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         int nq = 0;      // rounds whose Q is announced
         auto entry_of = [&](int label) { return label < kWinCap ? cs.win[label] : window_entry(p.g, label); };
         for (int r = 0; !dead && r < rounds; ++r) {
-            const Round rd = get_round(p, ct, r);
+            const Round rd = get_round<kSel>(p, ct, r);
             const int steps = max(rd.nb[0], rd.nb[1]);
             const int bh0 = rd.item[0] / Tb, bh1 = rd.item[1] / Tb;
             if (kChecked && is_k && p.idx) {
@@ -838,11 +836,11 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
                     const int32_t* hl = p.idx + (size_t)rd.item[h] * p.keep;
                     const int a = max(rd.tb[h], p.ntxt) - p.ntxt, b = rd.tb[h] + rd.nb[h] - p.ntxt;
                     for (int t = a + lane; t < b; t += 32) {
-                        const int raw = ld_list(p, hl + t);
+                        const int raw = ld_list<kSel>(hl + t);
                         bad |= raw < 0 || raw >= Tb;
-                        if (t > 0) bad |= raw <= ld_list(p, hl + t - 1);
+                        if (t > 0) bad |= raw <= ld_list<kSel>(hl + t - 1);
                     }
-                    if (lane == 0 && !p.sel_qb) {
+                    if (lane == 0 && !kSel) {
                         const int c = __ldg(p.cnt + rd.item[h]);
                         bad |= c < 0 || c > p.keep;
                     }
@@ -871,7 +869,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
                 for (int h = 0; h < 2; ++h) {
                     const int t = t0 + lane, i = rd.tb[h] + t - p.ntxt;  // entry of the item's list
                     if (t < rd.nb[h] && i >= 0)
-                        ent[h] = entry_of(p.idx ? clamp_label(ld_list(p, p.idx + (size_t)rd.item[h] * p.keep + i), Tb) : i);
+                        ent[h] = entry_of(p.idx ? clamp_label(ld_list<kSel>(p.idx + (size_t)rd.item[h] * p.keep + i), Tb) : i);
                 }
                 const int te = min(t0 + 32, steps);
                 for (int t = t0; t < te; ++t) {
@@ -930,7 +928,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         const uint32_t kbase = smem_u32(&sm.k[0][0]);
         uint32_t g = 0;
         for (int r = 0; r < rounds && !*abortf; ++r) {
-            const Round rd = get_round(p, ct, r);
+            const Round rd = get_round<kSel>(p, ct, r);
             const int steps = max(rd.nb[0], rd.nb[1]), both = min(rd.nb[0], rd.nb[1]);
             const uint32_t one_b = rd.nb[1] > rd.nb[0] ? 1u : 0u;  // the half of the steps past `both`
             const uint32_t qaddr = smem_u32(&sm.q[0]);
@@ -976,7 +974,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         const uint32_t vbase = smem_u32(&sm.v[0][0]);
         uint32_t g = 0;
         for (int r = 0; r < rounds && !*abortf; ++r) {
-            const Round rd = get_round(p, ct, r);
+            const Round rd = get_round<kSel>(p, ct, r);
             const int steps = max(rd.nb[0], rd.nb[1]);
             for (int t = 0; t < steps; ++t, ++g) {
                 const uint32_t pb = g & 1, st = g % kStages;
@@ -1027,7 +1025,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         // writes the rows of round r's item, whose last PV is that of step `last`
         auto finish = [&](uint32_t last, int r) {
             wait_pv(last);
-            const Round rd = get_round(p, ct, r);
+            const Round rd = get_round<kSel>(p, ct, r);
             store_row(p, half ? rd.item[1] : rd.item[0], row, ocol, done_m, done_l, nullptr, 1.f, 0.f);
             tc_fence_before();
             owed = false;
@@ -1037,7 +1035,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
             int nb, steps, mask_t;  // mask_t: the step of the last text block, if that one is ragged
             bool parted;            // half B has blocks (of a split item: there is something to merge)
             {
-                const Round rd = get_round(p, ct, r);
+                const Round rd = get_round<kSel>(p, ct, r);
                 nb = half ? rd.nb[1] : rd.nb[0];
                 steps = max(rd.nb[0], rd.nb[1]);
                 mask_t = (p.t_txt & 63) ? p.ntxt - 1 - (half ? rd.tb[1] : rd.tb[0]) : -1;
@@ -1081,19 +1079,12 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
                     for (int h2 = 0; h2 < 2; ++h2) {
                         uint32_t pk[16];
 #pragma unroll
-                        for (int b = 0; b < 16; b += 8) {
-                            float2 x[8];
-#pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                x[i] = __ffma2_rn(make_float2(__uint_as_float(sr[32 * h2 + 2 * (b + i)]),
-                                                              __uint_as_float(sr[32 * h2 + 2 * (b + i) + 1])), c2, nm2);
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) x[i] = make_float2(fast_exp2(x[i].x), fast_exp2(x[i].y));
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                ls2[i & 3] = __fadd2_rn(ls2[i & 3], x[i]);
-                                pk[b + i] = pack_bf16(x[i].x, x[i].y);
-                            }
+                        for (int i = 0; i < 16; ++i) {
+                            const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[32 * h2 + 2 * i]),
+                                                                    __uint_as_float(sr[32 * h2 + 2 * i + 1])), c2, nm2);
+                            const float2 pp = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+                            ls2[i & 3] = __fadd2_rn(ls2[i & 3], pp);
+                            pk[i] = pack_bf16(pp.x, pp.y);
                         }
                         tmem_st_32x32b_x16(tq + kColP + (g & 1) * 32 + h2 * 16, pk);
                     }
@@ -1230,6 +1221,12 @@ PerDeviceOnce g_attn_attr;  // the kernel's shared-memory attributes, set once p
 }  // namespace
 
 namespace {
+// Items per SM up to which the selection (and the pooling) run inside the attention launch. A CTA has
+// 16 warps, one item each; beyond that its rows queue up while the tensor pipe waits, and separate
+// launches, which give every SM several CTAs' warps, are faster: 2048 px (40 items) 395 -> 360 us a
+// layer, four 1024 px images (40) 187 -> 176; at one 1024 px image (10) the single launch is (48.2
+// against 49.3 us).
+constexpr int kSelItems = 16;
 int max_grid() { return num_sms(); }
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 }  // namespace
@@ -1271,6 +1268,15 @@ int launch_attn_tc_bf16(const ssba_desc& d, const Grid& g, int keep, float scale
         return SSBA_ERR_WORKSPACE;
     }
     const int BH = d.B * d.heads;
+    if (sel_qb && withhold == 0 && BH * g.Tb() > kSelItems * max_grid()) {
+        int rc = pool ? launch_pool_blocks(d, g, Q, K, const_cast<float*>(sel_qb), const_cast<float*>(sel_kb), st)
+                      : SSBA_OK;
+        if (rc == SSBA_OK)
+            rc = launch_select(d, g, keep, sel_qb, sel_kb, const_cast<int32_t*>(idx), const_cast<int32_t*>(cnt),
+                               sel_scores, st);
+        if (rc != SSBA_OK) return rc;
+        return launch_attn_tc_bf16(d, g, keep, scale, Q, K, V, idx, cnt, O, lse, ws, ws_bytes, st, budget_ns);
+    }
     TileMaps maps;
     memset(&maps, 0, sizeof(maps));
     if (!encode_window_maps(maps.q, Q, BH, g.H, g.W) || !encode_window_maps(maps.k, K, BH, g.H, g.W) ||
@@ -1310,9 +1316,10 @@ int launch_attn_tc_bf16(const ssba_desc& d, const Grid& g, int keep, float scale
     }
     const size_t smem = sizeof(SmemLayout) + 1024;
     g_attn_attr.run([smem] {
-        cudaFuncSetAttribute(ssba_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(ssba_attn_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+        for (auto k : {ssba_attn_tc_kernel<false>, ssba_attn_tc_kernel<true>}) {
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        }
     });
     // One CTA fits an SM (shared memory), so each CTA runs kSlots pipelines; the persistent
     // grid has one CTA per SM, fewer for small problems (one item a pipeline: with one a CTA the next
@@ -1332,7 +1339,7 @@ int launch_attn_tc_bf16(const ssba_desc& d, const Grid& g, int keep, float scale
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, ssba_attn_tc_kernel, maps, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, sel_qb ? ssba_attn_tc_kernel<true> : ssba_attn_tc_kernel<false>, maps, p);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("ssba_attn_tc_kernel launch: %s", cudaGetErrorString(e));

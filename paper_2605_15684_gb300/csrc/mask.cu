@@ -6,13 +6,13 @@
 //                       means q_b, k_b (Eq. for q_b/k_b) to the workspace. Dominant cost:
 //                       reading Q and K once (algorithmic bytes 2 * B * heads * N *
 //                       head_dim * elem); HBM-bound.
-//   ssba_select_kernel  one warp per query block: S row = q_b[i] . k_b[j] for all j in
-//                       fp32, then an exact selection of the `keep` largest entries under
-//                       the total order (S descending, label ascending), i.e. the k_drop
+//   ssba_select64_kernel  (head_dim 64; ssba_select_kernel for other widths) S rows = q_b[i] . k_b[j]
+//                       for all j in fp32, then an exact selection of the `keep` largest entries
+//                       under the total order (S descending, label ascending), i.e. the k_drop
 //                       smallest are dropped and ties keep the lower label; the kept labels
 //                       are written in ascending order.
 //   ssba_mask_fused_kernel  both steps in one launch for head_dim 64, 8x8 blocks and at
-//                       most 256 blocks: a cluster of 8 CTAs per (batch, head) pools its
+//                       most 128 blocks: a cluster of 8 CTAs per (batch, head) pools its
 //                       blocks into shared memory, reads the head's k_b from the other CTAs
 //                       of the cluster (distributed shared memory), and selects its rows
 //                       (keys in registers, the radix walk of sel::ballot_select). No
@@ -154,15 +154,100 @@ __global__ void __launch_bounds__(128) ssba_pool_generic_kernel(const T* __restr
 constexpr int kSelWarps = 8;
 constexpr int kSelKeyChunk = 256;
 constexpr int kMaxTb = 2048;
-constexpr int kRankMaxTb = 256;  // rows up to this length use rank counting, longer ones radix select
+
+// Gating of `rows` rows of keys in shared memory (row r at S + r * Tb); kept labels of row r to
+// dst + r * keep.
+template <int kPer>
+__device__ __forceinline__ void select_rows(const uint32_t* S, int Tb, int keep, int lane, int32_t* dst, int rows)
+{
+    for (int r = 0; r < rows; ++r) {
+        uint32_t key[kPer];
+#pragma unroll
+        for (int m = 0; m < kPer; ++m) {
+            const int j = lane + 32 * m;
+            key[m] = j < Tb ? S[(size_t)r * Tb + j] : 0u;
+        }
+        sel::ballot_select<kPer>(key, Tb, keep, lane, dst + (size_t)r * keep);
+    }
+}
+
+// Affinity and gating for head_dim 64: a CTA takes kSelWarps * kRows rows of one head, warp w the rows
+// [w kRows, (w + 1) kRows) of them; the keys' means pass through shared memory 128 at a time (rows of
+// 68 floats: 8 consecutive rows cover the banks), a lane scores 4 keys against its warp's kRows rows,
+// and the walks (ballot_select) read the finished rows of keys back from shared memory.
+// What bounds it: the shared-memory reads of the scores (4 + kRows 16-byte chunks for 16 kRows
+// multiply-adds) and the counts of the gating. kRows (24 heads, us for 1, 2, 4): 510 blocks 94, 69, 64;
+// 324 blocks 50, 44, 40; 256 blocks 31, 25, 28; 64 blocks at batch 4 12.8, 9.9, 10.6, at batch 1 7.4,
+// 6.2, 9.6; 16 blocks 3.8, 4.5, 6.0 (fewer CTAs than SMs). The kernel before (one row a warp, keys
+// transposed one word at a time, a 32-bit radix walk over shared memory): 195, 91, 99, 15, 6.8, 3.0.
+constexpr int kSel64Keys = 128, kSel64Ld = 68;
+template <int kRows>
+__global__ void __launch_bounds__(kSelWarps * 32, kRows == 2 ? 3 : 2) ssba_select64_kernel(const float* __restrict__ qb,
+                                                                       const float* __restrict__ kb, int Tb, int keep,
+                                                                       int32_t* __restrict__ idx,
+                                                                       int32_t* __restrict__ cnt,
+                                                                       float* __restrict__ scores)
+{
+    constexpr int kD = 64, kCta = kSelWarps * kRows, kPerLane = kSel64Keys / 32;
+    extern __shared__ float4 raw[];
+    float* ks = reinterpret_cast<float*>(raw);
+    float* qs = ks + kSel64Keys * kSel64Ld;                      // [kCta][64]
+    uint32_t* S = reinterpret_cast<uint32_t*>(qs + kCta * kD);   // [kCta][Tb]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bh = blockIdx.y;
+    const int row0 = blockIdx.x * kCta + warp * kRows, rows = min(max(Tb - row0, 0), kRows);
+    const float4* kbh = reinterpret_cast<const float4*>(kb + (size_t)bh * Tb * kD);
+    ptx::grid_dep_wait();  // the means may come from the grid launched just before this one
+    ptx::grid_dep_launch();
+    // rows past Tb are zeros; a warp reads only its own rows
+    for (int e = lane; e < kRows * (kD / 4); e += 32)
+        reinterpret_cast<float4*>(qs + warp * kRows * kD)[e] =
+            e / (kD / 4) < rows ? __ldg(reinterpret_cast<const float4*>(qb + ((size_t)bh * Tb + row0) * kD) + e)
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t* Sw = S + (size_t)warp * kRows * Tb;
+    for (int j0 = 0; j0 < Tb; j0 += kSel64Keys) {
+        const int nk = min(kSel64Keys, Tb - j0);
+        __syncthreads();  // the last keys are consumed
+#pragma unroll
+        for (int i = 0; i < kSel64Keys * (kD / 4) / (kSelWarps * 32); ++i) {
+            const int e = threadIdx.x + i * kSelWarps * 32, j = e / (kD / 4), c = e % (kD / 4);
+            if (j < nk) *reinterpret_cast<float4*>(ks + j * kSel64Ld + 4 * c) = __ldg(kbh + (size_t)(j0 + j) * (kD / 4) + c);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < kPerLane; ++m) {
+            const int j = lane + 32 * m;
+            if (j >= nk) break;
+            float acc[kRows];
+            sel::affinity<kRows>(acc, qs + warp * kRows * kD, kD, [&](int c) {
+                return *reinterpret_cast<const float4*>(ks + j * kSel64Ld + 4 * c);
+            });
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+                if (r >= rows) break;
+                Sw[(size_t)r * Tb + j0 + j] = sel::order_key(acc[r]);
+                if (scores) scores[((size_t)bh * Tb + row0 + r) * Tb + j0 + j] = acc[r];
+            }
+        }
+    }
+    __syncwarp();
+    int32_t* dst = idx + ((size_t)bh * Tb + row0) * keep;
+    // only the lengths that launch_select gives to this kRows
+    if constexpr (kRows == 4) {
+        if (Tb <= 512) select_rows<16>(Sw, Tb, keep, lane, dst, rows);
+        else select_rows<32>(Sw, Tb, keep, lane, dst, rows);
+    } else {
+        if (Tb <= 64) select_rows<2>(Sw, Tb, keep, lane, dst, rows);
+        else if (kRows == 2 || Tb <= 256) select_rows<8>(Sw, Tb, keep, lane, dst, rows);
+        else select_rows<64>(Sw, Tb, keep, lane, dst, rows);
+    }
+    if (lane < rows) cnt[(size_t)bh * Tb + row0 + lane] = keep;
+}
 
 // One warp per query block (row i of S), kSelWarps rows per CTA.
 // smem: kbT [d][kSelKeyChunk + 1] (padded transpose of a key chunk) | q rows [kSelWarps][d]
 //       | S rows as order keys [kSelWarps][Tb]
 // S[i][j] = q_b[i] . k_b[j] in fp32 (FMA over d in order); the row is then reduced to its
-// `keep` largest entries under (S descending, label ascending): rank(j) = #{k : key_k > key_j,
-// or key_k == key_j and k < j} is unique, and j is kept iff rank(j) < keep. Kept labels
-// are written in ascending order.
+// `keep` largest entries under (S descending, label ascending), kept labels ascending.
 __global__ void __launch_bounds__(kSelWarps * 32) ssba_select_kernel(const float* __restrict__ qb,
                                                                      const float* __restrict__ kb, int Tb,
                                                                      int d, int keep,
@@ -221,10 +306,8 @@ __global__ void __launch_bounds__(kSelWarps * 32) ssba_select_kernel(const float
     if (!active) return;
     int32_t* dst = idx + rowoff * keep;
 
-    if (Tb <= 32) sel::rank_select<1>(S, Tb, keep, lane, dst);
-    else if (Tb <= 64) sel::rank_select<2>(S, Tb, keep, lane, dst);
-    else if (Tb <= 128) sel::rank_select<4>(S, Tb, keep, lane, dst);
-    else if (Tb <= kRankMaxTb) sel::rank_select<8>(S, Tb, keep, lane, dst);
+    if (Tb <= 64) select_rows<2>(S, Tb, keep, lane, dst, 1);
+    else if (Tb <= 256) select_rows<8>(S, Tb, keep, lane, dst, 1);
     else {
         // keep-th largest key by MSB-first radix select
         uint32_t prefix = 0, pmask = 0;
@@ -262,14 +345,14 @@ __global__ void __launch_bounds__(kSelWarps * 32) ssba_select_kernel(const float
 
 constexpr int kFuseCluster = 8;    // CTAs per (batch, head)
 constexpr int kFuseWarps = 8;
-constexpr int kFuseMaxTb = 256;
+// Longest rows of the fused build. With 256 blocks a head (2048 px) its 192 CTAs are 32 rows each and
+// fall unevenly on the SMs: 43 us, against 13 (pooling) + 25 (selection) for the two kernels; at 144
+// blocks 24 against 21; at 64 it takes 8.8 against 4.2 + 6.2.
+constexpr int kFuseMaxTb = 128;
 
-// Affinity row of one query block (S_j = q_b . k_b[j], four interleaved partial sums over d
-// combined in a fixed order, as ssba_select_kernel) with the keys kept in registers (lane l:
-// labels l + 32 m), then the radix walk of sel::ballot_select, which keeps the same labels as
-// sel::rank_select. kbs: the head's k_b by rows, the 16-byte chunk c4 of row j at chunk
-// c4 ^ (j & 15) (the 32 lanes reading one chunk of 32 rows cover all 32 banks: four wavefronts,
-// the least for 512 bytes).
+// Affinity row of one query block with the keys held in registers (lane l: labels l + 32 m), then
+// the gating. kbs: the head's k_b by rows, the 16-byte chunk c4 of row j at chunk c4 ^ (j & 15) (the 32
+// lanes reading one chunk of 32 rows cover all 32 banks: four wavefronts, the least for 512 bytes).
 template <int kPer>
 __device__ __forceinline__ void affinity_select(const float* q, const float* kbs, int Tb, int keep, int lane,
                                                 float* srow, int32_t* dst)
@@ -282,20 +365,12 @@ __device__ __forceinline__ void affinity_select(const float* q, const float* kbs
         key[m] = 0u;
         if (j < Tb) {
             const float* row = kbs + j * kD;
-            const int sw = j & 15;
-            float a[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int c = 0; c < kD; c += 4) {
-                const float4 qv = *reinterpret_cast<const float4*>(q + c);
-                const float4 kv = *reinterpret_cast<const float4*>(row + 4 * ((c >> 2) ^ sw));
-                a[0] = fmaf(qv.x, kv.x, a[0]);
-                a[1] = fmaf(qv.y, kv.y, a[1]);
-                a[2] = fmaf(qv.z, kv.z, a[2]);
-                a[3] = fmaf(qv.w, kv.w, a[3]);
-            }
-            const float acc = (a[0] + a[1]) + (a[2] + a[3]);
-            if (srow) srow[j] = acc;
-            key[m] = sel::order_key(acc);
+            float acc[1];
+            sel::affinity<1>(acc, q, kD, [&](int c) {
+                return *reinterpret_cast<const float4*>(row + 4 * (c ^ (j & 15)));
+            });
+            if (srow) srow[j] = acc[0];
+            key[m] = sel::order_key(acc[0]);
         }
     }
     sel::ballot_select<kPer>(key, Tb, keep, lane, dst);
@@ -421,8 +496,7 @@ __global__ void __launch_bounds__(kFuseWarps * 32) ssba_mask_fused_kernel(const 
         int32_t* dst = idx + rowoff * keep;
         if (Tb <= 32) affinity_select<1>(q, kbs, Tb, keep, lane, srow, dst);
         else if (Tb <= 64) affinity_select<2>(q, kbs, Tb, keep, lane, srow, dst);
-        else if (Tb <= 128) affinity_select<4>(q, kbs, Tb, keep, lane, srow, dst);
-        else affinity_select<8>(q, kbs, Tb, keep, lane, srow, dst);
+        else affinity_select<4>(q, kbs, Tb, keep, lane, srow, dst);
         if (lane == 0) cnt[rowoff] = keep;
     }
 }
@@ -566,6 +640,33 @@ int launch_select(const ssba_desc& d, const Grid& g, int keep, const float* qb, 
         set_error("ssba_build_mask: Tb=%d exceeds the selection kernel's limit of %d blocks", Tb, kMaxTb);
         return SSBA_ERR_UNSUPPORTED;
     }
+    if (d.head_dim == 64) {
+        const int BH = d.B * d.heads;
+        // rows a warp (see the kernel): few where every row counts for the spread over the SMs; one where
+        // four would not fit their keys
+        const int rows = Tb > 1024 ? 1 : (Tb > 256 ? 4 : ((long long)BH * Tb >= 10ll * device_sm_count() ? 2 : 1));
+        const int cta = kSelWarps * rows;
+        const size_t sm = ((size_t)kSel64Keys * kSel64Ld + (size_t)cta * 64 + (size_t)cta * Tb) * sizeof(float);
+        auto kernel = rows == 4 ? ssba_select64_kernel<4> : (rows == 2 ? ssba_select64_kernel<2> : ssba_select64_kernel<1>);
+        if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((Tb + cta - 1) / cta, BH, 1);
+        cfg.blockDim = dim3(kSelWarps * 32, 1, 1);
+        cfg.dynamicSmemBytes = sm;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, qb, kb, Tb, keep, idx, cnt, scores);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e != cudaSuccess) {
+            set_error("ssba_select64_kernel launch: %s", cudaGetErrorString(e));
+            return SSBA_ERR_CUDA;
+        }
+        return SSBA_OK;
+    }
     size_t smem = ((size_t)d.head_dim * (kSelKeyChunk + 1) + (size_t)kSelWarps * d.head_dim +
                    (size_t)kSelWarps * Tb) * sizeof(float);
     if (smem > 220 * 1024) {
@@ -598,7 +699,11 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     const int Tb = g.Tb();
     if (d.head_dim != 64 || g.blk != 8 || Tb > kFuseMaxTb) return SSBA_ERR_UNSUPPORTED;
     const int bpc = (Tb + kFuseCluster - 1) / kFuseCluster;
-    const size_t smem = ((size_t)bpc * 64 + (size_t)Tb * 64) * sizeof(float);
+    size_t smem = ((size_t)bpc * 64 + (size_t)Tb * 64) * sizeof(float);
+    // The kernel's registers let three CTAs share an SM. A grid of up to two an SM asks for shared memory
+    // that only two fit in, so that its clusters spread: 1024 px mask and forward 49.6 -> 46.8 us, 768 x
+    // 1408 px 56.3 -> 53.1 (batch 4, with more CTAs than that, is faster with three: 29.9 -> 28.7).
+    if (d.B * d.heads * kFuseCluster <= 2 * device_sm_count() && smem < 80 * 1024) smem = 80 * 1024;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kFuseCluster, d.B * d.heads, 1);
     cfg.blockDim = dim3(kFuseWarps * 32, 1, 1);
@@ -613,18 +718,15 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e;
-    if (d.dtype == SSBA_BF16) {
-        auto k = ssba_mask_fused_kernel<__nv_bfloat16>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        e = cudaLaunchKernelEx(&cfg, k, static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K),
-                               g, keep, bpc, idx, cnt, scores);
-    } else {
-        auto k = ssba_mask_fused_kernel<float>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        e = cudaLaunchKernelEx(&cfg, k, static_cast<const float*>(Q), static_cast<const float*>(K), g, keep, bpc, idx,
-                               cnt, scores);
-    }
+    auto launch = [&](auto kernel, auto q, auto k) {
+        if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return cudaLaunchKernelEx(&cfg, kernel, q, k, g, keep, bpc, idx, cnt, scores);
+    };
+    const cudaError_t e =
+        d.dtype == SSBA_BF16
+            ? launch(ssba_mask_fused_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(Q),
+                     static_cast<const __nv_bfloat16*>(K))
+            : launch(ssba_mask_fused_kernel<float>, static_cast<const float*>(Q), static_cast<const float*>(K));
     if (e != cudaSuccess) {
         set_error("ssba_mask_fused_kernel launch: %s", cudaGetErrorString(e));
         return SSBA_ERR_CUDA;

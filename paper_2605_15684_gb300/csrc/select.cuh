@@ -16,48 +16,81 @@ __device__ __forceinline__ uint32_t order_key(float s)
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Kept labels of one row by rank counting; lane l owns labels l + 32m, m < kPer.
-template <int kPer>
-__device__ __forceinline__ void rank_select(const uint32_t* S, int Tb, int keep, int lane, int32_t* dst)
+// The float whose key is u.
+__device__ __forceinline__ float key_value(uint32_t u)
 {
-    uint32_t mine[kPer];
-    int rank[kPer];
-#pragma unroll
-    for (int m = 0; m < kPer; ++m) {
-        const int j = lane + 32 * m;
-        mine[m] = j < Tb ? S[j] : 0u;
-        rank[m] = 0;
-    }
-#pragma unroll 8
-    for (int k = 0; k < Tb; ++k) {
-        const uint32_t v = S[k];  // broadcast read
-#pragma unroll
-        for (int m = 0; m < kPer; ++m) rank[m] += (v > mine[m]) || (v == mine[m] && k < lane + 32 * m);
-    }
-    int out = 0;
-#pragma unroll
-    for (int m = 0; m < kPer; ++m) {
-        const int j = lane + 32 * m;
-        const bool kept = j < Tb && rank[m] < keep;
-        const uint32_t km = __ballot_sync(0xffffffffu, kept);
-        if (kept) dst[out + __popc(km & ((1u << lane) - 1u))] = j;
-        out += __popc(km);
-    }
+    return __uint_as_float((u & 0x80000000u) ? (u ^ 0x80000000u) : ~u);
 }
 
-// The same selection with the keys in registers (lane l holds the keys of labels l + 32 m,
-// 0 for labels >= Tb): an MSB-first radix walk over ballots narrows the keys whose high bits
-// equal a prefix to the group that holds the keep-th largest key; keys above the group are
-// kept, and within it the largest ones, the first equal ones in label order. The walk stops as
-// soon as the group holds exactly the keys still to keep (all of it is then kept; for random
-// scores after about a dozen of the 32 bits). Same total order, so the same lists as
-// rank_select; kPer ballots a round instead of Tb shared-memory reads.
+// Kept labels of one row, ascending, with the keys in registers (lane l holds the keys of labels
+// l + 32 m, anything for labels >= Tb): the keep largest under the total order (S descending, label
+// ascending), every path's rule, so the same scores give the same lists.
+//   1. Rows of more than 128 labels: a threshold with exactly keep keys at or above it is looked for
+//      between the row's smallest and largest value, each guess interpolated from the counts at the
+//      two ends (and halfway where two guesses in a row moved the same end): about five counts for
+//      random scores, a count being one ballot per 32 keys. Where there is one, the kept set is unique
+//      and this is it.
+//   2. Shorter rows, and otherwise (equal scores across the cut, infinities, NaN): an MSB-first radix
+//      walk narrows the keys whose high bits equal a prefix to the group that holds the keep-th largest
+//      key; keys above the group are kept, and within it the largest ones, the first equal ones in
+//      label order. It stops once the group holds exactly the keys still to keep: about sixteen
+//      counts, half of them over exponent bits that every score shares.
+// Selection with the walk alone against both: 510 labels 83 -> 65 us, 256 labels 26 -> 24. With 64
+// labels a count is two ballots and the code costs more than the counts: a 1024 px mask and forward 46.8
+// us with the walk, 49.2 with both.
 template <int kPer>
 __device__ __forceinline__ void ballot_select(const uint32_t (&key)[kPer], int Tb, int keep, int lane, int32_t* dst)
 {
     bool valid[kPer];
 #pragma unroll
     for (int m = 0; m < kPer; ++m) valid[m] = lane + 32 * m < Tb;
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+    if (kPer >= 8) {
+#pragma unroll
+        for (int m = 0; m < kPer; ++m)
+            if (valid[m]) {
+                kmin = min(kmin, key[m]);
+                kmax = max(kmax, key[m]);
+            }
+        kmin = __reduce_min_sync(0xffffffffu, kmin);
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
+    }
+    uint32_t at = kmin;  // keys >= at are kept, if n == keep
+    int n = Tb;
+    const float inf = __uint_as_float(0x7f800000u);
+    if (kPer >= 8 && n != keep && key_value(kmin) > -inf && key_value(kmax) < inf) {
+        float lo = key_value(kmin), hi = key_value(kmax);  // n_lo >= keep keys at or above lo, n_hi < keep above hi
+        int n_lo = Tb, n_hi = 0, moved = 0;
+        for (int step = 0; step < 16; ++step) {
+            const float f = (moved >= 2 || moved <= -2) ? 0.5f : __fdividef((float)(n_lo - keep) + 0.5f, (float)(n_lo - n_hi) + 1.f);
+            const float mid = lo + (hi - lo) * f;
+            at = order_key(mid);
+            n = 0;
+#pragma unroll
+            for (int m = 0; m < kPer; ++m) n += __popc(__ballot_sync(0xffffffffu, valid[m] && key[m] >= at));
+            if (n == keep) break;
+            if (n > keep) {
+                lo = mid;
+                n_lo = n;
+                moved = moved > 0 ? moved + 1 : 1;
+            } else {
+                hi = mid;
+                n_hi = n;
+                moved = moved < 0 ? moved - 1 : -1;
+            }
+        }
+    }
+    if (kPer >= 8 && n == keep) {
+        int out = 0;
+#pragma unroll
+        for (int m = 0; m < kPer; ++m) {
+            const bool kept = valid[m] && key[m] >= at;
+            const uint32_t km = __ballot_sync(0xffffffffu, kept);
+            if (kept) dst[out + __popc(km & ((1u << lane) - 1u))] = lane + 32 * m;
+            out += __popc(km);
+        }
+        return;
+    }
     uint32_t prefix = 0u, pmask = 0u;
     int remaining = keep, group = Tb;  // keys still to keep; keys whose bits under pmask equal prefix
     for (int bit = 31; bit >= 0 && group != remaining; --bit) {
@@ -87,6 +120,31 @@ __device__ __forceinline__ void ballot_select(const uint32_t (&key)[kPer], int T
         out += __popc(km);
         eq_seen += __popc(eqm);
     }
+}
+
+// One affinity S = q_b . k_b: four interleaved partial sums over d (components of 16-byte chunks, in
+// chunk order), added as (a0 + a1) + (a2 + a3), for kRows rows of q at once (each k chunk is read
+// once for all of them). q: row r at q + r * qld; chunk(c) gives k_b's c-th 16-byte chunk. Every
+// path uses this order, so the same means give the same scores and lists. The pairs (a0, a1) and
+// (a2, a3) go out as packed multiply-adds, with the roundings of single ones.
+template <int kRows, class Chunk>
+__device__ __forceinline__ void affinity(float (&s)[kRows], const float* q, int qld, Chunk chunk)
+{
+    float2 lo[kRows], hi[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) lo[r] = hi[r] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const float4 k = chunk(c);
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+            const float4 v = *reinterpret_cast<const float4*>(q + r * qld + 4 * c);
+            lo[r] = __ffma2_rn(make_float2(v.x, v.y), make_float2(k.x, k.y), lo[r]);
+            hi[r] = __ffma2_rn(make_float2(v.z, v.w), make_float2(k.z, k.w), hi[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) s[r] = (lo[r].x + lo[r].y) + (hi[r].x + hi[r].y);
 }
 
 }  // namespace sel
