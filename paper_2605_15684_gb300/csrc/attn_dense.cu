@@ -1,28 +1,35 @@
 // attn_dense.cu -- dense bf16 softmax attention on the sm_103a tensor cores: the 0 % sparsity
 // baseline of Table 2 (every key of the head), the denominator of the sparse kernel's speed-up.
 //
-// Without index lists every query shares every key, so tiles are 128 contiguous tokens and the
-// products run at M=128 (the sparse kernel's 64-row tiles are forced by its per-query-block
-// lists, and M=64 products run at half the per-SM rate):
+// Without index lists every query shares every key, so tiles are 128 contiguous tokens:
 //   S = Q_u K_j^T   tcgen05.mma kind::f16, M=128 N=128 K=16 x 4 (A = Q tile, B = K tile, both
 //                   K-major SW128 in shared memory)
 //   O += P V_j      M=128 N=64 K=16 x 8 (A = P, bf16, from tensor memory; B = V tile MN-major)
 // Work unit = one tile of 128 query rows of one (batch, head); it visits all N/128 key tiles.
 // Persistent CTAs, one per SM (their shared memory fills it), each running two independent
-// streams of units (unit v + r V for stream v of V), warp-specialised:
-//   warps 0, 1     TMA producers of stream 0, 1: the unit's Q tile (double-buffered), then K_j and
-//                  V_j into 2-stage rings (16 KB tiles, 128-row boxes of a [B*heads][N][64] map)
-//   warps 2, 3     MMA issuers of stream 0, 1 (one elected lane): QK_j once the softmax has
-//                  loaded S_{j-1}, then PV_{j-1} once its P is stored, so the tensor pipe has the
-//                  next QK while the softmax works
-//   warps 4-7      softmax of stream 0, warps 8-11 of stream 1: one thread per row (TMEM lane),
-//                  128 scores a tile read in four 32-column chunks twice (maximum, then exp2s and
-//                  the bf16 P store), lazy rescale of O by more than 2^8 as in the sparse kernel
-//   warps 12-15    epilogue of stream 0, warps 16-19 of stream 1: O / l in bf16 and lse
+// streams of units (unit v + r V for stream v of V), warp-specialised, 8 warps a stream (512
+// threads, 128 registers each):
+//   K producer, V producer   TMA: the unit's Q tile, then the key tiles into rings of three 16 KB
+//                  stages each (128-row boxes of a [B*heads][N][64] map)
+//   QK issuer      QK_j once the softmax has read S_{j-1}
+//   PV issuer      PV_j once P_j is stored and V_j has landed
+//   softmax        four warps, one thread per row (TMEM lane). Exp2 in the log2-scaled domain against a
+//                  reference max m, the first tile's row maximum: a tile's 128 scores are read once, in
+//                  four 32-column chunks, and become P at once. S is released when the last chunk is
+//                  in registers and the first three have been seen to sum to at most 2^24; where they
+//                  do not, the tile's maximum is taken, m raised, O rescaled and P formed again (as in
+//                  attn_tc.cu); where the last chunk alone does not, m is raised by a whole number and
+//                  P rescaled. At the end of a unit they write O / l in bf16 and lse.
 // TMEM of a stream: S 128 + P 64 (bf16 pairs) + O 64 = 256 columns; the two streams take 512.
-// Every mbarrier wait is bounded (globaltimer budget + CTA abort flag); a timeout is reported in
+// What bounds it: a tile takes about 1130 cycles of an SM, of which the tensor pipe is busy 608 (QK 4 x
+// 80, PV 8 x 36) and a scheduler's softmax warps about 800 (128 exp2s a row and what is around them).
+// 24 heads: 1024 px 137 -> 116 us (890 TFLOP/s; its last round of tiles leaves half the SMs idle), 2048
+// px 1852 -> 1513 us (1090 TFLOP/s), against the kernel that read S twice (maximum, then exp2s), had
+// one issuer for both products and 2-stage rings. Releasing S only after the last exp2s: 131 and 1772.
+// Every wait is bounded (globaltimer budget + CTA abort flag); a timeout is reported in
 // the device status word and the roles drain their copies and products before the CTA exits.
 #include <cuda.h>
+#include <cmath>
 #include <cstring>
 
 #include "common.cuh"
@@ -36,35 +43,41 @@ using namespace ptx;
 constexpr int kD = 64;
 constexpr int kTile = 128;                        // query rows of a unit = keys of a key tile
 constexpr uint32_t kTileBytes = kTile * kD * 2;   // 16 KB
-constexpr int kStages = 2;                        // K and V rings
+constexpr int kStages = 3;                        // K and V rings
 constexpr int kStreams = 2;
-constexpr int kWarps = 20;
-constexpr int kThreads = kWarps * 32;
+constexpr int kSoftWarps = 4;                     // softmax warps of a stream
+constexpr int kRoleWarps = 4;                     // K producer, QK issuer, V producer, PV issuer of a stream
+constexpr int kThreads = kStreams * (kSoftWarps + kRoleWarps) * 32;
+enum Role { kLoadK = 0, kQK = 1, kLoadV = 2, kPV = 3, kSoftmax = 4 };
 constexpr uint32_t kStreamCols = 256;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColS = 0;    // [0,128)
 constexpr uint32_t kColP = 128;  // [128,192)
 constexpr uint32_t kColO = 192;  // [192,256)
-constexpr float kRescaleLog2 = 8.0f;
+constexpr float kRaise = 16777216.f;  // 2^24: row sum of a tile above which the reference max is raised
 constexpr uint32_t kIdescQK = idesc_bf16_f32(128, 128, false, false);
 constexpr uint32_t kIdescPV = idesc_bf16_f32(128, 64, false, true);
 
 struct __align__(1024) StreamSmem {
-    uint8_t q[2][kTileBytes];
+    uint8_t q[kTileBytes];
     uint8_t k[kStages][kTileBytes];
     uint8_t v[kStages][kTileBytes];
-    float2 stats[2][kTile];  // (max in log2 units, row sum) per unit parity
-    uint64_t q_full[2], q_empty[2];
+};
+
+struct StreamCtl {
+    uint64_t q_full, q_empty;
     uint64_t k_full[kStages], k_empty[kStages];
     uint64_t v_full[kStages], v_empty[kStages];
-    uint64_t s_full, s_free, p_full, p_empty;
-    uint64_t stats_full[2], stats_free[2];
-    uint64_t o_full, o_free;
+    uint64_t s_full;  // QK_g has finished
+    uint64_t s_free;  // the four softmax warps have read S_g
+    uint64_t p_full;  // the four softmax warps have stored P_g (and read the last unit's O)
+    uint64_t o_full;  // PV_g has finished
     uint64_t drain[2];
 };
 
 struct __align__(1024) DenseSmem {
     StreamSmem st[kStreams];
+    StreamCtl ctl[kStreams];
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -107,33 +120,6 @@ __device__ __forceinline__ bool wait_raw(uint32_t bar, uint32_t parity, uint64_t
     return true;
 }
 
-// 32 lanes x 32 bits, 32 consecutive columns: thread i gets lane (base + i).
-__device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&r)[32])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-}
-
-__device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_t (&r)[32])
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-        : "memory");
-}
-
 // Units of stream v (V streams): v, v + V, v + 2V, ...
 __device__ __forceinline__ int stream_units(const DenseParams& p, int v, int V)
 {
@@ -141,7 +127,7 @@ __device__ __forceinline__ int stream_units(const DenseParams& p, int v, int V)
 }
 
 __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid_constant__ DenseMaps maps,
-                                                                    const __grid_constant__ DenseParams p)
+                                                                    const DenseParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     DenseSmem& cs = *reinterpret_cast<DenseSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -150,35 +136,29 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
     if (threadIdx.x == 0) {
         cs.abort_flag = 0;
         for (int s = 0; s < kStreams; ++s) {
-            StreamSmem& sm = cs.st[s];
-            for (int b = 0; b < 2; ++b) {
-                mbar_init(smem_u32(&sm.q_full[b]), 1);
-                mbar_init(smem_u32(&sm.q_empty[b]), 1);
-                mbar_init(smem_u32(&sm.stats_full[b]), 4);
-                mbar_init(smem_u32(&sm.stats_free[b]), 4);
-            }
+            StreamCtl& c = cs.ctl[s];
             for (int b = 0; b < kStages; ++b) {
-                mbar_init(smem_u32(&sm.k_full[b]), 1);
-                mbar_init(smem_u32(&sm.k_empty[b]), 1);
-                mbar_init(smem_u32(&sm.v_full[b]), 1);
-                mbar_init(smem_u32(&sm.v_empty[b]), 1);
+                mbar_init(smem_u32(&c.k_full[b]), 1);
+                mbar_init(smem_u32(&c.k_empty[b]), 1);
+                mbar_init(smem_u32(&c.v_full[b]), 1);
+                mbar_init(smem_u32(&c.v_empty[b]), 1);
             }
-            mbar_init(smem_u32(&sm.s_full), 1);
-            mbar_init(smem_u32(&sm.s_free), 4);
-            mbar_init(smem_u32(&sm.p_full), 4);
-            mbar_init(smem_u32(&sm.p_empty), 1);
-            mbar_init(smem_u32(&sm.o_full), 1);
-            mbar_init(smem_u32(&sm.o_free), 4);
-            mbar_init(smem_u32(&sm.drain[0]), 1);
-            mbar_init(smem_u32(&sm.drain[1]), 1);
+            mbar_init(smem_u32(&c.q_full), 1);
+            mbar_init(smem_u32(&c.q_empty), 1);
+            mbar_init(smem_u32(&c.s_full), 1);
+            mbar_init(smem_u32(&c.s_free), kSoftWarps);
+            mbar_init(smem_u32(&c.p_full), kSoftWarps);
+            mbar_init(smem_u32(&c.o_full), 1);
+            mbar_init(smem_u32(&c.drain[0]), 1);
+            mbar_init(smem_u32(&c.drain[1]), 1);
         }
         fence_mbar_init();
     }
-    if (warp == 2) {
+    if (warp == 1) {
         tmem_alloc(smem_u32(&cs.tmem_base), kTmemCols);
         tmem_relinquish();
     }
-    if (warp < 2 && lane == 0) {
+    if (warp == 2 && lane == 0) {
         tma_prefetch_desc(&maps.q);
         tma_prefetch_desc(&maps.k);
         tma_prefetch_desc(&maps.v);
@@ -190,261 +170,248 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
     // grid launched before this one)
     grid_dep_wait();
     grid_dep_launch();
-    // roles: stream of the warp, and its role
-    int stream, role;  // role 0 producer, 1 MMA, 2 softmax, 3 epilogue
-    if (warp < 2) { stream = warp; role = 0; }
-    else if (warp < 4) { stream = warp - 2; role = 1; }
-    else if (warp < 12) { stream = (warp - 4) / 4; role = 2; }
-    else { stream = (warp - 12) / 4; role = 3; }
+    // the softmax warps first, so that a stream's four are one per TMEM lane quadrant
+    const bool soft = warp < kStreams * kSoftWarps;
+    const int stream = soft ? warp / kSoftWarps : (warp - kStreams * kSoftWarps) / kRoleWarps;
+    const int role = soft ? kSoftmax : (warp - kStreams * kSoftWarps) % kRoleWarps;
     StreamSmem& sm = cs.st[stream];
+    StreamCtl& ct = cs.ctl[stream];
     const int V = gridDim.x * kStreams;
     const int v = stream * gridDim.x + blockIdx.x;  // stream-major numbering of the grid's streams
     const int nunits = stream_units(p, v, V);
     const uint32_t tbase = cs.tmem_base + stream * kStreamCols;
     volatile int* abortf = &cs.abort_flag;
+    const uint32_t abort_at = smem_u32(&cs.abort_flag);
     bool dead = false;
 
-    if (role == 0) {
-        // ------------------------------------------------------------ TMA producer
-        uint32_t gk = 0;  // key tiles loaded by this stream
+    if (role == kLoadK || role == kLoadV) {
+        // ------------------------------------------------------------ TMA producers
+        const bool is_k = role == kLoadK;
+        const uint32_t empty0 = smem_u32(is_k ? &ct.k_empty[0] : &ct.v_empty[0]);
+        const uint32_t full0 = smem_u32(is_k ? &ct.k_full[0] : &ct.v_full[0]);
+        const uint32_t tile0 = smem_u32(is_k ? &sm.k[0][0] : &sm.v[0][0]);
+        const CUtensorMap* map = is_k ? &maps.k : &maps.v;
+        uint32_t g = 0;  // key tiles announced
+        int nq = 0;      // units whose Q is announced
         if (lane == 0) {
             for (int n = 0; n < nunits && !dead; ++n) {
                 const int u = v + n * V, bh = u / p.nt, qt = u - bh * p.nt;
-                const uint32_t qb = n & 1;
-                if (!mbar_wait(smem_u32(&sm.q_empty[qb]), ((n >> 1) & 1) ^ 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
-                mbar_arrive_expect_tx(smem_u32(&sm.q_full[qb]), kTileBytes);
-                tma_load_3d(smem_u32(&sm.q[qb][0]), &maps.q, smem_u32(&sm.q_full[qb]), 0, qt * kTile, bh);
-                for (int j = 0; j < p.nt; ++j, ++gk) {
-                    const uint32_t slot = gk % kStages, ph = ((gk / kStages) & 1) ^ 1;
-                    if (!mbar_wait(smem_u32(&sm.k_empty[slot]), ph, abortf, p.budget_ns)) {
+                for (int j = 0; j < p.nt; ++j) {
+                    const uint32_t st = g % kStages;
+                    if (!mbar_wait(empty0 + 8 * st, ((g / kStages) & 1) ^ 1, abortf, p.budget_ns)) {
                         dead = true;
                         break;
                     }
-                    mbar_arrive_expect_tx(smem_u32(&sm.k_full[slot]), kTileBytes);
-                    tma_load_3d(smem_u32(&sm.k[slot][0]), &maps.k, smem_u32(&sm.k_full[slot]), 0, j * kTile, bh);
-                    if (!mbar_wait(smem_u32(&sm.v_empty[slot]), ph, abortf, p.budget_ns)) {
-                        dead = true;
-                        break;
+                    mbar_arrive_expect_tx(full0 + 8 * st, kTileBytes);
+                    tma_load_3d(tile0 + st * kTileBytes, map, full0 + 8 * st, 0, j * kTile, bh);
+                    ++g;
+                    if (is_k && j == 0) {  // the unit's Q after its first K: it waits longest
+                        if (!mbar_wait(smem_u32(&ct.q_empty), (n & 1) ^ 1, abortf, p.budget_ns)) {
+                            dead = true;
+                            break;
+                        }
+                        mbar_arrive_expect_tx(smem_u32(&ct.q_full), kTileBytes);
+                        tma_load_3d(smem_u32(&sm.q[0]), &maps.q, smem_u32(&ct.q_full), 0, qt * kTile, bh);
+                        ++nq;
                     }
-                    mbar_arrive_expect_tx(smem_u32(&sm.v_full[slot]), kTileBytes);
-                    tma_load_3d(smem_u32(&sm.v[slot][0]), &maps.v, smem_u32(&sm.v_full[slot]), 0, j * kTile, bh);
                 }
             }
             if (dead) {  // drain the copies that may still be in flight
-                for (uint32_t x = gk > kStages ? gk - kStages : 0; x < gk; ++x) {
-                    wait_raw(smem_u32(&sm.k_full[x % kStages]), (x / kStages) & 1, p.budget_ns);
-                    wait_raw(smem_u32(&sm.v_full[x % kStages]), (x / kStages) & 1, p.budget_ns);
-                }
+                for (uint32_t x = g > kStages ? g - kStages : 0; x < g; ++x)
+                    wait_raw(full0 + 8 * (x % kStages), (x / kStages) & 1, p.budget_ns);
+                if (nq > 0) wait_raw(smem_u32(&ct.q_full), (nq - 1) & 1, p.budget_ns);
             }
         }
         __syncwarp();
-    } else if (role == 1) {
-        // ------------------------------------------------------------ MMA issuer
-        // QK_j into S once the softmax has loaded S_{j-1}; then PV_{j-1} once P_{j-1} is stored.
+    } else if (role == kQK) {
+        // ------------------------------------------------------------ QK issuer
         const bool leader = elect_one_sync();
-        uint32_t gs = 0, gp = 0;  // key tiles through S; through P
-        auto do_pv = [&](int n, int j) -> bool {
-            const uint32_t slot = gp % kStages;
-            if (!mbar_wait(smem_u32(&sm.p_full), gp & 1, abortf, p.budget_ns)) return false;
-            if (j == 0 && n > 0 && !mbar_wait(smem_u32(&sm.o_free), (n - 1) & 1, abortf, p.budget_ns)) return false;
-            if (!mbar_wait(smem_u32(&sm.v_full[slot]), (gp / kStages) & 1, abortf, p.budget_ns)) return false;
-            tc_fence_after();
-            if (elect_one_sync()) {
-                const uint64_t vdesc = sdesc_sw128(smem_u32(&sm.v[slot][0]), 8192, 1024);
-#pragma unroll
-                for (int k = 0; k < kTile / 16; ++k)
-                    mma_ts(tbase + kColO, tbase + kColP + k * 8, vdesc + (uint64_t)(k * 128), kIdescPV,
-                           (j > 0 || k > 0) ? 1u : 0u);
-                mma_commit(smem_u32(&sm.v_empty[slot]));
-                mma_commit(smem_u32(&sm.p_empty));
-                if (j == p.nt - 1) mma_commit(smem_u32(&sm.o_full));
-            }
-            __syncwarp();
-            ++gp;
-            return true;
-        };
-        for (int n = 0; n < nunits && !dead; ++n) {
-            const uint32_t qb = n & 1;
-            if (!mbar_wait(smem_u32(&sm.q_full[qb]), (n >> 1) & 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            for (int j = 0; j < p.nt; ++j, ++gs) {
-                const uint32_t slot = gs % kStages;
-                if (gs >= 1u && !mbar_wait(smem_u32(&sm.s_free), (gs - 1) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
-                if (!mbar_wait(smem_u32(&sm.k_full[slot]), (gs / kStages) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
+        uint32_t g = 0;
+        for (int n = 0; n < nunits && !*abortf; ++n) {
+            wait_phase(smem_u32(&ct.q_full), n & 1, abort_at, p.budget_ns);
+            for (int j = 0; j < p.nt; ++j, ++g) {
+                const uint32_t st = g % kStages;
+                wait_phase(smem_u32(&ct.k_full[st]), (g / kStages) & 1, abort_at, p.budget_ns);
+                if (g >= 1) wait_phase(smem_u32(&ct.s_free), (g - 1) & 1, abort_at, p.budget_ns);
                 tc_fence_after();
                 if (elect_one_sync()) {
-                    const uint64_t adesc = sdesc_sw128(smem_u32(&sm.q[qb][0]), 16, 1024);
-                    const uint64_t bdesc = sdesc_sw128(smem_u32(&sm.k[slot][0]), 16, 1024);
+                    const uint64_t adesc = sdesc_sw128(smem_u32(&sm.q[0]), 16, 1024);
+                    const uint64_t bdesc = sdesc_sw128(smem_u32(&sm.k[st][0]), 16, 1024);
 #pragma unroll
                     for (int k = 0; k < kD / 16; ++k)
                         mma_ss(tbase + kColS, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), kIdescQK,
                                k > 0 ? 1u : 0u);
-                    mma_commit(smem_u32(&sm.s_full));
-                    mma_commit(smem_u32(&sm.k_empty[slot]));
-                    if (j == p.nt - 1) mma_commit(smem_u32(&sm.q_empty[qb]));
+                    mma_commit(smem_u32(&ct.s_full));
+                    mma_commit(smem_u32(&ct.k_empty[st]));
+                    if (j == p.nt - 1) mma_commit(smem_u32(&ct.q_empty));
                 }
                 __syncwarp();
-                if (j > 0 && !do_pv(n, j - 1)) {
-                    dead = true;
-                    break;
-                }
-            }
-            if (dead) break;
-            if (!do_pv(n, p.nt - 1)) {
-                dead = true;
-                break;
             }
         }
+        dead = *abortf != 0;
         if (dead && leader) {
-            mma_commit(smem_u32(&sm.drain[0]));
-            wait_raw(smem_u32(&sm.drain[0]), 0, p.budget_ns);
+            mma_commit(smem_u32(&ct.drain[0]));
+            wait_raw(smem_u32(&ct.drain[0]), 0, p.budget_ns);
         }
-    } else if (role == 2) {
-        // ------------------------------------------------------------ softmax
-        // Thread = row 32 quad + lane. Pass 1 reads the tile's 128 scores for the row maximum;
-        // pass 2 reads them again for exp2(s c - m), the row sum and the bf16 P store.
-        const int quad = warp & 3;
-        const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-        const uint32_t scol = tbase + lane_off + kColS, pcol = tbase + lane_off + kColP, ocol = tbase + lane_off + kColO;
+    } else if (role == kPV) {
+        // ------------------------------------------------------------ PV issuer
+        const bool leader = elect_one_sync();
+        uint32_t g = 0;
+        for (int n = 0; n < nunits && !*abortf; ++n)
+            for (int j = 0; j < p.nt; ++j, ++g) {
+                const uint32_t st = g % kStages;
+                wait_phase(smem_u32(&ct.v_full[st]), (g / kStages) & 1, abort_at, p.budget_ns);
+                wait_phase(smem_u32(&ct.p_full), g & 1, abort_at, p.budget_ns);
+                tc_fence_after();
+                if (elect_one_sync()) {
+                    const uint64_t vdesc = sdesc_sw128(smem_u32(&sm.v[st][0]), 8192, 1024);
+#pragma unroll
+                    for (int k = 0; k < kTile / 16; ++k)
+                        mma_ts(tbase + kColO, tbase + kColP + k * 8, vdesc + (uint64_t)(k * 128), kIdescPV,
+                               (j > 0 || k > 0) ? 1u : 0u);
+                    mma_commit(smem_u32(&ct.o_full));
+                    mma_commit(smem_u32(&ct.v_empty[st]));
+                }
+                __syncwarp();
+            }
+        dead = *abortf != 0;
+        if (dead && leader) {
+            mma_commit(smem_u32(&ct.drain[1]));
+            wait_raw(smem_u32(&ct.drain[1]), 0, p.budget_ns);
+        }
+    } else {
+        // ------------------------------------------------------------ softmax and output
+        const int quad = warp & 3, row = quad * 32 + lane;
+        const uint32_t tq = tbase + (static_cast<uint32_t>(quad * 32) << 16);
+        const uint32_t scol = tq + kColS, pcol = tq + kColP, ocol = tq + kColO;
         const float c = p.scale_log2;
-        uint32_t gs = 0;
-        for (int n = 0; n < nunits && !dead; ++n) {
+        uint32_t g = 0;
+        for (int n = 0; n < nunits && !*abortf; ++n) {
             float m_used = 0.f, l = 0.f;
-            for (int j = 0; j < p.nt; ++j, ++gs) {
-                if (!mbar_wait(smem_u32(&sm.s_full), gs & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
+            for (int j = 0; j < p.nt; ++j, ++g) {
+                wait_phase(smem_u32(&ct.s_full), g & 1, abort_at, p.budget_ns);
                 tc_fence_after();
-                float mx = -INFINITY;
-#pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {
-                    uint32_t a[32];
-                    tmem_ld_32x32b_x32(scol + 32 * ch, a);
-                    tmem_wait_ld();
-                    float t4[4] = {mx, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) t4[e & 3] = fmaxf(t4[e & 3], __uint_as_float(a[e]));
-                    mx = fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3]));
-                }
-                const float mx2 = mx * c;
-                // lazy rescale: the running max is raised only when it grows by more than
-                // 2^kRescaleLog2 (warp-uniform decision: O is rescaled by a warp-wide TMEM access)
-                bool rescale = false;
-                float alpha = 1.f;
-                if (j == 0) {
-                    m_used = mx2;
-                } else {
-                    const bool need = mx2 > m_used + kRescaleLog2;
-                    rescale = __any_sync(0xffffffffu, need);
-                    if (need) {
-                        alpha = fast_exp2(m_used - mx2);
-                        m_used = mx2;
-                    }
-                }
-                // the P buffer is free once PV_{j-1} has finished (O then holds every earlier PV)
-                if (gs >= 1u && !mbar_wait(smem_u32(&sm.p_empty), (gs - 1) & 1, abortf, p.budget_ns)) {
-                    dead = true;
-                    break;
-                }
-                tc_fence_after();
-                const float2 c2 = make_float2(c, c), nm2 = make_float2(-m_used, -m_used);
-                float2 ls2 = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {
-                    uint32_t r[32];
-                    tmem_ld_32x32b_x32(scol + 32 * ch, r);
-                    tmem_wait_ld();
-                    if (ch == 3) {  // S read in full: QK_{j+1} may overwrite it
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&sm.s_free));
-                    }
+                const float2 c2 = make_float2(c, c);
+                // P = exp2(s c - m) of one chunk in bf16 to tensor memory, its row sum onto ls2
+                float2 ls2[2];
+                auto exps = [&](int ch, const uint32_t (&r)[32]) {
+                    const float2 nm2 = make_float2(-m_used, -m_used);
                     uint32_t pk[16];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
-                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])),
-                                                    c2, nm2);
+                        const float2 x = __ffma2_rn(
+                            make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])), c2, nm2);
                         const float2 pp = make_float2(fast_exp2(x.x), fast_exp2(x.y));
-                        ls2 = __fadd2_rn(ls2, pp);
+                        ls2[e & 1] = __fadd2_rn(ls2[e & 1], pp);
                         pk[e] = pack_bf16(pp.x, pp.y);
                     }
                     tmem_st_32x32b_x16(pcol + 16 * ch, pk);
-                }
-                l = fmaf(l, alpha, ls2.x + ls2.y);
-                if (rescale) {
+                };
+                auto sum = [&] { return (ls2[0].x + ls2[1].x) + (ls2[0].y + ls2[1].y); };
+                auto rescale_o = [&](float alpha) {  // PV_{g-1} has finished
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        uint32_t o[32];
-                        tmem_ld_32x32b_x32(ocol + 32 * h, o);
+                    for (int h2 = 0; h2 < 4; ++h2) {
+                        uint32_t o[16];
+                        tmem_ld_32x32b_x16(ocol + h2 * 16, o);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                        tmem_st_32x32b_x32(ocol + 32 * h, o);
+                        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                        tmem_st_32x32b_x16(ocol + h2 * 16, o);
                     }
+                };
+                // P's buffer is free once PV_{g-1} has finished (O then holds every earlier PV)
+                if (g >= 1) wait_phase(smem_u32(&ct.o_full), (g - 1) & 1, abort_at, p.budget_ns);
+                tc_fence_after();
+                uint32_t r[32];
+                // chunks 0-2; the first tile takes its maximum first, and so does a tile whose sum
+                // comes out too large (S is still there)
+                bool over = j == 0;
+#pragma unroll 1
+                for (bool raise = j == 0;; raise = true) {
+                    if (raise) {
+                        float mx = -INFINITY;
+#pragma unroll
+                        for (int ch = 0; ch < 4; ++ch) {
+                            tmem_ld_32x32b_x32(scol + 32 * ch, r);
+                            tmem_wait_ld();
+                            float t4[4] = {mx, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                            for (int e = 0; e < 32; e += 2)
+                                t4[(e >> 1) & 3] = max3(t4[(e >> 1) & 3], __uint_as_float(r[e]), __uint_as_float(r[e + 1]));
+                            mx = fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3]));
+                        }
+                        const float mx2 = fmaxf(mx * c, -3.0e38f);  // finite, so that scores of -inf give P = 0
+                        const float alpha = over && j > 0 ? fast_exp2(m_used - mx2) : 1.f;
+                        m_used = over ? mx2 : m_used;
+                        l *= alpha;
+                        if (j > 0) rescale_o(alpha);
+                    }
+                    ls2[0] = ls2[1] = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int ch = 0; ch < 3; ++ch) {
+                        tmem_ld_32x32b_x32(scol + 32 * ch, r);
+                        tmem_wait_ld();
+                        exps(ch, r);
+                    }
+                    tmem_ld_32x32b_x32(scol + 96, r);
+                    over = !(sum() <= kRaise);
+                    tmem_wait_ld();
+                    if (raise || !__any_sync(0xffffffffu, over)) break;
                 }
+                const float ls012 = sum();
+                // S is read in full: QK_{g+1} may overwrite it
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ct.s_free));
+                exps(3, r);
+                float ls = sum();
+                over = j > 0 && !(ls <= kRaise);
+                if (__any_sync(0xffffffffu, over)) {
+                    // the last chunk alone came out too large: m is raised by a whole number, so that the
+                    // rest of P (bf16) is rescaled exactly
+                    float mx = __uint_as_float(r[0]);
+#pragma unroll
+                    for (int e = 1; e < 32; ++e) mx = fmaxf(mx, __uint_as_float(r[e]));
+                    const float up = over ? fmaxf(ceilf(mx * c - m_used), 0.f) : 0.f;
+                    const float alpha = fast_exp2(-up);
+                    rescale_o(alpha);
+#pragma unroll
+                    for (int ch = 0; ch < 3; ++ch) {
+                        uint32_t pk[16];
+                        tmem_wait_st();
+                        tmem_ld_32x32b_x16(pcol + 16 * ch, pk);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e)
+                            pk[e] = pack_bf16(__uint_as_float(pk[e] << 16) * alpha,
+                                              __uint_as_float(pk[e] & 0xffff0000u) * alpha);
+                        tmem_st_32x32b_x16(pcol + 16 * ch, pk);
+                    }
+                    l *= alpha;
+                    ls2[0] = ls2[1] = make_float2(0.f, 0.f);
+                    m_used += up;
+                    exps(3, r);
+                    ls = sum() + ls012 * alpha;
+                }
+                l += ls;
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sm.p_full));
+                if (lane == 0) mbar_arrive(smem_u32(&ct.p_full));
             }
-            if (dead) break;
-            const uint32_t eb = n & 1;
-            if (!mbar_wait(smem_u32(&sm.stats_free[eb]), ((n >> 1) & 1) ^ 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            sm.stats[eb][quad * 32 + lane] = make_float2(m_used, l);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sm.stats_full[eb]));
-        }
-    } else {
-        // ------------------------------------------------------------ epilogue
-        const int quad = warp & 3;
-        const int row = quad * 32 + lane;
-        const uint32_t ocol = tbase + (static_cast<uint32_t>(quad * 32) << 16) + kColO;
-        for (int n = 0; n < nunits && !dead; ++n) {
+            // the unit's rows: O / l in bf16 (two halves of 32 columns) and lse, after its last PV
             const int u = v + n * V, bh = u / p.nt, qt = u - bh * p.nt;
-            if (!mbar_wait(smem_u32(&sm.o_full), n & 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            // the row statistics first (the softmax hands them over after its last tile, before
-            // the last PV has finished), then O in two halves of 32 columns
-            const uint32_t eb = n & 1;
-            if (!mbar_wait(smem_u32(&sm.stats_full[eb]), (n >> 1) & 1, abortf, p.budget_ns)) {
-                dead = true;
-                break;
-            }
-            const float2 st = sm.stats[eb][row];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sm.stats_free[eb]));
-            const bool ok = st.y > 0.f;
-            const float inv = ok ? 1.f / st.y : 0.f;
+            wait_phase(smem_u32(&ct.o_full), (g - 1) & 1, abort_at, p.budget_ns);
+            tc_fence_after();
+            const bool ok = l > 0.f;
+            const float inv = ok ? 1.f / l : 0.f;
             const size_t tok = (size_t)bh * p.N + (size_t)qt * kTile + row;
             uint4* dst = reinterpret_cast<uint4*>(p.O + tok * kD);
-            tc_fence_after();
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 uint32_t o[32];
                 tmem_ld_32x32b_x32(ocol + 32 * h, o);
                 tmem_wait_ld();
-                if (h == 1) {  // O read in full: the next unit's first PV may overwrite it
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&sm.o_free));
-                }
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     uint4 w;
@@ -455,14 +422,16 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                     dst[4 * h + i] = w;
                 }
             }
-            p.lse[tok] = ok ? (st.x * 0.69314718055994531f + logf(st.y)) : -INFINITY;
+            p.lse[tok] = ok ? (m_used * 0.69314718055994531f + logf(l)) : -INFINITY;
+            tc_fence_before();  // the next unit's first PV, which waits for p_full, overwrites O
         }
+        dead = *abortf != 0;
     }
     if (dead) atomicExch(p.status, SSBA_ERR_TIMEOUT);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 2) tmem_dealloc(cs.tmem_base, kTmemCols);
+    if (warp == 1) tmem_dealloc(cs.tmem_base, kTmemCols);
 }
 
 // [B*heads][N][64] bf16 as a 3-D map with 128-row boxes (128-byte swizzle).

@@ -112,3 +112,26 @@ def test_infinite_values_stay_in_their_items():
     assert bool(hit.any()) and not bool(hit.all())
     assert torch.equal(O2[~hit], O[~hit]) and torch.equal(lse2, lse)
     assert not bool(torch.isfinite(O2[hit].float()).any())
+
+
+@pytest.mark.parametrize("scale,ramp", [(1.5, 1.0), (6.0, 1.0), (1.0, 12.0)])
+def test_dense_reference_maximum_raised(scale, ramp):
+    """The dense kernel's reference maximum: scores that outgrow the first tile's by more than 2^24, in the
+    first chunks of a tile (their P is formed again) and in the last one (the rest of P is rescaled)."""
+    H = W = 32
+    (q, k, v), _ = _inputs(3, H, W, 44)
+    k = (k.float() * torch.linspace(0.1, ramp, H * W).view(1, 1, -1, 1)).bfloat16()
+    if ramp > 1:  # every 128-key tile's largest scores in its last 32 keys
+        k = torch.where((torch.arange(H * W) % 128 < 96).view(1, 1, -1, 1), k * 0.05, k)
+    desc = api.SsbaDesc(1, 3, H, W, softmax_scale=scale)
+    O, lse = api.forward_dense(desc, q.cuda(), k.cuda(), v.cuda())
+    torch.cuda.synchronize()
+    for h in range(3):
+        s = (q[0, h].double() @ k[0, h].double().T).numpy() * np.float32(scale)
+        m = s.max(axis=1, keepdims=True)
+        e = np.exp(s - m)
+        ref = (e / e.sum(axis=1, keepdims=True)) @ v[0, h].double().numpy()
+        # as in test_reference_maximum_raised
+        tol = 2e-2 + 2.0 ** -20 * np.abs(m) * np.abs(v[0, h].double().numpy()).max()
+        assert np.all(np.abs(O[0, h].float().cpu().numpy() - ref) <= tol)
+        assert np.allclose(lse[0, h].cpu().numpy(), (m + np.log(e.sum(axis=1, keepdims=True)))[:, 0], rtol=1e-5, atol=1e-2)
