@@ -7,13 +7,19 @@
 //   Q, K = RoPE(Y_q), RoPE(Y_k), V = Y_v, each [B][heads][N][64] bf16
 //   q_b, k_b = block means of the bf16 Q and K, [B][heads][Tb][64] fp32
 //
-// Tile = 128 rows (two horizontally adjacent 8x8 windows of the shifted grid, one 16 x 8
-// token box per k step, so that the rows of a tile come from long runs of consecutive tokens:
-// measured, two 8 x 8 boxes per k step took the main loop from 35 to 47 us at 1024 px) x 256
-// output columns (four heads of 64) x the whole Dm, in 64-wide k steps through a 4-stage ring
-// of 48 KB (A 16 KB + B 32 KB, 128-byte swizzle). A pair that crosses the grid edge (shifted
-// layers) is cut into two or four boxes of 4, 8 or 12 columns and 4 or 8 rows. Persistent
-// CTAs, one per SM, 320 threads:
+// Two kernels of the same main loop: a tile is 128 rows x 256 output columns (four heads of 64) x the
+// whole Dm, in 64-wide k steps through a 4-stage ring of 48 KB (A 16 KB + B 32 KB, 128-byte swizzle).
+//   kWin  the rows are two horizontally adjacent 8x8 windows of the shifted grid, one 16 x 8 token box per
+//         k step (measured, two 8 x 8 boxes took the main loop from 35 to 47 us at 1024 px), and the
+//         epilogue sums the windows of Q and K. A pair that crosses the grid edge (shifted layers) is
+//         cut into two or four boxes of 4, 8 or 12 columns and 4 or 8 rows, which load more slowly
+//         and take a longer window sum.
+//   else  the rows are consecutive tokens, one 128-row box, and the pooling kernel of ssba_pool_blocks
+//         follows, reading Q and K from L2.
+// What bounds both: shared memory. A k step writes 48 KB and its products read 48 KB in 512 tensor cycles,
+// 188 bytes a cycle where the SM moves 128, so a tile's main loop takes about 9.6 us where its
+// products need 6.4.
+// Persistent CTAs, one per SM, 320 threads:
 //   warp 0      TMA producer (one elected lane)
 //   warp 1      MMA issuer: tcgen05.mma kind::f16 M=128 N=256 K=16, four per k step, into one
 //               of two 256-column TMEM accumulators (512 columns), so that the epilogue of
@@ -58,6 +64,7 @@ constexpr int kRopeCap = 128;     // grid rows / columns whose cos, sin are tabu
 
 struct QkvMaps {
     CUtensorMap x[8];  // X as [B*H][W][Dm]: boxes of 4, 8, 12, 16 columns x 8 rows, then x 4 rows
+    CUtensorMap rows;  // X as [B][N][Dm], 128-row boxes (rows past N read as zeros)
     CUtensorMap w;     // Wqkv as [1][3 Dm][Dm], 256-row boxes
 };
 
@@ -109,8 +116,10 @@ static_assert(offsetof(QkvSmem, bias) % 16 == 0 && (kBN * sizeof(float)) % 16 ==
 struct TileGeo {
     int b, nt, L0, wd, r0, c0, w1;
     bool rs, two;
+    int tok0;  // (not kWin) the first of the tile's consecutive tokens
 };
 
+template <bool kWin>
 __device__ __forceinline__ TileGeo tile_geo(const QkvParams& p, const Grid& g, int t)
 {
     TileGeo o;
@@ -118,6 +127,10 @@ __device__ __forceinline__ TileGeo tile_geo(const QkvParams& p, const Grid& g, i
     const int rest = t / p.n_tiles;
     const int mt = rest % p.m_tiles;
     o.b = rest / p.m_tiles;
+    if constexpr (!kWin) {
+        o.tok0 = mt * kBM;
+        return o;
+    }
     const int wr = mt / p.pairs, pp = mt - wr * p.pairs;
     o.L0 = wr * g.bw + 2 * pp;
     o.two = 2 * pp + 1 < g.bw;
@@ -199,7 +212,7 @@ __device__ __forceinline__ bool wait_raw_q(uint32_t bar, uint32_t parity, uint64
 
 // kTable: RoPE cos/sin from the per-CTA table (grids up to kRopeCap rows and columns); else
 // computed per element (a separate instantiation, so that the table path stays compact).
-template <bool kTable>
+template <bool kTable, bool kWin>
 __global__ void __launch_bounds__(kThreads, 1) ssba_qkv_rope_pool_kernel(const __grid_constant__ QkvMaps maps,
                                                                           const QkvParams p)
 {
@@ -231,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_qkv_rope_pool_kernel(const _
         }
         fence_mbar_init();
     }
-    if (warp == 0 && lane < 9) tma_prefetch_desc(lane < 8 ? &maps.x[lane] : &maps.w);
+    if (warp == 0 && lane < 10) tma_prefetch_desc(lane < 8 ? &maps.x[lane] : (lane < 9 ? &maps.rows : &maps.w));
     if constexpr (kTable) {
         const int npos = max(g.H, g.W);
         for (int e = threadIdx.x; e < kNumFreq * npos; e += kThreads) {
@@ -250,13 +263,16 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_qkv_rope_pool_kernel(const _
     tc_fence_after();
     const uint32_t tbase = sm.tmem_base;
     bool dead = false;
+    // everything above reads no input and writes no output (programmatic dependent launch)
+    grid_dep_wait();
+    grid_dep_launch();
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         uint32_t gstep = 0;
         if (lane == 0) {
             for (int t = blockIdx.x; t < p.tiles && !dead; t += gridDim.x) {
-                const TileGeo o = tile_geo(p, g, t);
+                const TileGeo o = tile_geo<kWin>(p, g, t);
                 for (int ks = 0; ks < ksteps; ++ks, ++gstep) {
                     const uint32_t s = gstep % kStages;
                     if (!mbar_wait(smem_u32(&sm.empty[s]), ((gstep / kStages) & 1) ^ 1, abortf, p.budget_ns)) {
@@ -264,8 +280,13 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_qkv_rope_pool_kernel(const _
                         break;
                     }
                     const uint32_t bar = smem_u32(&sm.full[s]);
-                    mbar_arrive_expect_tx(bar, 8 * o.wd * 128 + kBBytes);
-                    load_tile(maps, smem_u32(&sm.a[s][0]), bar, g, o, ks * kBK);
+                    if constexpr (kWin) {
+                        mbar_arrive_expect_tx(bar, 8 * o.wd * 128 + kBBytes);
+                        load_tile(maps, smem_u32(&sm.a[s][0]), bar, g, o, ks * kBK);
+                    } else {
+                        mbar_arrive_expect_tx(bar, kABytes + kBBytes);
+                        tma_load_3d(smem_u32(&sm.a[s][0]), &maps.rows, bar, ks * kBK, o.tok0, o.b);
+                    }
                     tma_load_3d(smem_u32(&sm.b[s][0]), &maps.w, bar, ks * kBK, o.nt * kBN, 0);
                 }
             }
@@ -335,12 +356,19 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_qkv_rope_pool_kernel(const _
         const bool collector = quad == 0;  // adds the four quadrants' sums and writes the means
         uint32_t it = 0, npool = 0;
         for (int t = blockIdx.x; t < p.tiles && !dead; t += gridDim.x, ++it) {
-            const TileGeo o = tile_geo(p, g, t);
-            int ra, rc;
-            tile_rc(o, rho, ra, rc);
-            const int win = rc >> 3;
-            const bool valid = rho < 8 * o.wd;
-            const int tok = valid ? g.token(o.L0 + win, ra * 8 + (rc & 7)) : 0;
+            const TileGeo o = tile_geo<kWin>(p, g, t);
+            int win = 0, tok;
+            bool valid;
+            if constexpr (kWin) {
+                int ra, rc;
+                tile_rc(o, rho, ra, rc);
+                win = rc >> 3;
+                valid = rho < 8 * o.wd;
+                tok = valid ? g.token(o.L0 + win, ra * 8 + (rc & 7)) : 0;
+            } else {
+                valid = o.tok0 + rho < N;
+                tok = valid ? o.tok0 + rho : 0;
+            }
             const int tpos[2] = {tok / g.W, tok % g.W};  // RoPE positions: row, column
             // stores go out transposed within groups of four lanes (see below): the tokens and
             // validity of the group's rows
@@ -351,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_qkv_rope_pool_kernel(const _
                 tokm[m] = __shfl_sync(0xffffffffu, tok, (lane & ~3) | m);
                 validm[m] = __shfl_sync(0xffffffffu, (int)valid, (lane & ~3) | m) != 0;
             }
-            const bool regular = o.wd == 16 && o.w1 == 0;  // window = bit 3 of the lane
+            const bool regular = kWin && o.wd == 16 && o.w1 == 0;  // window = bit 3 of the lane
             const int b = o.b, nt = o.nt;
             const uint32_t acc = it & 1;
             if (!mbar_wait(smem_u32(&sm.acc_full[acc]), (it >> 1) & 1, abortf, p.budget_ns)) {
@@ -364,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_qkv_rope_pool_kernel(const _
             // the warp's heads pool when they hold Q or K (the same for the four quadrants of a
             // head pair, so that their handshake counts agree)
             const int col0 = nt * kBN + hp * 2 * kD;
-            const bool pool_tile = col0 < 2 * p.Dm && p.qb != nullptr;
+            const bool pool_tile = kWin && col0 < 2 * p.Dm && p.qb != nullptr;
             float(*mypart)[2][2][32] = sm.part[hp][quad];
             if (pool_tile && !collector) {
                 // the collector must have taken the previous tile's sums
@@ -568,6 +596,16 @@ bool encode_maps(QkvMaps& m, const void* X, const void* Wqkv, int B, int H, int 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return false;
     }
+    {
+        cuuint64_t dims[3] = {(cuuint64_t)Dm, (cuuint64_t)H * W, (cuuint64_t)B};
+        cuuint64_t strides[2] = {(cuuint64_t)Dm * 2, (cuuint64_t)H * W * Dm * 2};
+        cuuint32_t box[3] = {kBK, kBM, 1};
+        cuuint32_t es[3] = {1, 1, 1};
+        if (fn(&m.rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(X), dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
     cuuint64_t dims[3] = {(cuuint64_t)Dm, (cuuint64_t)3 * Dm, 1};
     cuuint64_t strides[2] = {(cuuint64_t)Dm * 2, (cuuint64_t)3 * Dm * Dm * 2};
     cuuint32_t box[3] = {kBK, kBN, 1};
@@ -612,7 +650,15 @@ int launch_qkv_rope_pool(const ssba_desc& d, const Grid& g, const void* X, const
     p.heads = d.heads;
     p.Dm = Dm;
     p.pairs = (g.bw + 1) / 2;
-    p.m_tiles = (g.H / 8) * p.pairs;
+    // Window tiles (means in the epilogue) against row tiles and a pooling launch, 24 heads, us:
+    //   256 px 15.4 unshifted, 23.2 shifted / 14.6;  512 px 17.3, 24.4 / 18.9;  1024 px 43.1, 54.8 / 44.3;
+    //   two 1024 px images 78.4, 88.9 / 83.9;  1536 px 87.6, 92.8 / 95;  four 1024 px images 149, 164 /
+    //   170;  2048 px 151, 156 / 172.
+    // So rows where the layer is shifted and Q and K (here 50 MB at two 1024 px images) stay in L2 until
+    // they are pooled; and where no means are asked for (1024 px 38 us against 43 to 52).
+    const bool shifted = g.sr != 0 || g.sc != 0;
+    const bool win = qb && !(shifted && 4ll * d.B * g.H * g.W * Dm <= (48ll << 20));
+    p.m_tiles = win ? (g.H / 8) * p.pairs : (g.H * g.W + kBM - 1) / kBM;
     p.n_tiles = (3 * Dm + kBN - 1) / kBN;
     p.tiles = d.B * p.m_tiles * p.n_tiles;
     for (int i = 0; i < kNumFreq; ++i) p.theta[i] = (float)pow(10000.0, -(double)i / kNumFreq);
@@ -625,20 +671,31 @@ int launch_qkv_rope_pool(const ssba_desc& d, const Grid& g, const void* X, const
     const size_t smem = sizeof(QkvSmem) + 1024;
     static PerDeviceOnce attr;  // shared-memory attributes, set once per device
     attr.run([smem] {
-        cudaFuncSetAttribute(ssba_qkv_rope_pool_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(ssba_qkv_rope_pool_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        for (auto k : {ssba_qkv_rope_pool_kernel<true, true>, ssba_qkv_rope_pool_kernel<true, false>,
+                       ssba_qkv_rope_pool_kernel<false, true>, ssba_qkv_rope_pool_kernel<false, false>})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     const int grid = p.tiles < sm_count() ? p.tiles : sm_count();
-    if (g.H <= kRopeCap && g.W <= kRopeCap)
-        ssba_qkv_rope_pool_kernel<true><<<grid, kThreads, smem, st>>>(maps, p);
-    else
-        ssba_qkv_rope_pool_kernel<false><<<grid, kThreads, smem, st>>>(maps, p);
-    cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute la[1];
+    la[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    la[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = la;
+    cfg.numAttrs = 1;
+    const bool table = g.H <= kRopeCap && g.W <= kRopeCap;
+    auto kernel = table ? (win ? ssba_qkv_rope_pool_kernel<true, true> : ssba_qkv_rope_pool_kernel<true, false>)
+                        : (win ? ssba_qkv_rope_pool_kernel<false, true> : ssba_qkv_rope_pool_kernel<false, false>);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, maps, p);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("ssba_qkv_rope_pool_kernel launch: %s", cudaGetErrorString(e));
         return SSBA_ERR_CUDA;
     }
-    return SSBA_OK;
+    return qb && !win ? launch_pool_blocks(d, g, Q, K, qb, kb, st) : SSBA_OK;
 }
 
 }  // namespace ssba

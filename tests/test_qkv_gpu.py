@@ -148,3 +148,24 @@ def test_fused_path_feeds_the_forward():
     Oo, lo = oracle.forward(Q.double().numpy(), K.double().numpy(), V.double().numpy(), idx.cpu().numpy(), H, W, 8,
                             shift)
     check_out(O.float().cpu().numpy(), lse.cpu().numpy(), Oo, lo, "bf16")
+
+
+@pytest.mark.parametrize("B,heads,H,W,shift", [
+    (1, 24, 72, 88, (4, 4)),    # 6336 tokens, 39 MB of Q and K: row tiles (the last one of 64 rows) and a pooling launch
+    (2, 24, 72, 88, (4, 4)),    # above the limit: window tiles
+    (2, 24, 72, 88, (0, 0)),
+    (3, 2, 8, 24, (0, 4)),      # 192 tokens an image: a tile of 64 rows before the next image's
+])
+def test_row_tiles_and_window_tiles_give_the_same(B, heads, H, W, shift):
+    """The projection's two tilings, on one set of inputs: Q, K, V of a call that asks for means equal those of
+    one that does not (row tiles), bit for bit, and the means are those of its own Q and K."""
+    X, Wq, b = synthetic.projection_inputs(B, H * W, heads * 64, 5)
+    desc = api.SsbaDesc(B, heads, H, W, shift_r=shift[0], shift_c=shift[1], rho=0.8)
+    Q, K, V, qb, kb = api.qkv_rope_pool(desc, X.cuda(), Wq.cuda(), b.cuda())
+    Q2, K2, V2, _, _ = api.qkv_rope_pool(desc, X.cuda(), Wq.cuda(), b.cuda(), pooled=False)
+    qb2, kb2 = api.pool_blocks(desc, Q, K)
+    torch.cuda.synchronize()
+    for x, y in ((Q, Q2), (K, K2), (V, V2)):
+        assert torch.equal(x, y)
+    for x, y, t in ((qb, qb2, Q), (kb, kb2, K)):  # 64 fp32 additions in two orders
+        assert float((x - y).abs().max()) <= 2.0 ** -17 * float(t.abs().max())
