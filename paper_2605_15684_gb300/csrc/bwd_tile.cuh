@@ -89,8 +89,9 @@ struct BwdLayout {
 BwdLayout bwd_layout(const ssba_desc& d, const Grid& g, int keep);
 
 // The row kernel: D for every row and, when p.tlist is set, the rows' (lse log2(e), D) by block
-// in tile order, the counter reset and the transposed lists (one extra CTA per head). Launched plainly (it depends on all earlier work);
-// the gradient kernel that follows is its programmatic dependent.
+// in tile order, the counter reset and the transposed lists (one CTA per head). A programmatic dependent of the work
+// before it: every CTA waits for that work before it lets the gradient kernel that follows, its own
+// programmatic dependent, start, so that kernel may read inputs without waiting again.
 cudaError_t launch_bwd_rows(const BwdParams& p, int BH, cudaStream_t st);
 
 }  // namespace bwd
