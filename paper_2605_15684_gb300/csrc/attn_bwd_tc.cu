@@ -615,7 +615,9 @@ __global__ void __launch_bounds__(256) ssba_bwd_rows_kernel(const BwdParams p, c
         int label, pos;
         win::token_block(p.g, row - bh * N, label, pos);
         const int r = win::tile_row_of(p.g, label, pos);
-        p.ld[((size_t)bh * p.g.Tb() + label) * kT + r] = make_float2(__ldg(p.lse + row) * kLog2e, mine);
+        float* st = reinterpret_cast<float*>(p.ld + ((size_t)bh * p.g.Tb() + label) * (kT / 2) + (r >> 1)) + (r & 1);
+        st[0] = -(__ldg(p.lse + row) * kLog2e);
+        st[2] = -mine;
     }
 }
 

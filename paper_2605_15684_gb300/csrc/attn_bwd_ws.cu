@@ -11,7 +11,7 @@
 //              blocks: the forward's list for dQ, the transposed list the row kernel built for
 //              dK, dV) in one of two item slots; copies the item's resident tiles by TMA (two
 //              buffers, by item parity) and each pair's streamed tiles (a ring of three), each
-//              with the 512-byte row of (lse, D) values of its block that the compute warps
+//              with the 512-byte row of its block's statistics (lse, D) that the compute warps
 //              use (the row kernel writes them by block, in tile order: one bulk copy).
 //   warps 8-10 lane 0 of each issues a share of the MMAs: warp 8 S and dK += dS^T Q, warp 9
 //              dP and dV += P^T dO, warp 10 dQ += dS K. Per pair S, dP go into the same TMEM
@@ -22,8 +22,16 @@
 //              to global memory, fp32).
 // Pairs are counted across items: the next item's tiles arrive while the last item computes,
 // and its first products run while the compute warps store the last item's gradients.
+// What bounds it: a pair's chain of hand-offs (S, dP -> registers -> bf16 operands -> products), of which
+// two CTAs an SM hide half, with the compute warps' instructions on it: 2048 px 1700 cycles a pair and CTA,
+// the tensor pipe (44 cycles a product, 14 a pair) busy 620 of them for each CTA. So the statistics come as addends
+// for packed two-column arithmetic, the pair loop's waits return no verdict (wait_phase), and a thread
+// that issues nothing for a pair fences nothing. 24 heads, a call: 1024 px 139.4 -> 133.3 us, four 1024
+// px images 701 -> 668, 2048 px 1556 -> 1465 (the packed arithmetic alone 136.0, 683, 1505 -> those).
 // Tile rows follow the TMA box order (tile_row_pos). Every wait is bounded; on a timeout the
-// CTA records SSBA_ERR_TIMEOUT, waits (bounded) for its copies and MMAs in flight, and returns.
+// CTA records SSBA_ERR_TIMEOUT, waits (bounded) for its copies and MMAs in flight, and returns. (After one
+// the compute warps run to the end of their item on whatever their own tiles hold, and leave before its
+// epilogue or at the next item.)
 #include <algorithm>
 #include <cstdint>
 
@@ -64,8 +72,8 @@ struct alignas(1024) WsSmem {
     uint8_t x[kRing][kTile];  // pair tiles: dQ item K_j, dK/dV item Q_i
     uint8_t y[kRing][kTile];  //             V_j,         dO_i
     uint8_t e[2][kTile];      // bf16 operands: dS (e[0]); P^T and dS^T
-    float2 pld[kRing][kT];    // dK/dV pair: (lse log2(e), D) of its query rows (tile order)
-    float2 ild[2][kT];        // dQ item: (lse log2(e), D) of its rows
+    float4 pld[kRing][kT / 2];  // dK/dV pair: the statistics of its query rows (BwdParams::ld)
+    float4 ild[2][kT / 2];      // dQ item: of its rows
     int list[2][256];         // the item's other blocks, in pair order (producer only)
     uint32_t win[256];        // label -> packed window entry (window_entry)
     int4 info[2];             // role (0 dQ, 1 dK/dV, kDone), bh, label, n
@@ -111,7 +119,7 @@ __device__ __forceinline__ int tile_token(const Grid& g, int label, int r)
     return g.token(label, tile_row_pos(g, label, r));
 }
 
-constexpr uint32_t kLdRow = kT * sizeof(float2);  // 512 bytes of (lse, D) per block
+constexpr uint32_t kLdRow = kT * sizeof(float2);  // 512 bytes of statistics per block
 
 // An item slot's shape, read after its mbarrier wait.
 __device__ __forceinline__ int4 read_info(const int4* q)
@@ -176,7 +184,7 @@ __device__ bool produce(const WsMaps& maps, const BwdParams& p, WsSmem& sm, cons
             mbar_arrive_expect_tx(bar, 2 * kTile + (role ? 0 : kLdRow));
             window_boxes_e(role ? maps.k : maps.q, smem_u32(sm.a[s]), bar, e, bh);
             window_boxes_e(role ? maps.v : maps.o, smem_u32(sm.b[s]), bar, e, bh);
-            if (!role) bulk_load(smem_u32(sm.ild[s]), p.ld + brow * kT, kLdRow, bar);
+            if (!role) bulk_load(smem_u32(sm.ild[s]), p.ld + brow * (kT / 2), kLdRow, bar);
         }
         ++kab;
         // the pairs' streamed tiles, each once the pair three back has finished its products
@@ -194,7 +202,7 @@ __device__ bool produce(const WsMaps& maps, const BwdParams& p, WsSmem& sm, cons
                 if (!hold) {
                     window_boxes_e(role ? maps.q : maps.k, smem_u32(sm.x[r]), bar, e, bh);
                     window_boxes_e(role ? maps.o : maps.v, smem_u32(sm.y[r]), bar, e, bh);
-                    if (role) bulk_load(smem_u32(sm.pld[r]), p.ld + ((size_t)bh * Tb + j) * kT, kLdRow, bar);
+                    if (role) bulk_load(smem_u32(sm.pld[r]), p.ld + ((size_t)bh * Tb + j) * (kT / 2), kLdRow, bar);
                 }
             }
         }
@@ -210,11 +218,11 @@ __device__ bool produce(const WsMaps& maps, const BwdParams& p, WsSmem& sm, cons
 // dQ is issuer 2's. Each commits, so bar_a and tile_empty count three.
 __device__ __forceinline__ bool issue_acc(const BwdParams& p, WsSmem& sm, uint32_t q, int role, bool first, int which)
 {
-    if (!mbar_wait(smem_u32(&sm.e_full), q & 1, &sm.abort_flag, p.budget_ns)) return false;
-    tc_fence_after();
     const uint32_t tb0 = sm.tmem_base;
     const int r = (int)(q % kRing);
+    if (!mbar_wait(smem_u32(&sm.e_full), q & 1, &sm.abort_flag, p.budget_ns)) return false;
     if (role == 1) {
+        tc_fence_after();
         if (which == 0)
             mma_sb(tb0 + kColA1, smem_u32(sm.e[1]), smem_u32(sm.x[r]), !first);  // dK += dS^T Q
         else
@@ -279,7 +287,7 @@ __device__ bool issue(const BwdParams& p, WsSmem& sm, const int which)
         for (int t = 0; t < n; ++t, ++P) {
             const int r = (int)(P % kRing);
             if (!mbar_wait(smem_u32(&sm.tile_full[r]), (P / kRing) & 1, abortf, p.budget_ns)) return false;
-            if (P > 0 && !mbar_wait(smem_u32(&sm.s_free), (P - 1) & 1, abortf, p.budget_ns)) return false;
+            if (P > 0) wait_phase(smem_u32(&sm.s_free), (P - 1) & 1, smem_u32(&sm.abort_flag), p.budget_ns);
             tc_fence_after();
             if (which == 0)
                 mma_kk(tb0 + kColS, ab, smem_u32(sm.x[r]));  // S = Q K^T (dK/dV item: S^T = K Q^T)
@@ -336,24 +344,25 @@ __device__ bool compute(const BwdParams& p, WsSmem& sm)
     const uint32_t tb = sm.tmem_base + (static_cast<uint32_t>(q * 32) << 16) + 16 * (warp >> 2);
     const Grid& g = p.g;
     const int N = g.H * g.W;
-    const float c = p.scale * kLog2e;
+    const float2 c2 = make_float2(p.scale * kLog2e, p.scale * kLog2e);
     uint32_t P = 0;  // pairs done
     for (int k = 0;; ++k) {
         const int s = k & 1;
         if (!warp_wait(smem_u32(&sm.item_full[s]), (k >> 1) & 1, abortf, p.budget_ns)) return false;
         const int4 inf = read_info(&sm.info[s]);
-        float L2 = 0.f, Dr = 0.f;
+        float2 nl2 = make_float2(0.f, 0.f), nd2 = nl2;  // -lse log2(e) and -D, twice
         if (inf.x == 0) {  // the row's statistics came with the item's tiles
             if (!warp_wait(smem_u32(&sm.ab_full[s]), (k >> 1) & 1, abortf, p.budget_ns)) return false;
-            L2 = sm.ild[s][r].x;
-            Dr = sm.ild[s][r].y;
+            const float* st = reinterpret_cast<const float*>(&sm.ild[s][r >> 1]) + (r & 1);
+            nl2 = make_float2(st[0], st[0]);
+            nd2 = make_float2(st[2], st[2]);
         }
         warp_arrive(smem_u32(&sm.item_empty[s]));
         if (inf.x == kDone) return true;
         const int role = inf.x, bh = inf.y, label = inf.z, n = inf.w;
         for (int t = 0; t < n; ++t, ++P) {
             const int slot = (int)(P % kRing);
-            if (!warp_wait(smem_u32(&sm.bar_s), P & 1, abortf, p.budget_ns)) return false;
+            wait_phase(smem_u32(&sm.bar_s), P & 1, smem_u32(&sm.abort_flag), p.budget_ns);
             tc_fence_after();
             uint32_t sv[16], dp[16];
             tmem_ld_16x32bx2_x16_off32(tb + kColS, sv);
@@ -361,32 +370,38 @@ __device__ bool compute(const BwdParams& p, WsSmem& sm)
             tmem_wait_ld();
             tc_fence_before();
             warp_arrive(smem_u32(&sm.s_free));
+            auto pair_of = [](const uint32_t (&v)[16], int i) {
+                return make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+            };
+            auto probs = [&](const uint32_t (&v)[16], int i, float2 nl) {
+                const float2 x = __ffma2_rn(pair_of(v, i), c2, nl);
+                return make_float2(fast_exp2(x.x), fast_exp2(x.y));
+            };
             if (role == 1) {
                 // S^T, dP^T: columns are the query rows col0 + i of the pair's query block
-                if (!warp_wait(smem_u32(&sm.tile_full[slot]), (P / kRing) & 1, abortf, p.budget_ns)) return false;
-                const float4* ld = reinterpret_cast<const float4*>(sm.pld[slot] + col0);
+                wait_phase(smem_u32(&sm.tile_full[slot]), (P / kRing) & 1, smem_u32(&sm.abort_flag), p.budget_ns);
+                const float4* ld = sm.pld[slot] + (col0 >> 1);
                 uint32_t pp[8], dd[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const float4 qd = ld[i];  // (lse, D) of query rows col0 + 2 i and col0 + 2 i + 1
-                    const float p0 = fast_exp2(fmaf(__uint_as_float(sv[2 * i]), c, -qd.x));
-                    const float p1 = fast_exp2(fmaf(__uint_as_float(sv[2 * i + 1]), c, -qd.z));
-                    pp[i] = pack_bf16(p0, p1);
-                    dd[i] = pack_bf16(p0 * (__uint_as_float(dp[2 * i]) - qd.y), p1 * (__uint_as_float(dp[2 * i + 1]) - qd.w));
+                    const float4 qd = ld[i];  // of query rows col0 + 2 i and col0 + 2 i + 1
+                    const float2 pv = probs(sv, i, make_float2(qd.x, qd.y));
+                    const float2 ds = __fmul2_rn(pv, __fadd2_rn(pair_of(dp, i), make_float2(qd.z, qd.w)));
+                    pp[i] = pack_bf16(pv.x, pv.y);
+                    dd[i] = pack_bf16(ds.x, ds.y);
                 }
                 // the last pair's products have read e[] (and the tiles of its slot)
-                if (P > 0 && !warp_wait(smem_u32(&sm.bar_a), (P - 1) & 1, abortf, p.budget_ns)) return false;
+                if (P > 0) wait_phase(smem_u32(&sm.bar_a), (P - 1) & 1, smem_u32(&sm.abort_flag), p.budget_ns);
                 store_cols_bf16(sm.e[0], r, col0 >> 3, pp);
                 store_cols_bf16(sm.e[1], r, col0 >> 3, dd);
             } else {
                 uint32_t pk[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const float p0 = fast_exp2(fmaf(__uint_as_float(sv[2 * i]), c, -L2));
-                    const float p1 = fast_exp2(fmaf(__uint_as_float(sv[2 * i + 1]), c, -L2));
-                    pk[i] = pack_bf16(p0 * (__uint_as_float(dp[2 * i]) - Dr), p1 * (__uint_as_float(dp[2 * i + 1]) - Dr));
+                    const float2 ds = __fmul2_rn(probs(sv, i, nl2), __fadd2_rn(pair_of(dp, i), nd2));
+                    pk[i] = pack_bf16(ds.x, ds.y);
                 }
-                if (P > 0 && !warp_wait(smem_u32(&sm.bar_a), (P - 1) & 1, abortf, p.budget_ns)) return false;
+                if (P > 0) wait_phase(smem_u32(&sm.bar_a), (P - 1) & 1, smem_u32(&sm.abort_flag), p.budget_ns);
                 store_cols_bf16(sm.e[0], r, col0 >> 3, pk);
             }
             fence_proxy_async_smem();
@@ -531,7 +546,7 @@ int launch_backward_ws(const ssba_desc& d, const Grid& g, int keep, float scale,
     p.toff = reinterpret_cast<int*>(ws + lay.toff);
     p.tcnt = reinterpret_cast<int*>(ws + lay.tcnt);
     p.tlist = reinterpret_cast<int*>(ws + lay.tlist);
-    p.ld = reinterpret_cast<float2*>(ws + lay.ld);
+    p.ld = reinterpret_cast<float4*>(ws + lay.ld);
     p.g = g;
     p.keep = keep;
     p.scale = scale;

@@ -71,7 +71,8 @@ struct BwdParams {
     const int32_t* cnt;
     float *dQ, *dK, *dV, *Dbuf;
     int *ctr, *toff, *tcnt, *tlist;
-    float2* ld;  // [B*heads][Tb][64]: (lse log2(e), D) of each block's rows in TMA tile order
+    float4* ld;  // [B*heads][Tb][32]: (-lse log2(e) of two rows, -D of the same) of each block's rows, in
+                 // TMA tile order: addends of packed two-row arithmetic
     Grid g;
     int keep;
     float scale;
@@ -88,9 +89,9 @@ struct BwdLayout {
 };
 BwdLayout bwd_layout(const ssba_desc& d, const Grid& g, int keep);
 
-// The row kernel: D for every row and, when p.tlist is set, the rows' (lse log2(e), D) by block
-// in tile order, the counter reset and the transposed lists (one CTA per head). A programmatic dependent of the work
-// before it: every CTA waits for that work before it lets the gradient kernel that follows, its own
+// The row kernel: D for every row and, when p.tlist is set, the rows' statistics (ld) by
+// block, the counter reset and the transposed lists (one CTA per head). A programmatic dependent of the
+// work before it: every CTA waits for that work before it lets the gradient kernel that follows, its own
 // programmatic dependent, start, so that kernel may read inputs without waiting again.
 cudaError_t launch_bwd_rows(const BwdParams& p, int BH, cudaStream_t st);
 
