@@ -13,10 +13,11 @@
 //              buffers, by item parity) and each pair's streamed tiles (a ring of three), each
 //              with the 512-byte row of its block's statistics (lse, D) that the compute warps
 //              use (the row kernel writes them by block, in tile order: one bulk copy).
-//   warps 8-10 lane 0 of each issues a share of the MMAs: warp 8 S and dK += dS^T Q, warp 9
-//              dP and dV += P^T dO, warp 10 dQ += dS K. Per pair S, dP go into the same TMEM
-//              columns once the compute warps hold the last ones in registers; the
-//              accumulating products of a pair follow once its bf16 operands are stored.
+//   warps 8-10 lane 0 of each issues a share of the MMAs: warp 8 S, warp 9 dP, into the same
+//              TMEM columns once the compute warps hold the last pair's in registers; warp 10 the
+//              accumulating products of a pair, once its bf16 operands are stored. (Four products
+//              take a thread about 450 cycles to issue. With dK on S's thread and dV on dP's, a
+//              pair's S waited 860 cycles for its thread.)
 //   warps 0-7  the exps and the bf16 operands of each pair, two warps per TMEM lane quadrant
 //              (16 of a row's 64 columns a thread), and each item's epilogue (the accumulators
 //              to global memory, fp32).
@@ -49,10 +50,10 @@ using namespace win;
 using namespace bwd;
 
 constexpr int kCompute = 256;   // warps 0-7, two per TMEM lane quadrant
-constexpr int kIssuer0 = 256;   // lane 0 of warp 8: S, and dK += dS^T Q
-constexpr int kIssuer1 = 288;   // lane 0 of warp 9: dP, and dV += P^T dO
-constexpr int kIssuer2 = 320;   // lane 0 of warp 10: dQ += dS K
-constexpr int kIssuers = 3;     // commit to bar_a, tile_empty, drain
+constexpr int kIssuer0 = 256;   // lane 0 of warp 8: S
+constexpr int kIssuer1 = 288;   // lane 0 of warp 9: dP
+constexpr int kIssuer2 = 320;   // lane 0 of warp 10: the accumulating products
+constexpr int kIssuers = 3;     // commit to drain
 constexpr int kSdpIssuers = 2;  // commit to bar_s, ab_empty
 constexpr int kProducer = 11;   // warp
 constexpr int kThreads = 384;
@@ -82,11 +83,11 @@ struct alignas(1024) WsSmem {
     uint64_t ab_full[2];      // TMA bytes of the item tiles (and, for dQ, of its ild row)
     uint64_t ab_empty[2];     // MMA commits (the S and dP issuers) after the item's last S, dP
     uint64_t tile_full[kRing];   // TMA bytes of a pair's tiles (and, for dK/dV, of its pld row)
-    uint64_t tile_empty[kRing];  // MMA commits (all three issuers) after the pair's products
+    uint64_t tile_empty[kRing];  // MMA commit after the pair's accumulating products
     uint64_t bar_s;           // MMA commits (the S and dP issuers): S, dP of the pair in TMEM
     uint64_t s_free;          // 8 compute warps: S, dP in registers
     uint64_t e_full;          // 8 compute warps: the pair's bf16 operands stored
-    uint64_t bar_a;           // MMA commits (all three issuers): the pair's accumulating products
+    uint64_t bar_a;           // MMA commit: the pair's accumulating products
     uint64_t drain;
     uint32_t tmem_base;
     int abort_flag;
@@ -212,33 +213,11 @@ __device__ bool produce(const WsMaps& maps, const BwdParams& p, WsSmem& sm, cons
     }
 }
 
-// Issuer `which`'s share of the accumulating products of pair q (its role, and whether it opens
-// its item), once the pair's bf16 operands are stored: for a key-block pair issuer 0
-// dK += dS^T Q (x tile), issuer 1 dV += P^T dO (y tile); nothing for a query-block pair, whose
-// dQ is issuer 2's. Each commits, so bar_a and tile_empty count three.
-__device__ __forceinline__ bool issue_acc(const BwdParams& p, WsSmem& sm, uint32_t q, int role, bool first, int which)
-{
-    const uint32_t tb0 = sm.tmem_base;
-    const int r = (int)(q % kRing);
-    if (!mbar_wait(smem_u32(&sm.e_full), q & 1, &sm.abort_flag, p.budget_ns)) return false;
-    if (role == 1) {
-        tc_fence_after();
-        if (which == 0)
-            mma_sb(tb0 + kColA1, smem_u32(sm.e[1]), smem_u32(sm.x[r]), !first);  // dK += dS^T Q
-        else
-            mma_sb(tb0 + kColA0, smem_u32(sm.e[0]), smem_u32(sm.y[r]), !first);  // dV += P^T dO
-    }
-    mma_commit(smem_u32(&sm.bar_a));
-    mma_commit(smem_u32(&sm.tile_empty[r]));
-    return true;
-}
-
-// Lane 0 of warp 8 (which = 0) or 9 (which = 1): S or dP of every pair and its share of the
-// accumulating products, so that the issue latency of a tcgen05.mma (about 57 cycles from one
-// thread, 44 a product when several issue) is shared. Returns false on a timeout.
-// Lane 0 of warp 10: dQ += dS K of every query-block pair, in pair order, once its operands are
-// stored; for key-block pairs it only commits (bar_a and tile_empty count three commits).
-__device__ bool issue_dq(const BwdParams& p, WsSmem& sm)
+// Lane 0 of warp 10: every pair's accumulating products, in pair order, once its bf16 operands are stored:
+// dQ += dS K of a query-block pair, dV += P^T dO and dK += dS^T Q of a key-block pair. (A pair's operands
+// are made from its S and dP, so those are done with the tiles by then: the commits here are all that
+// bar_a and tile_empty count.) Returns false on a timeout.
+__device__ bool issue_acc(const BwdParams& p, WsSmem& sm)
 {
     volatile int* abortf = &sm.abort_flag;
     const uint32_t tb0 = sm.tmem_base;
@@ -251,37 +230,36 @@ __device__ bool issue_dq(const BwdParams& p, WsSmem& sm)
         if (inf.x == kDone) return true;
         const int role = inf.x, n = inf.w;
         for (int t = 0; t < n; ++t, ++P) {
+            const int r = (int)(P % kRing);
+            if (!mbar_wait(smem_u32(&sm.tile_full[r]), (P / kRing) & 1, abortf, p.budget_ns)) return false;
             if (!mbar_wait(smem_u32(&sm.e_full), P & 1, abortf, p.budget_ns)) return false;
             tc_fence_after();
-            const int r = (int)(P % kRing);
-            if (role == 0) mma_sb(tb0 + kColA0, smem_u32(sm.e[0]), smem_u32(sm.x[r]), t > 0);  // dQ += dS K
+            if (role == 0) {
+                mma_sb(tb0 + kColA0, smem_u32(sm.e[0]), smem_u32(sm.x[r]), t > 0);
+            } else {
+                mma_sb(tb0 + kColA0, smem_u32(sm.e[0]), smem_u32(sm.y[r]), t > 0);
+                mma_sb(tb0 + kColA1, smem_u32(sm.e[1]), smem_u32(sm.x[r]), t > 0);
+            }
             mma_commit(smem_u32(&sm.bar_a));
             mma_commit(smem_u32(&sm.tile_empty[r]));
         }
     }
 }
 
-__device__ bool issue(const BwdParams& p, WsSmem& sm, const int which)
+// Lane 0 of warp 8 (which = 0) or 9 (which = 1): S or dP of every pair, as soon as the compute warps hold
+// the last pair's in registers. Returns false on a timeout.
+__device__ bool issue_sdp(const BwdParams& p, WsSmem& sm, const int which)
 {
     volatile int* abortf = &sm.abort_flag;
     const uint32_t tb0 = sm.tmem_base;
-    uint32_t P = 0;  // pairs whose S, dP are issued
-    bool pending = false;  // pair P - 1's accumulating products not yet issued
-    int prole = 0;
-    bool pfirst = false;
+    uint32_t P = 0;  // pairs issued
     for (int k = 0;; ++k) {
         const int s = k & 1;
-        // the last item's final products first: its epilogue waits for them, and the next
-        // item's tiles may still be on their way
-        if (pending) {
-            if (!issue_acc(p, sm, P - 1, prole, pfirst, which)) return false;
-            pending = false;
-        }
         if (!mbar_wait(smem_u32(&sm.item_full[s]), (k >> 1) & 1, abortf, p.budget_ns)) return false;
         const int4 inf = read_info(&sm.info[s]);
         mbar_arrive(smem_u32(&sm.item_empty[s]));
         if (inf.x == kDone) return true;
-        const int role = inf.x, n = inf.w;
+        const int n = inf.w;
         if (!mbar_wait(smem_u32(&sm.ab_full[s]), (k >> 1) & 1, abortf, p.budget_ns)) return false;
         const uint32_t ab = smem_u32(which ? sm.b[s] : sm.a[s]);
         for (int t = 0; t < n; ++t, ++P) {
@@ -295,10 +273,6 @@ __device__ bool issue(const BwdParams& p, WsSmem& sm, const int which)
                 mma_kk(tb0 + kColDP, ab, smem_u32(sm.y[r]));  // dP = dO V^T (dP^T = V dO^T)
             mma_commit(smem_u32(&sm.bar_s));
             if (t == n - 1) mma_commit(smem_u32(&sm.ab_empty[s]));
-            if (pending && !issue_acc(p, sm, P - 1, prole, pfirst, which)) return false;
-            pending = true;
-            prole = role;
-            pfirst = t == 0;
         }
         if (n == 0) mma_commit(smem_u32(&sm.ab_empty[s]));
     }
@@ -448,12 +422,12 @@ __global__ void __launch_bounds__(kThreads, 2) ssba_bwd_ws_kernel(const __grid_c
         }
         for (int i = 0; i < kRing; ++i) {
             mbar_init(smem_u32(&sm.tile_full[i]), 1);
-            mbar_init(smem_u32(&sm.tile_empty[i]), kIssuers);
+            mbar_init(smem_u32(&sm.tile_empty[i]), 1);
         }
         mbar_init(smem_u32(&sm.bar_s), kSdpIssuers);
         mbar_init(smem_u32(&sm.s_free), kCompute / 32);
         mbar_init(smem_u32(&sm.e_full), kCompute / 32);
-        mbar_init(smem_u32(&sm.bar_a), kIssuers);
+        mbar_init(smem_u32(&sm.bar_a), 1);
         mbar_init(smem_u32(&sm.drain), kIssuers);
         fence_mbar_init();
     }
@@ -477,9 +451,9 @@ __global__ void __launch_bounds__(kThreads, 2) ssba_bwd_ws_kernel(const __grid_c
     if (warp < kCompute / 32)
         ok = compute(p, sm);
     else if (threadIdx.x == kIssuer0 || threadIdx.x == kIssuer1)
-        ok = issue(p, sm, threadIdx.x == kIssuer1 ? 1 : 0);
+        ok = issue_sdp(p, sm, threadIdx.x == kIssuer1 ? 1 : 0);
     else if (threadIdx.x == kIssuer2)
-        ok = issue_dq(p, sm);
+        ok = issue_acc(p, sm);
     else if (warp == kProducer)
         ok = produce(maps, p, sm, nk, P, kab);
     const bool dead = __syncthreads_or(!ok);
