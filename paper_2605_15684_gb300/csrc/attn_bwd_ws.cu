@@ -23,12 +23,13 @@
 //              to global memory, fp32).
 // Pairs are counted across items: the next item's tiles arrive while the last item computes,
 // and its first products run while the compute warps store the last item's gradients.
-// What bounds it: a pair's chain of hand-offs (S, dP -> registers -> bf16 operands -> products), of which
-// two CTAs an SM hide half, with the compute warps' instructions on it: 2048 px 1700 cycles a pair and CTA,
-// the tensor pipe (44 cycles a product, 14 a pair) busy 620 of them for each CTA. So the statistics come as addends
-// for packed two-column arithmetic, the pair loop's waits return no verdict (wait_phase), and a thread
-// that issues nothing for a pair fences nothing. 24 heads, a call: 1024 px 139.4 -> 133.3 us, four 1024
-// px images 701 -> 668, 2048 px 1556 -> 1465 (the packed arithmetic alone 136.0, 683, 1505 -> those).
+// What bounds it: the tensor pipe's 64 x 64 products and the chain of hand-offs between them (S, dP ->
+// registers -> bf16 operands -> products). At 2048 px a pair takes a CTA 1690 cycles, of which the products
+// of the SM's two CTAs take about 1230 (44 cycles each, 14 a pair); alone on its SM a CTA takes 1430. So
+// the compute warps' instructions count: the statistics come as addends for packed two-column
+// arithmetic, and the pair loop's waits return no verdict (wait_phase). 24 heads, a call, before these
+// and now: 1024 px 139.4, 132.2 us, four 1024 px images 701, 664, 2048 px 1556, 1460 (the threads that
+// issue are 1.2 us of the first).
 // Tile rows follow the TMA box order (tile_row_pos). Every wait is bounded; on a timeout the
 // CTA records SSBA_ERR_TIMEOUT, waits (bounded) for its copies and MMAs in flight, and returns. (After one
 // the compute warps run to the end of their item on whatever their own tiles hold, and leave before its
