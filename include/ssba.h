@@ -154,7 +154,7 @@ SSBA_API int ssba_forward_joint(const ssba_desc* desc, const void* Q, const void
 
 /* Bytes of the optional ssba_forward / ssba_forward_dense / ssba_forward_select workspace, and
  * of the required one of ssba_forward_fused, for desc on the current device (it scales with the
- * device's SM count: about 10 MB on 152 SMs);
+ * device's SM count: about 10 MB on 152 SMs, of which the last 256 bytes are used);
  * 0 for an fp32 or an invalid descriptor. Host only, no device work. */
 SSBA_API size_t ssba_forward_workspace_bytes(const ssba_desc* desc);
 
@@ -204,11 +204,12 @@ SSBA_API size_t ssba_backward_workspace_bytes(const ssba_desc* desc);
 SSBA_API int ssba_pool_blocks(const ssba_desc* desc, const void* Q, const void* K, float* qb, float* kb,
                               void* stream);
 
-/* Affinity, Top-k gating and sparse attention in one launch (Sec. 2.2, Algorithm 1 from
- * "S <- q_b k_b^T" on): each CTA computes the score rows and the kept-block lists of the query
- * blocks it will process (the arithmetic of ssba_build_mask, so the same means give the same
- * lists), writes them to kv_idx / kv_cnt (outputs here, same layout as ssba_build_mask), and
- * runs the forward of ssba_forward on them.
+/* Affinity, Top-k gating and sparse attention in one call (Sec. 2.2, Algorithm 1 from
+ * "S <- q_b k_b^T" on), with the arithmetic of ssba_build_mask, so the same means give the same
+ * lists. Up to 16 query blocks an SM (B * heads * Tb <= 16 * SMs) it is one launch: each CTA
+ * computes the score rows and the kept-block lists of the query blocks it will process, writes
+ * them to kv_idx / kv_cnt (outputs here, same layout as ssba_build_mask), and runs the forward of
+ * ssba_forward on them. Above, the selection is a launch of its own before the forward.
  *   qb, kb      device, fp32 block means from ssba_pool_blocks (or ssba_qkv_rope_pool).
  *   scores_opt  device out or NULL, fp32 [B][heads][Tb][Tb]: the scores of the selection.
  *   Q, K, V, O, lse, workspace as for ssba_forward.
@@ -218,18 +219,19 @@ SSBA_API int ssba_forward_select(const ssba_desc* desc, const void* Q, const voi
                                  float* scores_opt, void* O, float* lse, void* workspace, size_t ws_bytes,
                                  void* stream);
 
-/* The whole of Algorithm 1 after RoPE in one launch (Sec. 2.2): block compression (the means
+/* The whole of Algorithm 1 after RoPE in one call (Sec. 2.2): block compression (the means
  * q_b, k_b, with the pooling arithmetic of ssba_pool_blocks, so the same Q, K give the same
- * means and lists), affinity, Top-k gating and the sparse attention. The persistent grid (one
- * CTA per SM) first pools every block of the layer into qb / kb, meets at a grid-wide barrier
- * (bounded wait; a timeout returns through ssba_get_status as SSBA_ERR_TIMEOUT, with O and
- * the lists not written), then runs ssba_forward_select on those means.
+ * means and lists), affinity, Top-k gating and the sparse attention. Up to 16 query blocks an SM
+ * it is one launch: the persistent grid (one CTA per SM) first pools every block of the layer into
+ * qb / kb, meets at a grid-wide barrier (bounded wait; a timeout returns through ssba_get_status
+ * as SSBA_ERR_TIMEOUT, with O and the lists not written), then runs ssba_forward_select on those
+ * means. Above, it is ssba_pool_blocks and ssba_forward_select, with no grid-wide wait.
  *   qb, kb      device out, fp32 [B][heads][Tb][head_dim], 16-byte aligned: the block means.
  *   workspace   REQUIRED here, at least ssba_forward_workspace_bytes(desc) bytes: it holds the
  *               barrier's counters. The rules of ssba_forward's workspace hold (zero-filled before
  *               first use, left zero-filled, zeroed again after SSBA_ERR_TIMEOUT, one per stream).
  *   the rest    as ssba_forward_select.
- * The barrier needs every CTA of the grid (one per SM, at most the SM count) resident at once:
+ * The barrier of the one launch needs every CTA of the grid (one per SM, at most the SM count) resident at once:
  * work on other streams that holds SMs for longer than the wait budget (2 s) makes the call end
  * with SSBA_ERR_TIMEOUT instead of waiting for it. The fallback with no grid-wide wait is
  * ssba_pool_blocks then ssba_forward_select on the same buffers (the same means, lists and
@@ -282,7 +284,8 @@ SSBA_API int ssba_haar_iwt_pyramid(void* const* y, void* x, int32_t N, int32_t C
  *   bias    device fp32 [3 * Dm], or NULL.
  *   Q, K, V device out, bf16 [B][heads][N][64] (RoPE applied to Q and K).
  *   qb, kb  device out, fp32 [B][heads][Tb][64]: means of the bf16 Q and K over each block of
- *           the shifted grid (the layout ssba_select_mask reads); both NULL to skip them.
+ *           the shifted grid (the layout ssba_select_mask reads); both NULL to skip them. Summed
+ *           in the projection or by a pooling launch behind it, by shift and size.
  * desc: dtype SSBA_BF16, head_dim 64, block 8, shifts multiples of 4. All device pointers
  * 16-byte aligned. fp32 accumulation. Returns SSBA_ERR_UNSUPPORTED for other shapes. */
 SSBA_API int ssba_qkv_rope_pool(const ssba_desc* desc, const void* X, const void* Wqkv, const float* bias, void* Q,

@@ -391,7 +391,7 @@ def _forward_select_call(fn_name, desc, Q, K, V, qb, kb, kv_idx, kv_cnt, scores,
 
 def forward_select(desc: SsbaDesc, Q, K, V, qb, kb, kv_idx=None, kv_cnt=None, scores: bool | torch.Tensor = False,
                    O=None, lse=None, workspace="default", stream=None):
-    """ssba_forward_select: selection inside the attention launch. Returns (O, lse, kv_idx, kv_cnt[, S])."""
+    """ssba_forward_select: selection and attention on given block means. Returns (O, lse, kv_idx, kv_cnt[, S])."""
     if qb is None or kb is None:
         raise SsbaError(SSBA_ERR_INVALID, "forward_select needs the block means qb, kb")
     _, _, kv_idx, kv_cnt, S, O, lse = _forward_select_call("ssba_forward_select", desc, Q, K, V, qb, kb, kv_idx,
@@ -401,7 +401,7 @@ def forward_select(desc: SsbaDesc, Q, K, V, qb, kb, kv_idx=None, kv_cnt=None, sc
 
 def forward_fused(desc: SsbaDesc, Q, K, V, qb=None, kb=None, kv_idx=None, kv_cnt=None,
                   scores: bool | torch.Tensor = False, O=None, lse=None, workspace="default", stream=None):
-    """ssba_forward_fused: pooling, selection and attention in one launch.
+    """ssba_forward_fused: pooling, selection and attention in one call.
     Returns (O, lse, kv_idx, kv_cnt, qb, kb[, S])."""
     if workspace is None:
         raise SsbaError(SSBA_ERR_WORKSPACE, "forward_fused needs a forward workspace")
@@ -678,7 +678,7 @@ def realized_sparsity(desc: SsbaDesc) -> float:
 class BoundSelectLayer:
     """One SSBA layer on the one-launch selection path: ``pool()`` (ssba_pool_blocks) and
     ``attend()`` (ssba_forward_select, which also writes the kept-block lists), or ``fused()``
-    (ssba_forward_fused: both in one launch), buffers validated once and bare C calls after
+    (ssba_forward_fused: both in one call), buffers validated once and bare C calls after
     that."""
 
     def __init__(self, desc: SsbaDesc, Q, K, V, qb, kb, kv_idx, kv_cnt, O, lse, stream=None,

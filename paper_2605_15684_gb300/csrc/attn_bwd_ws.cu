@@ -24,8 +24,8 @@
 // Pairs are counted across items: the next item's tiles arrive while the last item computes,
 // and its first products run while the compute warps store the last item's gradients.
 // What bounds it: the tensor pipe's 64 x 64 products and the chain of hand-offs between them (S, dP ->
-// registers -> bf16 operands -> products). At 2048 px a pair takes a CTA 1690 cycles, of which the products
-// of the SM's two CTAs take about 1230 (44 cycles each, 14 a pair); alone on its SM a CTA takes 1430. So
+// registers -> bf16 operands -> products). At 2048 px a pair takes a CTA 1810 cycles, of which the products
+// of the SM's two CTAs take about 1230 (44 cycles each, 14 a pair); alone on its SM a CTA takes 1540. So
 // the compute warps' instructions count: the statistics come as addends for packed two-column
 // arithmetic, and the pair loop's waits return no verdict (wait_phase). 24 heads, a call, before these
 // and now: 1024 px 139.4, 132.2 us, four 1024 px images 701, 664, 2048 px 1556, 1460 (the threads that

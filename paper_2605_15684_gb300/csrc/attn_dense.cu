@@ -21,7 +21,7 @@
 //                  attn_tc.cu); where the last chunk alone does not, m is raised by a whole number and
 //                  P rescaled. At the end of a unit they write O / l in bf16 and lse.
 // TMEM of a stream: S 128 + P 64 (bf16 pairs) + O 64 = 256 columns; the two streams take 512.
-// What bounds it: a tile takes about 1130 cycles of an SM, of which the tensor pipe is busy 608 (QK 4 x
+// What bounds it: a tile takes about 1200 cycles of an SM, of which the tensor pipe is busy 608 (QK 4 x
 // 80, PV 8 x 36) and a scheduler's softmax warps about 800 (128 exp2s a row and what is around them).
 // 24 heads: 1024 px 137 -> 116 us (890 TFLOP/s; its last round of tiles leaves half the SMs idle), 2048
 // px 1852 -> 1513 us (1090 TFLOP/s), against the kernel that read S twice (maximum, then exp2s), had

@@ -15,7 +15,7 @@
 // hand-off where two tiles had two, and a softmax thread owns a whole row of 64 scores. An item
 // left over at the end of a pipeline's work takes both halves: the first half of its list in A,
 // the second in B, merged at the end (two partial softmax sums).
-// What bounds it: a step of each of the CTA's two pipelines takes about 1550 cycles, of which the
+// What bounds it: a step of each of the CTA's two pipelines takes 1430 (long lists) to 1600 cycles, of which the
 // tensor pipe is busy 2 x 608 (QK 4 x 80, PV 8 x 36) and the softmax needs 2 x 435 of its scheduler;
 // the rest is hand-offs (mbarrier waits, tensor-memory round trips) that two chains do not quite
 // cover. Forward on given lists, 24 heads, GPU time against the kernel with one 64-row tile per
