@@ -21,11 +21,14 @@
 //                  attn_tc.cu); where the last chunk alone does not, m is raised by a whole number and
 //                  P rescaled. At the end of a unit they write O / l in bf16 and lse.
 // TMEM of a stream: S 128 + P 64 (bf16 pairs) + O 64 = 256 columns; the two streams take 512.
-// What bounds it: a tile takes about 1200 cycles of an SM, of which the tensor pipe is busy 608 (QK 4 x
+// What bounds it: a tile takes about 1050 cycles of an SM, of which the tensor pipe is busy 608 (QK 4 x
 // 80, PV 8 x 36) and a scheduler's softmax warps about 800 (128 exp2s a row and what is around them).
-// 24 heads: 1024 px 137 -> 116 us (890 TFLOP/s; its last round of tiles leaves half the SMs idle), 2048
-// px 1852 -> 1513 us (1090 TFLOP/s), against the kernel that read S twice (maximum, then exp2s), had
-// one issuer for both products and 2-stage rings. Releasing S only after the last exp2s: 131 and 1772.
+// 24 heads: 1024 px 137 -> 98 us (1050 TFLOP/s; its last round of tiles leaves half the SMs idle), 2048
+// px 1852 -> 1310 us (1260 TFLOP/s), against the kernel that read S twice (maximum, then exp2s), had
+// one issuer for both products and 2-stage rings. With the wait for P's buffer in front of a tile's
+// exp2s instead of its second chunk's store: 115 and 1500. (In front of the first chunk's store: 101 and
+// 1330; of the third's: as of the second's.) Releasing S only after the last exp2s: 131 and 1772;
+// already when half of it is formed and the rest in registers: 2 % slower than as it is.
 // Every wait is bounded (globaltimer budget + CTA abort flag); a timeout is reported in
 // the device status word and the roles drain their copies and products before the CTA exits.
 #include <cuda.h>
@@ -294,6 +297,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                 const float2 c2 = make_float2(c, c);
                 // P = exp2(s c - m) of one chunk in bf16 to tensor memory, its row sum onto ls2
                 float2 ls2[2];
+                uint32_t pk0[16];  // chunk 0 of P, until the buffer is free
                 auto exps = [&](int ch, const uint32_t (&r)[32]) {
                     const float2 nm2 = make_float2(-m_used, -m_used);
                     uint32_t pk[16];
@@ -304,6 +308,17 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                         const float2 pp = make_float2(fast_exp2(x.x), fast_exp2(x.y));
                         ls2[e & 1] = __fadd2_rn(ls2[e & 1], pp);
                         pk[e] = pack_bf16(pp.x, pp.y);
+                    }
+                    if (ch == 0) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) pk0[e] = pk[e];
+                        return;
+                    }
+                    // P's buffer is free once PV_{g-1} has finished (O then holds every earlier PV)
+                    if (ch == 1) {
+                        if (g >= 1) wait_phase(smem_u32(&ct.o_full), (g - 1) & 1, abort_at, p.budget_ns);
+                        tc_fence_after();
+                        tmem_st_32x32b_x16(pcol, pk0);
                     }
                     tmem_st_32x32b_x16(pcol + 16 * ch, pk);
                 };
@@ -319,9 +334,6 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                         tmem_st_32x32b_x16(ocol + h2 * 16, o);
                     }
                 };
-                // P's buffer is free once PV_{g-1} has finished (O then holds every earlier PV)
-                if (g >= 1) wait_phase(smem_u32(&ct.o_full), (g - 1) & 1, abort_at, p.budget_ns);
-                tc_fence_after();
                 uint32_t r[32];
                 // chunks 0-2; the first tile takes its maximum first, and so does a tile whose sum
                 // comes out too large (S is still there)
@@ -344,7 +356,11 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                         const float alpha = over && j > 0 ? fast_exp2(m_used - mx2) : 1.f;
                         m_used = over ? mx2 : m_used;
                         l *= alpha;
-                        if (j > 0) rescale_o(alpha);
+                        if (j > 0) {
+                            wait_phase(smem_u32(&ct.o_full), (g - 1) & 1, abort_at, p.budget_ns);
+                            tc_fence_after();
+                            rescale_o(alpha);
+                        }
                     }
                     ls2[0] = ls2[1] = make_float2(0.f, 0.f);
 #pragma unroll
