@@ -344,7 +344,6 @@ __global__ void __launch_bounds__(kSelWarps * 32) ssba_select_kernel(const float
 
 
 constexpr int kFuseCluster = 8;    // CTAs per (batch, head)
-constexpr int kFuseWarps = 8;
 // Longest rows of the fused build. With 256 blocks a head (2048 px) its 192 CTAs are 32 rows each and
 // fall unevenly on the SMs: 43 us, against 13 (pooling) + 25 (selection) for the two kernels; at 144
 // blocks 24 against 21; at 64 it takes 8.8 against 4.2 + 6.2.
@@ -379,7 +378,7 @@ __device__ __forceinline__ void affinity_select(const float* q, const float* kbs
 // One cluster of kFuseCluster CTAs per (batch*head); CTA r of the cluster owns the blocks
 // [r * bpc, (r + 1) * bpc) ∩ [0, Tb).
 // smem: qown [bpc][64] | kbs [Tb][64] (the head's k_b, 16-byte chunks swizzled by row)
-//   1. pool: warp w takes (block, tensor) units w, w + 8, ... of its CTA; lane l covers
+//   1. pool: warp w takes (block, tensor) units w, w + kFuseWarps, ... of its CTA; lane l covers
 //      16-byte chunk l % CPR of rows l / CPR + RPI * i, summed in row order, then across
 //      lanes by shuffles (fixed order); a q_b mean goes to qown, a k_b mean into kbs of every
 //      CTA of the cluster (distributed shared memory stores, one per CTA and chunk).
@@ -387,7 +386,7 @@ __device__ __forceinline__ void affinity_select(const float* q, const float* kbs
 //      it, and none follow it, so a CTA may leave once it is done).
 //   3. one warp per owned query block: S row by four interleaved partial sums over d, its
 //      keys in registers, then the radix walk (affinity_select).
-template <typename T>
+template <typename T, int kFuseWarps>
 __global__ void __launch_bounds__(kFuseWarps * 32) ssba_mask_fused_kernel(const T* __restrict__ Q,
                                                                           const T* __restrict__ K, Grid g,
                                                                           int keep, int bpc,
@@ -704,9 +703,14 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     // that only two fit in, so that its clusters spread: 1024 px mask and forward 49.6 -> 46.8 us, 768 x
     // 1408 px 56.3 -> 53.1 (batch 4, with more CTAs than that, is faster with three: 29.9 -> 28.7).
     if (d.B * d.heads * kFuseCluster <= 2 * device_sm_count() && smem < 80 * 1024) smem = 80 * 1024;
+    // Warps of a CTA: one per block, where a CTA's nine to twelve blocks would be two rounds of eight warps and
+    // two such CTAs share an SM (768 x 1408 px, 66 blocks, mask and forward 54.5 -> 52.0 us, 1152 px 67.6
+    // -> 65.9; 16 warps 54.5 and 68.1). At up to eight blocks the four more are idle and only cost room
+    // (512 px 14.8 either way, four 1024 px images 183 -> 188).
+    const bool wide = bpc > 8 && bpc <= 12 && d.B * d.heads * kFuseCluster <= 2 * device_sm_count();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kFuseCluster, d.B * d.heads, 1);
-    cfg.blockDim = dim3(kFuseWarps * 32, 1, 1);
+    cfg.blockDim = dim3(wide ? 12 * 32 : 8 * 32, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -724,9 +728,10 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     };
     const cudaError_t e =
         d.dtype == SSBA_BF16
-            ? launch(ssba_mask_fused_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(Q),
-                     static_cast<const __nv_bfloat16*>(K))
-            : launch(ssba_mask_fused_kernel<float>, static_cast<const float*>(Q), static_cast<const float*>(K));
+            ? launch(wide ? ssba_mask_fused_kernel<__nv_bfloat16, 12> : ssba_mask_fused_kernel<__nv_bfloat16, 8>,
+                     static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K))
+            : launch(wide ? ssba_mask_fused_kernel<float, 12> : ssba_mask_fused_kernel<float, 8>,
+                     static_cast<const float*>(Q), static_cast<const float*>(K));
     if (e != cudaSuccess) {
         set_error("ssba_mask_fused_kernel launch: %s", cudaGetErrorString(e));
         return SSBA_ERR_CUDA;

@@ -87,3 +87,17 @@ def test_fused_with_many_items_equals_two_calls():
     for a, b, c in ((idx, idx2, idx3), (cnt, cnt2, cnt3), (O, O2, O3), (lse, lse2, lse3)):
         assert torch.equal(a, b) and torch.equal(a, c)
     assert bool(torch.isfinite(S3).all())
+
+
+@pytest.mark.parametrize("h,H,W", [(3, 64, 64), (3, 8, 520), (24, 48, 88), (2, 64, 96), (2, 72, 88), (40, 48, 88)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_one_launch_mask_by_blocks_a_cta(h, H, W, dtype):
+    """64 blocks a head (eight a CTA), 65 and 66 (nine), 96 (twelve), 99 (thirteen), and 66 with more CTAs than two
+    an SM: the lists of the same means, pooled and selected apart."""
+    desc = api.SsbaDesc(1, h, H, W, shift_r=4, shift_c=4, rho=0.84, dtype=dtype)
+    g = torch.Generator(device="cuda").manual_seed(H * W)
+    q, k = (torch.randn(1, h, H * W, 64, generator=g, device="cuda").to(dtype) for _ in range(2))
+    idx, cnt = api.build_mask(desc, q, k)
+    idx2, cnt2 = api.select_mask(desc, *api.pool_blocks(desc, q, k))
+    torch.cuda.synchronize()
+    assert torch.equal(idx, idx2) and torch.equal(cnt, cnt2)
