@@ -346,7 +346,10 @@ __global__ void __launch_bounds__(kSelWarps * 32) ssba_select_kernel(const float
 constexpr int kFuseCluster = 8;    // CTAs per (batch, head)
 // Longest rows of the fused build. With 256 blocks a head (2048 px) its 192 CTAs are 32 rows each and
 // fall unevenly on the SMs: 43 us, against 13 (pooling) + 25 (selection) for the two kernels; at 144
-// blocks 24 against 21; at 64 it takes 8.8 against 4.2 + 6.2.
+// blocks 24 against 21, at 128 22.8 against 25.6; at 64 it takes 8.8 against 4.2 + 6.2. Where its CTAs are
+// more than two an SM, rows of more than 64 blocks go to the two kernels as well (mask and forward of
+// two images, 81 blocks a head 118.9 -> 114.3 us, 120 blocks 210 -> 202; four images of 64 blocks 182.4
+// either way).
 constexpr int kFuseMaxTb = 128;
 
 // Affinity row of one query block with the keys held in registers (lane l: labels l + 32 m), then
@@ -696,18 +699,18 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
                       int32_t* cnt, float* scores, cudaStream_t st)
 {
     const int Tb = g.Tb();
-    if (d.head_dim != 64 || g.blk != 8 || Tb > kFuseMaxTb) return SSBA_ERR_UNSUPPORTED;
+    const bool spread = d.B * d.heads * kFuseCluster <= 2 * device_sm_count();
+    if (d.head_dim != 64 || g.blk != 8 || Tb > (spread ? kFuseMaxTb : 64)) return SSBA_ERR_UNSUPPORTED;
     const int bpc = (Tb + kFuseCluster - 1) / kFuseCluster;
     size_t smem = ((size_t)bpc * 64 + (size_t)Tb * 64) * sizeof(float);
     // The kernel's registers let three CTAs share an SM. A grid of up to two an SM asks for shared memory
     // that only two fit in, so that its clusters spread: 1024 px mask and forward 49.6 -> 46.8 us, 768 x
     // 1408 px 56.3 -> 53.1 (batch 4, with more CTAs than that, is faster with three: 29.9 -> 28.7).
-    if (d.B * d.heads * kFuseCluster <= 2 * device_sm_count() && smem < 80 * 1024) smem = 80 * 1024;
-    // Warps of a CTA: one per block, where a CTA's nine to twelve blocks would be two rounds of eight warps and
-    // two such CTAs share an SM (768 x 1408 px, 66 blocks, mask and forward 54.5 -> 52.0 us, 1152 px 67.6
+    if (spread && smem < 80 * 1024) smem = 80 * 1024;
+    // Warps of a CTA: one per block, where a CTA's nine to twelve blocks would be two rounds of eight warps (768 x 1408 px, 66 blocks, mask and forward 54.5 -> 52.0 us, 1152 px 67.6
     // -> 65.9; 16 warps 54.5 and 68.1). At up to eight blocks the four more are idle and only cost room
     // (512 px 14.8 either way, four 1024 px images 183 -> 188).
-    const bool wide = bpc > 8 && bpc <= 12 && d.B * d.heads * kFuseCluster <= 2 * device_sm_count();
+    const bool wide = bpc > 8 && bpc <= 12;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kFuseCluster, d.B * d.heads, 1);
     cfg.blockDim = dim3(wide ? 12 * 32 : 8 * 32, 1, 1);

@@ -93,7 +93,7 @@ def test_fused_with_many_items_equals_two_calls():
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_one_launch_mask_by_blocks_a_cta(h, H, W, dtype):
     """64 blocks a head (eight a CTA), 65 and 66 (nine), 96 (twelve), 99 (thirteen), and 66 with more CTAs than two
-    an SM: the lists of the same means, pooled and selected apart."""
+    an SM (two kernels): the lists of the same means, pooled and selected apart."""
     desc = api.SsbaDesc(1, h, H, W, shift_r=4, shift_c=4, rho=0.84, dtype=dtype)
     g = torch.Generator(device="cuda").manual_seed(H * W)
     q, k = (torch.randn(1, h, H * W, 64, generator=g, device="cuda").to(dtype) for _ in range(2))
