@@ -19,6 +19,7 @@
 //                       q_b/k_b round trip through global memory and no second launch.
 #include <cooperative_groups.h>
 #include <cstdio>
+#include <type_traits>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -173,13 +174,16 @@ __device__ __forceinline__ void select_rows(const uint32_t* S, int Tb, int keep,
 
 // Affinity and gating for head_dim 64: a CTA takes kSelWarps * kRows rows of one head, warp w the rows
 // [w kRows, (w + 1) kRows) of them; the keys' means pass through shared memory 128 at a time (rows of
-// 68 floats: 8 consecutive rows cover the banks), a lane scores 4 keys against its warp's kRows rows,
-// and the walks (ballot_select) read the finished rows of keys back from shared memory.
-// What bounds it: the shared-memory reads of the scores (4 + kRows 16-byte chunks for 16 kRows
-// multiply-adds) and the counts of the gating. kRows (24 heads, us for 1, 2, 4): 510 blocks 94, 69, 64;
-// 324 blocks 50, 44, 40; 256 blocks 31, 25, 28; 64 blocks at batch 4 12.8, 9.9, 10.6, at batch 1 7.4,
-// 6.2, 9.6; 16 blocks 3.8, 4.5, 6.0 (fewer CTAs than SMs). The kernel before (one row a warp, keys
-// transposed one word at a time, a 32-bit radix walk over shared memory): 195, 91, 99, 15, 6.8, 3.0.
+// 68 floats: 8 consecutive rows cover the banks), a lane scores 4 keys (2 or 1 of the last few) against
+// its warp's kRows rows at a time, and the walks (ballot_select) read the finished rows of keys back from
+// shared memory.
+// What bounds it: the latency of the gating's counts (36 of 53 us at 510 blocks) and the shared-memory
+// reads of the scores, 4 + kRows 16-byte chunks for 16 kRows multiply-adds of a lane. (One key at a time:
+// 510 blocks 62 us, 324 39.7, 256 24.0, 64 at batch 4 9.3; now 53, 35, 21 and 8.7.) kRows, 24 heads, us for
+// 2 and 4: 510 blocks 56, 53; 324 blocks 36.4, 35.5; 256 blocks 20.7, 23.0; for 1 and 2, one key at a
+// time: 64 blocks at batch 4 12.8, 9.9, at batch 1 7.4, 6.2; 16 blocks 3.8, 4.5 (fewer CTAs than SMs). The
+// kernel before (one row a warp, keys transposed one word at a time, a 32-bit radix walk over shared
+// memory): 510 blocks 195, 256 91, 64 at batch 4 15.
 constexpr int kSel64Keys = 128, kSel64Ld = 68;
 template <int kRows>
 __global__ void __launch_bounds__(kSelWarps * 32, kRows == 2 ? 3 : 2) ssba_select64_kernel(const float* __restrict__ qb,
@@ -213,21 +217,33 @@ __global__ void __launch_bounds__(kSelWarps * 32, kRows == 2 ? 3 : 2) ssba_selec
             if (j < nk) *reinterpret_cast<float4*>(ks + j * kSel64Ld + 4 * c) = __ldg(kbh + (size_t)(j0 + j) * (kD / 4) + c);
         }
         __syncthreads();
+        auto score = [&](auto n) {  // decltype(n)::value keys of a lane at a time; those past nk are not used
+            constexpr int kKeys = decltype(n)::value;
 #pragma unroll
-        for (int m = 0; m < kPerLane; ++m) {
-            const int j = lane + 32 * m;
-            if (j >= nk) break;
-            float acc[kRows];
-            sel::affinity<kRows>(acc, qs + warp * kRows * kD, kD, [&](int c) {
-                return *reinterpret_cast<const float4*>(ks + j * kSel64Ld + 4 * c);
-            });
+            for (int m0 = 0; m0 < kPerLane; m0 += kKeys) {
+                if (32 * m0 >= nk) break;
+                float acc[kKeys][kRows];
+                sel::affinity_keys<kRows, kKeys>(acc, qs + warp * kRows * kD, kD, [&](int k, int c) {
+                    return *reinterpret_cast<const float4*>(ks + (lane + 32 * (m0 + k)) * kSel64Ld + 4 * c);
+                });
 #pragma unroll
-            for (int r = 0; r < kRows; ++r) {
-                if (r >= rows) break;
-                Sw[(size_t)r * Tb + j0 + j] = sel::order_key(acc[r]);
-                if (scores) scores[((size_t)bh * Tb + row0 + r) * Tb + j0 + j] = acc[r];
+                for (int k = 0; k < kKeys; ++k) {
+                    const int j = lane + 32 * (m0 + k);
+#pragma unroll
+                    for (int r = 0; r < kRows; ++r) {
+                        if (r >= rows || j >= nk) break;
+                        Sw[(size_t)r * Tb + j0 + j] = sel::order_key(acc[k][r]);
+                        if (scores) scores[((size_t)bh * Tb + row0 + r) * Tb + j0 + j] = acc[k][r];
+                    }
+                }
             }
-        }
+        };
+        if (kRows > 1 && nk > kSel64Keys / 2)
+            score(std::integral_constant<int, 4>{});
+        else if (nk > 32)
+            score(std::integral_constant<int, 2>{});
+        else
+            score(std::integral_constant<int, 1>{});
     }
     __syncwarp();
     int32_t* dst = idx + ((size_t)bh * Tb + row0) * keep;

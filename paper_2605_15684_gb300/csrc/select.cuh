@@ -122,29 +122,47 @@ __device__ __forceinline__ void ballot_select(const uint32_t (&key)[kPer], int T
     }
 }
 
-// One affinity S = q_b . k_b: four interleaved partial sums over d (components of 16-byte chunks, in
-// chunk order), added as (a0 + a1) + (a2 + a3), for kRows rows of q at once (each k chunk is read
-// once for all of them). q: row r at q + r * qld; chunk(c) gives k_b's c-th 16-byte chunk. Every
+// Affinities S = q_b . k_b: four interleaved partial sums over d (components of 16-byte chunks, in
+// chunk order), added as (a0 + a1) + (a2 + a3), for kRows rows of q and kKeys of k_b at once (each
+// chunk is read once for all of them). q: row r at q + r * qld; chunk(k, c): key k's c-th chunk. Every
 // path uses this order, so the same means give the same scores and lists. The pairs (a0, a1) and
 // (a2, a3) go out as packed multiply-adds, with the roundings of single ones.
-template <int kRows, class Chunk>
-__device__ __forceinline__ void affinity(float (&s)[kRows], const float* q, int qld, Chunk chunk)
+template <int kRows, int kKeys, class Chunk>
+__device__ __forceinline__ void affinity_keys(float (&s)[kKeys][kRows], const float* q, int qld, Chunk chunk)
 {
-    float2 lo[kRows], hi[kRows];
+    float2 lo[kKeys][kRows], hi[kKeys][kRows];
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) lo[r] = hi[r] = make_float2(0.f, 0.f);
+    for (int k = 0; k < kKeys; ++k)
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) lo[k][r] = hi[k][r] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
-        const float4 k = chunk(c);
+        float4 kv[kKeys];
+#pragma unroll
+        for (int k = 0; k < kKeys; ++k) kv[k] = chunk(k, c);
 #pragma unroll
         for (int r = 0; r < kRows; ++r) {
             const float4 v = *reinterpret_cast<const float4*>(q + r * qld + 4 * c);
-            lo[r] = __ffma2_rn(make_float2(v.x, v.y), make_float2(k.x, k.y), lo[r]);
-            hi[r] = __ffma2_rn(make_float2(v.z, v.w), make_float2(k.z, k.w), hi[r]);
+#pragma unroll
+            for (int k = 0; k < kKeys; ++k) {
+                lo[k][r] = __ffma2_rn(make_float2(v.x, v.y), make_float2(kv[k].x, kv[k].y), lo[k][r]);
+                hi[k][r] = __ffma2_rn(make_float2(v.z, v.w), make_float2(kv[k].z, kv[k].w), hi[k][r]);
+            }
         }
     }
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) s[r] = (lo[r].x + lo[r].y) + (hi[r].x + hi[r].y);
+    for (int k = 0; k < kKeys; ++k)
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) s[k][r] = (lo[k][r].x + lo[k][r].y) + (hi[k][r].x + hi[k][r].y);
+}
+
+template <int kRows, class Chunk>
+__device__ __forceinline__ void affinity(float (&s)[kRows], const float* q, int qld, Chunk chunk)
+{
+    float t[1][kRows];
+    affinity_keys<kRows, 1>(t, q, qld, [&](int, int c) { return chunk(c); });
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) s[r] = t[0][r];
 }
 
 }  // namespace sel
