@@ -723,9 +723,10 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     // that only two fit in, so that its clusters spread: 1024 px mask and forward 49.6 -> 46.8 us, 768 x
     // 1408 px 56.3 -> 53.1 (batch 4, with more CTAs than that, is faster with three: 29.9 -> 28.7).
     if (spread && smem < 80 * 1024) smem = 80 * 1024;
-    // Warps of a CTA: one per block, where a CTA's nine to twelve blocks would be two rounds of eight warps (768 x 1408 px, 66 blocks, mask and forward 54.5 -> 52.0 us, 1152 px 67.6
-    // -> 65.9; 16 warps 54.5 and 68.1). At up to eight blocks the four more are idle and only cost room
-    // (512 px 14.8 either way, four 1024 px images 183 -> 188).
+    // Warps of a CTA: one per block, where a CTA's nine to twelve blocks would be two rounds of eight warps
+    // (768 x 1408 px, 66 blocks, mask and forward 54.5 -> 52.0 us, 1152 px 67.6 -> 65.9; 16 warps 54.5 and
+    // 68.1). At up to eight blocks the four more are idle and only cost room (512 px 14.8 either way, four
+    // 1024 px images 183 -> 188).
     const bool wide = bpc > 8 && bpc <= 12;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kFuseCluster, d.B * d.heads, 1);
