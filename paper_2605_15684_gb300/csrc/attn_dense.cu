@@ -384,7 +384,9 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                 over = j > 0 && !(ls <= kRaise);
                 if (__any_sync(0xffffffffu, over)) {
                     // the last chunk alone came out too large: m is raised by a whole number, so that the
-                    // rest of P (bf16) is rescaled exactly
+                    // rest of P (bf16) is rescaled exactly; or, where nothing of that rest is left (alpha is 0),
+                    // to the chunk's maximum itself, as the sum with a very low m (scores of -inf, or of -1e10)
+                    // would not hold it
                     float mx = __uint_as_float(r[0]);
 #pragma unroll
                     for (int e = 1; e < 32; ++e) mx = fmaxf(mx, __uint_as_float(r[e]));
@@ -405,7 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                     }
                     l *= alpha;
                     ls2[0] = ls2[1] = make_float2(0.f, 0.f);
-                    m_used += up;
+                    m_used = up > 256.f ? mx * c : m_used + up;
                     exps(3, r);
                     ls = sum() + ls012 * alpha;
                 }

@@ -135,3 +135,32 @@ def test_dense_reference_maximum_raised(scale, ramp):
         tol = 2e-2 + 2.0 ** -20 * np.abs(m) * np.abs(v[0, h].double().numpy()).max()
         assert np.all(np.abs(O[0, h].float().cpu().numpy() - ref) <= tol)
         assert np.allclose(lse[0, h].cpu().numpy(), (m + np.log(e.sum(axis=1, keepdims=True)))[:, 0], rtol=1e-5, atol=1e-2)
+
+
+@pytest.mark.parametrize("low", [float("-inf"), -2.0 ** 37])
+@pytest.mark.parametrize("far", [16.0, -16.0])
+def test_dense_first_keys_masked_by_low_scores(low, far):
+    """Every key but the last 32 of the second tile scores -inf, or -2^37: the reference maximum is that low
+    until those 32 come, in a tile's last chunk. Their scaled scores lie around +-177, where exp2 against a
+    reference of 0 is out of fp32's range. Softmax over those 32 keys in fp64 is what both must give."""
+    H = W = 16
+    (q, k, v), _ = _inputs(2, H, W, 45)
+    k = k.clone()
+    q, real = (q * 0.5).bfloat16(), torch.arange(H * W) >= 224
+    q[..., 0], q[..., 1] = 1.0, 8.0
+    k[..., 0], k[..., 1] = torch.where(real, 0.0, low).bfloat16(), torch.where(real, far * 8, 0.0).bfloat16()
+    scale = np.float32(np.log(2.0) / 4)  # times log2(e) 0.25 exactly: the low scores have no rounding of their own
+    assert np.float32(scale * np.float32(1.4426950408889634)) == np.float32(0.25)
+    desc = api.SsbaDesc(1, 2, H, W, softmax_scale=float(scale))
+    O, lse = api.forward_dense(desc, q.cuda(), k.cuda(), v.cuda())
+    torch.cuda.synchronize()
+    for h in range(2):
+        s = (q[0, h].double() @ k[0, h, 224:].double().T).numpy() * float(scale)
+        m = s.max(axis=1, keepdims=True)
+        assert (np.abs(m) > 100).all()
+        e = np.exp(s - m)
+        ref = (e / e.sum(axis=1, keepdims=True)) @ v[0, h, 224:].double().numpy()
+        # as in test_reference_maximum_raised
+        tol = 2e-2 + 2.0 ** -20 * np.abs(m) * np.abs(v[0, h].double().numpy()).max()
+        assert np.all(np.abs(O[0, h].float().cpu().numpy() - ref) <= tol)
+        assert np.allclose(lse[0, h].cpu().numpy(), (m + np.log(e.sum(axis=1, keepdims=True)))[:, 0], rtol=1e-5, atol=1e-2)
