@@ -525,9 +525,12 @@ __device__ __forceinline__ void mma_ts_half(int h, uint32_t d_tmem, uint32_t a_t
 
 // Row of a finished item: O / l in bf16 and lse to global memory, O (unnormalised) read from TMEM
 // in two chunks, the other part of a split item (b_o: its row in shared memory, 16-byte chunks
-// swizzled by row) added with weights wa, wb first.
+// swizzled by row) added with weights wa, wb first. A part whose a_ok, b_ok is false has a sum of 0 and
+// counts for nothing; a weight that vanishes does not drop its part, so that an infinity or NaN of V
+// under it comes out as it does where O is rescaled within one half.
 __device__ __forceinline__ void store_row(const TcParams& p, int item, int row, uint32_t ocol, float m, float l,
-                                          const float* b_o, float wa, float wb)
+                                          const float* b_o = nullptr, float wa = 1.f, float wb = 0.f,
+                                          bool a_ok = true, bool b_ok = false)
 {
     const int Tb = p.g.Tb(), N = p.g.H * p.g.W;
     const int bh = item / Tb, label = item - bh * Tb;
@@ -547,8 +550,8 @@ __device__ __forceinline__ void store_row(const TcParams& p, int item, int row, 
                 const float xb[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float a = wa > 0.f ? __uint_as_float(o[4 * i + e]) * wa : 0.f;
-                    o[4 * i + e] = __float_as_uint(wb > 0.f ? fmaf(xb[e], wb, a) : a);
+                    const float a = a_ok ? __uint_as_float(o[4 * i + e]) * wa : 0.f;
+                    o[4 * i + e] = __float_as_uint(b_ok ? fmaf(xb[e], wb, a) : a);
                 }
             }
         }
@@ -959,7 +962,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         auto finish = [&](uint32_t last, int r) {
             wait_pv(last);
             const Round rd = get_round<kSel>(p, ct, r);
-            store_row(p, half ? rd.item[1] : rd.item[0], row, ocol, done_m, done_l, nullptr, 1.f, 0.f);
+            store_row(p, half ? rd.item[1] : rd.item[0], row, ocol, done_m, done_l);
             tc_fence_before();
             owed = false;
         };
@@ -977,7 +980,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
                 if (steps == 0) {  // empty lists: nothing was multiplied; O = 0, lse = -inf
                     if (owed) finish(g - 1, r - 1);
                     if (!split || half == 0)
-                        store_row(p, half ? rd.item[1] : rd.item[0], row, ocol, 0.f, 0.f, nullptr, 1.f, 0.f);
+                        store_row(p, half ? rd.item[1] : rd.item[0], row, ocol, 0.f, 0.f);
                     split = false;
                     continue;
                 }
@@ -1114,10 +1117,11 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
             } else {
                 wait_phase(smem_u32(&ct.merged), 0, abort_at, p.budget_ns);
                 const float2 os = *stat;
-                const bool b_ok = os.y != 0.f;  // an empty part contributes nothing; its O was never written
-                const float m = b_ok ? fmaxf(done_m, os.x) : done_m;
-                const float wa = fast_exp2(done_m - m), wb = b_ok ? fast_exp2(os.x - m) : 0.f;
-                store_row(p, ct.last, row, ocol, m, done_l * wa + (b_ok ? os.y * wb : 0.f), part, wa, wb);
+                const bool a_ok = done_l != 0.f, b_ok = os.y != 0.f;
+                const float m = a_ok ? (b_ok ? fmaxf(done_m, os.x) : done_m) : os.x;
+                const float wa = a_ok ? fast_exp2(done_m - m) : 0.f, wb = b_ok ? fast_exp2(os.x - m) : 0.f;
+                store_row(p, ct.last, row, ocol, m, (a_ok ? done_l * wa : 0.f) + (b_ok ? os.y * wb : 0.f), part, wa,
+                          wb, a_ok, b_ok);
             }
             tc_fence_before();
         }
