@@ -8,6 +8,7 @@ library must exist (``paper_2605_15684_gb300.build.build()`` makes it).
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 import threading
@@ -241,19 +242,36 @@ def forward_workspace_bytes(desc: SsbaDesc) -> int:
     return int(lib.ssba_forward_workspace_bytes(ctypes.byref(d)))
 
 
-def _out(t, name: str, shape, dtype, dev):
+def _empty(shape, dtype, dev, stream=None, scratch=False):
+    """Memory that a call on ``stream`` (None: the current one) writes, from that stream's pool: whatever
+    had it before is done when the call's kernels run, and what takes a scratch area once the call has
+    dropped it runs after them. An output is recorded on the current stream too, where the caller reads
+    and frees it."""
+    if stream is None:
+        return torch.empty(shape, dtype=dtype, device=dev)
+    cur = torch.cuda.current_stream(dev)
+    if stream == cur:
+        return torch.empty(shape, dtype=dtype, device=dev)
+    with torch.cuda.stream(stream):
+        t = torch.empty(shape, dtype=dtype, device=dev)
+    if not scratch:
+        t.record_stream(cur)
+    return t
+
+
+def _out(t, name: str, shape, dtype, dev, stream=None):
     """An output: allocated when the caller gave none, else checked."""
     if t is None:
-        return torch.empty(shape, dtype=dtype, device=dev)
+        return _empty(shape, dtype, dev, stream)
     _check(t, name, shape, dtype)
     return t
 
 
-def _scores_out(scores, pl: _Plan, dev):
+def _scores_out(scores, pl: _Plan, dev, stream=None):
     if isinstance(scores, torch.Tensor):
         _check(scores, "scores", pl.scores, torch.float32)
         return scores
-    return torch.empty(pl.scores, dtype=torch.float32, device=dev) if scores else None
+    return _empty(pl.scores, torch.float32, dev, stream) if scores else None
 
 
 _fwd_ws: dict = {}
@@ -276,7 +294,9 @@ def default_forward_workspace(desc: SsbaDesc, device, stream=None) -> torch.Tens
     with _lock:
         ws = _fwd_ws.get(key)
         if ws is None or ws.numel() < need:
-            ws = torch.zeros(max(need, 1), dtype=torch.uint8, device=dev)
+            # allocated and filled on the stream that uses it
+            with torch.cuda.stream(stream) if stream is not None else contextlib.nullcontext():
+                ws = torch.zeros(max(need, 1), dtype=torch.uint8, device=dev)
             _fwd_ws[key] = ws
     return ws
 
@@ -297,11 +317,11 @@ def build_mask(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, kv_idx=None, kv
     _check(Q, "Q", pl.x, pl.dtype)
     _check(K, "K", pl.x, pl.dtype)
     dev = Q.device
-    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev)
-    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev)
-    S = _scores_out(scores, pl, dev)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, stream)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, stream)
+    S = _scores_out(scores, pl, dev, stream)
     if workspace is None:
-        workspace = torch.empty(int(lib.ssba_mask_workspace_bytes(pl.ref)), dtype=torch.uint8, device=dev)
+        workspace = _empty(int(lib.ssba_mask_workspace_bytes(pl.ref)), torch.uint8, dev, stream, scratch=True)
     rc = lib.ssba_build_mask(pl.ref, Q.data_ptr(), K.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
                              S.data_ptr() if S is not None else None, workspace.data_ptr(),
                              workspace.numel() * workspace.element_size(), _stream_ptr(stream))
@@ -322,8 +342,8 @@ def qkv_rope_pool(desc: SsbaDesc, X: torch.Tensor, Wqkv: torch.Tensor, bias=None
         _check(bias, "bias", (3 * Dm,), torch.float32)
     dev = X.device
     if out is None:
-        out = [torch.empty(pl.x, dtype=torch.bfloat16, device=dev) for _ in range(3)]
-        out += [torch.empty(pl.means, dtype=torch.float32, device=dev) for _ in range(2)] if pooled else [None, None]
+        out = [_empty(pl.x, torch.bfloat16, dev, stream) for _ in range(3)]
+        out += [_empty(pl.means, torch.float32, dev, stream) for _ in range(2)] if pooled else [None, None]
     Q, K, V, qb, kb = out
     for t, n in ((Q, "Q"), (K, "K"), (V, "V")):
         _check(t, n, pl.x, torch.bfloat16)
@@ -345,9 +365,9 @@ def select_mask(desc: SsbaDesc, qb: torch.Tensor, kb: torch.Tensor, kv_idx=None,
     _check(qb, "qb", pl.means, torch.float32)
     _check(kb, "kb", pl.means, torch.float32)
     dev = qb.device
-    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev)
-    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev)
-    S = _scores_out(scores, pl, dev)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, stream)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, stream)
+    S = _scores_out(scores, pl, dev, stream)
     _raise_on(lib.ssba_select_mask(pl.ref, qb.data_ptr(), kb.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
                                    S.data_ptr() if S is not None else None, _stream_ptr(stream)))
     return (kv_idx, kv_cnt, S) if S is not None else (kv_idx, kv_cnt)
@@ -359,8 +379,8 @@ def pool_blocks(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, qb=None, kb=No
     pl = _plan(lib, desc)
     _check(Q, "Q", pl.x, pl.dtype)
     _check(K, "K", pl.x, pl.dtype)
-    qb = _out(qb, "qb", pl.means, torch.float32, Q.device)
-    kb = _out(kb, "kb", pl.means, torch.float32, Q.device)
+    qb = _out(qb, "qb", pl.means, torch.float32, Q.device, stream)
+    kb = _out(kb, "kb", pl.means, torch.float32, Q.device, stream)
     _raise_on(lib.ssba_pool_blocks(pl.ref, Q.data_ptr(), K.data_ptr(), qb.data_ptr(), kb.data_ptr(),
                                    _stream_ptr(stream)))
     return qb, kb
@@ -373,13 +393,13 @@ def _forward_select_call(fn_name, desc, Q, K, V, qb, kb, kv_idx, kv_cnt, scores,
     _check(K, "K", pl.x, pl.dtype)
     _check(V, "V", pl.x, pl.dtype)
     dev = Q.device
-    qb = _out(qb, "qb", pl.means, torch.float32, dev)
-    kb = _out(kb, "kb", pl.means, torch.float32, dev)
-    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev)
-    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev)
-    S = _scores_out(scores, pl, dev)
-    O = _out(O, "O", pl.x, pl.dtype, dev)
-    lse = _out(lse, "lse", pl.rows, torch.float32, dev)
+    qb = _out(qb, "qb", pl.means, torch.float32, dev, stream)
+    kb = _out(kb, "kb", pl.means, torch.float32, dev, stream)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, stream)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, stream)
+    S = _scores_out(scores, pl, dev, stream)
+    O = _out(O, "O", pl.x, pl.dtype, dev, stream)
+    lse = _out(lse, "lse", pl.rows, torch.float32, dev, stream)
     if isinstance(workspace, str):
         workspace = default_forward_workspace(desc, dev, stream)
     wp, wn = _ws_args(workspace)
@@ -419,9 +439,9 @@ def build_mask_noalloc(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, kv_idx=
     _check(Q, "Q", pl.x, pl.dtype)
     _check(K, "K", pl.x, pl.dtype)
     dev = Q.device
-    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev)
-    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev)
-    S = _scores_out(scores, pl, dev)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, stream)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, stream)
+    S = _scores_out(scores, pl, dev, stream)
     rc = lib.ssba_build_mask_noalloc(pl.ref, Q.data_ptr(), K.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
                                      S.data_ptr() if S is not None else None, _stream_ptr(stream))
     _raise_on(rc)
@@ -439,8 +459,8 @@ def forward(desc: SsbaDesc, Q, K, V, kv_idx, kv_cnt, O=None, lse=None, workspace
     _check(V, "V", pl.x, pl.dtype)
     _check(kv_idx, "kv_idx", pl.lists, torch.int32)
     _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
-    O = _out(O, "O", pl.x, pl.dtype, Q.device)
-    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device, stream)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, stream)
     if isinstance(workspace, str):
         # neither kernel uses one here (the fp32 one takes none; bf16 only checks what is given)
         workspace = None
@@ -467,8 +487,8 @@ def forward_joint(desc: SsbaDesc, Q, K, V, K_txt, V_txt, kv_idx, kv_cnt, O=None,
     _check(V_txt, "V_txt", tshp, pl.dtype)
     _check(kv_idx, "kv_idx", pl.lists, torch.int32)
     _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
-    O = _out(O, "O", pl.x, pl.dtype, Q.device)
-    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device, stream)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, stream)
     if isinstance(workspace, str):
         workspace = None  # not used by this call
     wp, wn = _ws_args(workspace)
@@ -487,8 +507,8 @@ def forward_dense(desc: SsbaDesc, Q, K, V, O=None, lse=None, workspace="default"
     _check(Q, "Q", pl.x, pl.dtype)
     _check(K, "K", pl.x, pl.dtype)
     _check(V, "V", pl.x, pl.dtype)
-    O = _out(O, "O", pl.x, pl.dtype, Q.device)
-    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device, stream)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, stream)
     if isinstance(workspace, str):
         workspace = None  # not used by this call
     wp, wn = _ws_args(workspace)
@@ -558,10 +578,10 @@ def backward(desc: SsbaDesc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, dQ=None, dK=No
     _check(lse, "lse", pl.rows, torch.float32)
     _check(kv_idx, "kv_idx", pl.lists, torch.int32)
     _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
-    outs = [_out(t, n, pl.x, torch.float32, Q.device) for t, n in ((dQ, "dQ"), (dK, "dK"), (dV, "dV"))]
+    outs = [_out(t, n, pl.x, torch.float32, Q.device, stream) for t, n in ((dQ, "dQ"), (dK, "dK"), (dV, "dV"))]
     if workspace is None:
         need = int(lib.ssba_backward_workspace_bytes(pl.ref))
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=Q.device)
+        workspace = _empty(max(need, 16), torch.uint8, Q.device, stream, scratch=True)
     wp, wn = _ws_args(workspace)
     args = (pl.ref, Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), lse.data_ptr(), dO.data_ptr(),
             kv_idx.data_ptr(), kv_cnt.data_ptr(), outs[0].data_ptr(), outs[1].data_ptr(), outs[2].data_ptr(), wp, wn)
@@ -595,7 +615,7 @@ def haar_dwt(x: torch.Tensor, nb: int = 4, y=None, stream=None) -> torch.Tensor:
     N, C, H, W = x.shape
     _check(x, "x", (N, C, H, W), x.dtype)
     if y is None:
-        y = torch.empty((N, nb * C, H // 2, W // 2), dtype=x.dtype, device=x.device)
+        y = _empty((N, nb * C, H // 2, W // 2), x.dtype, x.device, stream)
     _check(y, "y", (N, nb * C, H // 2, W // 2), x.dtype)
     _raise_on(lib.ssba_haar_dwt(x.data_ptr(), y.data_ptr(), N, C, H, W, nb, _dtype_code(x), _stream_ptr(stream)))
     return y
@@ -609,7 +629,7 @@ def haar_iwt(y: torch.Tensor, C: int, nb: int = 4, x=None, stream=None) -> torch
     N, nbC, h, w = y.shape
     _check(y, "y", (N, nb * C, h, w), y.dtype)
     if x is None:
-        x = torch.empty((N, C, 2 * h, 2 * w), dtype=y.dtype, device=y.device)
+        x = _empty((N, C, 2 * h, 2 * w), y.dtype, y.device, stream)
     _check(x, "x", (N, C, 2 * h, 2 * w), y.dtype)
     _raise_on(lib.ssba_haar_iwt(y.data_ptr(), x.data_ptr(), N, C, 2 * h, 2 * w, nb, _dtype_code(y), _stream_ptr(stream)))
     return x
@@ -633,7 +653,7 @@ def haar_dwt_pyramid(x: torch.Tensor, levels: int, nb: int = 4, ys=None, stream=
         raise SsbaError(SSBA_ERR_INVALID, f"levels must be 1..{HAAR_MAX_LEVELS}")
     shapes = [(N, nb * C, H >> l, W >> l) for l in range(1, levels + 1)]
     if ys is None:
-        ys = [torch.empty(shp, dtype=x.dtype, device=x.device) for shp in shapes]
+        ys = [_empty(shp, x.dtype, x.device, stream) for shp in shapes]
     if len(ys) != levels:
         raise SsbaError(SSBA_ERR_INVALID, f"ys must hold {levels} tensors")
     for l, (t, shp) in enumerate(zip(ys, shapes)):
@@ -654,7 +674,7 @@ def haar_iwt_pyramid(ys, C: int, nb: int = 4, x=None, stream=None) -> torch.Tens
     for l, t in enumerate(ys):
         _check(t, f"ys[{l}]", (N, nb * C, H >> (l + 1), W >> (l + 1)), ys[0].dtype)
     if x is None:
-        x = torch.empty((N, C, H, W), dtype=ys[0].dtype, device=ys[0].device)
+        x = _empty((N, C, H, W), ys[0].dtype, ys[0].device, stream)
     _check(x, "x", (N, C, H, W), ys[0].dtype)
     _raise_on(lib.ssba_haar_iwt_pyramid(_ptr_array(ys), x.data_ptr(), N, C, H, W, levels, nb, _dtype_code(x),
                                         _stream_ptr(stream)))
