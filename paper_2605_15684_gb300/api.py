@@ -296,6 +296,12 @@ def default_forward_workspace(desc: SsbaDesc, device, stream=None) -> torch.Tens
         if ws is None or ws.numel() < need:
             # allocated and filled on the stream that uses it
             with torch.cuda.stream(stream) if stream is not None else contextlib.nullcontext():
+                if torch.cuda.is_current_stream_capturing():
+                    # the fill is a node of the graph, so no later call may count on it: this area is the
+                    # capture's own, and of it only the barrier words, its last 256 bytes, need the fill
+                    ws = torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
+                    ws[-256:].zero_()
+                    return ws
                 ws = torch.zeros(max(need, 1), dtype=torch.uint8, device=dev)
             _fwd_ws[key] = ws
     return ws

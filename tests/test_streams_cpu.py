@@ -91,3 +91,17 @@ def test_what_a_call_allocates_belongs_to_its_stream(world, i):
     for same in (None, main):  # on the current stream nothing is recorded
         _calls(same)[i]()
         assert made and all(s is main for _, s in made) and not recorded
+
+
+def test_a_workspace_made_in_a_capture_is_not_kept(world, monkeypatch):
+    """Its fill runs when the graph does, so a call outside the graph must not find it; it is zero where a call
+    reads it, and one that exists already is used."""
+    d = api.SsbaDesc(1, 2, 16, 16, rho=0.5)
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: True)
+    ws = api.default_forward_workspace(d, "cuda:0")
+    assert ws.numel() == 1024 and not ws[-256:].any() and not api._fwd_ws
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: False)
+    kept = api.default_forward_workspace(d, "cuda:0")
+    assert not kept.any() and kept is api.default_forward_workspace(d, "cuda:0")
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: True)
+    assert kept is api.default_forward_workspace(d, "cuda:0")

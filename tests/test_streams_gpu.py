@@ -44,3 +44,25 @@ def test_side_stream_with_default_buffers():
         assert api.get_status() == api.SSBA_OK
         for a, b in zip(got, want):
             assert torch.equal(a, b)
+
+
+def test_fused_call_captured_before_any_other_on_its_stream():
+    """A graph whose fused calls are the first on their stream, then a call outside it before its first replay."""
+    q, k, v = (t.cuda() for t in synthetic.qkv(1, 4, 1024, 64, torch.bfloat16, 73))
+    desc = api.SsbaDesc(1, 4, 32, 32, shift_r=4, shift_c=4, rho=0.75)
+    want = api.forward_fused(desc, q, k, v)
+    torch.cuda.synchronize()
+    api._fwd_ws.clear()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        in_graph = [api.forward_fused(desc, q, k, v) for _ in range(2)]
+    s.wait_stream(torch.cuda.current_stream())
+    outside = api.forward_fused(desc, q, k, v, stream=s)
+    torch.cuda.current_stream().wait_stream(s)
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    assert api.get_status() == api.SSBA_OK
+    for got in (*in_graph, outside):
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
