@@ -367,6 +367,14 @@ SSBA_API int ssba_test_backward_timeout(const ssba_desc* desc, const void* Q, co
                                         const int32_t* kv_cnt, float* dQ, float* dK, float* dV, void* workspace,
                                         size_t ws_bytes, uint64_t budget_ns, void* stream);
 
+/* A second hook of the same kind, with the same arguments and outcome: CTA 0 issues its first dP product
+ * only once another of its waits has run out (or after 4 budget_ns), so that what was waited for does come,
+ * late. The status still reads SSBA_ERR_TIMEOUT. */
+SSBA_API int ssba_test_backward_late(const ssba_desc* desc, const void* Q, const void* K, const void* V,
+                                     const void* O, const float* lse, const void* dO, const int32_t* kv_idx,
+                                     const int32_t* kv_cnt, float* dQ, float* dK, float* dV, void* workspace,
+                                     size_t ws_bytes, uint64_t budget_ns, void* stream);
+
 /* Reads and clears the device status word of the current device (SSBA_OK or
  * SSBA_ERR_TIMEOUT). Synchronous: call after the caller's stream sync. Returns
  * SSBA_OK, or SSBA_ERR_CUDA if the read failed. */

@@ -29,7 +29,8 @@ _STATUS_NAMES = {0: "SSBA_OK", 1: "SSBA_ERR_INVALID", 2: "SSBA_ERR_UNSUPPORTED",
 
 EXPORTED = ("ssba_keep_count", "ssba_mask_workspace_bytes", "ssba_build_mask", "ssba_build_mask_noalloc",
             "ssba_forward", "ssba_forward_joint", "ssba_forward_workspace_bytes", "ssba_forward_dense",
-            "ssba_test_forward_timeout", "ssba_test_fused_timeout", "ssba_test_backward_timeout", "ssba_backward", "ssba_backward_workspace_bytes", "ssba_haar_dwt",
+            "ssba_test_forward_timeout", "ssba_test_fused_timeout", "ssba_test_backward_timeout",
+            "ssba_test_backward_late", "ssba_backward", "ssba_backward_workspace_bytes", "ssba_haar_dwt",
             "ssba_haar_iwt", "ssba_haar_dwt_pyramid", "ssba_haar_iwt_pyramid", "ssba_qkv_rope_pool",
             "ssba_select_mask", "ssba_pool_blocks", "ssba_forward_select", "ssba_forward_fused",
             "ssba_get_status", "ssba_last_error", "ssba_timeline_read")
@@ -138,6 +139,8 @@ def load_library(path: str | None = None):
         lib.ssba_test_backward_timeout.argtypes = [DP, P, P, P, P, P, P, P, P, P, P, P, P, ctypes.c_size_t,
                                                    ctypes.c_uint64, P]
         lib.ssba_test_backward_timeout.restype = ctypes.c_int
+        lib.ssba_test_backward_late.argtypes = lib.ssba_test_backward_timeout.argtypes
+        lib.ssba_test_backward_late.restype = ctypes.c_int
         lib.ssba_backward_workspace_bytes.argtypes = [DP]
         lib.ssba_backward_workspace_bytes.restype = ctypes.c_size_t
         I = ctypes.c_int32
@@ -573,10 +576,10 @@ def backward_workspace_bytes(desc: SsbaDesc) -> int:
 
 
 def backward(desc: SsbaDesc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, dQ=None, dK=None, dV=None, workspace=None,
-             stream=None, _timeout_budget_ns=None):
+             stream=None, _timeout_budget_ns=None, _hook="ssba_test_backward_timeout"):
     """ssba_backward: gradients (dQ, dK, dV) in fp32 of the sparse forward for output gradient dO.
-    With _timeout_budget_ns set it calls the failure-detection test hook ssba_test_backward_timeout
-    instead (see include/ssba.h): the gradients are then undefined."""
+    With _timeout_budget_ns set it calls the failure-detection test hook instead (see include/ssba.h):
+    the gradients are then undefined."""
     lib = load_library()
     pl = _plan(lib, desc)
     for t, n in ((Q, "Q"), (K, "K"), (V, "V"), (O, "O"), (dO, "dO")):
@@ -594,7 +597,7 @@ def backward(desc: SsbaDesc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, dQ=None, dK=No
     if _timeout_budget_ns is None:
         rc = lib.ssba_backward(*args, _stream_ptr(stream))
     else:
-        rc = lib.ssba_test_backward_timeout(*args, int(_timeout_budget_ns), _stream_ptr(stream))
+        rc = getattr(lib, _hook)(*args, int(_timeout_budget_ns), _stream_ptr(stream))
     _raise_on(rc)
     return tuple(outs)
 
@@ -603,6 +606,13 @@ def test_backward_timeout(desc: SsbaDesc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, b
                           stream=None) -> None:
     """ssba_test_backward_timeout: the backward's failure-detection test hook (include/ssba.h)."""
     backward(desc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, stream=stream, _timeout_budget_ns=budget_ns)
+
+
+def test_backward_late(desc: SsbaDesc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, budget_ns: int = 2_000_000,
+                       stream=None) -> None:
+    """ssba_test_backward_late: the hook whose product comes after the wait for it (include/ssba.h)."""
+    backward(desc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, stream=stream, _timeout_budget_ns=budget_ns,
+             _hook="ssba_test_backward_late")
 
 
 def _dtype_code(t: torch.Tensor) -> int:

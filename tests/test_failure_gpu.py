@@ -5,7 +5,8 @@ free its tensor memory and report SSBA_ERR_TIMEOUT in the device status word, an
 CUDA context must stay usable (a normal forward right after matches the oracle). A second
 hook makes one CTA of the fused launch withhold its arrival at the grid barrier, so that
 every CTA's barrier wait runs out, with the same requirements. A third makes one CTA of the
-persistent backward announce a pair's tile copies without issuing them."""
+persistent backward announce a pair's tile copies without issuing them, a fourth issue a
+product after the wait for it has run out."""
 import pytest
 import torch
 
@@ -79,10 +80,11 @@ def test_grid_barrier_timeout_reports_status_and_context_survives():
     assert int(ws[-256:].count_nonzero()) == 0
 
 
-def test_backward_timeout_reports_status_and_context_survives():
-    """CTA 0 of the persistent backward never receives its first pair's tiles: its issuers'
-    waits run out, it drains and reports SSBA_ERR_TIMEOUT, the other CTAs finish; a normal
-    backward right after matches the oracle."""
+@pytest.mark.parametrize("hook", ["test_backward_timeout", "test_backward_late"])
+def test_backward_timeout_reports_status_and_context_survives(hook):
+    """CTA 0 of the persistent backward never receives its first pair's tiles, or issues a product of
+    it only after the wait for that product has run out: it drains and reports SSBA_ERR_TIMEOUT, the other
+    CTAs finish; a normal backward right after matches the oracle."""
     build.build()
     api.load_library()
     H = W = 32
@@ -98,7 +100,7 @@ def test_backward_timeout_reports_status_and_context_survives():
     torch.cuda.synchronize()
     assert api.get_status() == api.SSBA_OK
 
-    api.test_backward_timeout(desc, qd, kd, vd, O, lse, god, idx, cnt, budget_ns=2_000_000)
+    getattr(api, hook)(desc, qd, kd, vd, O, lse, god, idx, cnt, budget_ns=2_000_000)
     torch.cuda.synchronize()  # the kernel returns: no hang, no CUDA error
     assert api.get_status() == api.SSBA_ERR_TIMEOUT
     assert api.get_status() == api.SSBA_OK
