@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(128) ssba_pool_generic_kernel(const T* __restr
 constexpr int kSelWarps = 8;
 constexpr int kSelKeyChunk = 256;
 constexpr int kMaxTb = 2048;
+constexpr int kMaxGridY = 65535;  // (batch, head) pairs of a launch; more take several
 
 // Gating of `rows` rows of keys in shared memory (row r at S + r * Tb); kept labels of row r to
 // dst + r * keep.
@@ -585,8 +586,9 @@ int launch_pool_blocks(const ssba_desc& d, const Grid& g, const void* Q, const v
                        cudaStream_t st)
 {
     if (d.head_dim != 64 || g.blk != 8) return launch_pool(d, g, Q, K, qb, kb, st);
+    const int BH = d.B * d.heads;
+    const size_t head = (size_t)g.H * g.W * 64, means = (size_t)g.Tb() * 64;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((g.Tb() + kPoolWin - 1) / kPoolWin, d.B * d.heads, 1);
     cfg.blockDim = dim3(2 * kPoolWin * 32, 1, 1);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -594,17 +596,20 @@ int launch_pool_blocks(const ssba_desc& d, const Grid& g, const void* Q, const v
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e;
-    if (d.dtype == SSBA_BF16)
-        e = cudaLaunchKernelEx(&cfg, ssba_pool_blocks_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(Q),
-                               static_cast<const __nv_bfloat16*>(K), g, qb, kb);
-    else
-        e = cudaLaunchKernelEx(&cfg, ssba_pool_blocks_kernel<float>, static_cast<const float*>(Q),
-                               static_cast<const float*>(K), g, qb, kb);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        set_error("ssba_pool_blocks_kernel launch: %s", cudaGetErrorString(e));
-        return SSBA_ERR_CUDA;
+    for (int h0 = 0; h0 < BH; h0 += kMaxGridY) {
+        cfg.gridDim = dim3((g.Tb() + kPoolWin - 1) / kPoolWin, min(kMaxGridY, BH - h0), 1);
+        auto launch = [&](auto kernel, auto* x) {
+            return cudaLaunchKernelEx(&cfg, kernel, x + h0 * head, static_cast<decltype(x)>(K) + h0 * head, g,
+                                      qb + h0 * means, kb + h0 * means);
+        };
+        cudaError_t e = d.dtype == SSBA_BF16
+                            ? launch(ssba_pool_blocks_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(Q))
+                            : launch(ssba_pool_blocks_kernel<float>, static_cast<const float*>(Q));
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e != cudaSuccess) {
+            set_error("ssba_pool_blocks_kernel launch: %s", cudaGetErrorString(e));
+            return SSBA_ERR_CUDA;
+        }
     }
     return SSBA_OK;
 }
@@ -668,7 +673,6 @@ int launch_select(const ssba_desc& d, const Grid& g, int keep, const float* qb, 
         auto kernel = rows == 4 ? ssba_select64_kernel<4> : (rows == 2 ? ssba_select64_kernel<2> : ssba_select64_kernel<1>);
         if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((Tb + cta - 1) / cta, BH, 1);
         cfg.blockDim = dim3(kSelWarps * 32, 1, 1);
         cfg.dynamicSmemBytes = sm;
         cfg.stream = st;
@@ -677,11 +681,16 @@ int launch_select(const ssba_desc& d, const Grid& g, int keep, const float* qb, 
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, qb, kb, Tb, keep, idx, cnt, scores);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) {
-            set_error("ssba_select64_kernel launch: %s", cudaGetErrorString(e));
-            return SSBA_ERR_CUDA;
+        for (int h0 = 0; h0 < BH; h0 += kMaxGridY) {
+            const size_t row = (size_t)h0 * Tb;
+            cfg.gridDim = dim3((Tb + cta - 1) / cta, min(kMaxGridY, BH - h0), 1);
+            cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, qb + row * 64, kb + row * 64, Tb, keep, idx + row * keep,
+                                               cnt + row, scores ? scores + row * Tb : nullptr);
+            if (e == cudaSuccess) e = cudaGetLastError();
+            if (e != cudaSuccess) {
+                set_error("ssba_select64_kernel launch: %s", cudaGetErrorString(e));
+                return SSBA_ERR_CUDA;
+            }
         }
         return SSBA_OK;
     }

@@ -101,3 +101,17 @@ def test_one_launch_mask_by_blocks_a_cta(h, H, W, dtype):
     idx2, cnt2 = api.select_mask(desc, *api.pool_blocks(desc, q, k))
     torch.cuda.synchronize()
     assert torch.equal(idx, idx2) and torch.equal(cnt, cnt2)
+
+
+def test_fused_with_more_heads_than_a_grid_dimension():
+    """65600 (batch, head) pairs, more than a launch's y dimension holds: as two calls of half of them."""
+    h, H, W = 65600, 8, 16
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, k, v = (torch.randn(1, h, H * W, 64, generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+    got = api.forward_fused(api.SsbaDesc(1, h, H, W, rho=0.5), q, k, v)
+    desc = api.SsbaDesc(1, h // 2, H, W, rho=0.5)
+    for part in (slice(0, h // 2), slice(h // 2, h)):
+        want = api.forward_fused(desc, *(t[:, part] for t in (q, k, v)))
+        for a, b in zip(got, want):
+            assert torch.equal(a[:, part], b)
+    assert api.get_status() == api.SSBA_OK
