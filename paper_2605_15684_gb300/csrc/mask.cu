@@ -155,6 +155,8 @@ __global__ void __launch_bounds__(128) ssba_pool_generic_kernel(const T* __restr
 constexpr int kSelWarps = 8;
 constexpr int kSelKeyChunk = 256;
 constexpr int kMaxTb = 2048;
+constexpr size_t kSelSmem = 220 * 1024;   // largest working set of ssba_select_kernel
+constexpr size_t kPoolSmem = 200 * 1024;  // of ssba_pool_generic_kernel
 constexpr int kMaxGridY = 65535;  // (batch, head) pairs of a launch; more take several
 
 // Gating of `rows` rows of keys in shared memory (row r at S + r * Tb); kept labels of row r to
@@ -368,6 +370,7 @@ constexpr int kFuseCluster = 8;    // CTAs per (batch, head)
 // two images, 81 blocks a head 118.9 -> 114.3 us, 120 blocks 210 -> 202; four images of 64 blocks 182.4
 // either way).
 constexpr int kFuseMaxTb = 128;
+constexpr size_t kFuseSmem = 80 * 1024;  // above every row length's need
 
 // Affinity row of one query block with the keys held in registers (lane l: labels l + 32 m), then
 // the gating. kbs: the head's k_b by rows, the 16-byte chunk c4 of row j at chunk c4 ^ (j & 15) (the 32
@@ -630,19 +633,23 @@ int launch_pool(const ssba_desc& d, const Grid& g, const void* Q, const void* K,
     } else {
         const int P = g.blk * g.blk;
         const size_t smem = (size_t)2 * P * d.head_dim * sizeof(float);
-        if (smem > 200 * 1024) {
+        if (smem > kPoolSmem) {
             set_error("ssba_build_mask: block*block*head_dim too large for the pooling kernel");
             return SSBA_ERR_UNSUPPORTED;
         }
+        static PerDeviceOnce attr;
+        attr.run([] {
+            const int n = (int)kPoolSmem;
+            cudaFuncSetAttribute(ssba_pool_generic_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+            cudaFuncSetAttribute(ssba_pool_generic_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+        });
         dim3 grid(g.Tb(), d.B * d.heads);
         if (d.dtype == SSBA_BF16) {
             auto k = ssba_pool_generic_kernel<__nv_bfloat16>;
-            if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             k<<<grid, 128, smem, st>>>(static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K), g,
                                        d.head_dim, qb, kb);
         } else {
             auto k = ssba_pool_generic_kernel<float>;
-            if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             k<<<grid, 128, smem, st>>>(static_cast<const float*>(Q), static_cast<const float*>(K), g, d.head_dim, qb,
                                        kb);
         }
@@ -671,7 +678,18 @@ int launch_select(const ssba_desc& d, const Grid& g, int keep, const float* qb, 
         const int cta = kSelWarps * rows;
         const size_t sm = ((size_t)kSel64Keys * kSel64Ld + (size_t)cta * 64 + (size_t)cta * Tb) * sizeof(float);
         auto kernel = rows == 4 ? ssba_select64_kernel<4> : (rows == 2 ? ssba_select64_kernel<2> : ssba_select64_kernel<1>);
-        if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        // the largest size of each instantiation, once: a limit set for each call could be lowered by another
+        // thread before this one's launch
+        static PerDeviceOnce attr64;
+        attr64.run([] {
+            auto largest = [](auto k, int rows, int longest) {
+                const size_t n = ((size_t)kSel64Keys * kSel64Ld + (size_t)kSelWarps * rows * (64 + longest)) * sizeof(float);
+                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+            };
+            largest(ssba_select64_kernel<1>, 1, kMaxTb);
+            largest(ssba_select64_kernel<2>, 2, 256);
+            largest(ssba_select64_kernel<4>, 4, 1024);
+        });
         cudaLaunchConfig_t cfg = {};
         cfg.blockDim = dim3(kSelWarps * 32, 1, 1);
         cfg.dynamicSmemBytes = sm;
@@ -696,14 +714,16 @@ int launch_select(const ssba_desc& d, const Grid& g, int keep, const float* qb, 
     }
     size_t smem = ((size_t)d.head_dim * (kSelKeyChunk + 1) + (size_t)kSelWarps * d.head_dim +
                    (size_t)kSelWarps * Tb) * sizeof(float);
-    if (smem > 220 * 1024) {
+    if (smem > kSelSmem) {
         set_error("ssba_build_mask: selection working set too large (%zu bytes)", smem);
         return SSBA_ERR_UNSUPPORTED;
     }
-    cudaFuncSetAttribute(ssba_select_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(ssba_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static PerDeviceOnce attr;
+    attr.run([] {
+        cudaFuncSetAttribute(ssba_select_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
+        cudaFuncSetAttribute(ssba_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem);
+    });
     dim3 grid((Tb + kSelWarps - 1) / kSelWarps, d.B * d.heads);
     ssba_select_kernel<<<grid, kSelWarps * 32, smem, st>>>(qb, kb, Tb, d.head_dim, keep, idx, cnt, scores);
     cudaError_t e = cudaGetLastError();
@@ -731,7 +751,15 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     // The kernel's registers let three CTAs share an SM. A grid of up to two an SM asks for shared memory
     // that only two fit in, so that its clusters spread: 1024 px mask and forward 49.6 -> 46.8 us, 768 x
     // 1408 px 56.3 -> 53.1 (batch 4, with more CTAs than that, is faster with three: 29.9 -> 28.7).
-    if (spread && smem < 80 * 1024) smem = 80 * 1024;
+    if (spread && smem < kFuseSmem) smem = kFuseSmem;
+    static PerDeviceOnce attr_once;
+    attr_once.run([] {
+        auto set = [](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFuseSmem); };
+        set(ssba_mask_fused_kernel<__nv_bfloat16, 8>);
+        set(ssba_mask_fused_kernel<__nv_bfloat16, 12>);
+        set(ssba_mask_fused_kernel<float, 8>);
+        set(ssba_mask_fused_kernel<float, 12>);
+    });
     // Warps of a CTA: one per block, where a CTA's nine to twelve blocks would be two rounds of eight warps
     // (768 x 1408 px, 66 blocks, mask and forward 54.5 -> 52.0 us, 1152 px 67.6 -> 65.9; 16 warps 54.5 and
     // 68.1). At up to eight blocks the four more are idle and only cost room (512 px 14.8 either way, four
@@ -752,7 +780,6 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     auto launch = [&](auto kernel, auto q, auto k) {
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         return cudaLaunchKernelEx(&cfg, kernel, q, k, g, keep, bpc, idx, cnt, scores);
     };
     const cudaError_t e =
