@@ -215,11 +215,12 @@ _plans: dict = {}
 
 
 def _plan(lib, desc: SsbaDesc) -> _Plan:
-    """The plan of a descriptor, kept by the bytes of its C struct (a model's layers share a few
-    descriptors; at the cap the table starts over). The struct is made anew each time, so whatever
-    it refuses is refused on every call."""
+    """The plan of a descriptor, kept by the bytes of its C struct and the sizes as given (a model's layers
+    share a few descriptors; at the cap the table starts over). The struct is made anew each time, so
+    whatever it refuses is refused on every call; it keeps 32 bits of a size, so that it alone would
+    give a descriptor with a larger one the plan, and the shapes, of another."""
     c = desc.c()
-    key = bytes(c)
+    key = (bytes(c), desc.B, desc.heads, desc.H_tok, desc.W_tok, desc.head_dim, desc.block)
     pl = _plans.get(key)
     if pl is None:
         pl = _Plan(lib, desc, c)

@@ -272,3 +272,14 @@ def test_python_binding_validates_before_calling(lib):
     with pytest.raises(api.SsbaError, match="workspace"):
         api.forward_fused(dsc, q, q, q, workspace=None)
     assert api.realized_sparsity(api.SsbaDesc(1, 24, 64, 64, rho=0.8416)) == 53 / 64
+
+
+def test_a_size_past_32_bits_does_not_take_or_leave_the_plan_of_another(lib):
+    """The C struct keeps 32 bits of a size: 2^32 + 1 images look like one to it, not to the shape checks."""
+    good = api.SsbaDesc(B=1, heads=2, H_tok=16, W_tok=24, rho=0.75)
+    for order in ((2 ** 32 + 1, 1), (1, 2 ** 32 + 1)):
+        api._plans.clear()
+        for B in order:
+            desc = api.SsbaDesc(B=B, heads=2, H_tok=16, W_tok=24, rho=0.75)
+            assert api._plan(lib, desc).x == (B, 2, 384, 64)
+    assert api.keep_count(good) == 2
