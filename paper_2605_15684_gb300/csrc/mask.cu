@@ -370,7 +370,6 @@ constexpr int kFuseCluster = 8;    // CTAs per (batch, head)
 // two images, 81 blocks a head 118.9 -> 114.3 us, 120 blocks 210 -> 202; four images of 64 blocks 182.4
 // either way).
 constexpr int kFuseMaxTb = 128;
-constexpr size_t kFuseSmem = 80 * 1024;  // above every row length's need
 
 // Affinity row of one query block with the keys held in registers (lane l: labels l + 32 m), then
 // the gating. kbs: the head's k_b by rows, the 16-byte chunk c4 of row j at chunk c4 ^ (j & 15) (the 32
@@ -409,8 +408,8 @@ __device__ __forceinline__ void affinity_select(const float* q, const float* kbs
 //      it, and none follow it, so a CTA may leave once it is done).
 //   3. one warp per owned query block: S row by four interleaved partial sums over d, its
 //      keys in registers, then the radix walk (affinity_select).
-template <typename T, int kFuseWarps>
-__global__ void __launch_bounds__(kFuseWarps * 32) ssba_mask_fused_kernel(const T* __restrict__ Q,
+template <typename T, int kFuseWarps, int kMinCtas>
+__global__ void __launch_bounds__(kFuseWarps * 32, kMinCtas) ssba_mask_fused_kernel(const T* __restrict__ Q,
                                                                           const T* __restrict__ K, Grid g,
                                                                           int keep, int bpc,
                                                                           int32_t* __restrict__ idx,
@@ -747,19 +746,15 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     const bool spread = d.B * d.heads * kFuseCluster <= 2 * device_sm_count();
     if (d.head_dim != 64 || g.blk != 8 || Tb > (spread ? kFuseMaxTb : 64)) return SSBA_ERR_UNSUPPORTED;
     const int bpc = (Tb + kFuseCluster - 1) / kFuseCluster;
-    size_t smem = ((size_t)bpc * 64 + (size_t)Tb * 64) * sizeof(float);
-    // The kernel's registers let three CTAs share an SM. A grid of up to two an SM asks for shared memory
-    // that only two fit in, so that its clusters spread: 1024 px mask and forward 49.6 -> 46.8 us, 768 x
-    // 1408 px 56.3 -> 53.1 (batch 4, with more CTAs than that, is faster with three: 29.9 -> 28.7).
-    if (spread && smem < kFuseSmem) smem = kFuseSmem;
-    static PerDeviceOnce attr_once;
-    attr_once.run([] {
-        auto set = [](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFuseSmem); };
-        set(ssba_mask_fused_kernel<__nv_bfloat16, 8>);
-        set(ssba_mask_fused_kernel<__nv_bfloat16, 12>);
-        set(ssba_mask_fused_kernel<float, 8>);
-        set(ssba_mask_fused_kernel<float, 12>);
-    });
+    const size_t smem = ((size_t)bpc * 64 + (size_t)Tb * 64) * sizeof(float);
+    static_assert((kFuseMaxTb / kFuseCluster + kFuseMaxTb) * 64 * sizeof(float) <= 48 * 1024, "no opt-in needed");
+    // CTAs an SM. A grid of up to two an SM takes the instantiation whose 128 registers (kMinCtas 2) let two and
+    // no more share one, so that its clusters spread; left to itself the compiler takes 80, three fit,
+    // and clusters crowd some SMs while others idle. Two against three, 24 heads, GPU time: 1024 px mask and
+    // forward 44.2 against 47.1 us, the mask alone 8.4 either way (28 heads 8.5 against 10.5); 99 blocks 80
+    // against 87 together. (Asking for 80 KB of shared memory spreads them too, but with 80 registers fewer
+    // loads are in flight: alone 8.8 us, fp32 9.5 against 8.7, 36 heads 11.5 against 8.9.) Grids above two
+    // an SM have more than one round of two and are faster with three (four 1024 px images 29.9 -> 28.7).
     // Warps of a CTA: one per block, where a CTA's nine to twelve blocks would be two rounds of eight warps
     // (768 x 1408 px, 66 blocks, mask and forward 54.5 -> 52.0 us, 1152 px 67.6 -> 65.9; 16 warps 54.5 and
     // 68.1). At up to eight blocks the four more are idle and only cost room (512 px 14.8 either way, four
@@ -784,9 +779,13 @@ int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q
     };
     const cudaError_t e =
         d.dtype == SSBA_BF16
-            ? launch(wide ? ssba_mask_fused_kernel<__nv_bfloat16, 12> : ssba_mask_fused_kernel<__nv_bfloat16, 8>,
+            ? launch(wide     ? ssba_mask_fused_kernel<__nv_bfloat16, 12, 0>
+                     : spread ? ssba_mask_fused_kernel<__nv_bfloat16, 8, 2>
+                              : ssba_mask_fused_kernel<__nv_bfloat16, 8, 0>,
                      static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K))
-            : launch(wide ? ssba_mask_fused_kernel<float, 12> : ssba_mask_fused_kernel<float, 8>,
+            : launch(wide     ? ssba_mask_fused_kernel<float, 12, 0>
+                     : spread ? ssba_mask_fused_kernel<float, 8, 2>
+                              : ssba_mask_fused_kernel<float, 8, 0>,
                      static_cast<const float*>(Q), static_cast<const float*>(K));
     if (e != cudaSuccess) {
         set_error("ssba_mask_fused_kernel launch: %s", cudaGetErrorString(e));
