@@ -178,18 +178,23 @@ __device__ __forceinline__ void select_rows(const uint32_t* S, int Tb, int keep,
 // Affinity and gating for head_dim 64: a CTA takes kSelWarps * kRows rows of one head, warp w the rows
 // [w kRows, (w + 1) kRows) of them; the keys' means pass through shared memory 128 at a time (rows of
 // 68 floats: 8 consecutive rows cover the banks), a lane scores 4 keys (2 or 1 of the last few) against
-// its warp's kRows rows at a time, and the walks (ballot_select) read the finished rows of keys back from
-// shared memory.
+// its warp's kRows rows at a time, and the walks (ballot_select, kPer keys a lane; 8: 2 up to 64 blocks) read the
+// finished rows of keys back from shared memory. One instantiation for each register layout of the walk, so that
+// the long rows' registers (64 keys a lane) do not cost the short ones theirs, and CTAs.
 // What bounds it: the latency of the gating's counts (36 of 53 us at 510 blocks) and the shared-memory
 // reads of the scores, 4 + kRows 16-byte chunks for 16 kRows multiply-adds of a lane. (One key at a time:
-// 510 blocks 62 us, 324 39.7, 256 24.0, 64 at batch 4 9.3; now 53, 35, 21 and 8.7.) kRows, 24 heads, us for
-// 2 and 4: 510 blocks 56, 53; 324 blocks 36.4, 35.5; 256 blocks 20.7, 23.0; for 1 and 2, one key at a
-// time: 64 blocks at batch 4 12.8, 9.9, at batch 1 7.4, 6.2; 16 blocks 3.8, 4.5 (fewer CTAs than SMs). The
-// kernel before (one row a warp, keys transposed one word at a time, a 32-bit radix walk over shared
-// memory): 510 blocks 195, 256 91, 64 at batch 4 15.
+// 510 blocks 62 us, 324 39.7, 256 24.0, 64 at batch 4 9.3; now 53, 35, 20 and 9.) The kernel before (one
+// row a warp, keys transposed one word at a time, a 32-bit radix walk over shared memory): 510 blocks
+// 195, 256 99, 64 at batch 4 15.
 constexpr int kSel64Keys = 128, kSel64Ld = 68;
-template <int kRows>
-__global__ void __launch_bounds__(kSelWarps * 32, kRows == 2 ? 3 : 2) ssba_select64_kernel(const float* __restrict__ qb,
+// CTAs an SM that the registers leave room for: as many as run without spills.
+constexpr int sel64_ctas(int rows, int per) { return per == 64 ? 1 : (rows == 4 || per == 32 ? 2 : (rows == 2 ? 3 : 4)); }
+constexpr size_t sel64_smem(int rows, int Tb)
+{
+    return ((size_t)kSel64Keys * kSel64Ld + (size_t)kSelWarps * rows * (64 + Tb)) * sizeof(float);
+}
+template <int kRows, int kPer>
+__global__ void __launch_bounds__(kSelWarps * 32, sel64_ctas(kRows, kPer)) ssba_select64_kernel(const float* __restrict__ qb,
                                                                        const float* __restrict__ kb, int Tb, int keep,
                                                                        int32_t* __restrict__ idx,
                                                                        int32_t* __restrict__ cnt,
@@ -198,8 +203,8 @@ __global__ void __launch_bounds__(kSelWarps * 32, kRows == 2 ? 3 : 2) ssba_selec
     constexpr int kD = 64, kCta = kSelWarps * kRows, kPerLane = kSel64Keys / 32;
     extern __shared__ float4 raw[];
     float* ks = reinterpret_cast<float*>(raw);
-    float* qs = ks + kSel64Keys * kSel64Ld;                      // [kCta][64]
-    uint32_t* S = reinterpret_cast<uint32_t*>(qs + kCta * kD);   // [kCta][Tb]
+    float* qs = ks + kSel64Keys * kSel64Ld;                     // [kCta][64]
+    uint32_t* S = reinterpret_cast<uint32_t*>(qs + kCta * kD);  // [kCta][Tb]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bh = blockIdx.y;
     const int row0 = blockIdx.x * kCta + warp * kRows, rows = min(max(Tb - row0, 0), kRows);
     const float4* kbh = reinterpret_cast<const float4*>(kb + (size_t)bh * Tb * kD);
@@ -250,15 +255,8 @@ __global__ void __launch_bounds__(kSelWarps * 32, kRows == 2 ? 3 : 2) ssba_selec
     }
     __syncwarp();
     int32_t* dst = idx + ((size_t)bh * Tb + row0) * keep;
-    // only the lengths that launch_select gives to this kRows
-    if constexpr (kRows == 4) {
-        if (Tb <= 512) select_rows<16>(Sw, Tb, keep, lane, dst, rows);
-        else select_rows<32>(Sw, Tb, keep, lane, dst, rows);
-    } else {
-        if (Tb <= 64) select_rows<2>(Sw, Tb, keep, lane, dst, rows);
-        else if (kRows == 2 || Tb <= 256) select_rows<8>(Sw, Tb, keep, lane, dst, rows);
-        else select_rows<64>(Sw, Tb, keep, lane, dst, rows);
-    }
+    if (kPer == 8 && Tb <= 64) select_rows<2>(Sw, Tb, keep, lane, dst, rows);
+    else select_rows<kPer>(Sw, Tb, keep, lane, dst, rows);
     if (lane < rows) cnt[(size_t)bh * Tb + row0 + lane] = keep;
 }
 
@@ -325,7 +323,8 @@ __global__ void __launch_bounds__(kSelWarps * 32) ssba_select_kernel(const float
     if (!active) return;
     int32_t* dst = idx + rowoff * keep;
 
-    if (Tb <= 64) select_rows<2>(S, Tb, keep, lane, dst, 1);
+    if (Tb <= 32) select_rows<1>(S, Tb, keep, lane, dst, 1);
+    else if (Tb <= 64) select_rows<2>(S, Tb, keep, lane, dst, 1);
     else if (Tb <= 256) select_rows<8>(S, Tb, keep, lane, dst, 1);
     else {
         // keep-th largest key by MSB-first radix select
@@ -671,27 +670,44 @@ int launch_select(const ssba_desc& d, const Grid& g, int keep, const float* qb, 
     }
     if (d.head_dim == 64) {
         const int BH = d.B * d.heads;
-        // rows a warp (see the kernel): few where every row counts for the spread over the SMs; one where
-        // four would not fit their keys
-        const int rows = Tb > 1024 ? 1 : (Tb > 256 ? 4 : ((long long)BH * Tb >= 10ll * device_sm_count() ? 2 : 1));
-        const int cta = kSelWarps * rows;
-        const size_t sm = ((size_t)kSel64Keys * kSel64Ld + (size_t)cta * 64 + (size_t)cta * Tb) * sizeof(float);
-        auto kernel = rows == 4 ? ssba_select64_kernel<4> : (rows == 2 ? ssba_select64_kernel<2> : ssba_select64_kernel<1>);
-        // the largest size of each instantiation, once: a limit set for each call could be lowered by another
-        // thread before this one's launch
+        // Rows a warp. Short rows: two where a CTA's eight warps of one each would be many CTAs an SM (24 heads,
+        // us, one row and two: 64 blocks 4.9, 5.1; at batch 4 9.9, 9.1; 256 blocks 25, 20), one below and up to 32
+        // blocks, where a row is little work (16 blocks at batch 8 5.4, 5.6). Rows of 257 to 1024: the fewest
+        // that leave a CTA an SM, since a warp's rows follow each other (one head of 510 blocks 15, 19
+        // and 25 us for one, two and four; 24 heads 78, 61, 54). Longer ones: two, what their keys leave room for
+        // (1280 blocks, 24 heads 726, 483; one head 55, 50).
+        const int sms = device_sm_count();
+        auto ctas = [&](int r) { return (long long)BH * ((Tb + kSelWarps * r - 1) / (kSelWarps * r)); };
+        const int rows = Tb <= 32     ? 1
+                         : Tb <= 256  ? ((long long)BH * Tb >= 10ll * sms ? 2 : 1)
+                         : Tb <= 1024 ? (ctas(1) <= sms ? 1 : (ctas(2) <= sms ? 2 : 4))
+                                      : 2;
+        const int per = Tb <= 32 ? 1 : (Tb <= 256 ? 8 : (Tb <= 512 ? 16 : (Tb <= 1024 ? 32 : 64)));
+        struct Variant {
+            int rows, per, longest;  // longest row it is given
+            decltype(&ssba_select64_kernel<1, 1>) kernel;
+        };
+        static const Variant variants[] = {
+            {1, 1, 32, ssba_select64_kernel<1, 1>},     {1, 8, 256, ssba_select64_kernel<1, 8>},
+            {2, 8, 256, ssba_select64_kernel<2, 8>},    {1, 16, 512, ssba_select64_kernel<1, 16>},
+            {2, 16, 512, ssba_select64_kernel<2, 16>},  {4, 16, 512, ssba_select64_kernel<4, 16>},
+            {1, 32, 1024, ssba_select64_kernel<1, 32>}, {2, 32, 1024, ssba_select64_kernel<2, 32>},
+            {4, 32, 1024, ssba_select64_kernel<4, 32>}, {2, 64, kMaxTb, ssba_select64_kernel<2, 64>},
+        };
+        // the largest size of each, once: a limit set for each call could be lowered by another thread before
+        // this one's launch
         static PerDeviceOnce attr64;
         attr64.run([] {
-            auto largest = [](auto k, int rows, int longest) {
-                const size_t n = ((size_t)kSel64Keys * kSel64Ld + (size_t)kSelWarps * rows * (64 + longest)) * sizeof(float);
-                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
-            };
-            largest(ssba_select64_kernel<1>, 1, kMaxTb);
-            largest(ssba_select64_kernel<2>, 2, 256);
-            largest(ssba_select64_kernel<4>, 4, 1024);
+            for (const Variant& v : variants)
+                cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sel64_smem(v.rows, v.longest));
         });
+        const Variant* v = variants;
+        while (v->rows != rows || v->per != per) ++v;
+        const int cta = kSelWarps * rows;
         cudaLaunchConfig_t cfg = {};
         cfg.blockDim = dim3(kSelWarps * 32, 1, 1);
-        cfg.dynamicSmemBytes = sm;
+        cfg.dynamicSmemBytes = sel64_smem(rows, Tb);
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -701,7 +717,7 @@ int launch_select(const ssba_desc& d, const Grid& g, int keep, const float* qb, 
         for (int h0 = 0; h0 < BH; h0 += kMaxGridY) {
             const size_t row = (size_t)h0 * Tb;
             cfg.gridDim = dim3((Tb + cta - 1) / cta, min(kMaxGridY, BH - h0), 1);
-            cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, qb + row * 64, kb + row * 64, Tb, keep, idx + row * keep,
+            cudaError_t e = cudaLaunchKernelEx(&cfg, v->kernel, qb + row * 64, kb + row * 64, Tb, keep, idx + row * keep,
                                                cnt + row, scores ? scores + row * Tb : nullptr);
             if (e == cudaSuccess) e = cudaGetLastError();
             if (e != cudaSuccess) {

@@ -122,6 +122,22 @@ __device__ __forceinline__ void ballot_select(const uint32_t (&key)[kPer], int T
     }
 }
 
+// Rows of up to 32 labels, one key a lane: its rank is counted over the others, read from their lanes. The
+// reads do not wait for each other, where the counts of a walk do.
+template <>
+__device__ __forceinline__ void ballot_select<1>(const uint32_t (&key)[1], int Tb, int keep, int lane, int32_t* dst)
+{
+    int rank = 0;
+#pragma unroll 8
+    for (int k = 0; k < Tb; ++k) {
+        const uint32_t other = __shfl_sync(0xffffffffu, key[0], k);
+        rank += other > key[0] || (other == key[0] && k < lane);
+    }
+    const bool kept = lane < Tb && rank < keep;
+    const uint32_t km = __ballot_sync(0xffffffffu, kept);
+    if (kept) dst[__popc(km & ((1u << lane) - 1u))] = lane;
+}
+
 // Affinities S = q_b . k_b: four interleaved partial sums over d (components of 16-byte chunks, in
 // chunk order), added as (a0 + a1) + (a2 + a3), for kRows rows of q and kKeys of k_b at once (each
 // chunk is read once for all of them). q: row r at q + r * qld; chunk(k, c): key k's c-th chunk. Every
