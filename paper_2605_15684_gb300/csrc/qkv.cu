@@ -9,6 +9,7 @@
 //
 // Two kernels of the same main loop: a tile is 128 rows x 256 output columns (four heads of 64) x the
 // whole Dm, in 64-wide k steps through a 4-stage ring of 48 KB (A 16 KB + B 32 KB, 128-byte swizzle).
+// (launch_qkv_rope_pool has the rule between them.)
 //   kWin  the rows are two horizontally adjacent 8x8 windows of the shifted grid, one 16 x 8 token box per
 //         k step (measured, two 8 x 8 boxes took the main loop from 35 to 47 us at 1024 px), and the
 //         epilogue sums the windows of Q and K. A pair that crosses the grid edge (shifted layers) is
@@ -650,14 +651,22 @@ int launch_qkv_rope_pool(const ssba_desc& d, const Grid& g, const void* X, const
     p.heads = d.heads;
     p.Dm = Dm;
     p.pairs = (g.bw + 1) / 2;
-    // Window tiles (means in the epilogue) against row tiles and a pooling launch, 24 heads, us:
-    //   256 px 15.4 unshifted, 23.2 shifted / 14.6;  512 px 17.3, 24.4 / 18.9;  1024 px 43.1, 54.8 / 44.3;
-    //   two 1024 px images 78.4, 88.9 / 83.9;  1536 px 87.6, 92.8 / 95;  four 1024 px images 149, 164 /
-    //   170;  2048 px 151, 156 / 172.
-    // So rows where the layer is shifted and Q and K (here 50 MB at two 1024 px images) stay in L2 until
-    // they are pooled; and where no means are asked for (1024 px 38 us against 43 to 52).
-    const bool shifted = g.sr != 0 || g.sc != 0;
-    const bool win = qb && !(shifted && 4ll * d.B * g.H * g.W * Dm <= (48ll << 20));
+    // Window tiles (means in the epilogue) against row tiles and a pooling launch over Q and K, us. The
+    // window sums cost the epilogue about the same a tile whatever the heads, so where the main loop is
+    // short it cannot hide them, and more where windows are cut; the pooling launch costs by its bytes.
+    //   12 heads    2048 px 74, 55;  four such images 257, 208.  16 heads 1920 px 83, 73;  2048 px 88, 86
+    //   24 heads    unshifted 512 px 17.3, 19.2;  1024 px 42.9, 44.6;  2048 px 150, 168
+    //               shifted 256 px 23.2, 14.6;  512 px 24.4, 18.9;  1024 px 53.2, 45.1;  1152 x 2048 px (54 MB
+    //               of Q and K) 96.0, 95.1;  1664 px (63 MB) 114.5, 113.2;  1792 px (74 MB) 123, 128;
+    //               2048 px 155, 166
+    //   32 heads    shifted, 64 MB 142.2, 141.9;  72 MB 154, 159
+    //   grids past the RoPE table (kRopeCap)  24 heads, a 4K frame 542, 362;  256 x 2176 px 79, 39
+    // So rows past the table (there the epilogue computes its own sines as well), at up to 12 heads, and up
+    // to 64 MB of Q and K where windows are cut or the heads are 16 or fewer; and where no means
+    // are asked for (1024 px 38 us).
+    const bool shifted = g.sr != 0 || g.sc != 0, table = g.H <= kRopeCap && g.W <= kRopeCap;
+    const bool small = 4ll * d.B * g.H * g.W * Dm <= (64ll << 20);
+    const bool win = qb && table && Dm > 768 && !(small && (shifted || Dm <= 1024));
     p.m_tiles = win ? (g.H / 8) * p.pairs : (g.H * g.W + kBM - 1) / kBM;
     p.n_tiles = (3 * Dm + kBN - 1) / kBN;
     p.tiles = d.B * p.m_tiles * p.n_tiles;
@@ -672,7 +681,7 @@ int launch_qkv_rope_pool(const ssba_desc& d, const Grid& g, const void* X, const
     static PerDeviceOnce attr;  // shared-memory attributes, set once per device
     attr.run([smem] {
         for (auto k : {ssba_qkv_rope_pool_kernel<true, true>, ssba_qkv_rope_pool_kernel<true, false>,
-                       ssba_qkv_rope_pool_kernel<false, true>, ssba_qkv_rope_pool_kernel<false, false>})
+                       ssba_qkv_rope_pool_kernel<false, false>})
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     const int grid = p.tiles < sm_count() ? p.tiles : sm_count();
@@ -685,10 +694,13 @@ int launch_qkv_rope_pool(const ssba_desc& d, const Grid& g, const void* X, const
     la[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     la[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = la;
-    cfg.numAttrs = 1;
-    const bool table = g.H <= kRopeCap && g.W <= kRopeCap;
-    auto kernel = table ? (win ? ssba_qkv_rope_pool_kernel<true, true> : ssba_qkv_rope_pool_kernel<true, false>)
-                        : (win ? ssba_qkv_rope_pool_kernel<false, true> : ssba_qkv_rope_pool_kernel<false, false>);
+    // The early launch saves the gap before the kernel (24 heads 256 px 16.7 -> 15.6 us, 1024 px 44.2 -> 42.9; row
+    // tiles of 12 heads 2048 px 55.4 -> 53.3), but it can cost more than that: window tiles of more than about five
+    // rounds an SM (16 heads 2048 px 88.4 -> 90.5, two such images 161 -> 171), row tiles of more than 16
+    // heads (32 heads 2048 px 268 -> 280), grids past the RoPE table (172 -> 187). Why was not found.
+    cfg.numAttrs = table && (p.tiles <= 4 * sm_count() || (!win && Dm <= 1024)) ? 1 : 0;
+    auto kernel = win ? ssba_qkv_rope_pool_kernel<true, true>
+                      : (table ? ssba_qkv_rope_pool_kernel<true, false> : ssba_qkv_rope_pool_kernel<false, false>);
     cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, maps, p);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {

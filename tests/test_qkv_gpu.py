@@ -69,6 +69,9 @@ def _check_pooled(qb, Q, H, W, shift):
     (2, 3, 24, 16, (4, -4)),    # 3 Dm = 576: a partial N tile, heads straddle tiles
     (1, 2, 8, 24, (0, 4)),      # Tb = 3: the last M tile holds one window
     (1, 5, 40, 24, (-4, 0)),    # 15 windows, five heads
+    (1, 17, 16, 16, (0, 0)),    # window tiles (above 16 heads): 3 Dm = 3264, a partial N tile, heads straddle tiles
+    (2, 18, 8, 24, (0, 0)),     # window tiles, the last M tile of one window
+    (1, 3, 8, 136, (0, 4)),     # past the RoPE table's positions
 ])
 def test_qkv_rope_pool_matches_oracle(B, heads, H, W, shift):
     desc, (X, Wq, b), (Q, K, V, qb, kb) = _run(B, heads, H, W, shift, seed=B * 100 + heads)
@@ -154,6 +157,9 @@ def test_fused_path_feeds_the_forward():
     (1, 24, 72, 88, (4, 4)),    # 6336 tokens, 39 MB of Q and K: row tiles (the last one of 64 rows) and a pooling launch
     (2, 24, 72, 88, (4, 4)),    # above the limit: window tiles
     (2, 24, 72, 88, (0, 0)),
+    (1, 12, 72, 88, (0, 0)),    # 12 heads: row tiles, unshifted too
+    (1, 20, 72, 88, (0, 0)),    # window tiles below the limit
+    (1, 20, 8, 136, (0, 0)),    # row tiles past the RoPE table's positions
     (3, 2, 8, 24, (0, 4)),      # 192 tokens an image: a tile of 64 rows before the next image's
 ])
 def test_row_tiles_and_window_tiles_give_the_same(B, heads, H, W, shift):
