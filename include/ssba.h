@@ -391,14 +391,13 @@ SSBA_API const char* ssba_last_error(void);
  *         stored, grid barrier passed, head means staged, lists selected, pipelines start,
  *         pipeline 0 done, pipeline 1 done, exit, and for warp 0's first item the start of
  *         its selection, its score row done, its list done (0 where a phase did not run);
- *   tile  host array of 8 x 128 x 12 uint32: for pipelines 0 and 1 of CTAs 0, 1, grid/2 and
- *         grid-1, per tile (the pipeline's running key-block count), SM clock stamps of: K copy
+ *   tile  host array of 8 x 128 x 10 uint32: for pipelines 0 and 1 of CTAs 0, 1, grid/2 and
+ *         grid-1, per step (the pipeline's running count of key blocks), SM clock stamps of: K copy
  *         issued, QK issued, softmax saw S, softmax exps done, P stored, PV issued, V copy
- *         issued, QK's wait for a free S buffer over, S in the softmax's registers, row maxima
- *         known, P buffer free, PV's waits over;
- *   item  host array of 8 x 32 x 4 uint32: per item of those pipelines, SM clock stamps of: the
- *         epilogue starts waiting for O, O ready, the epilogue done, and (item 0 only) the
- *         pipeline's start.
+ *         issued, QK's waits over, S in the softmax's registers, PV's waits over;
+ *   item  host array of 8 x 32 x 4 uint32: per round (two items) of those pipelines, SM clock
+ *         stamps of: the finished rows of the first item start waiting for O, O ready, the rows
+ *         written, and (round 0 only) the pipeline's start.
  * Synchronous (call after the caller's stream sync). The default build records nothing and
  * returns SSBA_ERR_UNSUPPORTED; SSBA_ERR_CUDA if a copy fails. */
 SSBA_API int ssba_timeline_read(uint64_t* cta, uint32_t* tile, uint32_t* item);

@@ -122,17 +122,17 @@ constexpr int kWinCap = 256;  // labels whose window (origin, box shape) is tabu
 
 // Timeline instrumentation, compiled only into the timeline build of the library (-DSSBA_TIMELINE;
 // the default build has none of it). Per CTA, globaltimer stamps (ns) of the launch's phases; per
-// tile of eight sampled pipelines (pipeline 0 and 1 of CTAs 0, 1, gridDim/2 and gridDim-1), SM
-// clock stamps of each role's step, and per item the epilogue's. ssba_timeline_read copies them out.
+// step of eight sampled pipelines (pipeline 0 and 1 of CTAs 0, 1, gridDim/2 and gridDim-1), SM
+// clock stamps of each role, and per round those of the finished rows. ssba_timeline_read copies them out.
 namespace tl {
-constexpr int kCtas = 256, kCtaEv = 16, kPipes = 4 * kSlots, kTiles = 128, kTileEv = 12, kItems = 32, kItemEv = 4;
+constexpr int kCtas = 256, kCtaEv = 16, kPipes = 4 * kSlots, kTiles = 128, kTileEv = 10, kItems = 32, kItemEv = 4;
 enum CtaEv { kEntry = 0, kDepWait, kPoolLanded, kPooled, kBarrier, kStaged, kSelected, kPipesStart, kSlot0End,
              kSlot1End, kEnd, kSelStart, kScoresDone, kWalkDone };
-// tile events: K copy issued, QK issued, softmax saw S, softmax done with the exps, P stored,
-// PV issued, V copy issued, QK's wait for a free S buffer over, S in the softmax's registers,
-// row maxima known, P buffer free (softmax), PV's waits over
-enum TileEv { kKIssue = 0, kQKIssue, kSmxStart, kSmxExp, kPStored, kPVIssue, kVIssue, kSFree, kSLoaded, kMaxDone,
-              kPFree, kPVReady };
+// step events: K copy issued, QK issued, softmax saw S, softmax done with the exps, P stored, PV
+// issued, V copy issued, QK's waits over, S in the softmax's registers, PV's waits over (the
+// softmax's of half A's first warp)
+enum TileEv { kKIssue = 0, kQKIssue, kSmxStart, kSmxExp, kPStored, kPVIssue, kVIssue, kSFree, kSLoaded, kPVReady };
+// round events: half A's rows are due (their wait for the last PV starts), O ready, rows written
 enum ItemEv { kEpiStart = 0, kEpiO, kEpiDone, kPipeClock0 };
 #ifdef SSBA_TIMELINE
 __device__ unsigned long long cta_ev[kCtas][kCtaEv];
@@ -412,14 +412,13 @@ __device__ __forceinline__ int ld_list(const int32_t* a) { return kSel ? __ldcg(
 
 // Score row and Top-k gating of one item (one warp), with the arithmetic and the selection code
 // of the mask kernels (S_j = q_b . k_b[j], four interleaved partial sums over d combined in a
-// fixed order; walked by sel::ballot_select on keys held
-// in registers), so the same means give the same lists. kbs: the head's k_b
+// fixed order; sel::ballot_select on keys held in registers), so the same means give the same lists.
+// kbs: the head's k_b
 // staged in shared memory, the 16-byte chunk c4 of row j at chunk c4 ^ (j & 15) (two lanes per
 // bank at most when 32 lanes read one column); qs: the item's q_b row in shared memory. Not
 // inlined, so that its registers do not weigh on the pipeline roles.
 template <int kPer>
-__device__ __noinline__ void select_item(const TcParams& p, int item, int lane, const float* kbs, const float* qs,
-                                         uint32_t* S)
+__device__ __noinline__ void select_item(const TcParams& p, int item, int lane, const float* kbs, const float* qs)
 {
     const int Tb = p.g.Tb();
     const bool stamp = threadIdx.x == 0 && item == sel_first_item(p, blockIdx.x, gridDim.x * kSlots);
@@ -438,7 +437,6 @@ __device__ __noinline__ void select_item(const TcParams& p, int item, int lane, 
             key[m] = sel::order_key(acc);
         }
     }
-    (void)S;
     if (stamp) TL_CTA(tl::kScoresDone);
     sel::ballot_select<kPer>(key, Tb, p.keep, lane, const_cast<int32_t*>(p.idx) + (size_t)item * p.keep);
     if (stamp) TL_CTA(tl::kWalkDone);
@@ -668,18 +666,17 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         const int h1a = f1 / Tb, h1b = n1 ? (f1 + n1 - 1) / Tb : h1a - 1;
         const int nh0 = max(0, h0b - h0a + 1), nh = nh0 + max(0, h1b - h1a + 1);
         auto head_of = [&](int hi) { return hi < nh0 ? h0a + hi : h1a + (hi - nh0); };
-        // staging: pipeline 0's k, v, q buffers end with the scratch (per warp 128 key words and
-        // a 64-float query row, then up to kSelQRows shared query rows); the rest of them and
-        // pipeline 1's hold the heads
+        // staging: pipeline 0's k, v, q buffers end with the scratch (a 64-float query row per warp, then
+        // up to kSelQRows shared query rows, more than the kSelItems an SM of a call that selects here;
+        // only the failure-detection hook can bring more); the rest of them and pipeline 1's hold the heads
         constexpr uint32_t kRegion = sizeof(SlotSmem);  // k, v, q of one pipeline
-        constexpr int kSelQRows = 48;
-        constexpr int kWarpScratch = 128 + kD;  // words per warp: keys, then its own query row
-        constexpr uint32_t kScratch = (kThreads / 32) * kWarpScratch * 4 + kSelQRows * kD * 4;
+        constexpr int kSelQRows = 24;
+        constexpr uint32_t kScratch = (kThreads / 32 + kSelQRows) * kD * 4;
         const uint32_t hb = (uint32_t)Tb * kD * 4;
         const int cap0 = (int)((kRegion - kScratch) / hb), cap = cap0 + (int)(kRegion / hb);
         uint8_t* r0 = &cs.slot[0].k[0][0];
-        uint32_t* keys = reinterpret_cast<uint32_t*>(r0 + kRegion - kScratch) + gwarp * kWarpScratch;
-        float* qrows = reinterpret_cast<float*>(r0 + kRegion - kScratch + (kThreads / 32) * kWarpScratch * 4);
+        float* own = reinterpret_cast<float*>(r0 + kRegion - kScratch) + gwarp * kD;
+        float* qrows = reinterpret_cast<float*>(r0 + kRegion - kScratch) + (kThreads / 32) * kD;
         auto staged = [&](int hi) {
             return reinterpret_cast<float*>(hi < cap0 ? r0 + hi * hb : &cs.slot[1].k[0][0] + (hi - cap0) * hb);
         };
@@ -713,17 +710,16 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
                 if (hi < 0 || hi >= m) continue;
                 const float* qs = qrows + q * kD;
                 if (q >= kSelQRows) {  // rows past the staged ones: this warp's own copy
-                    float* own = reinterpret_cast<float*>(keys) + 128;  // after its keys
                     if (lane < kD / 4)
                         reinterpret_cast<float4*>(own)[lane] =
                             __ldcg(reinterpret_cast<const float4*>(p.sel_qb + (size_t)item * kD) + lane);
                     __syncwarp();
                     qs = own;
                 }
-                if (Tb <= 32) select_item<1>(p, item, lane, staged(hi), qs, keys);
-                else if (Tb <= 64) select_item<2>(p, item, lane, staged(hi), qs, keys);
-                else if (Tb <= 128) select_item<4>(p, item, lane, staged(hi), qs, keys);
-                else select_item<8>(p, item, lane, staged(hi), qs, keys);
+                if (Tb <= 32) select_item<1>(p, item, lane, staged(hi), qs);
+                else if (Tb <= 64) select_item<2>(p, item, lane, staged(hi), qs);
+                else if (Tb <= 128) select_item<4>(p, item, lane, staged(hi), qs);
+                else select_item<8>(p, item, lane, staged(hi), qs);
             }
             __syncthreads();
         }
@@ -962,9 +958,12 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         };
         // writes the rows of round r's item, whose last PV is that of step `last`
         auto finish = [&](uint32_t last, int r) {
+            if (quad == 0 && lane == 0) TL_ITEM(slot, (uint32_t)r, tl::kEpiStart);
             wait_pv(last);
+            if (quad == 0 && lane == 0) TL_ITEM(slot, (uint32_t)r, tl::kEpiO);
             const Round rd = get_round<kSel>(p, ct, r);
             store_row(p, half ? rd.item[1] : rd.item[0], row, ocol, done_m, done_l);
+            if (quad == 0 && lane == 0) TL_ITEM(slot, (uint32_t)r, tl::kEpiDone);
             tc_fence_before();
             owed = false;
         };
@@ -1164,7 +1163,9 @@ namespace {
 // 16 warps, one item each; beyond that its rows queue up while the tensor pipe waits, and separate
 // launches, which give every SM several CTAs' warps, are faster: 2048 px (40 items) 395 -> 360 us a
 // layer, four 1024 px images (40) 187 -> 176; at one 1024 px image (10) the single launch is (48.2
-// against 49.3 us).
+// against 49.3 us). Against ssba_build_mask and ssba_forward the single launch loses at every size
+// (24 heads, GPU time, 256 px 12.3 against 8.8 us, 512 px 16.5 and 13.5, 1024 px 45.4 and 44.4): the mask kernel
+// pools without a grid barrier, but does not write the means that these calls return.
 constexpr int kSelItems = 16;
 int max_grid() { return num_sms(); }
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }

@@ -5,14 +5,15 @@ its pipelines, from the time stamps of the timeline build (build.py variant "tim
     python -m paper_2605_15684_gb300.timeline [--layers 24] [--isolated] [--phases-only] [--px 1024]
 
 Runs the benchmark's 1024 px step (64 x 64 grid, B = 1, 24 heads x 64, rho = 0.8416, layer l
-with seed l and shift (0,0) / (4,4) alternating, one ssba_forward_fused launch per layer; with
---px 512 or 2048 the 32 x 32 or 128 x 128 grid of those workloads) a few times, then reads the stamps of the last launch (layer 23 in the stream, or, with --isolated,
-one more launch of layer 1 alone) and prints:
+with seed l and shift (0,0) / (4,4) alternating, one ssba_forward_fused call per layer: one launch; with
+--px 512 or 2048 the 32 x 32 or 128 x 128 grid of those workloads, the latter in three launches, of which the
+last, on given lists, is stamped) a few times, then reads the stamps of the last launch (layer 23 in the
+stream, or, with --isolated, one more launch of layer 1 alone) and prints:
   * per phase, the min / median / max over the CTAs of globaltimer microseconds since the first
     CTA's entry (pooling copies landed, means stored, grid barrier, staging, selection,
     pipelines start and end);
-  * per sampled pipeline, the tile period (SM cycles between the softmax seeing S of
-    consecutive tiles) and the median latency of each hand-off in the tile loop.
+  * per sampled pipeline, the period of a step (SM cycles between the softmax seeing S of consecutive
+    key blocks), the median latency of each hand-off, and when the finished rows were written.
 A diagnostic: the numbers come from a build whose kernels carry extra stores, so read
 differences, not absolute times, and time the default build with bench.py.
 """
@@ -30,8 +31,8 @@ CTA_EVENTS = ["entry", "dep wait over", "pool rows landed", "means stored", "gri
               "head means staged", "lists selected", "pipelines start", "pipeline 0 done", "pipeline 1 done",
               "exit", "warp 0 selects", "its score row done", "its list done"]
 TILE_EVENTS = ["K issued", "QK issued", "softmax saw S", "exps done", "P stored", "PV issued", "V issued",
-               "S buffer free", "S loaded", "row max known", "P buffer free", "PV waits over"]
-N_CTA, CTA_EV, N_PIPE, N_TILE, TILE_EV, N_ITEM, ITEM_EV = 256, 16, 8, 128, 12, 32, 4
+               "QK waits over", "S loaded", "PV waits over"]
+N_CTA, CTA_EV, N_PIPE, N_TILE, TILE_EV, N_ITEM, ITEM_EV = 256, 16, 8, 128, 10, 32, 4
 
 
 def _read(lib):
@@ -52,12 +53,9 @@ def report(lib, grid: int, tag: str) -> None:
         if v:
             print(f"   {name:22s} {min(v):8.2f} {statistics.median(v):8.2f} {max(v):8.2f}")
     print(f"== {tag}: tile loop of the sampled pipelines (SM cycles, medians over tiles)")
-    hand = [("QK issued -> softmax saw S", 1, 2), ("saw S -> S loaded", 2, 8), ("S loaded -> max known", 8, 9),
-            ("max known -> exps done", 9, 3), ("exps done -> P buffer free", 3, 10), ("P buffer free -> P stored", 10, 4),
-            ("P stored -> next saw S", 4, -1),
-            ("P stored -> PV waits over", 4, 11), ("PV waits over -> PV issued", 11, 5),
-            ("K issued -> QK issued", 0, 1),
-            ("S buffer free -> QK issued", 7, 1)]
+    hand = [("QK issued -> softmax saw S", 1, 2), ("saw S -> S loaded", 2, 8), ("S loaded -> exps done", 8, 3),
+            ("exps done -> P stored", 3, 4), ("P stored -> next saw S", 4, -1), ("P stored -> PV waits over", 4, 9),
+            ("PV waits over -> PV issued", 9, 5), ("K issued -> QK issued", 0, 1), ("QK waits over -> QK issued", 7, 1)]
     for pi in range(N_PIPE):
         def ev(t, e):
             return tile[(pi * N_TILE + t) * TILE_EV + e]
@@ -84,8 +82,8 @@ def report(lib, grid: int, tag: str) -> None:
             if o and dn:
                 epi.append(((o - start) & 0xFFFFFFFF, (dn - o) & 0xFFFFFFFF))
         if epi:
-            print("      items: O ready at " + ", ".join(f"{a}" for a, _ in epi) +
-                  "; epilogue " + ", ".join(f"{b}" for _, b in epi) + " cycles")
+            print("      rounds: O ready at " + ", ".join(f"{a}" for a, _ in epi) +
+                  "; rows written in " + ", ".join(f"{b}" for _, b in epi) + " cycles")
 
 
 def main() -> None:
