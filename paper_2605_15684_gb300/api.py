@@ -246,36 +246,40 @@ def forward_workspace_bytes(desc: SsbaDesc) -> int:
     return int(lib.ssba_forward_workspace_bytes(ctypes.byref(d)))
 
 
-def _empty(shape, dtype, dev, stream=None, scratch=False):
-    """Memory that a call on ``stream`` (None: the current one) writes, from that stream's pool: whatever
+def _side(stream, dev):
+    """``stream`` where it is another than the current one, else None."""
+    if stream is None or stream.cuda_stream == torch._C._cuda_getCurrentRawStream(dev.index):
+        return None
+    return stream
+
+
+def _empty(shape, dtype, dev, side, scratch=False):
+    """Memory that a call on stream ``side`` (None: the current one) writes, from that stream's pool: whatever
     had it before is done when the call's kernels run, and what takes a scratch area once the call has
     dropped it runs after them. An output is recorded on the current stream too, where the caller reads
     and frees it."""
-    if stream is None:
+    if side is None:
         return torch.empty(shape, dtype=dtype, device=dev)
-    cur = torch.cuda.current_stream(dev)
-    if stream == cur:
-        return torch.empty(shape, dtype=dtype, device=dev)
-    with torch.cuda.stream(stream):
+    with torch.cuda.stream(side):
         t = torch.empty(shape, dtype=dtype, device=dev)
     if not scratch:
-        t.record_stream(cur)
+        t.record_stream(torch.cuda.current_stream(dev))
     return t
 
 
-def _out(t, name: str, shape, dtype, dev, stream=None):
+def _out(t, name: str, shape, dtype, dev, side):
     """An output: allocated when the caller gave none, else checked."""
     if t is None:
-        return _empty(shape, dtype, dev, stream)
+        return torch.empty(shape, dtype=dtype, device=dev) if side is None else _empty(shape, dtype, dev, side)
     _check(t, name, shape, dtype)
     return t
 
 
-def _scores_out(scores, pl: _Plan, dev, stream=None):
+def _scores_out(scores, pl: _Plan, dev, side):
     if isinstance(scores, torch.Tensor):
         _check(scores, "scores", pl.scores, torch.float32)
         return scores
-    return _empty(pl.scores, torch.float32, dev, stream) if scores else None
+    return _empty(pl.scores, torch.float32, dev, side) if scores else None
 
 
 _fwd_ws: dict = {}
@@ -327,11 +331,12 @@ def build_mask(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, kv_idx=None, kv
     _check(Q, "Q", pl.x, pl.dtype)
     _check(K, "K", pl.x, pl.dtype)
     dev = Q.device
-    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, stream)
-    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, stream)
-    S = _scores_out(scores, pl, dev, stream)
+    side = _side(stream, dev)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, side)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, side)
+    S = _scores_out(scores, pl, dev, side)
     if workspace is None:
-        workspace = _empty(int(lib.ssba_mask_workspace_bytes(pl.ref)), torch.uint8, dev, stream, scratch=True)
+        workspace = _empty(int(lib.ssba_mask_workspace_bytes(pl.ref)), torch.uint8, dev, side, scratch=True)
     rc = lib.ssba_build_mask(pl.ref, Q.data_ptr(), K.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
                              S.data_ptr() if S is not None else None, workspace.data_ptr(),
                              workspace.numel() * workspace.element_size(), _stream_ptr(stream))
@@ -351,9 +356,10 @@ def qkv_rope_pool(desc: SsbaDesc, X: torch.Tensor, Wqkv: torch.Tensor, bias=None
     if bias is not None:
         _check(bias, "bias", (3 * Dm,), torch.float32)
     dev = X.device
+    side = _side(stream, dev)
     if out is None:
-        out = [_empty(pl.x, torch.bfloat16, dev, stream) for _ in range(3)]
-        out += [_empty(pl.means, torch.float32, dev, stream) for _ in range(2)] if pooled else [None, None]
+        out = [_empty(pl.x, torch.bfloat16, dev, side) for _ in range(3)]
+        out += [_empty(pl.means, torch.float32, dev, side) for _ in range(2)] if pooled else [None, None]
     Q, K, V, qb, kb = out
     for t, n in ((Q, "Q"), (K, "K"), (V, "V")):
         _check(t, n, pl.x, torch.bfloat16)
@@ -375,9 +381,10 @@ def select_mask(desc: SsbaDesc, qb: torch.Tensor, kb: torch.Tensor, kv_idx=None,
     _check(qb, "qb", pl.means, torch.float32)
     _check(kb, "kb", pl.means, torch.float32)
     dev = qb.device
-    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, stream)
-    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, stream)
-    S = _scores_out(scores, pl, dev, stream)
+    side = _side(stream, dev)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, side)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, side)
+    S = _scores_out(scores, pl, dev, side)
     _raise_on(lib.ssba_select_mask(pl.ref, qb.data_ptr(), kb.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
                                    S.data_ptr() if S is not None else None, _stream_ptr(stream)))
     return (kv_idx, kv_cnt, S) if S is not None else (kv_idx, kv_cnt)
@@ -389,8 +396,9 @@ def pool_blocks(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, qb=None, kb=No
     pl = _plan(lib, desc)
     _check(Q, "Q", pl.x, pl.dtype)
     _check(K, "K", pl.x, pl.dtype)
-    qb = _out(qb, "qb", pl.means, torch.float32, Q.device, stream)
-    kb = _out(kb, "kb", pl.means, torch.float32, Q.device, stream)
+    side = _side(stream, Q.device)
+    qb = _out(qb, "qb", pl.means, torch.float32, Q.device, side)
+    kb = _out(kb, "kb", pl.means, torch.float32, Q.device, side)
     _raise_on(lib.ssba_pool_blocks(pl.ref, Q.data_ptr(), K.data_ptr(), qb.data_ptr(), kb.data_ptr(),
                                    _stream_ptr(stream)))
     return qb, kb
@@ -403,13 +411,14 @@ def _forward_select_call(fn_name, desc, Q, K, V, qb, kb, kv_idx, kv_cnt, scores,
     _check(K, "K", pl.x, pl.dtype)
     _check(V, "V", pl.x, pl.dtype)
     dev = Q.device
-    qb = _out(qb, "qb", pl.means, torch.float32, dev, stream)
-    kb = _out(kb, "kb", pl.means, torch.float32, dev, stream)
-    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, stream)
-    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, stream)
-    S = _scores_out(scores, pl, dev, stream)
-    O = _out(O, "O", pl.x, pl.dtype, dev, stream)
-    lse = _out(lse, "lse", pl.rows, torch.float32, dev, stream)
+    side = _side(stream, dev)
+    qb = _out(qb, "qb", pl.means, torch.float32, dev, side)
+    kb = _out(kb, "kb", pl.means, torch.float32, dev, side)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, side)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, side)
+    S = _scores_out(scores, pl, dev, side)
+    O = _out(O, "O", pl.x, pl.dtype, dev, side)
+    lse = _out(lse, "lse", pl.rows, torch.float32, dev, side)
     if isinstance(workspace, str):
         workspace = default_forward_workspace(desc, dev, stream)
     wp, wn = _ws_args(workspace)
@@ -449,9 +458,10 @@ def build_mask_noalloc(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, kv_idx=
     _check(Q, "Q", pl.x, pl.dtype)
     _check(K, "K", pl.x, pl.dtype)
     dev = Q.device
-    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, stream)
-    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, stream)
-    S = _scores_out(scores, pl, dev, stream)
+    side = _side(stream, dev)
+    kv_idx = _out(kv_idx, "kv_idx", pl.lists, torch.int32, dev, side)
+    kv_cnt = _out(kv_cnt, "kv_cnt", pl.counts, torch.int32, dev, side)
+    S = _scores_out(scores, pl, dev, side)
     rc = lib.ssba_build_mask_noalloc(pl.ref, Q.data_ptr(), K.data_ptr(), kv_idx.data_ptr(), kv_cnt.data_ptr(),
                                      S.data_ptr() if S is not None else None, _stream_ptr(stream))
     _raise_on(rc)
@@ -460,8 +470,8 @@ def build_mask_noalloc(desc: SsbaDesc, Q: torch.Tensor, K: torch.Tensor, kv_idx=
 
 def forward(desc: SsbaDesc, Q, K, V, kv_idx, kv_cnt, O=None, lse=None, workspace="default", stream=None):
     """ssba_forward: returns (O [B,h,N,d] in desc.dtype, lse [B,h,N] fp32).
-    ``workspace``: "default" (the per-stream one of default_forward_workspace), None or a
-    zero-filled uint8 CUDA tensor; the result is the same with each."""
+    ``workspace``: "default" or None (none: this call uses none), or a zero-filled uint8 CUDA tensor, which
+    is checked and left alone; the result is the same with each."""
     lib = load_library()
     pl = _plan(lib, desc)
     _check(Q, "Q", pl.x, pl.dtype)
@@ -469,8 +479,9 @@ def forward(desc: SsbaDesc, Q, K, V, kv_idx, kv_cnt, O=None, lse=None, workspace
     _check(V, "V", pl.x, pl.dtype)
     _check(kv_idx, "kv_idx", pl.lists, torch.int32)
     _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
-    O = _out(O, "O", pl.x, pl.dtype, Q.device, stream)
-    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, stream)
+    side = _side(stream, Q.device)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device, side)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, side)
     if isinstance(workspace, str):
         # neither kernel uses one here (the fp32 one takes none; bf16 only checks what is given)
         workspace = None
@@ -497,8 +508,9 @@ def forward_joint(desc: SsbaDesc, Q, K, V, K_txt, V_txt, kv_idx, kv_cnt, O=None,
     _check(V_txt, "V_txt", tshp, pl.dtype)
     _check(kv_idx, "kv_idx", pl.lists, torch.int32)
     _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
-    O = _out(O, "O", pl.x, pl.dtype, Q.device, stream)
-    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, stream)
+    side = _side(stream, Q.device)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device, side)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, side)
     if isinstance(workspace, str):
         workspace = None  # not used by this call
     wp, wn = _ws_args(workspace)
@@ -517,8 +529,9 @@ def forward_dense(desc: SsbaDesc, Q, K, V, O=None, lse=None, workspace="default"
     _check(Q, "Q", pl.x, pl.dtype)
     _check(K, "K", pl.x, pl.dtype)
     _check(V, "V", pl.x, pl.dtype)
-    O = _out(O, "O", pl.x, pl.dtype, Q.device, stream)
-    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, stream)
+    side = _side(stream, Q.device)
+    O = _out(O, "O", pl.x, pl.dtype, Q.device, side)
+    lse = _out(lse, "lse", pl.rows, torch.float32, Q.device, side)
     if isinstance(workspace, str):
         workspace = None  # not used by this call
     wp, wn = _ws_args(workspace)
@@ -588,10 +601,11 @@ def backward(desc: SsbaDesc, Q, K, V, O, lse, dO, kv_idx, kv_cnt, dQ=None, dK=No
     _check(lse, "lse", pl.rows, torch.float32)
     _check(kv_idx, "kv_idx", pl.lists, torch.int32)
     _check(kv_cnt, "kv_cnt", pl.counts, torch.int32)
-    outs = [_out(t, n, pl.x, torch.float32, Q.device, stream) for t, n in ((dQ, "dQ"), (dK, "dK"), (dV, "dV"))]
+    side = _side(stream, Q.device)
+    outs = [_out(t, n, pl.x, torch.float32, Q.device, side) for t, n in ((dQ, "dQ"), (dK, "dK"), (dV, "dV"))]
     if workspace is None:
         need = int(lib.ssba_backward_workspace_bytes(pl.ref))
-        workspace = _empty(max(need, 16), torch.uint8, Q.device, stream, scratch=True)
+        workspace = _empty(max(need, 16), torch.uint8, Q.device, side, scratch=True)
     wp, wn = _ws_args(workspace)
     args = (pl.ref, Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(), lse.data_ptr(), dO.data_ptr(),
             kv_idx.data_ptr(), kv_cnt.data_ptr(), outs[0].data_ptr(), outs[1].data_ptr(), outs[2].data_ptr(), wp, wn)
@@ -632,7 +646,7 @@ def haar_dwt(x: torch.Tensor, nb: int = 4, y=None, stream=None) -> torch.Tensor:
     N, C, H, W = x.shape
     _check(x, "x", (N, C, H, W), x.dtype)
     if y is None:
-        y = _empty((N, nb * C, H // 2, W // 2), x.dtype, x.device, stream)
+        y = _empty((N, nb * C, H // 2, W // 2), x.dtype, x.device, _side(stream, x.device))
     _check(y, "y", (N, nb * C, H // 2, W // 2), x.dtype)
     _raise_on(lib.ssba_haar_dwt(x.data_ptr(), y.data_ptr(), N, C, H, W, nb, _dtype_code(x), _stream_ptr(stream)))
     return y
@@ -646,7 +660,7 @@ def haar_iwt(y: torch.Tensor, C: int, nb: int = 4, x=None, stream=None) -> torch
     N, nbC, h, w = y.shape
     _check(y, "y", (N, nb * C, h, w), y.dtype)
     if x is None:
-        x = _empty((N, C, 2 * h, 2 * w), y.dtype, y.device, stream)
+        x = _empty((N, C, 2 * h, 2 * w), y.dtype, y.device, _side(stream, y.device))
     _check(x, "x", (N, C, 2 * h, 2 * w), y.dtype)
     _raise_on(lib.ssba_haar_iwt(y.data_ptr(), x.data_ptr(), N, C, 2 * h, 2 * w, nb, _dtype_code(y), _stream_ptr(stream)))
     return x
@@ -670,7 +684,7 @@ def haar_dwt_pyramid(x: torch.Tensor, levels: int, nb: int = 4, ys=None, stream=
         raise SsbaError(SSBA_ERR_INVALID, f"levels must be 1..{HAAR_MAX_LEVELS}")
     shapes = [(N, nb * C, H >> l, W >> l) for l in range(1, levels + 1)]
     if ys is None:
-        ys = [_empty(shp, x.dtype, x.device, stream) for shp in shapes]
+        ys = [_empty(shp, x.dtype, x.device, _side(stream, x.device)) for shp in shapes]
     if len(ys) != levels:
         raise SsbaError(SSBA_ERR_INVALID, f"ys must hold {levels} tensors")
     for l, (t, shp) in enumerate(zip(ys, shapes)):
@@ -691,7 +705,7 @@ def haar_iwt_pyramid(ys, C: int, nb: int = 4, x=None, stream=None) -> torch.Tens
     for l, t in enumerate(ys):
         _check(t, f"ys[{l}]", (N, nb * C, H >> (l + 1), W >> (l + 1)), ys[0].dtype)
     if x is None:
-        x = _empty((N, C, H, W), ys[0].dtype, ys[0].device, stream)
+        x = _empty((N, C, H, W), ys[0].dtype, ys[0].device, _side(stream, ys[0].device))
     _check(x, "x", (N, C, H, W), ys[0].dtype)
     _raise_on(lib.ssba_haar_iwt_pyramid(_ptr_array(ys), x.data_ptr(), N, C, H, W, levels, nb, _dtype_code(x),
                                         _stream_ptr(stream)))
@@ -782,7 +796,7 @@ class BoundLayer:
         if workspace.numel() * workspace.element_size() < need:
             raise SsbaError(SSBA_ERR_WORKSPACE, f"workspace needs {need} bytes")
         if isinstance(fwd_workspace, str):
-            fwd_workspace = default_forward_workspace(desc, Q.device, stream) if desc.dtype == torch.bfloat16 else None
+            fwd_workspace = None  # not used by ssba_forward
         fwp, fwn = _ws_args(fwd_workspace)
         if fwp is not None and fwn < forward_workspace_bytes(desc):
             raise SsbaError(SSBA_ERR_WORKSPACE, f"forward workspace needs {forward_workspace_bytes(desc)} bytes")
