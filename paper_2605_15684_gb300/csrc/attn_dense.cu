@@ -186,6 +186,8 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
     volatile int* abortf = &cs.abort_flag;
     const uint32_t abort_at = smem_u32(&cs.abort_flag);
     bool dead = false;
+    uint32_t g = 0;  // key tiles that the role is through with
+    int nq = 0;      // (K producer) units whose Q is announced
 
     if (role == kLoadK || role == kLoadV) {
         // ------------------------------------------------------------ TMA producers
@@ -194,8 +196,6 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
         const uint32_t full0 = smem_u32(is_k ? &ct.k_full[0] : &ct.v_full[0]);
         const uint32_t tile0 = smem_u32(is_k ? &sm.k[0][0] : &sm.v[0][0]);
         const CUtensorMap* map = is_k ? &maps.k : &maps.v;
-        uint32_t g = 0;  // key tiles announced
-        int nq = 0;      // units whose Q is announced
         if (lane == 0) {
             for (int n = 0; n < nunits && !dead; ++n) {
                 const int u = v + n * V, bh = u / p.nt, qt = u - bh * p.nt;
@@ -219,17 +219,10 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                     }
                 }
             }
-            if (dead) {  // drain the copies that may still be in flight
-                for (uint32_t x = g > kStages ? g - kStages : 0; x < g; ++x)
-                    wait_raw(full0 + 8 * (x % kStages), (x / kStages) & 1, p.budget_ns);
-                if (nq > 0) wait_raw(smem_u32(&ct.q_full), (nq - 1) & 1, p.budget_ns);
-            }
         }
         __syncwarp();
     } else if (role == kQK) {
         // ------------------------------------------------------------ QK issuer
-        const bool leader = elect_one_sync();
-        uint32_t g = 0;
         for (int n = 0; n < nunits && !*abortf; ++n) {
             wait_phase(smem_u32(&ct.q_full), n & 1, abort_at, p.budget_ns);
             for (int j = 0; j < p.nt; ++j, ++g) {
@@ -252,14 +245,8 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
             }
         }
         dead = *abortf != 0;
-        if (dead && leader) {
-            mma_commit(smem_u32(&ct.drain[0]));
-            wait_raw(smem_u32(&ct.drain[0]), 0, p.budget_ns);
-        }
     } else if (role == kPV) {
         // ------------------------------------------------------------ PV issuer
-        const bool leader = elect_one_sync();
-        uint32_t g = 0;
         for (int n = 0; n < nunits && !*abortf; ++n)
             for (int j = 0; j < p.nt; ++j, ++g) {
                 const uint32_t st = g % kStages;
@@ -278,17 +265,12 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
                 __syncwarp();
             }
         dead = *abortf != 0;
-        if (dead && leader) {
-            mma_commit(smem_u32(&ct.drain[1]));
-            wait_raw(smem_u32(&ct.drain[1]), 0, p.budget_ns);
-        }
     } else {
         // ------------------------------------------------------------ softmax and output
         const int quad = warp & 3, row = quad * 32 + lane;
         const uint32_t tq = tbase + (static_cast<uint32_t>(quad * 32) << 16);
         const uint32_t scol = tq + kColS, pcol = tq + kColP, ocol = tq + kColO;
         const float c = p.scale_log2;
-        uint32_t g = 0;
         for (int n = 0; n < nunits && !*abortf; ++n) {
             float m_used = 0.f, l = 0.f;
             for (int j = 0; j < p.nt; ++j, ++g) {
@@ -445,7 +427,22 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_dense_tc_kernel(const __grid
         }
         dead = *abortf != 0;
     }
-    if (dead) atomicExch(p.status, SSBA_ERR_TIMEOUT);
+    if (__syncthreads_or(dead)) {
+        // a wait ran out: nothing more is issued, but a role that was done before may have left copies or products in
+        // flight, which the ones that gave up have not waited for
+        if ((role == kLoadK || role == kLoadV) && lane == 0) {
+            const uint32_t full0 = smem_u32(role == kLoadK ? &ct.k_full[0] : &ct.v_full[0]);
+            for (uint32_t x = g > kStages ? g - kStages : 0; x < g; ++x)
+                wait_raw(full0 + 8 * (x % kStages), (x / kStages) & 1, p.budget_ns);
+            if (nq > 0) wait_raw(smem_u32(&ct.q_full), (nq - 1) & 1, p.budget_ns);
+        }
+        if ((role == kQK || role == kPV) && elect_one_sync()) {
+            const uint32_t bar = smem_u32(&ct.drain[role == kPV]);
+            mma_commit(bar);
+            wait_raw(bar, 0, p.budget_ns);
+        }
+        if (threadIdx.x == 0) atomicExch(p.status, SSBA_ERR_TIMEOUT);
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

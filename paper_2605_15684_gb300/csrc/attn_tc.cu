@@ -737,6 +737,8 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
     const int rounds = ct.rounds;
     const uint32_t abort_at = smem_u32(&cs.abort_flag);
     bool dead = false;
+    uint32_t g = 0;  // steps that the role is through with
+    int nq = 0;      // (K producer) rounds whose Q is announced
     if (threadIdx.x == 0) TL_CTA(tl::kPipesStart);
     if (soft && threadIdx.x % (kSoftWarps * 32) == 0) TL_ITEM(slot, 0u, tl::kPipeClock0);
 
@@ -755,8 +757,6 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         const CUtensorMap* mt = is_k ? &maps.kt : &maps.vt;
         // test hook: the first K copies of pipeline 0 never land
         const bool hold = p.withhold == 1 && is_k && vcta == 0;
-        uint32_t g = 0;  // steps announced
-        int nq = 0;      // rounds whose Q is announced
         auto entry_of = [&](int label) { return label < kWinCap ? cs.win[label] : window_entry(p.g, label); };
         for (int r = 0; !dead && r < rounds; ++r) {
             const Round rd = get_round<kSel>(p, ct, r);
@@ -843,13 +843,6 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
                 }
             }
         }
-        if (dead && lane == 0) {
-            // drain: wait for the copies of this warp that may still be in flight
-            for (uint32_t x = g > kStages ? g - kStages : 0; x < g; ++x)
-                wait_raw(full0 + 8 * (x % kStages), (x / kStages) & 1, p.budget_ns);
-            if (nq > 0) wait_raw(smem_u32(&ct.q_full), (nq - 1) & 1, p.budget_ns);
-        }
-        __syncwarp();
     } else if (role == kQK) {
         // ------------------------------------------------------------ QK issuer
         // S_g = [Q_A; Q_B] [K_A; K_B]^T once the softmax holds S_{g-1} in registers (N=64 on the one
@@ -858,9 +851,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         // (measured: 4 MMAs + commit issue in about 280 cycles, against about 480 under a
         // precomputed lane test). elect.sync picks the same lane of a full warp every time, so a
         // commit always follows the MMAs of its own thread.
-        const bool leader = elect_one_sync();
         const uint32_t kbase = smem_u32(&sm.k[0][0]);
-        uint32_t g = 0;
         for (int r = 0; r < rounds && !*abortf; ++r) {
             const Round rd = get_round<kSel>(p, ct, r);
             const int steps = max(rd.nb[0], rd.nb[1]), both = min(rd.nb[0], rd.nb[1]);
@@ -895,18 +886,12 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
             }
         }
         dead = *abortf != 0;
-        if (dead && leader) {
-            mma_commit(smem_u32(&ct.drain[0]));
-            wait_raw(smem_u32(&ct.drain[0]), 0, p.budget_ns);
-        }
     } else if (role == kPV) {
         // ------------------------------------------------------------ PV issuer
         // O_h += P_h V_h of both halves once the softmax has stored P_g and V_g has landed; all PVs
         // of a pipeline are issued by this one thread, so they accumulate into O in order. (One
         // issuer for QK and PV took 2000 cycles a step: its waits and issues do not overlap.)
-        const bool leader = elect_one_sync();
         const uint32_t vbase = smem_u32(&sm.v[0][0]);
-        uint32_t g = 0;
         for (int r = 0; r < rounds && !*abortf; ++r) {
             const Round rd = get_round<kSel>(p, ct, r);
             const int steps = max(rd.nb[0], rd.nb[1]);
@@ -935,10 +920,6 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
             }
         }
         dead = *abortf != 0;
-        if (dead && leader) {
-            mma_commit(smem_u32(&ct.drain[1]));
-            wait_raw(smem_u32(&ct.drain[1]), 0, p.budget_ns);
-        }
     } else if (role == kSoftmax) {
         // ------------------------------------------------------------ softmax and output
         const int quad = gwarp & 3;  // TMEM lane quadrant of this warp
@@ -947,7 +928,6 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         const uint32_t tq = tbase + (static_cast<uint32_t>(quad * 32) << 16);
         const uint32_t scol = tq + kColS + half * 64, ocol = tq + kColO;
         const float c = p.scale_log2;
-        uint32_t g = 0;
         // The last round's item, whose O is written after this round's first exps: its row statistics
         // stay here; its last PV is that of step g - 1.
         bool owed = false;
@@ -1129,7 +1109,22 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
         dead = *abortf != 0;
     }
 
-    if (dead) atomicExch(p.status, SSBA_ERR_TIMEOUT);
+    if (__syncthreads_or(dead)) {
+        // a wait ran out: nothing more is issued, but a role that was done before may have left copies or products in
+        // flight, which the ones that gave up have not waited for
+        if ((role == kLoadK || role == kLoadV) && lane == 0) {
+            const uint32_t full0 = smem_u32(role == kLoadK ? &ct.k_full[0] : &ct.v_full[0]);
+            for (uint32_t x = g > kStages ? g - kStages : 0; x < g; ++x)
+                wait_raw(full0 + 8 * (x % kStages), (x / kStages) & 1, p.budget_ns);
+            if (nq > 0) wait_raw(smem_u32(&ct.q_full), (nq - 1) & 1, p.budget_ns);
+        }
+        if ((role == kQK || role == kPV) && elect_one_sync()) {
+            const uint32_t bar = smem_u32(&ct.drain[role == kPV]);
+            mma_commit(bar);
+            wait_raw(bar, 0, p.budget_ns);
+        }
+        if (threadIdx.x == 0) atomicExch(p.status, SSBA_ERR_TIMEOUT);
+    }
     if (soft && threadIdx.x % (kSoftWarps * 32) == 0) TL_CTA(slot == 0 ? tl::kSlot0End : tl::kSlot1End);
     tc_fence_before();
     __syncthreads();
