@@ -86,9 +86,9 @@ def whole_job_tflops(world: int, flops_per_rank: float, seconds: float) -> float
 
 
 def mask_launches(head_dim: int, Tb: int, blk: int = 8) -> int:
-    """Kernels one ssba_build_mask call launches: the fused build (head_dim 64, 8x8 blocks,
-    at most 256 blocks) is one, the pooling + selection pair is two."""
-    return 1 if (head_dim == 64 and blk == 8 and Tb <= 256) else 2
+    """Kernels one ssba_build_mask call of one image launches: the fused build (head_dim 64, 8x8 blocks, at
+    most 128 blocks a head, 64 above 38 heads) is one, the pooling + selection pair is two."""
+    return 1 if (head_dim == 64 and blk == 8 and Tb <= 128) else 2
 
 
 def kept_flops(B, h, Tb, keep, d, blk=8):

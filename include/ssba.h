@@ -224,7 +224,7 @@ SSBA_API int ssba_forward_select(const ssba_desc* desc, const void* Q, const voi
  * means and lists), affinity, Top-k gating and the sparse attention. Up to 16 query blocks an SM
  * it is one launch: the persistent grid (one CTA per SM) first pools every block of the layer into
  * qb / kb, meets at a grid-wide barrier (bounded wait; a timeout returns through ssba_get_status
- * as SSBA_ERR_TIMEOUT, with O and the lists not written), then runs ssba_forward_select on those
+ * as SSBA_ERR_TIMEOUT, with O not written and the lists undefined), then runs ssba_forward_select on those
  * means. Above, it is ssba_pool_blocks and ssba_forward_select, with no grid-wide wait.
  *   qb, kb      device out, fp32 [B][heads][Tb][head_dim], 16-byte aligned: the block means.
  *   workspace   REQUIRED here, at least ssba_forward_workspace_bytes(desc) bytes: it holds the

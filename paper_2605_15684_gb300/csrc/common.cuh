@@ -103,7 +103,7 @@ int launch_pool_blocks(const ssba_desc& d, const Grid& g, const void* Q, const v
                        cudaStream_t st);
 int launch_select(const ssba_desc& d, const Grid& g, int keep, const float* qb, const float* kb,
                   int32_t* idx, int32_t* cnt, float* scores, cudaStream_t st);
-// Pool + affinity + selection in one launch (head_dim 64, 8x8 blocks, Tb <= 256); returns
+// Pool + affinity + selection in one launch (head_dim 64, 8x8 blocks, Tb <= 128, or 64 with many heads); returns
 // SSBA_ERR_UNSUPPORTED without launching for other shapes.
 int launch_mask_fused(const ssba_desc& d, const Grid& g, int keep, const void* Q, const void* K, int32_t* idx,
                       int32_t* cnt, float* scores, cudaStream_t st);
@@ -125,7 +125,7 @@ int launch_dense_m128(const ssba_desc& d, float scale, const void* Q, const void
                       float* lse, cudaStream_t st);
 int launch_dense_tc_bf16(const ssba_desc& d, float scale, const void* Q, const void* K, const void* V,
                          void* O, float* lse, void* ws, size_t ws_bytes, cudaStream_t st);
-// Bytes of the split-merge workspace of the bf16 forward on the current device.
+// Bytes of the forward workspace on the current device (the grid barrier's counters are its last 256).
 size_t attn_tc_workspace_bytes();
 // Copies out the attention kernel's time stamps (timeline build; else SSBA_ERR_UNSUPPORTED).
 int timeline_read(unsigned long long* cta, unsigned* tile, unsigned* item);

@@ -54,6 +54,6 @@ def test_reference_arm_runs_on_rank_zero_only(capsys):
 
 def test_launch_count_of_the_mask_build():
     assert bench.mask_launches(64, 64) == 1
-    assert bench.mask_launches(64, 256) == 1
-    assert bench.mask_launches(64, 289) == 2
+    assert bench.mask_launches(64, 128) == 1
+    assert bench.mask_launches(64, 256) == 2
     assert bench.mask_launches(128, 64) == 2
