@@ -285,7 +285,7 @@ SSBA_API int ssba_haar_iwt_pyramid(void* const* y, void* x, int32_t N, int32_t C
  *   Q, K, V device out, bf16 [B][heads][N][64] (RoPE applied to Q and K).
  *   qb, kb  device out, fp32 [B][heads][Tb][64]: means of the bf16 Q and K over each block of
  *           the shifted grid (the layout ssba_select_mask reads); both NULL to skip them. Summed
- *           in the projection or by a pooling launch behind it, by shift and size.
+ *           in the projection or by a pooling launch behind it, by heads, grid, shift and size.
  * desc: dtype SSBA_BF16, head_dim 64, block 8, shifts multiples of 4. All device pointers
  * 16-byte aligned. fp32 accumulation. Returns SSBA_ERR_UNSUPPORTED for other shapes. */
 SSBA_API int ssba_qkv_rope_pool(const ssba_desc* desc, const void* X, const void* Wqkv, const float* bias, void* Q,

@@ -25,7 +25,8 @@ __device__ __forceinline__ float key_value(uint32_t u)
 // Kept labels of one row, ascending, with the keys in registers (lane l holds the keys of labels
 // l + 32 m, anything for labels >= Tb): the keep largest under the total order (S descending, label
 // ascending), every path's rule, so the same scores give the same lists.
-//   1. Rows of more than 128 labels: a threshold with exactly keep keys at or above it is looked for
+//   1. kPer of 8 and more (rows of more than 128 labels; where the keys pass through shared memory, more than
+//      64): a threshold with exactly keep keys at or above it is looked for
 //      between the row's smallest and largest value, each guess interpolated from the counts at the
 //      two ends (and halfway where two guesses in a row moved the same end): about five counts for
 //      random scores, a count being one ballot per 32 keys. Where there is one, the kept set is unique
@@ -37,7 +38,7 @@ __device__ __forceinline__ float key_value(uint32_t u)
 //      counts, half of them over exponent bits that every score shares.
 // Selection with the walk alone against both: 510 labels 83 -> 65 us, 256 labels 26 -> 24. With 64
 // labels a count is two ballots and the code costs more than the counts: a 1024 px mask and forward 46.8
-// us with the walk, 49.2 with both.
+// us with the walk, 49.2 with both. (One key a lane: ballot_select<1> below.)
 template <int kPer>
 __device__ __forceinline__ void ballot_select(const uint32_t (&key)[kPer], int Tb, int keep, int lane, int32_t* dst)
 {
