@@ -464,9 +464,7 @@ __device__ __forceinline__ Round get_round(const TcParams& p, const SlotCtl& c, 
         rd.nb[h] = n;
     }
     if (rd.split) {
-        // a list of three or fewer stays with half A: the merge costs more than the step it saves (144
-        // single items of 2 blocks 7.2 -> 7.0 us, of 3 7.7 -> 7.6; of 4, unsplit 8.1 against 7.85)
-        rd.tb[1] = rd.nb[0] < 4 ? rd.nb[0] : (rd.nb[0] + 1) >> 1;
+        rd.tb[1] = (rd.nb[0] + 1) >> 1;
         rd.nb[1] = rd.nb[0] - rd.tb[1];
         rd.nb[0] = rd.tb[1];
     }
@@ -1066,7 +1064,7 @@ __global__ void __launch_bounds__(kThreads, 1) ssba_attn_tc_kernel(const __grid_
                     mbar_arrive(smem_u32(&ct.p_full[g & 1]));
                 }
             }
-            if (split && !parted) {  // a short list: half A has all of it
+            if (split && !parted) {  // one block: half A has all of it
                 split = false;
                 if (half) break;
             }

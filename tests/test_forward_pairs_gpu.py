@@ -166,27 +166,27 @@ def test_dense_first_keys_masked_by_low_scores(low, far):
         assert np.allclose(lse[0, h].cpu().numpy(), (m + np.log(e.sum(axis=1, keepdims=True)))[:, 0], rtol=1e-5, atol=1e-2)
 
 
-@pytest.mark.parametrize("heads", [1, 20])  # 4 items: one a pipeline, its blocks in the two halves; 1280: pairs too
+@pytest.mark.parametrize("heads", [1, 20])  # 4 items: one a pipeline, its two blocks in the two halves; 1280: pairs too
 @pytest.mark.parametrize("low", [0, 1])
 def test_infinite_value_under_a_vanishing_weight(heads, low):
-    """Lists of four blocks, the scores of two (the first or the last) 400 below the others', where exp gives 0, and a
-    column of their V infinite: that column of O is no number (0 x inf), wherever the item runs, and the rest is
-    the other blocks'."""
+    """Lists of two blocks, the scores of one (the `low`-th) 400 below the other's, where exp gives 0, and a column of its
+    V infinite: that column of O is no number (0 x inf), wherever the item runs, and the rest is the other block's."""
     H = W = 16 if heads == 1 else 64
     (_, _, _), (q, k, v) = _inputs(heads, H, W, 46)
-    desc = api.SsbaDesc(1, heads, H, W, rho=0.0 if heads == 1 else 60 / 64)
+    desc = api.SsbaDesc(1, heads, H, W, rho=0.5 if heads == 1 else 62 / 64)
     Tb = desc.Tb
     lab = torch.from_numpy(np.asarray(oracle.partition(H, W, 8, (0, 0)))).long().cuda()
-    far, near = (lab // 2 == low), (lab // 2 == 1 - low)  # the lists hold blocks 0 to 3
+    blocks = (0, 2)
     q[..., 0] = 16.0
-    k[..., 0] = torch.where(far, -200.0, 0.0).bfloat16()
-    v[:, :, far, 5] = float("inf")
-    idx = torch.arange(4, dtype=torch.int32, device="cuda").expand(1, heads, Tb, 4).contiguous()
-    cnt = torch.full((1, heads, Tb), 4, dtype=torch.int32, device="cuda")
+    k[..., 0] = torch.where(lab == blocks[low], -200.0, 0.0).bfloat16()
+    v[:, :, lab == blocks[low], 5] = float("inf")
+    idx = torch.tensor(blocks, dtype=torch.int32, device="cuda").expand(1, heads, Tb, 2).contiguous()
+    cnt = torch.full((1, heads, Tb), 2, dtype=torch.int32, device="cuda")
     O, lse = api.forward(desc, q, k, v, idx, cnt)
     torch.cuda.synchronize()
     assert not bool(torch.isfinite(O[..., 5]).any())
-    s = q.float() @ k[:, :, near].float().transpose(-1, -2) / 8
-    want, rest = torch.softmax(s, -1) @ v[:, :, near].float(), torch.arange(64, device="cuda") != 5
+    kk, vv = (t[:, :, lab == blocks[1 - low]].float() for t in (k, v))
+    s = q.float() @ kk.transpose(-1, -2) / 8
+    want, rest = torch.softmax(s, -1) @ vv, torch.arange(64, device="cuda") != 5
     assert float((O.float() - want)[..., rest].abs().max()) <= 2e-2  # the bf16 bound of tests/parity.py
     assert float((lse - torch.logsumexp(s, -1)).abs().max()) <= 1e-2
