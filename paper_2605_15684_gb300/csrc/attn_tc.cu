@@ -19,10 +19,10 @@
 // tensor pipe is busy 2 x 608 (QK 4 x 80, PV 8 x 36) and the softmax needs 2 x 435 of its scheduler;
 // the rest is hand-offs (mbarrier waits, tensor-memory round trips) that two chains do not quite
 // cover. Forward on given lists, 24 heads, GPU time in a graph of distinct layers, against the kernel with one
-// 64-row tile per product: 4K (128 of 510 blocks) 2395 -> 1800 us, 2048 px (41 of 256) 400 -> 324, four 1024
-// px images (16 of 64) 171 -> 152, one (11 of 64) 39.4 -> 36.5, 512 px (3 of 16) 10.6 -> 9.7. Where there is
-// about one block for each of the 304 pipelines and a list is short, the longer step shows: 288 blocks of 3
-// 8.1 -> 8.4 us.
+// 64-row tile per product: 4K (128 of 510 blocks) 2400 -> 1770 us, 2048 px (41 of 256) 400 -> 319, four 1024
+// px images (16 of 64) 171 -> 150, one (11 of 64) 39.1 -> 35.8, 512 px (3 of 16) 10.6 -> 10.2. Where there is
+// about one block for each of the 304 pipelines and a list is short, the longer step and the merge show: 288
+// blocks of 3 8.1 -> 8.5 us.
 // Persistent CTAs, one per SM (its 226 KB of shared memory fills the SM), each running two
 // independent pipelines of 8 warps (512 threads, 128 registers each), warp-specialised:
 //   K producer  (TMA, one lane). Q of each item and K, V of each listed key block arrive as 8 KB tiles
@@ -1160,7 +1160,7 @@ namespace {
 // layer, four 1024 px images (40) 187 -> 176; at one 1024 px image (10) the single launch is (48.2
 // against 49.3 us). ssba_build_mask and ssba_forward are two launches (the mask kernel, which pools without a
 // grid barrier but does not write the means that these calls return): 24 heads, one launch and those two,
-// 256 px 12.1, 9.1 us, 512 px 15.5, 13.6, 1024 px 47.1, 46.6.
+// 256 px 12.0, 9.2 us, 512 px 16.0, 14.4, 1024 px 47.0, 46.9.
 constexpr int kSelItems = 16;
 int max_grid() { return num_sms(); }
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
